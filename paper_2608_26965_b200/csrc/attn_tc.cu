@@ -2,36 +2,56 @@
 // cores (eq. 2 over the selected clusters; Appendix A: an excluded cluster
 // enters through its centroid key/value with weight |c| exp(q . kbar / sqrt(d))).
 //
-// One CTA per tile of 128 query rows (one query cluster, half of a 256-row one,
-// or a 64-row one in a half-filled tile).  Per CTA the half-steps of 64 keys form
-// one dependent chain, so what counts is the number of chains per SM: at d = 64 a
-// CTA holds one 64-column score buffer and 64 output columns in tensor memory and
-// four CTAs share an SM; at d = 128 two score buffers and 128 output columns, two
-// CTAs per SM (TcCfg).  Key and value rows stream through shared memory by TMA in
-// slots of 64 rows (128-byte swizzle, 64-column panels), loaded in the order the
-// tensor core consumes them:
-//     S_b = Q K_h^T        tcgen05.mma, Q and K from shared memory (K-major)
-//     P_b = exp2(S_b c - m) four softmax warps, one query row per thread; P is
-//                          written back over S_b as packed bf16; row sums in fp32
-//                          registers
-//     O  += P_b V_h        tcgen05.mma, P from tensor memory, V from shared memory (MN-major)
-// issued as S(0) [S(1)] | PV(0) S(NBUF) | PV(1) S(NBUF + 1) | ...  The softmax keeps
-// a reference m per row instead of the exact running maximum: it is measured on a
-// row's first half-step, afterwards gathered with the exponentials and raised one
-// half-step late (by an integer, when a half-step exceeded it by 2^8), the softmax
-// warps then rescale O in tensor memory themselves after waiting for the one
-// product that can still be in flight; a climb beyond 2^96 inside one half-step
-// marks the tile for the second pass of the fp32 kernel.  After the selected
-// clusters the key centroids are streamed as extra keys, 64 per half-step: their
-// tile holds bf16 hi parts in rows 0-63 and lo parts in rows 64-127, accumulated
-// by two products so the centroid logits keep fp32-level accuracy; logit bias
-// ln|c|, selected clusters masked; values are the value centroids.  Block lists
-// may be ragged (a length per query cluster).  Warp 0 issues TMA, warp 1 issues
-// MMAs (all lanes run the loop, one elected lane issues), warps 2-5 do the softmax
-// and the epilogue (rows scattered back to the original order).
+// Persistent CTAs, one per SM, each walking over tiles of 128 query rows (one query
+// cluster, half of a 256-row one, or a 64-row one).  Keys are
+// consumed in steps of 128:
+//     S   = Q K_s^T        tcgen05.mma, Q and K from shared memory (K-major)
+//     P   = exp2(S c - m)  one query row per thread; P is written back over S as
+//                          packed bf16; row sums in fp32 registers
+//     O  += P V_s          tcgen05.mma, P from tensor memory, V from shared memory (MN-major)
+// A softmax warp needs about twice the time of its exponentials for a step (latencies of
+// tensor-memory loads, barriers, conversions), so the steps go round three groups of
+// four softmax warps, each with a score buffer of its own (3 x 128 + D columns of
+// tensor memory), and the tensor core works up to three steps ahead: neither the
+// products nor the hand-offs between the units are on a softmax warp's path.  Roles:
+// warp 0 loads Q and K, warp 3 V (TMA, 128-byte swizzle, 64-column panels), warp 1
+// issues all products, warp 2 walks over tiles and block lists and writes a descriptor
+// per step (rows to load, masks, additive terms) into a ring, warps 4-15 are the
+// softmax groups.  The roles run ahead of one another across tiles, so that the start
+// of a tile hides behind the end of the one before.
+// The rows of a 64-row query cluster are loaded twice, into both halves of a tile: the
+// upper half takes keys 0-63 of every step and the lower half keys 64-127 (the other
+// probabilities of a row are stored as zeros), so that all four softmax warps of a group
+// work and each on half of the columns; the two halves are independent rows with sums,
+// references and outputs of their own, merged at the end of the tile.
+// All roles run at the same time on one SM and have to fit its instruction cache
+// together: with the loops of the single-warp roles unrolled (105 KB of code) the same
+// kernel took 1.40 ms where it now takes 0.73 (2 x 16 heads of 20,000 rows, d = 128, 10
+// clusters of 256 kept), so loops stay rolled unless a step is shorter for it.
+// What bounds it: at d = 128 every step brings 64 KB through L2, which delivers 43 bytes
+// per cycle and SM (1,520 cycles; a step takes 1,850), since the lists of two query
+// clusters share nothing; at d = 64 the exponentials (1,024 of 1,340 cycles per step)
+// and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
+// four at d = 64, half-steps of 64 keys in one chain per CTA): 40 heads of 32,760 rows,
+// d = 128, 32 of 256 clusters kept 2.91 -> 2.44 ms; 8 heads of 16,384 x 131,072, d = 64,
+// 128 of 1,024 kept 0.88 -> 0.82; 12 heads of 16,385 in clusters of 64 0.373 -> 0.356.
+//
+// The softmax keeps a reference m per row instead of the exact running maximum: it is
+// measured on a row's first step and raised (by an integer) when a sum of 32
+// probabilities exceeded 2^32, at the group's next step; the reference of every step is
+// handed from group to group through shared memory, and the group that raises it
+// rescales O in tensor memory itself.  A climb beyond 2^96 inside the steps in
+// flight marks the tile for the second pass of the fp32 kernel.
+// After the selected clusters the key centroids are streamed as extra keys, 64 per
+// step: their tile holds bf16 hi parts in rows 0-63 and lo parts in rows 64-127, whose
+// scores are added when they are read, with an additive term ln|c|, selected clusters
+// masked; values are the value centroids.  Block lists may be ragged (a length per
+// query cluster); tiles are handed out by a counter.
 // Indices that come from the caller (block lists, list lengths, perm_q) are range-
 // checked before use: a bad one sets CA_ERR_BAD_INDEX in the status word and the
 // access is skipped (the cluster is masked, the row is not written).
+#include <type_traits>
+
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
@@ -39,11 +59,25 @@ namespace ca {
 
 using namespace ptx;
 
-constexpr int kTcThreads = 192;
-constexpr int kTile = 128;                 // query rows per CTA, key rows per tile
-constexpr int kHalf = 64;                  // keys per half-step
-constexpr float kRescaleThreshold = 8.0f;  // log2 units
-constexpr float kDanger = 96.0f;            // log2 units: exp2 arguments stay below this
+constexpr int kGroups = 3;                 // softmax groups of 128 threads, score buffers
+constexpr int kTcThreads = 128 + kGroups * 128;
+constexpr int kTile = 128;                 // query rows per tile, key rows per step
+constexpr int kCen = 64;                   // key centroids per step
+constexpr int kRing = 8;                   // step descriptors in flight
+constexpr int kParts = 6;                  // steps s - 2 .. s + 3 can have row sums on their way while step s ends a tile
+constexpr int kMergeInts = 18;             // row pitch of the hand-over between the halves of a 64-row query cluster
+// first rows of a step's boxes (key clusters of 16 rows: eight boxes), of its value centroids, of Q
+constexpr int kRowCenV = 8, kRowQ = 9, kRowInts = 12;
+// A reference is raised when a sum of 32 probabilities exceeds 2^32: P is bf16, O and l are fp32, so
+// probabilities far above 1 cost no precision, and the climbs that remain below the limit
+// (nearly all) need no rescaling of O, which stalls all three groups for some 2,000 cycles.
+constexpr float kRescaleThreshold = 32.0f;  // log2 units
+constexpr float kSumLimit = 4294967296.0f;  // 2^kRescaleThreshold
+constexpr float kDangerSum = 7.9228163e28f;  // 2^96
+
+// flags of a step descriptor
+constexpr int kFMasked = 1, kFCentroid = 2, kFFirst = 4, kFLast = 8, kFStop = 16;
+constexpr int kFIndexShift = 8, kFRestShift = 12;   // min(15, index in the tile), min(15, steps after it)
 
 // F8: queries, keys and key centroids arrive as E4M3 codes (one byte per element: a 128-byte row
 // of a panel holds 128 of them) and Q K^T runs as kind::f8f6f4 products; values stay bf16.
@@ -53,46 +87,29 @@ struct TcCfg {
   static constexpr int QK_PANELS = F8 ? D / 128 : D / 64;    // query / key panels
   static constexpr int QK_PANEL_COLS = F8 ? 128 : 64;        // elements per panel row
   static constexpr int QK_KSTEP = F8 ? 32 : 16;              // elements per tensor-core instruction (32 bytes)
-  static constexpr int PANEL_BYTES = kTile * 128;            // query tile: 128 rows x 128 bytes per panel
-  static constexpr int TILE_BYTES = QK_PANELS * PANEL_BYTES;
-  static constexpr int HALF_PANEL_BYTES = kHalf * 128;       // key/value slot: 64 rows x 128 bytes per panel
-  static constexpr int HALF_BYTES = PANELS * HALF_PANEL_BYTES;        // a value slot
-  static constexpr int KHALF_BYTES = QK_PANELS * HALF_PANEL_BYTES;    // a key slot
-  static constexpr int CEN_PARTS = F8 ? 1 : 2;               // key slots of a centroid half-step (bf16: hi and lo parts)
-  // Per CTA the half-steps form one dependent chain (scores -> softmax -> P V -> next scores) whose
-  // length is set by latencies, not by any pipe, and an SM has throughput to spare: what counts is
-  // the number of such chains per SM.  d = 64: one 64-column score buffer + 64 output columns =
-  // 128 columns of tensor memory and 48 KB of shared memory per CTA, four CTAs per SM.  d = 128: the
-  // output alone takes 128 columns; two score buffers, 256 columns, two CTAs per SM.
-  static constexpr int NBUF = (D == 64) ? 1 : 2;
-  static constexpr int NBAR = 2;                              // barrier rings (>= every lead below)
-  static constexpr uint32_t TMEM_COLS = (D == 64) ? 128 : 256;
-  static constexpr int CTAS_PER_SM = (D == 64) ? 4 : 2;
-  // key and value slots of 64 rows (one half-step each; a centroid half-step takes two key slots).
-  // The keys of half-step i are loaded once S(i - K_LEAD) has completed, so the slots of at most
-  // K_LEAD half-steps are live (K_LEAD_CEN for centroid half-steps); likewise for the values.
-  static constexpr int NK = 2;
-  static constexpr int NV = 2;
-  static constexpr int K_LEAD = 2;
-  static constexpr int K_LEAD_CEN = 1;
-  static constexpr int PV_N = D;
-  // How the softmax notices a probability above 2^threshold.  d = 128: it keeps the largest
-  // exponent of the half-step.  d = 64: no exponent is tracked; such a probability shows in its
-  // chunk's row sum, and the sum bounds it from above, so the reference moves up by the sum's
-  // exponent (too far by at most log2(32), which costs nothing in fp32 / bf16).  Measured: d = 64
-  // 0.916 -> 0.895 ms without the tracking, d = 128 2.90 -> 2.95 ms.
-  static constexpr bool TRACK_MAX = D != 64;
-  static constexpr bool Q_IN_TMEM = false;
-  static constexpr int TMEM_Q = 0;
+  static constexpr int PANEL_BYTES = kTile * 128;            // 128 rows x 128 bytes
+  static constexpr int QK_BYTES = QK_PANELS * PANEL_BYTES;   // a query tile, a key tile
+  static constexpr int V_BYTES = PANELS * PANEL_BYTES;       // a value tile
+  static constexpr uint32_t TMEM_COLS = 512;                 // kGroups x 128 score columns (P over 64 of them), D of O
+  static constexpr int NK = kGroups;                         // key tiles in shared memory: one per score buffer
+  static constexpr int NV = (D == 64 || F8) ? 3 : 2;         // value tiles
   // shared memory layout (offsets from a 1024-byte aligned base)
   static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + TILE_BYTES;
-  static constexpr int OFF_V = OFF_K + NK * KHALF_BYTES;
-  static constexpr int OFF_BIAS = OFF_V + NV * HALF_BYTES;                     // 8 x 64 floats
-  static constexpr int OFF_BAR = OFF_BIAS + 8 * kHalf * 4;
-  static constexpr int NUM_BARS = 3 + 3 * NBAR + NK + NV;           // q_full, o_done, q_tmem, three rings, per slot
-  static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;           // tmem base, abort flag
-  static constexpr int OFF_BITMAP = OFF_MISC + 16;
+  static constexpr int OFF_K = OFF_Q + QK_BYTES;
+  static constexpr int OFF_V = OFF_K + NK * QK_BYTES;
+  static constexpr int OFF_BIAS = OFF_V + NV * V_BYTES;                  // [kRing][128] floats
+  static constexpr int OFF_LPART = OFF_BIAS + kRing * kTile * 4;         // [kParts steps][128 rows] {row sum, reference}
+  static constexpr int OFF_MERGE = OFF_LPART + kParts * kTile * 8;       // [64 rows][kMergeInts] 16 columns of O, sum, reference
+  static constexpr int OFF_REF = OFF_MERGE + 64 * kMergeInts * 4;        // [128 rows] {reference, step}
+  static constexpr int OFF_ROWS = OFF_REF + kTile * 8;                   // [kRing][kRowInts]
+  static constexpr int OFF_TILE = OFF_ROWS + kRing * kRowInts * 4;       // [kRing] head, first position, redo word, tile
+  static constexpr int OFF_FLAGS = OFF_TILE + kRing * 16;
+  static constexpr int OFF_SCALE = OFF_FLAGS + kRing * 4;                // [kRing][2] scales of the keys (F8)
+  static constexpr int OFF_BAR = OFF_SCALE + kRing * 8;
+  static constexpr int NUM_BARS = 2 + 4 + 2 * kGroups + 2 * kRing + NK + 2 * NV + 4;
+  static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;                // tmem base, abort flag, redo counts x 4
+  static constexpr int OFF_BITMAP = OFF_MISC + 32;
+  static_assert(OFF_TILE % 16 == 0 && OFF_BAR % 8 == 0 && OFF_MISC % 8 == 0, "alignment");
 };
 
 struct TcParams {
@@ -103,8 +120,9 @@ struct TcParams {
   __nv_bfloat16* O;
   float* lse;
   int* status;
-  int32_t* redo;                  // [B*H, n_qc, 2] per CTA: scores left the range of the fast softmax
-  int n_q, n_k, c_q, c_k, keep, list_stride, n_qc, n_kc, cen_tiles, compensate, bitmap_words;
+  int* next_tile;                 // counter that hands out tiles, zero at the start
+  int32_t* redo;                  // [B*H, n_qc, 2] per tile: scores left the range of the fast softmax
+  int n_q, n_k, c_q, c_k, keep, list_stride, n_qc, n_kc, cen_tiles, compensate, bitmap_words, n_tiles;
   float scale_log2;
   // quantised Q K^T: de-quantisation scales of the query rows [B*H*n_qc*c_q], of the key clusters
   // [B*H*n_kc] and of the runs of 64 key centroids [B*H*cen_tiles]; null otherwise
@@ -122,8 +140,12 @@ __host__ __device__ inline int selected_tiles(int keep, int c_k) {
   return c_k >= kTile ? keep * (c_k / kTile) : (keep * c_k + kTile - 1) / kTile;
 }
 
+// A value that all lanes of a (converged) warp hold, made known as such to the compiler: branches on it
+// and addresses from it stay in the uniform datapath.
+__device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 template <int D, bool F8>
-__global__ void __launch_bounds__(kTcThreads, TcCfg<D, F8>::CTAS_PER_SM)
+__global__ void __launch_bounds__(kTcThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ck,
                const __grid_constant__ CUtensorMap tm_cv, const TcParams prm) {
@@ -134,60 +156,54 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const uint32_t s_base = smem_u32(smem);
   const uint32_t s_q = s_base + C::OFF_Q, s_k = s_base + C::OFF_K, s_v = s_base + C::OFF_V;
   float* bias = reinterpret_cast<float*>(smem + C::OFF_BIAS);
+  float2* lpart = reinterpret_cast<float2*>(smem + C::OFF_LPART);
+  const uint32_t s_ref = s_base + C::OFF_REF;
+  int* st_rows = reinterpret_cast<int*>(smem + C::OFF_ROWS);
+  int4* st_tile = reinterpret_cast<int4*>(smem + C::OFF_TILE);
+  int* st_flags = reinterpret_cast<int*>(smem + C::OFF_FLAGS);
+  float* st_scale = reinterpret_cast<float*>(smem + C::OFF_SCALE);
   const uint32_t bar0 = s_base + C::OFF_BAR;
-  const uint32_t b_q_full = bar0, b_o_done = bar0 + 8, b_q_tmem = bar0 + 16;
-  auto b_s_full = [&](int b) { return bar0 + 24 + 8 * b; };
-  auto b_p_ready = [&](int b) { return bar0 + 24 + 8 * (C::NBAR + b); };
-  auto b_pv_done = [&](int b) { return bar0 + 24 + 8 * (2 * C::NBAR + b); };
-  auto b_k_full = [&](int s) { return bar0 + 24 + 8 * (3 * C::NBAR + s); };
-  auto b_v_full = [&](int s) { return bar0 + 24 + 8 * (3 * C::NBAR + C::NK + s); };
+  const uint32_t b_q_empty = bar0, b_o_empty = bar0 + 8;
+  // O of tile t is complete.  With tiles of one step three groups wait for three tiles at a time: a
+  // barrier for each, so that no parity stands for two of them.
+  auto b_o_full = [&](int t) { return bar0 + 16 + 8 * (t & 3); };
+  const uint32_t bar1 = bar0 + 48;
+  auto b_s_full = [&](int b) { return bar1 + 8 * b; };
+  auto b_p_ready = [&](int b) { return bar1 + 8 * (kGroups + b); };
+  auto b_step_full = [&](int s) { return bar1 + 8 * (2 * kGroups + s); };
+  auto b_step_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + kRing + s); };
+  auto b_k_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + s); };
+  auto b_v_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + s); };
+  auto b_v_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + C::NV + s); };
+  auto b_m_full = [&](int w) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + 2 * C::NV + w); };
+  auto b_m_empty = [&](int w) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + 2 * C::NV + 2 + w); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
-  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 8);
+  int* redo_acc = reinterpret_cast<int*>(smem + C::OFF_MISC + 8);
   unsigned* bitmap = reinterpret_cast<unsigned*>(smem + C::OFF_BITMAP);
-  // member counts of the selected clusters, in list order: looked up every half-step, so they are
-  // fetched from global memory once instead of sitting on each half-step's critical path
-  uint16_t* members_of = reinterpret_cast<uint16_t*>(bitmap + prm.bitmap_words);
-  // quantised Q K^T: de-quantisation scale of every selected key cluster, in list order
-  float* kscale_of = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(members_of) +
-                                              (((size_t)prm.list_stride * 2 + 15) & ~(size_t)15));
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int p = blockIdx.y;
-  // a query cluster of 256 rows takes two CTAs; one of 64 rows fills the upper half of a tile
-  // (the lower half is zeros and the warps that own those rows only keep the barriers going)
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
+  // a query cluster of 256 rows takes two tiles; one of 64 rows is loaded into both halves of one
   const int tiles_per_qc = prm.c_q >= kTile ? prm.c_q / kTile : 1;
-  const int q_rows = prm.c_q >= kTile ? kTile : prm.c_q;
-  const int qc = blockIdx.x / tiles_per_qc, half = blockIdx.x % tiles_per_qc;
-  const int32_t* sel = prm.block_idx + ((size_t)p * prm.n_qc + qc) * prm.list_stride;
-  int keep = prm.keep_count ? prm.keep_count[(size_t)p * prm.n_qc + qc] : prm.keep;
-  if (keep < 0 || keep > prm.list_stride) {            // a list length that does not fit its row
-    if (tid == 0) atomicCAS(prm.status, 0, kErrBadIndex);
-    keep = keep < 0 ? 0 : prm.list_stride;
-  }
-  const int sel_tiles = selected_tiles(keep, prm.c_k);
-  const int cen_tiles = prm.compensate ? prm.cen_tiles : 0;
-  const int steps = 2 * sel_tiles + cen_tiles;         // half-steps of 64 keys
+  const bool twice = prm.c_q < kTile;
 
   if (tid == 0) {
-    mbar_init(b_q_full, 1);
-    mbar_init(b_q_tmem, 4);
-    mbar_init(b_o_done, 1);
-    for (int b = 0; b < C::NBAR; ++b) { mbar_init(b_s_full(b), 1); mbar_init(b_p_ready(b), 4); mbar_init(b_pv_done(b), 1); }
+    mbar_init(b_q_empty, 1); mbar_init(b_o_empty, 4);
+#pragma unroll 1
+    for (int b = 0; b < kGroups; ++b) { mbar_init(b_s_full(b), 1); mbar_init(b_p_ready(b), 4); }
+#pragma unroll 1
+    for (int s = 0; s < kRing; ++s) { mbar_init(b_step_full(s), 1); mbar_init(b_step_empty(s), 6); }
+#pragma unroll 1
     for (int s = 0; s < C::NK; ++s) mbar_init(b_k_full(s), 1);
-    for (int s = 0; s < C::NV; ++s) mbar_init(b_v_full(s), 1);
+#pragma unroll 1
+    for (int s = 0; s < C::NV; ++s) { mbar_init(b_v_full(s), 1); mbar_init(b_v_empty(s), 1); }
+#pragma unroll 1
+    for (int w = 0; w < 4; ++w) { mbar_init(b_m_full(w), 1); mbar_init(b_o_full(w), 1); }
     *abort_flag = 0;
-    *redo_flag = 0;
+    for (int b = 0; b < 4; ++b) redo_acc[b] = 0;
     fence_mbar_init();
   }
-  if (q_rows < kTile) {
-    // rows [q_rows, 128) of every Q panel: zeros (read by the tensor core through the async proxy)
-    for (int e = tid; e < C::QK_PANELS * (kTile - q_rows) * 8; e += kTcThreads) {
-      const int pn = e / ((kTile - q_rows) * 8), rem = e % ((kTile - q_rows) * 8);
-      *reinterpret_cast<uint4*>(smem + C::OFF_Q + pn * C::PANEL_BYTES + q_rows * 128 + rem * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    fence_proxy_async();
-  }
+  if (tid < kTile) reinterpret_cast<int2*>(smem + C::OFF_REF)[tid] = make_int2(0, -1);
   if (warp == 1) {                       // this warp owns the TMEM allocation
     tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
     tmem_relinquish();
@@ -195,307 +211,410 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + C::NBUF * kHalf;
-  // key slots used before half-step u (a centroid half-step takes two: hi and lo parts)
-  auto kslot_of = [&](int u) { return u < 2 * sel_tiles ? u : 2 * sel_tiles + C::CEN_PARTS * (u - 2 * sel_tiles); };
+  const uint32_t tmem_base = warp_uniform(*tmem_slot);
+  const uint32_t tmem_o = tmem_base + kGroups * kTile;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    // Loads run in the order the tensor core consumes them: the keys of half-step i (needed by
-    // S(i), issued NBUF half-steps early) and the values of half-step i - NBUF.  A slot is free
-    // again when the product that read it has completed, which is what the barriers s_full and
-    // pv_done of that half-step announce; no separate "empty" barriers or commits.
-    if (lane == 0) {
-      prefetch_tensormap(&tm_q); prefetch_tensormap(&tm_k); prefetch_tensormap(&tm_v);
-      const int q_row = (p * prm.n_qc + qc) * prm.c_q + half * kTile;
-      mbar_expect_tx(b_q_full, C::QK_PANELS * q_rows * 128);
-      for (int pn = 0; pn < C::QK_PANELS; ++pn)
-        tma_load_2d(s_q + pn * C::PANEL_BYTES, &tm_q, pn * C::QK_PANEL_COLS, q_row, b_q_full);
-      bool ok = true;
-      // `key`: rows of keys or key centroids (their panels), otherwise rows of values
-      auto load_rows = [&](uint32_t dst, const CUtensorMap* map, int row, uint32_t bar, bool key) {
-        const int panels = key ? C::QK_PANELS : C::PANELS, cols = key ? C::QK_PANEL_COLS : 64;
-        for (int pn = 0; pn < panels; ++pn) tma_load_2d(dst + pn * C::HALF_PANEL_BYTES, map, pn * cols, row, bar);
-      };
-      // the 64 rows of half-step u of the selected clusters: one box, or several boxes of c_k rows
-      auto load_selected = [&](uint32_t dst, const CUtensorMap* map, int u, uint32_t bar, bool key) {
-        if (prm.c_k >= kHalf) {
-          const int pos = u * kHalf;                       // position in the concatenated selected rows
-          int j = sel[min(pos / prm.c_k, keep - 1)];     // a filler half-step repeats the last cluster (masked)
-          j = min(max(j, 0), prm.n_kc - 1);                // out-of-range entries are flagged and masked by the softmax warps
-          load_rows(dst, map, (p * prm.n_kc + j) * prm.c_k + pos % prm.c_k, bar, key);
-        } else {
-          const int per = kHalf / prm.c_k;
-          for (int x = 0; x < per; ++x) {
-            int e = u * per + x;
-            if (e >= keep) e = keep - 1;                   // filler rows, masked by the softmax
-            const int j = min(max(sel[e], 0), prm.n_kc - 1);
-            const int panels = key ? C::QK_PANELS : C::PANELS, cols = key ? C::QK_PANEL_COLS : 64;
-            for (int pn = 0; pn < panels; ++pn)
-              tma_load_2d(dst + pn * C::HALF_PANEL_BYTES + x * prm.c_k * 128, map, pn * cols,
-                          (p * prm.n_kc + j) * prm.c_k, bar);
+  if (warp < 4) {
+    auto relaxed = [&](uint32_t bar, uint32_t phase) {
+      return mbar_wait_relaxed(bar, phase & 1, abort_flag, prm.status, prm.wait_limit);
+    };
+    if (warp == 0 || warp == 3) {
+      // ---------------------------------------------------------- TMA producers: Q and K, V
+      if (lane == 0) {
+        prefetch_tensormap(warp == 0 ? &tm_q : &tm_v);
+        prefetch_tensormap(warp == 0 ? &tm_k : &tm_cv);
+        const int boxes = prm.c_k >= kTile ? 1 : kTile / prm.c_k;
+        auto produce = [&](auto is_key) {
+          constexpr bool key = decltype(is_key)::value;
+          constexpr int panels = key ? C::QK_PANELS : C::PANELS, cols = key ? C::QK_PANEL_COLS : 64;
+          constexpr int slots = key ? C::NK : C::NV, bytes = key ? C::QK_BYTES : C::V_BYTES;
+          static_assert(!key || slots == kGroups, "a key slot goes with a score buffer");
+          int tiles = 0, stops = 0;
+          int ring = 0, slot = 0;               // of step i
+          uint32_t ph_ring = 0, ph_slot = 1;    // of its descriptor; of the product that read the slot before
+#pragma unroll 1
+          for (int i = 0;; ++i) {
+            if (!relaxed(b_step_full(ring), ph_ring)) return;
+            const int fl = st_flags[ring];
+            const int* rows = st_rows + ring * kRowInts;
+            // A slot is free when the product that read it has completed: for keys the scores of step
+            // i - slots, whose barrier takes its next phase behind this load.
+            if (i >= slots && !relaxed(key ? b_s_full(slot) : b_v_empty(slot), ph_slot)) return;
+            const uint32_t dst = (key ? s_k : s_v) + slot * bytes, bar = key ? b_k_full(slot) : b_v_full(slot);
+            if (fl & kFStop) {                             // passed on to the issuer
+              if (!key) return;
+              mbar_arrive(bar);
+              if (++stops == kGroups) return;
+            } else {
+              if (key && (fl & kFFirst)) {
+                if (tiles > 0 && !relaxed(b_q_empty, tiles - 1)) return;
+                ++tiles;
+                mbar_expect_more(bar, C::QK_BYTES);           // Q arrives with the tile's first keys
+#pragma unroll 1
+                for (int half = 0; half <= (twice ? 1 : 0); ++half)
+#pragma unroll
+                  for (int pn = 0; pn < C::QK_PANELS; ++pn)
+                    tma_load_2d(s_q + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ], bar);
+              }
+              if (!(fl & kFCentroid)) {
+                // 128 rows: one box, or several boxes of c_k rows
+                if (!key || i != (prm.skip_key_load >> 1)) {     // diagnostic: this slot never fills, its waiters time out
+                  mbar_expect_tx(bar, bytes);
+#pragma unroll 1
+                  for (int x = 0; x < boxes; ++x)
+#pragma unroll
+                    for (int pn = 0; pn < panels; ++pn)
+                      tma_load_2d(dst + pn * C::PANEL_BYTES + x * prm.c_k * 128, key ? &tm_k : &tm_v, pn * cols, rows[x], bar);
+                }
+              } else {
+                // keys as bf16: 64 rows of hi parts and 64 rows of lo parts; as codes, and values: 64 rows
+                mbar_expect_tx(bar, panels * ((key && !F8) ? kTile : kCen) * 128);
+#pragma unroll
+                for (int pn = 0; pn < panels; ++pn)
+                  tma_load_2d(dst + pn * C::PANEL_BYTES, key ? &tm_ck : &tm_cv, pn * cols, rows[key ? 0 : kRowCenV], bar);
+              }
+              mbar_arrive(b_step_empty(ring));
+            }
+            if (++slot == slots) { slot = 0; ph_slot ^= 1; }
+            if (++ring == kRing) { ring = 0; ph_ring ^= 1; }
           }
-        }
-      };
-      // A slot is reused when the product that read it has completed.  Products complete in the
-      // order of their issue, so it is enough to wait for a later one; the one waited for is chosen
-      // so that its barrier cannot complete another phase before this thread has looked (the next
-      // product on the same score buffer needs the very load that follows the wait).
-      for (int i = 0; i < steps + C::NBUF && ok; ++i) {
-        if (i < steps) {
-          const bool centroid = i >= 2 * sel_tiles;
-          const int parts = centroid ? C::CEN_PARTS : 1;
-          const int w = i - (centroid ? C::K_LEAD_CEN : C::K_LEAD);
-          if (w >= 0) ok = mbar_wait_relaxed(b_s_full(w % C::NBAR), (w / C::NBAR) & 1, abort_flag, prm.status, prm.wait_limit);
-          for (int g = 0; g < parts && ok; ++g) {
-            const int kc = kslot_of(i) + g, slot = kc % C::NK;
-            if (i == prm.skip_key_load) continue;          // diagnostic: this slot never fills, its waiters time out
-            mbar_expect_tx(b_k_full(slot), C::KHALF_BYTES);
-            const uint32_t dst = s_k + slot * C::KHALF_BYTES;
-            if (!centroid) load_selected(dst, &tm_k, i, b_k_full(slot), true);
-            else load_rows(dst, &tm_ck, (p * prm.cen_tiles + (i - 2 * sel_tiles)) * (C::CEN_PARTS * kHalf) + g * kHalf,
-                           b_k_full(slot), true);
-          }
-        }
-        const int j = i - C::NBUF;
-        if (j >= 0 && ok) {
-          const int slot = j % C::NV;
-          const int w = j - C::NV;
-          if (w >= 0) ok = mbar_wait_relaxed(b_pv_done(w % C::NBAR), (w / C::NBAR) & 1, abort_flag, prm.status, prm.wait_limit);
-          if (!ok) break;
-          mbar_expect_tx(b_v_full(slot), C::HALF_BYTES);
-          const uint32_t dst = s_v + slot * C::HALF_BYTES;
-          if (j < 2 * sel_tiles) load_selected(dst, &tm_v, j, b_v_full(slot), false);
-          else load_rows(dst, &tm_cv, (p * prm.cen_tiles + (j - 2 * sel_tiles)) * kHalf, b_v_full(slot), false);
-        }
+        };
+        if (warp == 0) produce(std::true_type{});
+        else produce(std::false_type{});
       }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    // every lane runs the loop (waits and descriptor arithmetic stay warp-uniform); one elected
-    // lane issues the tensor-core instructions
-    {
-      constexpr uint32_t idesc_qk = F8 ? idesc_e4m3_f32(kTile, kHalf) : idesc_bf16_f32(kTile, kHalf, 0, 0);
-      constexpr uint32_t idesc_pv = idesc_bf16_f32(kTile, C::PV_N, 0, 1);
-      bool ok = __all_sync(0xffffffffu, mbar_wait(b_q_full, 0, abort_flag, prm.status, prm.wait_limit));
+    } else if (warp == 1) {
+      // ---------------------------------------------------------- MMA issuer
+      // Every lane runs the loop (descriptor arithmetic stays warp-uniform); one elected lane issues
+      // the tensor-core instructions.  A wait on a barrier that has completed costs some 130
+      // cycles, so everything a step needs is waited for at once, one barrier per lane.
+      constexpr uint32_t idesc_qk = F8 ? idesc_e4m3_f32(kTile, kTile) : idesc_bf16_f32(kTile, kTile, 0, 0);
+      constexpr uint32_t idesc_qc = F8 ? idesc_e4m3_f32(kTile, kCen) : idesc_qk;      // centroid steps
+      constexpr uint32_t idesc_pv = idesc_bf16_f32(kTile, D, 0, 1);
+      auto wait = [&](uint32_t bar, uint32_t phase) {
+        return __all_sync(0xffffffffu, mbar_wait(bar, phase & 1, abort_flag, prm.status, prm.wait_limit));
+      };
       // descriptors differ from a base one only in the start-address field (units of 16 bytes):
       // the base descriptors are built once, the per-instruction part is an addition
       const uint64_t q_desc0 = smem_desc_sw128(s_q, 16, 1024);
       const uint64_t k_desc0 = smem_desc_sw128(s_k, 16, 1024);
-      const uint64_t v_desc0 = smem_desc_sw128(s_v, C::HALF_PANEL_BYTES, 1024);
-      // The tensor core sits idle between the softmax's arrival and the next product, so that
-      // stretch is kept short: everything a product needs besides the probabilities -- its key and
-      // value slots (loaded long before) and their descriptors -- is waited for and computed BEFORE
-      // the wait for the softmax, and P V (u) and S(u + NBUF) are then issued back to back.
-      auto wait_keys = [&](int un) {
-        const int parts = un >= 2 * sel_tiles ? C::CEN_PARTS : 1;      // centroid keys as bf16: hi parts, then lo parts
-        bool got = true;
-        for (int g = 0; g < parts && got; ++g) {
-          const int kc = kslot_of(un) + g;
-          got = __all_sync(0xffffffffu, mbar_wait(b_k_full(kc % C::NK), (kc / C::NK) & 1, abort_flag, prm.status, prm.wait_limit));
+      const uint64_t v_desc0 = smem_desc_sw128(s_v, C::PANEL_BYTES, 1024);
+      int o_tiles = 0;
+      // scores of step u + kGroups, by one thread, into the buffer that P V (u) was issued from just before
+      auto scores = [&](int fl, int buf) {
+        if (fl & kFStop) {                    // wakes the group of this step, which ends with it
+          mbar_arrive(b_s_full(buf));
+          return;
         }
-        return got;
-      };
-      // first key slot and number of parts of S(un); fire_s (elected lane) issues it
-      auto fire_s = [&](uint32_t d_cols, int kc0, int parts, uint32_t bar) {
-        for (int g = 0; g < parts; ++g) {
-          const uint64_t kd = k_desc0 + ((((kc0 + g) % C::NK) * C::KHALF_BYTES) >> 4);
+        const uint32_t d_cols = tmem_base + buf * kTile;
+        const uint64_t kd = k_desc0 + ((buf * C::QK_BYTES) >> 4);
+        const uint32_t idesc = (fl & kFCentroid) ? idesc_qc : idesc_qk;
 #pragma unroll
-          for (int ks = 0; ks < D / C::QK_KSTEP; ++ks) {
-            // K-major operands: 32 bytes (16 bf16 or 32 E4M3 elements) per step, four steps per panel
-            const uint32_t qoff = ((ks / 4) * C::PANEL_BYTES + (ks % 4) * 32) >> 4;
-            const uint32_t koff = ((ks / 4) * C::HALF_PANEL_BYTES + (ks % 4) * 32) >> 4;
-            if (F8) mma_ss_f8(d_cols, q_desc0 + qoff, kd + koff, idesc_qk, (g > 0 || ks > 0) ? 1u : 0u);
-            else mma_ss(d_cols, q_desc0 + qoff, kd + koff, idesc_qk, (g > 0 || ks > 0) ? 1u : 0u);
-          }
+        for (int ks = 0; ks < D / C::QK_KSTEP; ++ks) {
+          // K-major operands: 32 bytes (16 bf16 or 32 E4M3 elements) per instruction, four per panel
+          const uint32_t off = ((ks / 4) * C::PANEL_BYTES + (ks % 4) * 32) >> 4;
+          if (F8) mma_ss_f8(d_cols, q_desc0 + off, kd + off, idesc, ks > 0 ? 1u : 0u);
+          else mma_ss(d_cols, q_desc0 + off, kd + off, idesc, ks > 0 ? 1u : 0u);
         }
-        mma_commit(bar);
+        mma_commit(b_s_full(buf));
+        if (fl & kFLast) mma_commit(b_q_empty);
       };
-      for (int u = 0; u < C::NBUF && u < steps && ok; ++u) {
-        ok = wait_keys(u);
+      static_assert(C::NK == kGroups, "key slots and score buffers go round together");
+      bool ok = true, first = true;           // `first`: P V of this step is the first one of a tile
+      int buf = 0, slot_v = 0, ring = 0;      // of the scores to issue; of P V
+      int fl0 = 0, fl1 = 0, fl2 = 0;          // flags of steps u, u + 1, u + 2
+      uint32_t ph_s = 0, ph_p = 0, ph_v = 0;  // phases of the keys of step u + kGroups, of P and of V of step u
+#pragma unroll 1
+      for (int u = -kGroups; ok; ++u) {
+        uint32_t bar = b_k_full(buf), phase = ph_s;
+        const int fl = fl0;
+        if (u >= 0) {
+          if (fl & kFStop) break;
+          if (lane == 1) { bar = b_p_ready(buf); phase = ph_p; }
+          if (lane == 2) { bar = b_v_full(slot_v); phase = ph_v; }
+        }
+        ok = wait(bar, phase);
+        if (u >= 0 && first && o_tiles > 0) ok = ok && wait(b_o_empty, o_tiles - 1);   // O of the tile before has been read
         if (!ok) break;
-        tc_fence_after();
-        if (elect_one())
-          fire_s(tmem_s + (u % C::NBUF) * kHalf, kslot_of(u), u >= 2 * sel_tiles ? C::CEN_PARTS : 1, b_s_full(u % C::NBAR));
-        __syncwarp();
-      }
-      for (int u = 0; u < steps && ok; ++u) {
-        const int slot = u % C::NV, un = u + C::NBUF;
-        ok = __all_sync(0xffffffffu, mbar_wait(b_v_full(slot), (u / C::NV) & 1, abort_flag, prm.status, prm.wait_limit));
-        if (ok && un < steps) ok = wait_keys(un);
-        // V is MN-major: 16 key rows (2048 bytes) per instruction; panels along d
-        const uint64_t vd = v_desc0 + ((slot * C::HALF_BYTES) >> 4);
-        const uint32_t p_cols = tmem_s + (u % C::NBUF) * kHalf;
-        const uint32_t s_cols = tmem_s + (un % C::NBUF) * kHalf, s_bar = b_s_full(un % C::NBAR), pv_bar = b_pv_done(u % C::NBAR);
-        const int s_kc0 = kslot_of(un), s_parts = un >= steps ? 0 : (un >= 2 * sel_tiles ? C::CEN_PARTS : 1);
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(b_p_ready(u % C::NBAR), (u / C::NBAR) & 1, abort_flag, prm.status, prm.wait_limit));
-        if (!ok) break;
+        const int fl_s = warp_uniform(st_flags[ring]);      // published: its keys have arrived
         tc_fence_after();
         if (elect_one()) {
+          if (u >= 0) {
+            // V is MN-major: 16 key rows (2048 bytes) per instruction; panels along d
+            const uint64_t vd = v_desc0 + ((slot_v * C::V_BYTES) >> 4);
+            const uint32_t p_cols = tmem_base + buf * kTile;
 #pragma unroll
-          for (int ks = 0; ks < kHalf / 16; ++ks)
-            mma_ts(tmem_o, p_cols + ks * 8, vd + (uint64_t)(ks * (2048 >> 4)), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
-          mma_commit(pv_bar);
-          if (s_parts) fire_s(s_cols, s_kc0, s_parts, s_bar);
+            for (int ks = 0; ks < 4; ++ks)
+              mma_ts(tmem_o, p_cols + ks * 8, vd + (uint64_t)(ks * (2048 >> 4)), idesc_pv, (ks > 0 || !first) ? 1u : 0u);
+            if (!(fl & kFCentroid)) {
+#pragma unroll
+              for (int ks = 4; ks < 8; ++ks)
+                mma_ts(tmem_o, p_cols + ks * 8, vd + (uint64_t)(ks * (2048 >> 4)), idesc_pv, 1u);
+            }
+            mma_commit(b_v_empty(slot_v));
+            if (fl & kFLast) mma_commit(b_o_full(o_tiles));
+          }
+          scores(fl_s, buf);
         }
         __syncwarp();
+        fl0 = fl1; fl1 = fl2; fl2 = fl_s;
+        if (++buf == kGroups) { buf = 0; ph_s ^= 1; if (u >= 0) ph_p ^= 1; }
+        if (++ring == kRing) ring = 0;
+        if (u >= 0) {
+          first = (fl & kFLast) != 0;
+          if (first) ++o_tiles;
+          if (++slot_v == C::NV) { slot_v = 0; ph_v ^= 1; }
+        }
       }
-      if (elect_one()) mma_commit(b_o_done);
+    } else {
+      // ---------------------------------------------------------- tiles, lists, step descriptors
+      const int per_head = prm.n_qc * tiles_per_qc;
+      const int ck_shift = __ffs(prm.c_k) - 1;
+      const int boxes = prm.c_k >= kTile ? 1 : kTile / prm.c_k;      // list entries per step, at most 8
+      int s = 0, ord = 0;
+      bool ok = true;
+      auto claim = [&]() {
+        if (s >= kRing) ok = __all_sync(0xffffffffu, relaxed(b_step_empty(s % kRing), s / kRing - 1));
+        return ok;
+      };
+      auto publish = [&]() {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b_step_full(s % kRing));
+        ++s;
+      };
+#pragma unroll 1
+      for (int tile = blockIdx.x; tile < prm.n_tiles && ok; ++ord) {
+        int next = 0;
+        if (lane == 0) next = (int)gridDim.x + atomicAdd(prm.next_tile, 1);
+        const int p = tile / per_head, x = tile % per_head;
+        const int qc = x / tiles_per_qc, half = x % tiles_per_qc;
+        const int32_t* sel = prm.block_idx + ((size_t)p * prm.n_qc + qc) * prm.list_stride;
+        const int32_t* cnt = prm.count_k + (size_t)p * prm.n_kc;
+        int keep = prm.keep_count ? prm.keep_count[(size_t)p * prm.n_qc + qc] : prm.keep;
+        if (keep < 0 || keep > prm.list_stride) {            // a list length that does not fit its row
+          if (lane == 0) atomicCAS(prm.status, 0, kErrBadIndex);
+          keep = keep < 0 ? 0 : prm.list_stride;
+        }
+        const int sel_steps = selected_tiles(keep, prm.c_k);
+        const int cen_steps = prm.compensate ? prm.cen_tiles : 0;
+        const int n = max(sel_steps + cen_steps, 1);      // nothing to attend to: one step with every column masked
+        if (prm.compensate) {
+#pragma unroll 1
+          for (int w = lane; w < prm.bitmap_words; w += 32) bitmap[w] = 0u;
+          __syncwarp();
+        }
+        int base = -32, my_j = 0, my_members = 0;            // list entries [base, base + 32), one per lane
+        float my_scale = 0.f;
+#pragma unroll 1
+        for (int u = 0; u < n && ok; ++u) {
+          int fl = (u == 0 ? kFFirst : 0) | (u == n - 1 ? kFLast : 0) | (min(u, 15) << kFIndexShift) |
+                   (min(n - 1 - u, 15) << kFRestShift);
+          const int e0 = prm.c_k >= kTile ? u >> (ck_shift - 7) : u * boxes;
+          if (u < sel_steps && e0 >= base + 32) {
+            base = e0 & ~31;
+            const int e = base + lane;
+            my_members = 0;
+            my_j = 0;
+            my_scale = 0.f;
+            if (e < keep) {
+              const int j = sel[e];
+              my_j = min(max(j, 0), prm.n_kc - 1);
+              if (j != my_j) {                             // not a key cluster: flagged, all of its columns masked
+                atomicCAS(prm.status, 0, kErrBadIndex);
+              } else {
+                my_members = min(max(cnt[j], 0), prm.c_k);
+                if (F8) my_scale = prm.k_scale[(size_t)p * prm.n_kc + j];
+                if (prm.compensate) atomicOr(&bitmap[j >> 5], 1u << (j & 31));
+              }
+            }
+          }
+          if (!claim()) break;
+          int* rows = st_rows + (s % kRing) * kRowInts;
+          float* bz = bias + (s % kRing) * kTile;
+          float sc = 0.f;
+          if (u < sel_steps) {
+            // filler boxes behind the end of the list repeat its last entry, masked
+            const int at = e0 - base;
+            const int src = prm.c_k >= kTile ? at : min(at + (lane & 7), keep - 1 - base);
+            const int j = __shfl_sync(0xffffffffu, my_j, src);
+            int members = __shfl_sync(0xffffffffu, my_members, src);
+            if (F8) sc = __shfl_sync(0xffffffffu, my_scale, src);
+            const int first = prm.c_k >= kTile ? (u << 7) & (prm.c_k - 1) : 0;    // row of the step's first column
+            members -= first;
+            if (prm.c_k < kTile && e0 + (lane & 7) >= keep) members = 0;
+            if (lane < boxes) rows[lane] = (p * prm.n_kc + j) * prm.c_k + first;
+            const int width = min(prm.c_k, kTile);
+            if (__any_sync(0xffffffffu, lane < boxes && members < width)) {
+              fl |= kFMasked;
+#pragma unroll 1
+              for (int c = lane; c < kTile; c += 32) {
+                const int m = __shfl_sync(0xffffffffu, members, c / width);
+                bz[c] = (c & (width - 1)) < m ? 0.f : -INFINITY;
+              }
+            }
+          } else {
+            fl |= kFMasked;
+            if (cen_steps > 0) {
+              const int i = u - sel_steps;
+              fl |= kFCentroid;
+              __syncwarp();
+#pragma unroll
+              for (int g = 0; g < 2; ++g) {
+                const int j = i * kCen + lane + 32 * g;
+                const bool use = j < prm.n_kc && !((bitmap[j >> 5] >> (j & 31)) & 1u);
+                bz[lane + 32 * g] = use ? log2f((float)cnt[min(j, prm.n_kc - 1)]) : -INFINITY;
+              }
+              if (lane == 0) rows[0] = (p * prm.cen_tiles + i) * (F8 ? kCen : kTile);
+              if (lane == 1) rows[kRowCenV] = (p * prm.cen_tiles + i) * kCen;
+              if (F8) sc = prm.c_scale[(size_t)p * prm.cen_tiles + i];
+            } else {
+#pragma unroll 1
+              for (int c = lane; c < kTile; c += 32) bz[c] = -INFINITY;
+              if (lane < boxes) rows[lane] = p * prm.n_kc * prm.c_k;
+            }
+          }
+          if (F8 && lane < 2) st_scale[(s % kRing) * 2 + lane] = sc;
+          if (lane == 0) {
+            st_flags[s % kRing] = fl;
+            rows[kRowQ] = (p * prm.n_qc + qc) * prm.c_q + half * kTile;
+            st_tile[s % kRing] = make_int4(p, qc * prm.c_q + half * kTile, (p * prm.n_qc + qc) * 2 + half, ord);
+          }
+          publish();
+        }
+        tile = __shfl_sync(0xffffffffu, next, 0);
+      }
+#pragma unroll 1
+      for (int g = 0; g < kGroups && ok; ++g) {
+        if (!claim()) break;
+        if (lane == 0) st_flags[s % kRing] = kFStop;
+        publish();
+      }
     }
   } else {
-    // ------------------------------------------------------------ softmax + epilogue (128 threads)
-    const int st = tid - 64;                       // 0..127
+    // ------------------------------------------------------------ softmax groups and epilogue
+    const int group = (warp >> 2) - 1;
     const int quarter = warp & 3;                  // TMEM lanes this warp may touch
-    const int row = quarter * 32 + lane;           // query row within the tile
+    const int row = quarter * 32 + lane;           // row within the tile
+    const int qrow = twice ? row & 63 : row;       // query row
+    const int half = quarter >> 1;                 // of the tile
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-    const int32_t* cnt = prm.count_k + (size_t)p * prm.n_kc;
-    for (int w = st; w < prm.bitmap_words; w += 128) bitmap[w] = 0u;
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    for (int e = st; e < keep; e += 128) {
-      const int j = sel[e];
-      if (j < 0 || j >= prm.n_kc) {                        // not a key cluster: flagged, all of its columns masked
-        atomicCAS(prm.status, 0, kErrBadIndex);
-        members_of[e] = 0;
-        if (F8) kscale_of[e] = 0.f;
-        continue;
-      }
-      members_of[e] = (uint16_t)min(max(cnt[j], 0), prm.c_k);
-      if (F8) kscale_of[e] = prm.k_scale[(size_t)p * prm.n_kc + j];
-      if (prm.compensate) atomicOr(&bitmap[j >> 5], 1u << (j & 31));
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-
-    if (C::Q_IN_TMEM) {
-      // this thread's query row: eight 16-byte chunks, stored at chunk position c ^ (row & 7)
-      bool q_ok = __all_sync(0xffffffffu, mbar_wait(b_q_full, 0, abort_flag, prm.status, prm.wait_limit));
-      uint32_t qw[32];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const uint4 v = *reinterpret_cast<const uint4*>(smem + C::OFF_Q + row * 128 + ((c ^ (row & 7)) << 4));
-        qw[4 * c] = v.x; qw[4 * c + 1] = v.y; qw[4 * c + 2] = v.z; qw[4 * c + 3] = v.w;
-      }
-      (void)q_ok;
-      tmem_st32(tmem_base + C::TMEM_Q + lane_addr, qw);
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(b_q_tmem);
-    }
-    float m_ref = -INFINITY, l_run = 0.f, pend = 0.f;
-    const int ck_shift = __ffs(prm.c_k) - 1;
+    const uint32_t t_s = tmem_base + group * kTile + lane_addr;
+    auto wait = [&](uint32_t bar, uint32_t phase) {
+      return __all_sync(0xffffffffu, mbar_wait(bar, phase & 1, abort_flag, prm.status, prm.wait_limit));
+    };
+    float m_own = -INFINITY, l_run = 0.f, pend = 0.f;
     // factor from a raw score to log2 units: the softmax scale, and with quantised Q K^T the scale
-    // of this thread's query row (times, per half-step, the scale of the key cluster or centroid run)
+    // of this thread's query row (times, per 64 keys, the scale of the key cluster or centroid run)
     float row_sc = prm.scale_log2;
-    if (F8) {
-      const int qrow = (p * prm.n_qc + qc) * prm.c_q + half * kTile + (row < q_rows ? row : 0);
-      row_sc *= prm.q_scale[qrow];
-    }
-    // A warp whose wait gave up goes through the remaining half-steps without touching anything
-    // (`dead`), so that it still meets the other softmax warps at the barriers they share.
-    bool dead = false;
-    for (int u = 0; u < steps; ++u) {
-      const int b = u & 1;                               // half of a 128-row tile (geometry of the keys)
-      const int buf = u % C::NBUF;                       // score buffer
-      const uint32_t t_s = tmem_s + lane_addr + buf * kHalf;
-      // per-column additive term (log2 units): only half-steps with masked or weighted columns need
-      // it.  `masked` depends on the half-step only, so it is uniform over the 128 threads.
-      bool masked = false;
-      // eight buffers: a thread can run at most NBUF half-steps ahead of the slowest one
-      float* bz = bias + (u & 7) * kHalf;
-      if (u < 2 * sel_tiles) {
-        // cluster sizes are powers of two: positions are split with shifts and masks
-        const int t = u >> 1;
-        bool use = true;
-        if (prm.c_k >= kTile) {
-          const int e = t >> (ck_shift - 7);                      // c_k / 128 tiles per cluster
-          const int members = members_of[e];
-          const int first = ((t << 7) & (prm.c_k - 1)) + b * kHalf;   // row of this half-step's first column
-          masked = members < first + kHalf;
-          use = first + (st & 63) < members;
-        } else {
-          const int col0 = t * kTile + b * kHalf;                // position in the list of selected rows
-          const int e_first = col0 >> ck_shift, e_last = (col0 + kHalf - 1) >> ck_shift;
-          for (int e = e_first; e <= e_last; ++e)
-            if (e >= keep || members_of[e] < prm.c_k) masked = true;
-          const int e = (col0 + (st & 63)) >> ck_shift;
-          use = e < keep && ((col0 + (st & 63)) & (prm.c_k - 1)) < members_of[min(e, keep - 1)];
-        }
-        if (masked && st < kHalf) bz[st] = use ? 0.f : -INFINITY;
-      } else {
-        masked = true;
-        const int j = (u - 2 * sel_tiles) * kHalf + (st & 63);
-        const bool use = j < prm.n_kc && !((bitmap[j >> 5] >> (j & 31)) & 1u);
-        if (st < kHalf) bz[st] = use ? log2f((float)cnt[min(j, prm.n_kc - 1)]) : -INFINITY;
-      }
-      if (masked) asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (dead) continue;
-      // scale of this half-step's scores.  A zero scale (an all-zero query row or key group) makes
-      // every logit 0: the raw scores are then dropped and the additive terms enter with scale 1.
-      float sc_used = prm.scale_log2;
-      bool keep_raw = true;
-      if (F8) {
-        const float ks = u < 2 * sel_tiles ? kscale_of[min((u * kHalf) >> ck_shift, max(keep - 1, 0))]
-                                           : prm.c_scale[(size_t)p * prm.cen_tiles + (u - 2 * sel_tiles)];
-        const float sc_eff = row_sc * ks;
-        keep_raw = sc_eff > 0.f;
-        sc_used = keep_raw ? sc_eff : (masked ? 1.f : 0.f);
-      }
-
-      if (!__all_sync(0xffffffffu, mbar_wait(b_s_full(u % C::NBAR), (u / C::NBAR) & 1, abort_flag, prm.status, prm.wait_limit))) {
-        dead = true;
-        continue;
-      }
-      tc_fence_after();
-      if (quarter * 32 >= q_rows) {          // this warp's rows are padding of a 64-row query cluster
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b_p_ready(u % C::NBAR));
-        continue;
-      }
-      // The loops over the two 32-column chunks are kept rolled: the body of a half-step is
-      // executed by every softmax warp of both resident CTAs at different places, and an unrolled
-      // body does not stay in the instruction cache.
-      // ---- masked / weighted half-steps (short clusters, centroid columns): the additive term is
-      // folded into the scores in tensor memory first, so that the common path below has no bias
-      if (masked) {
-        const float inv_scale_log2 = __fdividef(1.f, sc_used);
-        const float raw_factor = keep_raw ? 1.f : 0.f;
+    uint32_t ph_s = 0;
 #pragma unroll 1
-        for (int c4 = 0; c4 < 2; ++c4) {
+    for (int s = group;; s += kGroups) {
+      const int ring = s % kRing;
+      if (!wait(b_s_full(group), ph_s)) break;
+      ph_s ^= 1;
+      tc_fence_after();
+      const int fl = warp_uniform(st_flags[ring]);
+      if (fl & kFStop) break;
+      const int index = (fl >> kFIndexShift) & 15, rest = (fl >> kFRestShift) & 15;
+      const bool cen = (fl & kFCentroid) != 0, masked = (fl & kFMasked) != 0;
+      if (index < kGroups) {                       // this group's first step of the tile
+        m_own = -INFINITY;
+        l_run = 0.f;
+        pend = 0.f;
+        if (F8) {
+          const int4 tl = st_tile[ring];
+          row_sc = prm.scale_log2 * prm.q_scale[(size_t)tl.x * prm.n_qc * prm.c_q + tl.y + qrow];
+        }
+      }
+      // scales of this step's scores, per run of 64 columns.  A zero scale (an all-zero query row or
+      // key group) makes every logit 0: the raw scores are then dropped and the additive terms
+      // enter with scale 1.
+      float sc_h[2] = {prm.scale_log2, prm.scale_log2};
+      float raw_h[2] = {1.f, 1.f};
+      if (F8) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float sc_eff = row_sc * st_scale[ring * 2 + h];
+          raw_h[h] = sc_eff > 0.f ? 1.f : 0.f;
+          sc_h[h] = sc_eff > 0.f ? sc_eff : (masked ? 1.f : 0.f);
+        }
+      }
+      const float* bz = bias + ring * kTile;
+      // chunks [c_begin, c_end) of 32 columns; of a 64-row query cluster's halves the lower one has no part in
+      // the 64 columns of a centroid step
+      const int c_begin = twice && !cen ? 2 * half : 0;
+      const int c_end = twice ? (cen ? 2 - 2 * half : c_begin + 2) : (cen ? 2 : 4);
+      // ---- masked or weighted steps: scores of hi and lo parts of centroids are added and the additive
+      // term is folded into the scores in tensor memory first, so that the common path below has
+      // no bias
+      if (masked) {
+#pragma unroll 1
+        for (int c4 = c_begin; c4 < c_end; ++c4) {
+          const float inv = __fdividef(1.f, F8 && c4 >= 2 ? sc_h[1] : sc_h[0]);
+          const float raw = F8 && c4 >= 2 ? raw_h[1] : raw_h[0];
           uint32_t r[32];
           tmem_ld32(t_s + c4 * 32, r);
-          tmem_wait_ld();
+          if (!F8 && cen) {
+            uint32_t lo[32];
+            tmem_ld32(t_s + kCen + c4 * 32, lo);
+            tmem_wait_ld32(r);
+            tmem_wait_ld32(lo);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(lo[j]));
+          } else {
+            tmem_wait_ld32(r);
+          }
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
-            const float raw = F8 ? __uint_as_float(r[j]) * raw_factor : __uint_as_float(r[j]);
-            r[j] = __float_as_uint(fmaf(bz[c4 * 32 + j], inv_scale_log2, raw));
+            const float x = F8 ? __uint_as_float(r[j]) * raw : __uint_as_float(r[j]);
+            r[j] = __float_as_uint(fmaf(bz[c4 * 32 + j], inv, x));
           }
           tmem_st32(t_s + c4 * 32, r);
         }
         tmem_wait_st();
       }
-      // ---- reference maximum.  The softmax needs no exact row maximum, only a reference m_ref
-      // that keeps exp2(x - m_ref) in range.  The first half-step of a row (and any later one while
-      // the row has seen only masked columns) measures the maximum of its scores first; afterwards
-      // the maximum of a half-step is gathered while its exponentials are computed, and a row
-      // whose values exceeded 2^threshold moves its reference up at the start of the NEXT
-      // half-step (`pend`).  Values between 2^threshold and 2^kDanger are exact all the same: P is
-      // bf16, which has the exponent range of fp32, and O and l are fp32.  A jump beyond 2^kDanger
-      // within one half-step may overflow: the CTA then marks its query tile in `redo`, and the
-      // launcher's second pass recomputes marked tiles with the fp32 kernel (exact row maxima).
-      float alpha = 1.f;
-      bool rescale = false;
-      if (__any_sync(0xffffffffu, m_ref == -INFINITY || pend > 0.f)) {
-        bool raise = false;
-        float tmax = 0.f;
-        if (__any_sync(0xffffffffu, m_ref == -INFINITY)) {
-          float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+      // ---- reference.  The softmax needs no exact row maximum, only a reference m that keeps
+      // exp2(x - m) in range.  The first step of a row (and any later one while the row has seen only
+      // masked columns) measures the maximum of its scores; afterwards a row whose probabilities
+      // exceeded 2^threshold (seen in the sum of 32 of them) moves its reference up at its group's
+      // NEXT step (`pend`).  Values between 2^threshold and 2^96 are exact all the same: P is
+      // bf16, which has the exponent range of fp32, and O and l are fp32.  A sum beyond 2^96 may
+      // overflow: the row sum then becomes NaN, which marks the tile in `redo`, and the launcher's
+      // second pass recomputes marked tiles with the fp32 kernel (exact row maxima).
+      // The reference of step s - 1 comes from the group before through shared memory.
+      float m_prev;
+      {
+        int at;
+        bool got = true;
+        long long t0 = 0;
 #pragma unroll 1
-          for (int c4 = 0; c4 < 2; ++c4) {
+        for (uint32_t it = 0;; ++it) {
+          asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=f"(m_prev), "=r"(at) : "r"(s_ref + row * 8) : "memory");
+          if (__all_sync(0xffffffffu, at >= s - 1)) break;
+          if ((it & 255u) == 255u) {
+            if (t0 == 0) t0 = clock64();
+            const bool late = *abort_flag != 0 || clock64() - t0 > prm.wait_limit;
+            if (__any_sync(0xffffffffu, late)) {
+              *abort_flag = 1;
+              if (lane == 0) atomicCAS(prm.status, 0, 5 /* CA_ERR_TIMEOUT */);
+              got = false;
+              break;
+            }
+          }
+        }
+        if (!got) break;
+      }
+      if (index == 0) m_prev = -INFINITY;
+      float m_ref = m_prev;
+      if (__any_sync(0xffffffffu, m_prev == -INFINITY || m_prev != m_own || pend > 0.f)) {
+        if (pend > 0.f) m_ref = fmaxf(m_ref, m_own + pend);
+        if (c_end > 0 && __any_sync(0xffffffffu, m_ref == -INFINITY)) {
+          float tmax = -INFINITY;
+#pragma unroll 1
+          for (int c4 = c_begin; c4 < c_end; ++c4) {
             uint32_t r[32];
             tmem_ld32(t_s + c4 * 32, r);
-            tmem_wait_ld();
+            tmem_wait_ld32(r);
+            float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
               mx0 = max3(mx0, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
@@ -503,58 +622,44 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               mx2 = max3(mx2, __uint_as_float(r[j + 4]), __uint_as_float(r[j + 5]));
               mx3 = max3(mx3, __uint_as_float(r[j + 6]), __uint_as_float(r[j + 7]));
             }
+            tmax = fmaxf(tmax, fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * (F8 && c4 >= 2 ? sc_h[1] : sc_h[0]));
           }
-          tmax = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * sc_used;
-          raise = tmax > m_ref + kRescaleThreshold || (m_ref == -INFINITY && tmax > -INFINITY);
+          if (tmax > m_ref + kRescaleThreshold || m_ref == -INFINITY) m_ref = fmaxf(m_ref, tmax);
         }
-        if (raise) {
-          alpha = (m_ref == -INFINITY) ? 0.f : ex2_approx(m_ref - tmax);
-          m_ref = tmax;
-        } else if (pend > 0.f) {
-          alpha = ex2_approx(-pend);
-          m_ref += pend;
-        }
-        rescale = __any_sync(0xffffffffu, raise || pend > 0.f);
-      }
-      pend = 0.f;
-      if (rescale) {
-        l_run *= alpha;
-        if (u > 0) {
-          // products complete in the order of their issue: once P V (u-1) is complete, all earlier are
-          if (!__all_sync(0xffffffffu, mbar_wait(b_pv_done((u - 1) % C::NBAR), ((u - 1) / C::NBAR) & 1, abort_flag, prm.status, prm.wait_limit))) {
-            dead = true;
-            continue;
-          }
+        if (m_own > -INFINITY) l_run *= ex2_approx(m_own - m_ref);
+        if (index > 0 && __any_sync(0xffffffffu, m_ref != m_prev)) {
+          // P V (s - 1) is complete when its value slot is free again; P V (s) waits for this warp
+          if (!wait(b_v_empty((s - 1) % C::NV), (s - 1) / C::NV)) break;
           tc_fence_after();
+          const float alpha = m_prev == -INFINITY ? 0.f : ex2_approx(m_prev - m_ref);
 #pragma unroll 1
           for (int c4 = 0; c4 < D / 32; ++c4) {
             uint32_t o[32];
             tmem_ld32(tmem_o + lane_addr + c4 * 32, o);
-            tmem_wait_ld();
+            tmem_wait_ld32(o);
 #pragma unroll
             for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
             tmem_st32(tmem_o + lane_addr + c4 * 32, o);
           }
+          tmem_wait_st();
         }
+        pend = 0.f;
       }
-      // ---- P = exp2(x - m_ref), packed to bf16 over the first 32 columns of the buffer (chunk 0
-      // goes to columns [0,16) while chunk 1 is still unread in [32,64); chunk 1 to [16,32))
-      float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-      const f32x2 sc2 = pack2(sc_used, sc_used);
-      float cm0 = -INFINITY, cm1 = -INFINITY;            // maximum of x - m_ref over the half-step
-      float big = 0.f;                                   // larger of the two chunk sums of the half-step
-#pragma unroll 1
-      for (int c4 = 0; c4 < 2; ++c4) {
-        uint32_t r[32];
-        tmem_ld32(t_s + c4 * 32, r);
-        tmem_wait_ld();
-        // The special-function unit takes one exponential per 8 cycles and sub-core and is the
-        // busiest unit of the kernel at d = 64: scaling and sums use two-value fp32 instructions,
-        // and the other work of the chunk is interleaved with the exponentials in groups of four,
-        // two groups behind, so that it issues in the shadow of that unit.
+      m_own = m_ref;
+      asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(s_ref + row * 8), "f"(m_ref), "r"(s) : "memory");
+
+      // ---- P = exp2(x - m), packed to bf16: the 32 columns of chunk c go to columns [16 c, 16 c + 16),
+      // which have been read by then.  A chunk is loaded while the one before it is computed.
+      const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
+      const f32x2 nm2 = pack2(neg_m, neg_m);
+      float big = 0.f;                                   // largest sum of a chunk
+      auto chunk = [&](uint32_t (&r)[32], f32x2 sc2, uint32_t dst) {
+        // The special-function unit takes one exponential per 8 cycles and sub-core: scaling and
+        // sums use two-value fp32 instructions, and the other work of the chunk is interleaved
+        // with the exponentials in groups of four, two groups behind, so that it issues in the
+        // shadow of that unit.
         float x[32];
         uint32_t pk[16];
-        const f32x2 nm2 = pack2(neg_m, neg_m);
         f32x2 s01 = pack2(0.f, 0.f), s23 = s01;
         auto scale4 = [&](int j) {
           unpack2(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2, nm2), x[j], x[j + 1]);
@@ -565,13 +670,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
         for (int g = 0; g < 10; ++g) {
           if (g < 8) {
-            const int j = 4 * g;
-            if (C::TRACK_MAX) {
-              cm0 = max3(cm0, x[j], x[j + 1]);
-              cm1 = max3(cm1, x[j + 2], x[j + 3]);
-            }
 #pragma unroll
-            for (int e = j; e < j + 4; ++e) x[e] = ex2_approx(x[e]);
+            for (int e = 4 * g; e < 4 * g + 4; ++e) x[e] = ex2_approx(x[e]);
           }
           if (g + 2 < 8) scale4(4 * (g + 2));
           if (g >= 2) {
@@ -585,73 +685,150 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         float sa, sb, sc, sd;
         unpack2(s01, sa, sb);
         unpack2(s23, sc, sd);
-        const float chunk_sum = (sa + sb) + (sc + sd);
-        l_run += chunk_sum;
-        if (!C::TRACK_MAX) big = fmaxf(big, chunk_sum);
-        tmem_st16(t_s + c4 * 16, pk);
+        const float sum = (sa + sb) + (sc + sd);
+        l_run += sum;
+        big = fmaxf(big, sum);
+        if (!(sum < kDangerSum)) l_run = __int_as_float(0x7fffffff);
+        tmem_st16(dst, pk);
+      };
+      uint32_t ra[32], rb[32];
+      tmem_ld32(t_s + c_begin * 32, ra);
+      tmem_wait_ld32(ra);
+#pragma unroll 1
+      for (int h = c_begin >> 1; 2 * h < c_end; ++h) {
+        const float sc = F8 && h > 0 ? sc_h[1] : sc_h[0];
+        const f32x2 sc2 = pack2(sc, sc);
+        tmem_ld32(t_s + h * 64 + 32, rb);
+        chunk(ra, sc2, t_s + h * 32);
+        tmem_wait_ld32(rb);
+        if (2 * h + 2 < c_end) tmem_ld32(t_s + h * 64 + 64, ra);
+        chunk(rb, sc2, t_s + h * 32 + 16);
+        tmem_wait_ld32(ra);
       }
-      if (C::TRACK_MAX) {
-        const float hm = fmaxf(cm0, cm1);
-        if (hm > kRescaleThreshold) pend = ceilf(hm);
-        if (__any_sync(0xffffffffu, hm > kDanger)) *redo_flag = 1;
-      } else {
-        // a sum that is not below 2^kDanger (infinite or NaN included) marks the tile
-        if (big > 256.0f) pend = ceilf(log2f(big));
-        if (__any_sync(0xffffffffu, !(big < 7.9228163e28f))) *redo_flag = 1;
+      if (twice && (!cen || half == 1)) {                  // the other half's keys
+#pragma unroll
+        for (int j = 0; j < 32; ++j) ra[j] = 0u;
+        tmem_st32(t_s + (cen || half == 1 ? 0 : 32), ra);
       }
+      if (big > kSumLimit) pend = ceilf(log2f(big));
+      // the group's last step of the tile: its row sums go to the group that ends the tile
+      if (rest > 0 && rest < kGroups) lpart[s % kParts * kTile + row] = make_float2(l_run, m_ref);
+      const int4 tl = st_tile[ring];
       // one arrival per warp: 128 arrivals on one barrier word would be serialised in shared memory
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(b_p_ready(u % C::NBAR));
-    }
+      if (lane == 0) { mbar_arrive(b_p_ready(group)); mbar_arrive(b_step_empty(ring)); }
+      if (rest > 0) continue;
 
-    // epilogue: O / l, rows back to their original positions
-    bool ok = !dead;
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(b_o_done, 0, abort_flag, prm.status, prm.wait_limit));
-    tc_fence_after();
-    if (ok) {                                          // warp-uniform: TMEM loads are warp-collective
-      const int pos = qc * prm.c_q + half * kTile + row;
-      bool live = row < q_rows && pos < prm.n_q;        // rows of the padding are not written
-      int orig = live ? prm.perm_q[(size_t)p * prm.n_q + pos] : 0;
+      // ---- epilogue: O / l, rows back to their original positions
+      const int pos = tl.y + qrow;
+      bool live = pos < prm.n_q;                        // rows of the padding are not written
+      int orig = live ? prm.perm_q[(size_t)tl.x * prm.n_q + pos] : 0;
       if (orig < 0 || orig >= prm.n_q) {                // not a row of O: flagged, nothing written
         atomicCAS(prm.status, 0, kErrBadIndex);
         live = false;
         orig = 0;
       }
+      // products complete in order, and the sums were written before the probabilities were handed over
+      if (!wait(b_o_full(tl.w), tl.w >> 2)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int g = 1; g < kGroups; ++g) {
+        if (g <= index) {
+          const float2 other = lpart[(s - g) % kParts * kTile + row];
+          if (other.y > -INFINITY) l_run += other.x * ex2_approx(other.y - m_ref);
+        }
+      }
+      // the halves of a 64-row query cluster: the lower one hands over its sums and 16 columns of O at a
+      // time, scaled to the larger reference by the upper one
+      float* merge = reinterpret_cast<float*>(smem + C::OFF_MERGE) + qrow * kMergeInts;
+      const int pair = quarter & 1, uses = tl.w * (D / 16);
+      bool got = true;
+      if (twice && half == 1) {
+#pragma unroll 1
+        for (int c = 0; c < D / 16 && got; ++c) {
+          const int use = uses + c;
+          uint32_t o[16];
+          tmem_ld16(tmem_o + lane_addr + c * 16, o);
+          tmem_wait_ld();
+          if (use > 0) got = wait(b_m_empty(pair), use - 1);
+          if (!got) break;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) merge[j] = __uint_as_float(o[j]);
+          merge[16] = l_run;
+          merge[17] = m_ref;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_m_full(pair));
+        }
+      }
+      float l_all = l_run, m_all = m_ref, w_own = 1.f, w_other = 0.f;
+      if (twice && half == 0) {
+        got = wait(b_m_full(pair), uses);
+        if (!got) break;
+        const float l_other = merge[16], m_other = merge[17];
+        m_all = fmaxf(m_ref, m_other);
+        w_own = m_ref > -INFINITY ? ex2_approx(m_ref - m_all) : 0.f;
+        w_other = m_other > -INFINITY ? ex2_approx(m_other - m_all) : 0.f;
+        l_all = l_run * w_own + l_other * w_other;
+      }
+      if (!got) break;
       // a row without a single live entry (an empty list without compensation): zeros, lse = -inf
-      const bool empty = !(l_run > 0.f);
-      const float inv = empty ? 0.f : 1.f / l_run;
-      __nv_bfloat16* out = prm.O + ((size_t)p * prm.n_q + orig) * D;
+      const bool lost = !(l_all < INFINITY);            // left the range: the second pass computes it
+      const bool empty = !(l_all > 0.f);
+      const float inv = empty ? 0.f : 1.f / l_all;
+      __nv_bfloat16* out = prm.O + ((size_t)tl.x * prm.n_q + orig) * D;
+      const bool write = live && !(twice && half == 1);
+      if (!(twice && half == 1)) {
+        const float inv_own = inv * w_own, inv_other = inv * w_other;
+#pragma unroll 1
+        for (int c = 0; c < D / 16; ++c) {
+          uint32_t o[16];
+          tmem_ld16(tmem_o + lane_addr + c * 16, o);
+          tmem_wait_ld();
 #pragma unroll
-      for (int c4 = 0; c4 < D / 32; ++c4) {
-        uint32_t o[32];
-        tmem_ld32(tmem_o + lane_addr + c4 * 32, o);
-        tmem_wait_ld();
-        if (live) {
-          uint4* dst = reinterpret_cast<uint4*>(out + c4 * 32);
+          for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv_own);
+          if (twice) {
+            if (c > 0) got = wait(b_m_full(pair), uses + c);
+            if (!got) break;
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint4 w;
-            w.x = pack_bf16x2(__uint_as_float(o[8 * v + 0]) * inv, __uint_as_float(o[8 * v + 1]) * inv);
-            w.y = pack_bf16x2(__uint_as_float(o[8 * v + 2]) * inv, __uint_as_float(o[8 * v + 3]) * inv);
-            w.z = pack_bf16x2(__uint_as_float(o[8 * v + 4]) * inv, __uint_as_float(o[8 * v + 5]) * inv);
-            w.w = pack_bf16x2(__uint_as_float(o[8 * v + 6]) * inv, __uint_as_float(o[8 * v + 7]) * inv);
-            if (empty) w = make_uint4(0u, 0u, 0u, 0u);   // no product was issued: the accumulator holds no data
-            dst[v] = w;
+            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(fmaf(merge[j], inv_other, __uint_as_float(o[j])));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(b_m_empty(pair));
+          }
+          if (write) {
+            uint4* dst = reinterpret_cast<uint4*>(out + c * 16);
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+              uint4 w;
+              w.x = pack_bf16x2(__uint_as_float(o[8 * v + 0]), __uint_as_float(o[8 * v + 1]));
+              w.y = pack_bf16x2(__uint_as_float(o[8 * v + 2]), __uint_as_float(o[8 * v + 3]));
+              w.z = pack_bf16x2(__uint_as_float(o[8 * v + 4]), __uint_as_float(o[8 * v + 5]));
+              w.w = pack_bf16x2(__uint_as_float(o[8 * v + 6]), __uint_as_float(o[8 * v + 7]));
+              if (empty) w = make_uint4(0u, 0u, 0u, 0u);   // every column masked: the accumulator may hold 0 x inf
+              dst[v] = w;
+            }
           }
         }
       }
-      if (live && prm.lse)
-        prm.lse[(size_t)p * prm.n_q + orig] = empty ? -INFINITY : (m_ref + log2f(l_run)) * 0.6931471805599453f;
+      if (!got) break;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_o_empty);
+      if (write && prm.lse)
+        prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_all + log2f(l_all)) * 0.6931471805599453f;
+      // one word per tile, written on every launch by the last of its four warps: 1 = recompute
+      const bool redo = __any_sync(0xffffffffu, lost && !(twice && half == 1));
+      if (lane == 0) {
+        int* acc = &redo_acc[tl.w & 3];
+        if ((atomicAdd(acc, redo ? 257 : 1) & 255) == 3) prm.redo[tl.z] = atomicExch(acc, 0) >= 256 ? 1 : 0;
+      }
     }
   }
 
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
-  // one word per CTA, written on every launch: 1 = this tile is to be recomputed
-  if (tid == 0) prm.redo[((size_t)p * prm.n_qc + qc) * 2 + half] = *redo_flag;
 }
 
 // ---------------------------------------------------------------------------
@@ -664,7 +841,7 @@ __global__ void centroid_prep_kernel(const float* __restrict__ ck, const float* 
                                      __nv_bfloat16* __restrict__ vb) {
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= cen_tiles * kHalf * D) return;
+  if (e >= cen_tiles * kCen * D) return;
   const int j = e / D, col = e % D;
   float k = 0.f, v = 0.f;
   if (j < n_kc) {
@@ -672,10 +849,10 @@ __global__ void centroid_prep_kernel(const float* __restrict__ ck, const float* 
     v = cv[(size_t)p * n_kc * D + e];
   }
   const __nv_bfloat16 h = __float2bfloat16_rn(k);
-  const size_t tile = (size_t)p * cen_tiles + j / kHalf;
-  kmix[(tile * kTile + (j % kHalf)) * D + col] = h;
-  kmix[(tile * kTile + kHalf + (j % kHalf)) * D + col] = __float2bfloat16_rn(k - __bfloat162float(h));
-  vb[((size_t)p * cen_tiles * kHalf + j) * D + col] = __float2bfloat16_rn(v);
+  const size_t tile = (size_t)p * cen_tiles + j / kCen;
+  kmix[(tile * kTile + (j % kCen)) * D + col] = h;
+  kmix[(tile * kTile + kCen + (j % kCen)) * D + col] = __float2bfloat16_rn(k - __bfloat162float(h));
+  vb[((size_t)p * cen_tiles * kCen + j) * D + col] = __float2bfloat16_rn(v);
 }
 
 // ---------------------------------------------------------------------------
@@ -724,30 +901,29 @@ bool attn_tc_supported(const ca_problem_t& pr) {
 // quantised Q K^T: head dimension 128 (one 128-byte panel row of codes), key clusters of at least
 // 64 rows (one scale per half-step)
 bool attn_tc_fp8_supported(const ca_problem_t& pr) {
-  return attn_tc_supported(pr) && pr.head_dim == 128 && pr.cluster_k >= kHalf;
+  return attn_tc_supported(pr) && pr.head_dim == 128 && pr.cluster_k >= kCen;
 }
 
 size_t attn_tc_workspace_bytes(const ca_problem_t& pr) {
   const size_t P = (size_t)pr.batch * pr.heads;
-  const size_t cen_tiles = (size_t)ceil_div(ceil_div(pr.n_k, pr.cluster_k), kHalf);
+  const size_t cen_tiles = (size_t)ceil_div(ceil_div(pr.n_k, pr.cluster_k), kCen);
   const size_t n_qc = (size_t)ceil_div(pr.n_q, pr.cluster_q);
   size_t bytes = kStatusBytes + align_up(P * cen_tiles * kTile * pr.head_dim * sizeof(__nv_bfloat16), 256) +
-                 align_up(P * cen_tiles * kHalf * pr.head_dim * sizeof(__nv_bfloat16), 256) +
+                 align_up(P * cen_tiles * kCen * pr.head_dim * sizeof(__nv_bfloat16), 256) +
                  align_up(P * n_qc * 2 * sizeof(int32_t), 256);
   if (pr.flags & CA_ATTN_FP8_QK) {
     const size_t n_kc = (size_t)ceil_div(pr.n_k, pr.cluster_k), D = pr.head_dim;
     const size_t q_rows = P * n_qc * pr.cluster_q, k_rows = P * n_kc * pr.cluster_k;
     bytes += align_up(q_rows * D, 256) + align_up(q_rows * 4, 256) + align_up(k_rows * D, 256) +
-             align_up(P * n_kc * 4, 256) + align_up(P * cen_tiles * kHalf * D, 256) + align_up(P * cen_tiles * 4, 256);
+             align_up(P * n_kc * 4, 256) + align_up(P * cen_tiles * kCen * D, 256) + align_up(P * cen_tiles * 4, 256);
   }
   return bytes;
 }
 
 template <int D, bool F8>
-static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, dim3 grid, cudaStream_t st) {
+static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, cudaStream_t st) {
   using C = TcCfg<D, F8>;
-  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4 + (((size_t)prm.list_stride * 2 + 15) & ~(size_t)15) +
-                      (F8 ? (size_t)prm.list_stride * 4 : 0);
+  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4;
   auto k = attn_tc_kernel<D, F8>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k<<<grid, kTcThreads, smem, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], prm);
@@ -770,11 +946,11 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
                    cudaStream_t st) {
   const int P = pr.batch * pr.heads, D = pr.head_dim;
   const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
-  const int cen_tiles = ceil_div(n_kc, kHalf);
+  const int cen_tiles = ceil_div(n_kc, kCen);
   Carver c(ws);
   int* status = c.take<int>(kStatusBytes / sizeof(int));
   __nv_bfloat16* kmix = c.take<__nv_bfloat16>((size_t)P * cen_tiles * kTile * D);
-  __nv_bfloat16* vb = c.take<__nv_bfloat16>((size_t)P * cen_tiles * kHalf * D);
+  __nv_bfloat16* vb = c.take<__nv_bfloat16>((size_t)P * cen_tiles * kCen * D);
   int32_t* redo = c.take<int32_t>((size_t)P * n_qc * 2);
   const bool f8 = (pr.flags & CA_ATTN_FP8_QK) != 0;
   unsigned char *q8 = nullptr, *k8 = nullptr, *c8 = nullptr;
@@ -784,7 +960,7 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
     const size_t q_rows = (size_t)P * n_qc * pr.cluster_q, k_rows = (size_t)P * n_kc * pr.cluster_k;
     q8 = c.take<unsigned char>(q_rows * D);  sq = c.take<float>(q_rows);
     k8 = c.take<unsigned char>(k_rows * D);  sk = c.take<float>((size_t)P * n_kc);
-    c8 = c.take<unsigned char>((size_t)P * cen_tiles * kHalf * D);  sc = c.take<float>((size_t)P * cen_tiles);
+    c8 = c.take<unsigned char>((size_t)P * cen_tiles * kCen * D);  sc = c.take<float>((size_t)P * cen_tiles);
     ProfScope ps(kProfAttnPrep, st);
     const int rq = launch_quantize_qk(Qp, Kp, pr.compensate ? ck : nullptr, P, n_qc, pr.cluster_q, n_kc, pr.cluster_k,
                                       cen_tiles, D, q8, sq, k8, sk, c8, sc, st);
@@ -792,23 +968,23 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   }
   if (pr.compensate) {
     ProfScope ps(kProfAttnPrep, st);
-    centroid_prep_kernel<<<dim3(ceil_div(cen_tiles * kHalf * D, 256), P), 256, 0, st>>>(ck, cv, n_kc, cen_tiles, D,
+    centroid_prep_kernel<<<dim3(ceil_div(cen_tiles * kCen * D, 256), P), 256, 0, st>>>(ck, cv, n_kc, cen_tiles, D,
                                                                                         kmix, vb);
     CA_LAUNCH_CHECK();
   }
   CUtensorMap maps[5];
-  const int kbox = pr.cluster_k < kHalf ? pr.cluster_k : kHalf;      // key/value slots hold 64 rows
+  const int kbox = pr.cluster_k < kTile ? pr.cluster_k : kTile;
   const int qbox = pr.cluster_q < kTile ? pr.cluster_q : kTile;
   bool ok = make_map(&maps[2], Vp, (size_t)P * n_kc * pr.cluster_k, D, kbox) &&
-            make_map(&maps[4], vb, (size_t)P * cen_tiles * kHalf, D, kHalf);
+            make_map(&maps[4], vb, (size_t)P * cen_tiles * kCen, D, kCen);
   if (f8)
     ok = ok && make_map(&maps[0], q8, (size_t)P * n_qc * pr.cluster_q, D, qbox, true) &&
          make_map(&maps[1], k8, (size_t)P * n_kc * pr.cluster_k, D, kbox, true) &&
-         make_map(&maps[3], c8, (size_t)P * cen_tiles * kHalf, D, kHalf, true);
+         make_map(&maps[3], c8, (size_t)P * cen_tiles * kCen, D, kCen, true);
   else
     ok = ok && make_map(&maps[0], Qp, (size_t)P * n_qc * pr.cluster_q, D, qbox) &&
          make_map(&maps[1], Kp, (size_t)P * n_kc * pr.cluster_k, D, kbox) &&
-         make_map(&maps[3], kmix, (size_t)P * cen_tiles * kTile, D, kHalf);
+         make_map(&maps[3], kmix, (size_t)P * cen_tiles * kTile, D, kTile);
   if (!ok) return CA_ERR_CUDA;
   TcParams prm;
   prm.count_k = count_k; prm.block_idx = block_idx; prm.keep_count = keep_count; prm.perm_q = perm_q;
@@ -816,12 +992,18 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   prm.O = static_cast<__nv_bfloat16*>(O); prm.lse = lse; prm.status = status; prm.redo = redo;
   prm.n_q = pr.n_q; prm.n_k = pr.n_k; prm.c_q = pr.cluster_q; prm.c_k = pr.cluster_k; prm.keep = pr.keep;
   prm.n_qc = n_qc; prm.n_kc = n_kc; prm.cen_tiles = cen_tiles; prm.compensate = pr.compensate;
-  prm.bitmap_words = (cen_tiles * kHalf + 31) / 32;
+  prm.bitmap_words = (cen_tiles * kCen + 31) / 32;
   prm.scale_log2 = scale * 1.4426950408889634f;
   prm.wait_limit = g_wait_limit;
   prm.skip_key_load = g_skip_key_load;
   prm.q_scale = sq; prm.k_scale = sk; prm.c_scale = sc;
-  dim3 grid(n_qc * (pr.cluster_q >= kTile ? pr.cluster_q / kTile : 1), P);
+  const int tiles_per_qc = pr.cluster_q >= kTile ? pr.cluster_q / kTile : 1;
+  prm.n_tiles = P * n_qc * tiles_per_qc;
+  prm.next_tile = status + kTileWord;
+  int sms = 0, dev = 0;
+  CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
+  CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int grid = prm.n_tiles < sms ? prm.n_tiles : sms;
   int rc;
   {
     ProfScope ps(kProfAttn, st);
@@ -833,7 +1015,7 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   // second pass: query tiles whose scores left the range of the fast softmax (a climb of more than
   // 2^96 within 64 keys) are recomputed by the fp32 kernel; its CTAs return at once for the others
   return launch_attn_ref(pr, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, scale, O, lse,
-                         status, st, redo, (int)grid.x / n_qc, status + kRecomputedWord);
+                         status, st, redo, tiles_per_qc, status + kRecomputedWord);
 }
 
 }  // namespace ca
