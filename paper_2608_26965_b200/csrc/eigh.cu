@@ -6,7 +6,7 @@ namespace ca {
 
 // ---------------------------------------------------------------------------
 // Factor of a positive semi-definite matrix: lower-triangular F with F F^T = A
-// (right-looking Cholesky in double, one CTA of 1024 threads per matrix).  A pivot
+// (right-looking Cholesky in double, one CTA per matrix).  A pivot
 // that is not above 1e-12 of the largest diagonal entry marks a direction in
 // which the (pseudo-)metric is zero: its column of F is set to zero, which is the
 // counterpart of clamping small or negative eigenvalues (Section 3.2.2).
@@ -18,147 +18,166 @@ namespace ca {
 // Besides F in double and float, F^T can be written as bf16 hi + lo parts, the layout in which the
 // tensor-core projection takes its weights (the query representation multiplies by F).
 //
-// Thread (i, q) = (warp, lane) keeps the entries (i + 32 a, q + 32 b), a, b < d / 32, in registers
-// for the whole elimination: rows and columns both dealt out cyclically, so that the shrinking
-// trailing block stays spread over all threads.  A step is bound by the instructions it issues,
-// not by the arithmetic: with a whole row per eight threads every multiply-add came with a
-// shared-memory load and three index tests, a dozen instructions per entry; a tile takes d / 32
-// entries of column j for its rows and d / 32 for its columns, and the only tests left are
-// uniform ones per tile row and per step (the body of a step is compiled once per position of
-// column j among the tile columns, so that finished tile columns cost nothing).  Step j needs
-// column j, which its owners publish to shared memory during step j - 1 (right after their last
-// update of it), so a step takes one barrier; the trailing block takes
-// A[r][k] -= A[r][j] A[k][j] / pivot_j with the unscaled column, and the columns are scaled by
-// 1 / sqrt(pivot) at the end.  The one division of a step is made by the thread that completes
-// the next pivot, also a step ahead.  A dropped pivot (reciprocal 0) leaves the trailing block
-// alone and gives a zero column.  Entries above the diagonal inside a diagonal tile block take the
-// same updates as their mirror images; they are never read and are written as zeros.
+// The elimination goes by panels of eight columns.  One warp factors a panel with its rows in
+// registers and shuffles instead of barriers (the chain of a column: pivot, reciprocal, update), then all
+// threads take the eight columns off the trailing block at once: two barriers per eight columns.  With a
+// column and a barrier of 1,024 threads per step, and the one division of the step in its chain, a factor
+// took 26 us at d = 64 and 59 us at d = 128 (per launch); now 17.5 and 50.  Warp w keeps the entries (w + NW a, q + 32 b) of the trailing block in
+// registers, rows dealt out cyclically, so that the shrinking block stays spread over all warps and tests on
+// rows are uniform; finished columns stay in shared memory, unscaled, and are scaled by 1 / sqrt(pivot)
+// on the way out.  The trailing block takes A[r][k] -= A[r][j] A[k][j] / pivot_j with the unscaled columns;
+// a dropped pivot (reciprocal 0) leaves it alone and gives a zero column.
 // ---------------------------------------------------------------------------
-// One elimination step for the case that column j + 1 lies in tile column B0 (tile columns and
-// tile rows below B0 are final).
-template <int TB, int B0, typename T>
-__device__ __forceinline__ void cholesky_step(T (&a)[TB][TB], const T* __restrict__ col, T* __restrict__ col_next,
-                                              T* __restrict__ ip_next, T ip, T tol, int i, int q, int j) {
-  T c[TB];
-#pragma unroll
-  for (int tb = B0; tb < TB; ++tb) {
-    const int k = q + 32 * tb;
-    c[tb] = (tb > B0 || k > j) ? col[k] : (T)0;            // columns up to j are final: they take a - f * 0
-  }
-#pragma unroll
-  for (int ta = B0; ta < TB; ++ta) {
-    const int r = i + 32 * ta;
-    if (ta == B0 && r <= j) continue;                      // uniform over the warp: rows up to j are final
-    const T f = col[r] * ip;
-#pragma unroll
-    for (int tb = B0; tb <= ta; ++tb) a[ta][tb] -= f * c[tb];
-  }
-  if (q == ((j + 1) & 31)) {                               // column j + 1 is complete: publish it
-#pragma unroll
-    for (int ta = B0; ta < TB; ++ta) {
-      const int r = i + 32 * ta;
-      if (r > j) {
-        col_next[r] = a[ta][B0];
-        if (r == j + 1) *ip_next = a[ta][B0] > tol ? (T)1 / a[ta][B0] : (T)0;
-      }
-    }
-  }
+constexpr int kPanel = 8;
+
+// reciprocal by Newton's iteration on the hardware's estimate (relative error of a few 1e-16)
+__device__ __forceinline__ double reciprocal(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
 }
 
-template <int D, typename T>
-__global__ void __launch_bounds__(1024) cholesky_factor_kernel(const double* __restrict__ gram,
-                                                               const double* __restrict__ sum, double n,
-                                                               double scale, double* __restrict__ out64,
-                                                               float* __restrict__ out32,
-                                                               __nv_bfloat16* __restrict__ wt_hi,
-                                                               __nv_bfloat16* __restrict__ wt_lo) {
-  constexpr int TB = D / 32;       // rows and columns of a thread's tile
-  static_assert(TB >= 1 && TB <= 4, "tile of at most 4 x 4 entries per thread");
-  __shared__ T colbuf[2][D];       // column j of the trailing matrix, rows >= j (two in rotation)
-  __shared__ T pivots[D];          // diagonal entries; afterwards 1 / sqrt(pivot) per column
-  __shared__ T s_ip[2];
-  __shared__ T s_tol;
-  const T kDrop = sizeof(T) == 8 ? (T)1e-12 : (T)1e-6;   // share of the largest diagonal entry below which a pivot drops out
-  const int tid = threadIdx.x;
-  const int i = tid >> 5, q = tid & 31;
-  const double* G = gram + (size_t)blockIdx.x * D * D;
+template <int D>
+__global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __restrict__ gram,
+                                                                const double* __restrict__ sum, double n,
+                                                                double scale, double* __restrict__ out64,
+                                                                float* __restrict__ out32,
+                                                                __nv_bfloat16* __restrict__ wt_hi,
+                                                                __nv_bfloat16* __restrict__ wt_lo) {
+  constexpr int NT = 4 * D, NW = NT / 32;
+  constexpr int RT = D / NW, CT = D / 32;     // rows and columns of a thread's tile
+  constexpr int LD = D + 1;                   // pitch of a column
+  extern __shared__ __align__(16) double chol_smem[];
+  double* F = chol_smem;                      // [D][LD]  finished columns and the panel, column-major, unscaled
+  double* G = F + D * LD;                     // [kPanel][D]  panel columns over their pivots
+  double* pivots = G + kPanel * D;            // [D]
+  __shared__ double s_tol;
+  constexpr double kDrop = 1e-12;             // share of the largest diagonal entry below which a pivot drops out
+  const int tid = threadIdx.x, w = tid >> 5, q = tid & 31;
+  const double* A = gram + (size_t)blockIdx.x * D * D;
   const double* sm = sum ? sum + (size_t)blockIdx.x * D : nullptr;
-  T a[TB][TB];
+  double a[RT][CT];
+  const double per_n = sm ? scale / n : 0.0;
 #pragma unroll
-  for (int ta = 0; ta < TB; ++ta) {
-    const int r = i + 32 * ta;
+  for (int ta = 0; ta < RT; ++ta) {
+    const int r = w + NW * ta;
     // the centring needs double precision: the Gram matrix is n mean^2 + scatter
-    const double row_term = sm ? sm[r] * (scale / n) : 0.0;
+    const double row_term = sm ? sm[r] * per_n : 0.0;
 #pragma unroll
-    for (int tb = 0; tb < TB; ++tb) {
+    for (int tb = 0; tb < CT; ++tb) {
       const int k = q + 32 * tb;
-      a[ta][tb] = (T)0;
-      if (k <= r) a[ta][tb] = (T)(sm ? fma(-row_term, sm[k], G[r * D + k] * scale) : G[r * D + k] * scale);
+      a[ta][tb] = 0.0;
+      if (k <= r) a[ta][tb] = sm ? fma(-row_term, sm[k], A[r * D + k] * scale) : A[r * D + k] * scale;
       if (k == r) pivots[r] = a[ta][tb];
-      if (k == 0) colbuf[0][r] = a[ta][tb];
     }
   }
   __syncthreads();
   if (tid < 32) {
-    T mx = (T)0;
+    double mx = 0.0;
     for (int t = tid; t < D; t += 32) mx = max(mx, pivots[t]);
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (tid == 0) {
-      s_tol = kDrop * mx;
-      s_ip[0] = pivots[0] > kDrop * mx ? (T)1 / pivots[0] : (T)0;
-    }
+    if (tid == 0) s_tol = kDrop * mx;
   }
-  __syncthreads();
-  const T tol = s_tol;
-  for (int j = 0; j < D - 1; ++j) {
-    const T* col = colbuf[j & 1];
-    T* col_next = colbuf[(j + 1) & 1];
-    T* ip_next = &s_ip[(j + 1) & 1];
-    const T ip = s_ip[j & 1];
-    switch ((j + 1) >> 5) {                                // uniform over the CTA
-      case 0: cholesky_step<TB, 0>(a, col, col_next, ip_next, ip, tol, i, q, j); break;
-      case 1: if constexpr (TB > 1) cholesky_step<TB, 1>(a, col, col_next, ip_next, ip, tol, i, q, j); break;
-      case 2: if constexpr (TB > 2) cholesky_step<TB, 2>(a, col, col_next, ip_next, ip, tol, i, q, j); break;
-      default: if constexpr (TB > 3) cholesky_step<TB, 3>(a, col, col_next, ip_next, ip, tol, i, q, j); break;
+#pragma unroll 1
+  for (int p0 = 0; p0 < D; p0 += kPanel) {
+    // the panel's columns, from their owners to shared memory
+    const int b0 = p0 >> 5, at = q - (p0 & 31);
+    if (at >= 0 && at < kPanel) {
+#pragma unroll
+      for (int ta = 0; ta < RT; ++ta) {
+        double v = a[ta][0];
+#pragma unroll
+        for (int tb = 1; tb < CT; ++tb) v = tb == b0 ? a[ta][tb] : v;
+        F[(p0 + at) * LD + w + NW * ta] = v;
+      }
     }
     __syncthreads();
-  }
-  if (q == i) {
+    if (w == 0) {
+      const double tol = s_tol;
+      double x[CT][kPanel];                   // rows q + 32 s
 #pragma unroll
-    for (int t = 0; t < TB; ++t) pivots[i + 32 * t] = a[t][t];
-  }
-  __syncthreads();
-  if (tid < D) pivots[tid] = pivots[tid] > tol ? (T)rsqrt((double)pivots[tid]) : (T)0;
-  __syncthreads();
-  double* o64 = out64 + (size_t)blockIdx.x * D * D;
-  float* o32 = out32 ? out32 + (size_t)blockIdx.x * D * D : nullptr;
+      for (int s = 0; s < CT; ++s)
 #pragma unroll
-  for (int ta = 0; ta < TB; ++ta) {
-    const int r = i + 32 * ta;
+        for (int c = 0; c < kPanel; ++c) x[s][c] = F[(p0 + c) * LD + q + 32 * s];
 #pragma unroll
-    for (int tb = 0; tb < TB; ++tb) {
-      const int k = q + 32 * tb;
-      const double v = (k <= r) ? (double)(a[ta][tb] * pivots[k]) : 0.0;
-      o64[r * D + k] = v;
-      if (o32) o32[r * D + k] = (float)v;
-      if (wt_hi) {                                          // F^T [out k][in r] = F[r][k] as bf16 hi + lo
-        const float vf = (float)v;
-        const __nv_bfloat16 h = __float2bfloat16_rn(vf);
-        wt_hi[(size_t)blockIdx.x * D * D + (size_t)k * D + r] = h;
-        wt_lo[(size_t)blockIdx.x * D * D + (size_t)k * D + r] = __float2bfloat16_rn(vf - __bfloat162float(h));
+      for (int c = 0; c < kPanel; ++c) {
+        // rows p0 .. p0 + 7 of the panel lie in slot b0 of eight neighbouring lanes
+        double own = x[0][c];
+#pragma unroll
+        for (int s = 1; s < CT; ++s) own = s == b0 ? x[s][c] : own;
+        const double pivot = __shfl_sync(0xffffffffu, own, (p0 + c) & 31);
+        double head[kPanel];
+#pragma unroll
+        for (int k = c + 1; k < kPanel; ++k) head[k] = __shfl_sync(0xffffffffu, own, (p0 + k) & 31);
+        const double ip = pivot > tol ? reciprocal(pivot) : 0.0;
+#pragma unroll
+        for (int s = 0; s < CT; ++s) {
+          const double f = x[s][c] * ip;
+#pragma unroll
+          for (int k = c + 1; k < kPanel; ++k) x[s][k] = fma(-f, head[k], x[s][k]);
+          F[(p0 + c) * LD + q + 32 * s] = x[s][c];
+          G[c * D + q + 32 * s] = f;
+        }
+        if (q == 0) pivots[p0 + c] = pivot > tol ? pivot : 0.0;
+      }
+    }
+    __syncthreads();
+    // trailing block: columns from p0 + 8 on
+#pragma unroll
+    for (int half = 0; half < kPanel; half += 4) {
+      double cv[CT][4];
+#pragma unroll
+      for (int tb = 0; tb < CT; ++tb)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) cv[tb][c] = q + 32 * tb >= p0 + kPanel ? F[(p0 + half + c) * LD + q + 32 * tb] : 0.0;
+#pragma unroll
+      for (int ta = 0; ta < RT; ++ta) {
+        const int r = w + NW * ta;
+        if (r < p0 + kPanel) continue;        // uniform over the warp
+        double f[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) f[c] = G[(half + c) * D + r];
+#pragma unroll
+        for (int tb = 0; tb < CT; ++tb) {
+          if (32 * tb > r || 32 * tb + 31 < p0 + kPanel) continue;   // uniform: above the diagonal, or finished
+#pragma unroll
+          for (int c = 0; c < 4; ++c) a[ta][tb] = fma(-f[c], cv[tb][c], a[ta][tb]);
+        }
       }
     }
   }
+  __syncthreads();
+  if (tid < D) pivots[tid] = pivots[tid] > 0.0 ? rsqrt(pivots[tid]) : 0.0;
+  __syncthreads();
+  const size_t mat = (size_t)blockIdx.x * D * D;
+#pragma unroll 4
+  for (int e = tid; e < D * D; e += NT) {
+    const int r = e / D, k = e % D;
+    const double v = k <= r ? F[k * LD + r] * pivots[k] : 0.0;
+    out64[mat + e] = v;
+    if (out32) out32[mat + e] = (float)v;
+  }
+  if (wt_hi) {                                // F^T [out k][in r] = F[r][k] as bf16 hi + lo
+#pragma unroll 4
+    for (int e = tid; e < D * D; e += NT) {
+      const int k = e / D, r = e % D;
+      const float vf = k <= r ? (float)(F[k * LD + r] * pivots[k]) : 0.f;
+      const __nv_bfloat16 h = __float2bfloat16_rn(vf);
+      wt_hi[mat + e] = h;
+      wt_lo[mat + e] = __float2bfloat16_rn(vf - __bfloat162float(h));
+    }
+  }
 }
-
-typedef double CholT;   // arithmetic of the elimination (float32 was measured: no faster, and less exact)
 
 int launch_cholesky_factor(const double* gram, const double* sum, double n, double scale, int count, int D,
                            double* out64, float* out32, void* wt_hi, void* wt_lo, cudaStream_t st) {
   __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(wt_hi);
   __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(wt_lo);
-  if (D == 64) cholesky_factor_kernel<64, CholT><<<count, 1024, 0, st>>>(gram, sum, n, scale, out64, out32, hi, lo);
-  else cholesky_factor_kernel<128, CholT><<<count, 1024, 0, st>>>(gram, sum, n, scale, out64, out32, hi, lo);
+  const size_t smem = sizeof(double) * ((size_t)D * (D + 1) + kPanel * D + D);
+  auto k = D == 64 ? cholesky_factor_kernel<64> : cholesky_factor_kernel<128>;
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<count, 4 * D, smem, st>>>(gram, sum, n, scale, out64, out32, hi, lo);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
