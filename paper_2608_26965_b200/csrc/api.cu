@@ -107,7 +107,8 @@ ClusterWs carve_cluster(const ca_problem_t* p, void* base, bool need_yq, bool ne
     w.WK32 = c.take<float>(P * DD);
     w.biasK = c.take<float>(P * D);
     w.biasQ = c.take<float>(P * D);
-    w.Qprime = c.take<float>(P * (size_t)p->n_q * D);
+    // r(q) of fp32 storage; the tensor-core kernels of bf16 storage recompute it
+    if (p->dtype == CA_DTYPE_FP32) w.Qprime = c.take<float>(P * (size_t)p->n_q * D);
     w.wt_hi = c.take<__nv_bfloat16>(P * DD);
     w.wt_lo = c.take<__nv_bfloat16>(P * DD);
     w.wt2_hi = c.take<__nv_bfloat16>(P * DD);
@@ -242,8 +243,6 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     float* yk_out = Yk ? Yk : w.Yk;
     // bf16 storage runs the O(n d^2) passes on the tensor cores; fp32 storage on the CUDA cores
     const bool tc = p->dtype == CA_DTYPE_BF16;
-    __nv_bfloat16* qp_hi = reinterpret_cast<__nv_bfloat16*>(w.Qprime);          // r(q) as bf16 hi + lo parts
-    __nv_bfloat16* qp_lo = qp_hi + (size_t)P * p->n_q * D;
     // Factors F_q F_q^T = M = Q^T Q / n_q and F_k F_k^T = C_K (Section 3.2.2; they stand in for the
     // symmetric roots: any factor yields the same principal-component coordinates).  The
     // un-normalised query representation (Appendix B.1) takes the root of K_c^T K_c / n_k, the
@@ -270,8 +269,8 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     {
       ProfScope ps(kProfGram, st);
       if (tc) {
-        CA_TRY(launch_gram_tc(Q, nullptr, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, st));
-        CA_TRY(launch_gram_tc(K, nullptr, P, p->n_k, D, w.partial2, w.gramK, w.sumK, w.status, sq));
+        CA_TRY(launch_gram_tc(Q, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, st));
+        CA_TRY(launch_gram_tc(K, P, p->n_k, D, w.partial2, w.gramK, w.sumK, w.status, sq));
       } else {
         CA_TRY(launch_moments(Q, p->dtype, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, st));
         CA_TRY(launch_moments(K, p->dtype, P, p->n_k, D, w.partial2, w.gramK, w.sumK, sq));
@@ -286,21 +285,21 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     }
     // ---- query side (side stream)
     // query representation r(q) = F_k^T q / |F_k^T q|, its covariance and principal components E_Q
-    // (one kernel), the coordinates Y = (r(q) - mean) E_Q
+    // (one kernel), the coordinates Y = (r(q) - mean) E_Q.  fp32 storage keeps r(q); bf16 storage
+    // sums its moments without storing it and projects from Q once more: E_Q is orthogonal, so
+    // r(q) E_Q = q W / |q W| with W = F_k E_Q.  Reading Q (2 d bytes per row) twice replaces writing and
+    // twice reading r(q) in 4 d bytes.
     float* EQ32 = w.basis32 + (size_t)P * DD;
     {
       ProfScope ps(kProfTransform, sq);
-      if (tc) {
-        CA_TRY(launch_transform_tc(Q, nullptr, P, p->n_q, D, Fk32, nullptr, unnormalized ? 0 : 1, nullptr, qp_hi, qp_lo,
-                                   w.wt2_hi, w.wt2_lo, w.status, sq, nullptr, true));
-      } else {
+      if (!tc)
         CA_TRY(launch_transform_rows(Q, p->dtype, P, p->n_q, D, Fk32, nullptr, unnormalized ? 0 : 1, w.Qprime, sq));
-      }
     }
     {
       ProfScope ps(kProfGram, sq);
       if (tc) {
-        CA_TRY(launch_gram_tc(qp_hi, qp_lo, P, p->n_q, D, w.partial2, w.gramQp, w.sumQp, w.status, sq));
+        CA_TRY(launch_rep_gram_tc(Q, P, p->n_q, D, unnormalized ? 0 : 1, w.partial2, w.gramQp, w.sumQp, w.wt2_hi,
+                                  w.wt2_lo, w.status, sq));
       } else {
         CA_TRY(launch_moments(w.Qprime, CA_DTYPE_FP32, P, p->n_q, D, w.partial2, w.gramQp, w.sumQp, sq));
       }
@@ -310,8 +309,8 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
       PcaArgs a{};
       a.mode = kPcaQueries;
       a.gram = w.gramQp; a.sum = w.sumQp; a.n = (double)p->n_q;
-      a.lift = Fk; a.out_lifted = 0;
-      a.mean_sum = w.sumQp; a.mean_n = (double)p->n_q;
+      a.lift = Fk; a.out_lifted = tc ? 1 : 0;
+      a.mean_sum = w.sumQp; a.mean_n = (double)p->n_q; a.mean_lifted = 1;
       a.W32 = EQ32; a.bias = w.biasQ;
       a.wt_hi = tc ? w.wt2_hi : nullptr; a.wt_lo = tc ? w.wt2_lo : nullptr;
       CA_TRY(launch_pca(a, P, D, sq));
@@ -319,8 +318,8 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     {
       ProfScope ps(kProfTransform, sq);
       if (tc) {
-        CA_TRY(launch_transform_tc(qp_hi, qp_lo, P, p->n_q, D, EQ32, w.biasQ, 0, yq_out, nullptr, nullptr, w.wt2_hi,
-                                   w.wt2_lo, w.status, sq, w.Ytq, true));
+        CA_TRY(launch_transform_tc(Q, P, p->n_q, D, w.biasQ, unnormalized ? 0 : 1, yq_out, w.wt2_hi, w.wt2_lo,
+                                   w.status, sq, w.Ytq));
       } else {
         CA_TRY(launch_transform_rows(w.Qprime, CA_DTYPE_FP32, P, p->n_q, D, EQ32, w.biasQ, 0, yq_out, sq));
       }
@@ -351,8 +350,7 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     {
       ProfScope ps(kProfTransform, st);
       if (tc) {
-        CA_TRY(launch_transform_tc(K, nullptr, P, p->n_k, D, w.WK32, w.biasK, 0, yk_out, nullptr, nullptr, w.wt_hi,
-                                   w.wt_lo, w.status, st, w.Ytk, true));
+        CA_TRY(launch_transform_tc(K, P, p->n_k, D, w.biasK, 0, yk_out, w.wt_hi, w.wt_lo, w.status, st, w.Ytk));
       } else {
         CA_TRY(launch_transform_rows(K, p->dtype, P, p->n_k, D, w.WK32, w.biasK, 0, yk_out, st));
       }
@@ -524,8 +522,8 @@ int cluster_qk_basic(const ca_problem_t* p, const void* Q, const void* K, const 
   if (!(p->flags & CA_METRIC_IN)) {
     // keys are compared in the query metric Q^T Q / n_q, queries in K_c^T K_c / n_k (Section 3.2.2)
     if (p->dtype == CA_DTYPE_BF16) {
-      CA_TRY(launch_gram_tc(Q, nullptr, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, st));
-      CA_TRY(launch_gram_tc(K, nullptr, P, p->n_k, D, w.partial, w.gramK, w.sumK, w.status, st));
+      CA_TRY(launch_gram_tc(Q, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, st));
+      CA_TRY(launch_gram_tc(K, P, p->n_k, D, w.partial, w.gramK, w.sumK, w.status, st));
     } else {
       CA_TRY(launch_moments(Q, p->dtype, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, st));
       CA_TRY(launch_moments(K, p->dtype, P, p->n_k, D, w.partial, w.gramK, w.sumK, st));

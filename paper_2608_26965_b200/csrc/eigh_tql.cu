@@ -946,14 +946,15 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
       const double other = lam[k];
       rank += (other > mine) || (other == mine && k < tid);
     }
-    // sign rule on column tid of F E (of E when no factor is given); bias = -mean . (output column)
+    // sign rule on column tid of F E (of E when no factor is given); bias = -mean . that column, or
+    // . column tid of E where the mean is one of transformed rows
     float best = -1.f, sgn = 1.f, dot = 0.f;
 #pragma unroll 8
     for (int i = 0; i < D; ++i) {
       const float e_i = Qt[tid * LDA + i];
       const float w_i = a.lift ? A[i * LDA + tid] : e_i;
       if (fabsf(w_i) > best) { best = fabsf(w_i); sgn = (w_i < 0.f) ? -1.f : 1.f; }
-      dot = fmaf(mean[i], lifted_out ? w_i : e_i, dot);
+      dot = fmaf(mean[i], a.mean_lifted ? e_i : w_i, dot);
     }
     rank_of[tid] = rank;
     sign_of[tid] = sgn;

@@ -17,12 +17,14 @@ int launch_gram_finalize(const float* partial, int problems, int n_chunks, int D
                          double* colsum, cudaStream_t st);
 
 // tc_linear.cu (bf16 storage: tensor-core versions of the two kernels above)
-int launch_gram_tc(const void* X_hi, const void* X_lo, int problems, int n_rows, int D, float* partial,
-                   double* gram, double* colsum, int* status, cudaStream_t st);
-int launch_transform_tc(const void* X_hi, const void* X_lo, int problems, int n_rows, int D, const float* W,
-                        const float* bias, int normalize, float* out, void* out_hi, void* out_lo,
-                        void* wt_hi, void* wt_lo, int* status, cudaStream_t st, float* out_t = nullptr,
-                        bool weights_ready = false);
+int launch_gram_tc(const void* X, int problems, int n_rows, int D, float* partial, double* gram, double* colsum,
+                   int* status, cudaStream_t st);
+// Gram matrix and column sums of the rows x W (divided by their norm when `normalize`); W as bf16 hi + lo parts
+int launch_rep_gram_tc(const void* X, int problems, int n_rows, int D, int normalize, float* partial, double* gram,
+                       double* colsum, const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st);
+// out = x W (divided by the row's norm when `normalize`) + bias
+int launch_transform_tc(const void* X, int problems, int n_rows, int D, const float* bias, int normalize, float* out,
+                        const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st, float* out_t = nullptr);
 
 // eigh_tql.cu: covariance + principal components + projection matrix of one side, one CTA per head
 enum { kPcaMatrix = 0, kPcaKeys = 1, kPcaQueries = 2 };
@@ -39,8 +41,9 @@ struct PcaArgs {
                             // column t of F E); null: the sign rule applies to E itself
   int out_lifted;           // 1: the projection written is F E (rows are projected from the original
                             // space); 0: E (rows are already transformed)
-  const double* mean_sum;   // [P][D] column sums of the rows that will be projected, and their count:
-  double mean_n;            //   bias = -(mean_sum / mean_n) . projection   (null: zero bias)
+  const double* mean_sum;   // [P][D] column sums of the rows, and their count (null: zero bias):
+  double mean_n;            //   bias = -(mean_sum / mean_n) . F E,
+  int mean_lifted;          //   or . E where the sums are of transformed rows
   float* W32;               // [P][D in][D out] projection matrix
   float* bias;              // [P][D] or null
   __nv_bfloat16* wt_hi;     // [P][D out][D in] transposed projection as bf16 hi + lo parts, or null

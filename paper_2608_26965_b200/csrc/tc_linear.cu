@@ -1,10 +1,11 @@
 // Tensor-core (tcgen05 + TMEM + TMA) kernels for the tall-skinny linear algebra
 // of the clustering stage (Section 3.2.2 metric matrices, Section 3.2.1
 // covariance and projection on the principal components):
-//   gram_tc       G = X^T X and column sums of X   (X [N, d] bf16, optionally hi + lo parts)
-//   transform_tc  Y = g(X W + b), g = identity or row normalisation
-//                 (W [d, d] fp32 used as bf16 hi + lo parts; Y fp32, or bf16 hi + lo parts)
-// A value v stored as hi + lo (hi = bf16(v), lo = bf16(v - hi)) keeps 16 bits of
+//   gram_tc       G = X^T X and column sums of X   (X [N, d] bf16)
+//   transform_tc  Y = g(X W) + b, g = identity or row normalisation
+//                 (W [d, d] fp32 used as bf16 hi + lo parts; Y fp32)
+//   rep_gram_tc   G = R^T R and column sums of R = g(X W), R never written to memory
+// A value v kept as hi + lo (hi = bf16(v), lo = bf16(v - hi)) keeps 16 bits of
 // mantissa; products use hi*hi + hi*lo + lo*hi with fp32 accumulation.
 #include "kernels.h"
 #include "tc_ptx.cuh"
@@ -46,19 +47,43 @@ struct GramCfg {
 struct GramParams {
   float* partial;        // [(p * n_chunks + chunk) * (D*D + D)]
   int* status;
-  int n_rows, chunk_rows, n_chunks, has_lo, stages;
+  int n_rows, chunk_rows, n_chunks, stages, normalize;    // normalize: of the representation
 };
+
+// One of the four epilogue warps writes its rows of the accumulated Gram matrix and column sums.
+template <int D>
+__device__ __forceinline__ void write_gram(uint32_t tmem_acc, uint32_t tmem_sum, int quarter, int lane, bool any,
+                                           float* __restrict__ out) {
+  // accumulator row m sits in lane m (D = 128) or in lane (m % 16) + 32 (m / 16) (D = 64)
+  const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+  const int m = D == 128 ? quarter * 32 + lane : quarter * 16 + lane;
+  const bool live = any && (D == 128 || lane < 16);
+#pragma unroll
+  for (int c4 = 0; c4 < D / 32; ++c4) {
+    uint32_t v[32];
+    tmem_ld32(tmem_acc + lane_addr + c4 * 32, v);
+    tmem_wait_ld();
+    if (live) {
+      float4* dst = reinterpret_cast<float4*>(out + m * D + c4 * 32);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        dst[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                             __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+    }
+  }
+  const uint32_t sum = tmem_ld1(tmem_sum + lane_addr);     // one of 16 identical sums
+  tmem_wait_ld();
+  if (live) out[D * D + m] = __uint_as_float(sum);
+}
 
 template <int D>
 __global__ void __launch_bounds__(kLinThreads, 1)
-gram_tc_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
-               const GramParams prm) {
+gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const GramParams prm) {
   using C = GramCfg<D>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
-  const int parts = prm.has_lo ? 2 : 1;
-  const int stage_bytes = parts * C::TILE_BYTES;
+  constexpr int stage_bytes = C::TILE_BYTES;
   const uint32_t s_base = smem_u32(smem);
   const uint32_t s_ones = s_base + prm.stages * stage_bytes;                // 2 KB of bf16 1.0
   const uint32_t bar0 = s_ones + 2048;
@@ -100,11 +125,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
         if (!ok) break;
         mbar_expect_tx(b_full(s), stage_bytes);
         const uint32_t dst = s_base + s * stage_bytes;
-        for (int pn = 0; pn < C::PANELS; ++pn) {
-          tma_load_3d(dst + pn * C::PANEL_BYTES, &tm_hi, pn * 64, r_begin + t * kRows, p, b_full(s));
-          if (prm.has_lo)
-            tma_load_3d(dst + C::TILE_BYTES + pn * C::PANEL_BYTES, &tm_lo, pn * 64, r_begin + t * kRows, p, b_full(s));
-        }
+        for (int pn = 0; pn < C::PANELS; ++pn)
+          tma_load_3d(dst + pn * C::PANEL_BYTES, &tm_x, pn * 64, r_begin + t * kRows, p, b_full(s));
       }
     }
   } else if (warp == 1) {
@@ -117,21 +139,15 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
         ok = mbar_wait(b_full(s), (t / prm.stages) & 1, abort_flag, prm.status);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t hi = s_base + s * stage_bytes, lo = hi + C::TILE_BYTES;
+        const uint32_t x = s_base + s * stage_bytes;
 #pragma unroll
         for (int ks = 0; ks < kRows / 16; ++ks) {
           // 16 rows (the contraction index) per step = 2048 bytes; 64-column panels along M and N
-          const uint64_t dh = smem_desc_sw128(hi + ks * 2048, C::PANEL_BYTES, 1024);
+          const uint64_t dh = smem_desc_sw128(x + ks * 2048, C::PANEL_BYTES, 1024);
           const uint64_t ones = smem_desc_sw128(s_ones, C::PANEL_BYTES, 1024);
           const uint32_t acc = (t > 0 || ks > 0) ? 1u : 0u;
           mma_ss(tmem_acc, dh, dh, idesc, acc);
           mma_ss(tmem_sum, dh, ones, idesc_sum, acc);
-          if (prm.has_lo) {
-            const uint64_t dl = smem_desc_sw128(lo + ks * 2048, C::PANEL_BYTES, 1024);
-            mma_ss(tmem_acc, dh, dl, idesc, 1u);
-            mma_ss(tmem_acc, dl, dh, idesc, 1u);
-            mma_ss(tmem_sum, dl, ones, idesc_sum, 1u);
-          }
         }
         mma_commit(b_empty(s));
       }
@@ -139,31 +155,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant_
     }
   } else {
     const int quarter = warp & 3;
-    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const bool ok = __all_sync(0xffffffffu, mbar_wait(b_done, 0, abort_flag, prm.status));
     tc_fence_after();
     if (ok) {
-      // accumulator row m sits in lane m (M = 128) or in lane (m % 16) + 32 (m / 16) (M = 64)
-      const int m = (C::M == 128) ? quarter * 32 + lane : quarter * 16 + lane;
-      const bool live = (C::M == 128) || lane < 16;
-      float* out = prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D);
-#pragma unroll
-      for (int c4 = 0; c4 < D / 32; ++c4) {
-        uint32_t v[32];
-        tmem_ld32(tmem_acc + lane_addr + c4 * 32, v);
-        tmem_wait_ld();
-        if (live && n_tiles > 0) {
-          float4* dst = reinterpret_cast<float4*>(out + m * D + c4 * 32);
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            dst[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                 __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-        }
-      }
-      uint32_t sv[32];
-      tmem_ld32(tmem_sum + lane_addr, sv);          // 16 identical sums; columns beyond are unused
-      tmem_wait_ld();
-      if (live && n_tiles > 0) out[D * D + m] = __uint_as_float(sv[0]);
+      write_gram<D>(tmem_acc, tmem_sum, quarter, lane, n_tiles > 0,
+                    prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D));
     }
   }
   tc_fence_before();
@@ -181,28 +177,26 @@ struct LinCfg {
   static constexpr int TILE_BYTES = PANELS * PANEL_BYTES;       // one part of an X tile
   static constexpr int W_PANEL_BYTES = D * 128;                 // W^T panels: D rows x 128 bytes
   static constexpr int W_BYTES = PANELS * W_PANEL_BYTES;        // one part of W^T
-  static constexpr int OUT_BYTES = kRows * D * 4;               // fp32 tile, or hi + lo bf16 tiles
+  static constexpr int OUT_BYTES = kRows * D * 4;               // fp32 tile
 };
 
 struct LinParams {
   const float* bias;      // [P][D] or null
   float* out_t;           // [P][D][n_rows] or null: the fp32 result once more, coordinate-major
   int* status;
-  int n_rows, tiles_per_cta, has_lo, stages, normalize, out_split;
+  int n_rows, tiles_per_cta, stages, normalize;       // normalize: rows are divided by their norm before the bias
 };
 
 template <int D>
 __global__ void __launch_bounds__(kLinThreads, 1)
-transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_constant__ CUtensorMap tm_xlo,
-                    const __grid_constant__ CUtensorMap tm_whi, const __grid_constant__ CUtensorMap tm_wlo,
-                    const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ CUtensorMap tm_out_lo,
+transform_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_whi,
+                    const __grid_constant__ CUtensorMap tm_wlo, const __grid_constant__ CUtensorMap tm_out,
                     const LinParams prm) {
   using C = LinCfg<D>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
-  const int parts = prm.has_lo ? 2 : 1;
-  const int stage_bytes = parts * C::TILE_BYTES;
+  constexpr int stage_bytes = C::TILE_BYTES;
   const uint32_t s_base = smem_u32(smem);
   const uint32_t s_w = s_base;                                   // W^T hi, W^T lo
   const uint32_t s_x = s_w + 2 * C::W_BYTES;
@@ -256,8 +250,7 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
         const uint32_t dst = s_x + s * stage_bytes;
         const int row = (t_begin + t) * kRows;
         for (int pn = 0; pn < C::PANELS; ++pn) {
-          tma_load_3d(dst + pn * C::PANEL_BYTES, &tm_xhi, pn * 64, row, p, b_full(s));
-          if (prm.has_lo) tma_load_3d(dst + C::TILE_BYTES + pn * C::PANEL_BYTES, &tm_xlo, pn * 64, row, p, b_full(s));
+          tma_load_3d(dst + pn * C::PANEL_BYTES, &tm_x, pn * 64, row, p, b_full(s));
         }
       }
     }
@@ -271,7 +264,7 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
         if (ok) ok = mbar_wait(b_full(s), (t / prm.stages) & 1, abort_flag, prm.status);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t xh = s_x + s * stage_bytes, xl = xh + C::TILE_BYTES;
+        const uint32_t xh = s_x + s * stage_bytes;
         const uint32_t acc = tmem_base + a * D;
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
@@ -282,7 +275,6 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
           const uint64_t dwl = smem_desc_sw128(s_w + C::W_BYTES + wo, 16, 1024);
           mma_ss(acc, dxh, dwh, idesc, ks > 0 ? 1u : 0u);
           mma_ss(acc, dxh, dwl, idesc, 1u);
-          if (prm.has_lo) mma_ss(acc, smem_desc_sw128(xl + xo, 16, 1024), dwh, idesc, 1u);
         }
         mma_commit(b_empty(s));
         mma_commit(b_acc_full(a));
@@ -306,7 +298,7 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
         tmem_ld32(tmem_base + a * D + lane_addr + c4 * 32, r);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[c4 * 32 + j] = __uint_as_float(r[j]) + s_bias[c4 * 32 + j];
+        for (int j = 0; j < 32; ++j) v[c4 * 32 + j] = __uint_as_float(r[j]);
       }
       tc_fence_before();
       mbar_arrive(b_acc_empty(a));                    // the accumulator may be overwritten
@@ -317,7 +309,10 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
         const float nrm = sqrtf(ss);
         const float inv = nrm >= 1e-30f ? 1.f / nrm : 0.f;
 #pragma unroll
-        for (int j = 0; j < D; ++j) v[j] *= inv;
+        for (int j = 0; j < D; ++j) v[j] = fmaf(v[j], inv, s_bias[j]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < D; ++j) v[j] += s_bias[j];
       }
       if (prm.out_t) {
         // coordinate-major copy: for one coordinate the 128 threads of the tile write 512
@@ -334,46 +329,19 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
       // the previous tile's stores must have finished reading the staging buffer
       if (st == 0) tma_store_wait_read();
       asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (!prm.out_split) {
-        // fp32 tile as 32-column panels with the 128-byte swizzle the store expects
+      // fp32 tile as 32-column panels with the 128-byte swizzle the store expects
 #pragma unroll
-        for (int pn = 0; pn < D / 32; ++pn)
+      for (int pn = 0; pn < D / 32; ++pn)
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            float4 w = make_float4(v[pn * 32 + 4 * c], v[pn * 32 + 4 * c + 1], v[pn * 32 + 4 * c + 2], v[pn * 32 + 4 * c + 3]);
-            *reinterpret_cast<float4*>(out_ptr + pn * 16384 + row * 128 + ((c ^ (row & 7)) * 16)) = w;
-          }
-      } else {
-        // bf16 hi and lo tiles as 64-column panels
-#pragma unroll
-        for (int pn = 0; pn < D / 64; ++pn)
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            uint32_t h[4], l[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float x0 = v[pn * 64 + 8 * c + 2 * j], x1 = v[pn * 64 + 8 * c + 2 * j + 1];
-              const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-              h[j] = pack_bf16x2(__bfloat162float(h0), __bfloat162float(h1));
-              l[j] = pack_bf16x2(x0 - __bfloat162float(h0), x1 - __bfloat162float(h1));
-            }
-            const int off = pn * 16384 + row * 128 + ((c ^ (row & 7)) * 16);
-            *reinterpret_cast<uint4*>(out_ptr + off) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(out_ptr + C::OUT_BYTES / 2 + off) = make_uint4(l[0], l[1], l[2], l[3]);
-          }
-      }
+        for (int c = 0; c < 8; ++c) {
+          float4 w = make_float4(v[pn * 32 + 4 * c], v[pn * 32 + 4 * c + 1], v[pn * 32 + 4 * c + 2], v[pn * 32 + 4 * c + 3]);
+          *reinterpret_cast<float4*>(out_ptr + pn * 16384 + row * 128 + ((c ^ (row & 7)) * 16)) = w;
+        }
       fence_proxy_async();
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (st == 0) {
         const int grow = (t_begin + t) * kRows;
-        if (!prm.out_split) {
-          for (int pn = 0; pn < D / 32; ++pn) tma_store_3d(&tm_out, pn * 32, grow, p, s_out + pn * 16384);
-        } else {
-          for (int pn = 0; pn < D / 64; ++pn) {
-            tma_store_3d(&tm_out, pn * 64, grow, p, s_out + pn * 16384);
-            tma_store_3d(&tm_out_lo, pn * 64, grow, p, s_out + C::OUT_BYTES / 2 + pn * 16384);
-          }
-        }
+        for (int pn = 0; pn < D / 32; ++pn) tma_store_3d(&tm_out, pn * 32, grow, p, s_out + pn * 16384);
         tma_store_commit();
       }
     }
@@ -384,17 +352,211 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_xhi, const __grid_con
   if (warp == 1) tmem_dealloc(tmem_base, kCols);
 }
 
-// W [P][D in][D out] fp32  ->  W^T hi / lo [P][D out][D in] bf16
-__global__ void weight_prep_kernel(const float* __restrict__ W, int D, __nv_bfloat16* __restrict__ hi,
-                                   __nv_bfloat16* __restrict__ lo) {
-  const int p = blockIdx.y;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= D * D) return;
-  const int n = e / D, k = e % D;
-  const float w = W[(size_t)p * D * D + k * D + n];
-  const __nv_bfloat16 h = __float2bfloat16_rn(w);
-  hi[(size_t)p * D * D + e] = h;
-  lo[(size_t)p * D * D + e] = __float2bfloat16_rn(w - __bfloat162float(h));
+// ===========================================================================
+// Gram matrix and column sums of the row representation R = g(X W), g = identity or division by the row's norm
+// ===========================================================================
+// Two chained products per tile of 128 rows: T = X W into tensor memory, from where the epilogue
+// warps normalise a row per thread and write it to shared memory as H + L, bf16 hi + lo parts in the
+// layout of a loaded tile, then the Gram matrix.  H^T H + H^T 2L is what is accumulated: its
+// symmetric part is H^T H + H^T L + L^T H, and the decomposition takes the symmetric part of what it is given.
+// T of the next tile is issued before R of this one is waited for.
+// r(q) used to be written by the row transform and read back by its Gram matrix and by the projection
+// (12 d bytes per row): the query side of 40 heads of 32,760 rows, d = 128, took 0.63 ms in these
+// kernels and takes 0.39.
+template <int D>
+struct RepCfg {
+  static constexpr int PANELS = D / 64;
+  static constexpr int PANEL_BYTES = kRows * 128;
+  static constexpr int TILE_BYTES = PANELS * PANEL_BYTES;
+  static constexpr int W_PANEL_BYTES = D * 128;
+  static constexpr int W_BYTES = PANELS * W_PANEL_BYTES;
+  static constexpr int STAGES = D == 64 ? 3 : 2;
+  static constexpr int OFF_X = 2 * W_BYTES;
+  static constexpr int OFF_R = OFF_X + STAGES * TILE_BYTES;             // hi tile, 2 lo tile
+  static constexpr int OFF_ONES = OFF_R + 2 * TILE_BYTES;               // 2 KB of bf16 1.0, 2 KB of 0.5
+  static constexpr int OFF_BAR = OFF_ONES + 4096;
+  static constexpr int NUM_BARS = 2 + 2 * STAGES + 4 + 2;               // weights, done; x full/empty; acc full/empty x 2; r full/empty
+  static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
+  static constexpr int SMEM = 1024 + OFF_MISC + 16;
+  static constexpr uint32_t TMEM_COLS = D == 64 ? 256 : 512;            // two T accumulators, G, sums
+  static constexpr int CTAS_PER_SM = D == 64 ? 2 : 1;
+};
+
+template <int D>
+__global__ void __launch_bounds__(kLinThreads, 1)
+rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_whi,
+                   const __grid_constant__ CUtensorMap tm_wlo, const GramParams prm) {
+  using C = RepCfg<D>;
+  extern __shared__ unsigned char smem_unaligned[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
+  const uint32_t s_base = smem_u32(smem);
+  const uint32_t s_w = s_base, s_x = s_base + C::OFF_X, s_r = s_base + C::OFF_R, s_ones = s_base + C::OFF_ONES;
+  unsigned char* r_ptr = smem + C::OFF_R;
+  const uint32_t bar0 = s_base + C::OFF_BAR;
+  const uint32_t b_w = bar0, b_done = bar0 + 8;
+  auto b_full = [&](int s) { return bar0 + 16 + 8 * s; };
+  auto b_empty = [&](int s) { return bar0 + 16 + 8 * (C::STAGES + s); };
+  auto b_acc_full = [&](int a) { return bar0 + 16 + 8 * (2 * C::STAGES + a); };
+  auto b_acc_empty = [&](int a) { return bar0 + 16 + 8 * (2 * C::STAGES + 2 + a); };
+  const uint32_t b_r_full = bar0 + 16 + 8 * (2 * C::STAGES + 4), b_r_empty = b_r_full + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int p = blockIdx.y, chunk = blockIdx.x;
+  const int r_begin = chunk * prm.chunk_rows;
+  const int r_end = min(prm.n_rows, r_begin + prm.chunk_rows);
+  const int n_tiles = (r_end - r_begin + kRows - 1) / kRows;
+
+  if (tid == 0) {
+    mbar_init(b_w, 1);
+    mbar_init(b_done, 1);
+    for (int s = 0; s < C::STAGES; ++s) { mbar_init(b_full(s), 1); mbar_init(b_empty(s), 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(b_acc_full(a), 1); mbar_init(b_acc_empty(a), 4); }
+    mbar_init(b_r_full, 4);
+    mbar_init(b_r_empty, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  for (int e = tid; e < 2048; e += kLinThreads)
+    reinterpret_cast<__nv_bfloat16*>(smem + C::OFF_ONES)[e] = __float2bfloat16_rn(e < 1024 ? 1.0f : 0.5f);
+  fence_proxy_async();                 // the ones are read by the tensor core (async proxy)
+  if (warp == 1) { tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS); tmem_relinquish(); }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_t = *tmem_slot, tmem_g = tmem_t + 2 * D, tmem_sum = tmem_g + D;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      mbar_expect_tx(b_w, 2 * C::W_BYTES);
+      for (int pn = 0; pn < C::PANELS; ++pn) {
+        tma_load_2d(s_w + pn * C::W_PANEL_BYTES, &tm_whi, pn * 64, p * D, b_w);
+        tma_load_2d(s_w + C::W_BYTES + pn * C::W_PANEL_BYTES, &tm_wlo, pn * 64, p * D, b_w);
+      }
+      bool ok = true;
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        const int s = t % C::STAGES;
+        if (t >= C::STAGES) ok = mbar_wait(b_empty(s), ((t / C::STAGES) - 1) & 1, abort_flag, prm.status);
+        if (!ok) break;
+        mbar_expect_tx(b_full(s), C::TILE_BYTES);
+        for (int pn = 0; pn < C::PANELS; ++pn)
+          tma_load_3d(s_x + s * C::TILE_BYTES + pn * C::PANEL_BYTES, &tm_x, pn * 64, r_begin + t * kRows, p, b_full(s));
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc_t = idesc_bf16_f32(kRows, D, 0, 0);     // X (K-major) times W^T (K-major)
+      constexpr uint32_t idesc_g = idesc_bf16_f32(D, D, 1, 1);         // R^T R: both operands MN-major
+      constexpr uint32_t idesc_s = idesc_bf16_f32(D, 16, 1, 1);
+      bool ok = mbar_wait(b_w, 0, abort_flag, prm.status);
+      auto product_t = [&](int t) {
+        const int s = t % C::STAGES, a = t & 1;
+        if (t >= 2 && !mbar_wait(b_acc_empty(a), ((t >> 1) - 1) & 1, abort_flag, prm.status)) return false;
+        if (!mbar_wait(b_full(s), (t / C::STAGES) & 1, abort_flag, prm.status)) return false;
+        tc_fence_after();
+        const uint32_t x = s_x + s * C::TILE_BYTES, acc = tmem_t + a * D;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) {
+          const uint64_t dx = smem_desc_sw128(x + (ks / 4) * C::PANEL_BYTES + (ks % 4) * 32, 16, 1024);
+          const uint32_t wo = (ks / 4) * C::W_PANEL_BYTES + (ks % 4) * 32;
+          mma_ss(acc, dx, smem_desc_sw128(s_w + wo, 16, 1024), idesc_t, ks > 0 ? 1u : 0u);
+          mma_ss(acc, dx, smem_desc_sw128(s_w + C::W_BYTES + wo, 16, 1024), idesc_t, 1u);
+        }
+        mma_commit(b_empty(s));
+        mma_commit(b_acc_full(a));
+        return true;
+      };
+      if (ok && n_tiles > 0) ok = product_t(0);
+      for (int t = 0; t < n_tiles && ok; ++t) {
+        if (t + 1 < n_tiles) ok = product_t(t + 1);
+        if (ok) ok = mbar_wait(b_r_full, t & 1, abort_flag, prm.status);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t ones = smem_desc_sw128(s_ones, C::PANEL_BYTES, 1024);
+        const uint64_t halves = smem_desc_sw128(s_ones + 2048, C::PANEL_BYTES, 1024);
+#pragma unroll
+        for (int ks = 0; ks < kRows / 16; ++ks) {
+          // 16 rows (the contraction index) per step = 2048 bytes; 64-column panels along M and N
+          const uint64_t dh = smem_desc_sw128(s_r + ks * 2048, C::PANEL_BYTES, 1024);
+          const uint64_t dl = smem_desc_sw128(s_r + C::TILE_BYTES + ks * 2048, C::PANEL_BYTES, 1024);
+          const uint32_t acc = (t > 0 || ks > 0) ? 1u : 0u;
+          mma_ss(tmem_g, dh, dh, idesc_g, acc);
+          mma_ss(tmem_g, dh, dl, idesc_g, 1u);
+          mma_ss(tmem_sum, dh, ones, idesc_s, acc);
+          mma_ss(tmem_sum, dl, halves, idesc_s, 1u);
+        }
+        mma_commit(b_r_empty);
+      }
+      mma_commit(b_done);
+    }
+  } else {
+    const int quarter = warp & 3;
+    const int row = quarter * 32 + lane;
+    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, prm.status));
+    };
+    bool ok = true;
+    for (int t = 0; t < n_tiles && ok; ++t) {
+      const int a = t & 1;
+      ok = wait(b_acc_full(a), (t >> 1) & 1);
+      if (!ok) break;
+      tc_fence_after();
+      float v[D];
+#pragma unroll
+      for (int c4 = 0; c4 < D / 32; ++c4) {
+        uint32_t r[32];
+        tmem_ld32(tmem_t + a * D + lane_addr + c4 * 32, r);
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[c4 * 32 + j] = __uint_as_float(r[j]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_acc_empty(a));
+      if (prm.normalize) {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+        for (int j = 0; j < D; j += 4) {
+          s0 = fmaf(v[j], v[j], s0); s1 = fmaf(v[j + 1], v[j + 1], s1);
+          s2 = fmaf(v[j + 2], v[j + 2], s2); s3 = fmaf(v[j + 3], v[j + 3], s3);
+        }
+        const float nrm = sqrtf((s0 + s1) + (s2 + s3));
+        const float inv = nrm >= 1e-30f ? 1.f / nrm : 0.f;
+#pragma unroll
+        for (int j = 0; j < D; ++j) v[j] *= inv;
+      }
+      if (t > 0) ok = wait(b_r_empty, (t - 1) & 1);
+      if (!ok) break;
+#pragma unroll
+      for (int pn = 0; pn < D / 64; ++pn)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          uint32_t h[4], l[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float x0 = v[pn * 64 + 8 * c + 2 * j], x1 = v[pn * 64 + 8 * c + 2 * j + 1];
+            h[j] = pack_bf16x2(x0, x1);
+            l[j] = pack_bf16x2(2.f * (x0 - __uint_as_float(h[j] << 16)), 2.f * (x1 - __uint_as_float(h[j] & 0xffff0000u)));
+          }
+          const int off = pn * C::PANEL_BYTES + row * 128 + ((c ^ (row & 7)) * 16);
+          *reinterpret_cast<uint4*>(r_ptr + off) = make_uint4(h[0], h[1], h[2], h[3]);
+          *reinterpret_cast<uint4*>(r_ptr + C::TILE_BYTES + off) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_r_full);
+    }
+    if (ok) ok = wait(b_done, 0);
+    tc_fence_after();
+    if (ok) write_gram<D>(tmem_g, tmem_sum, quarter, lane, n_tiles > 0,
+                          prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D));
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem_t, C::TMEM_COLS);
 }
 
 // ---------------------------------------------------------------------------
@@ -481,54 +643,59 @@ int gram_tc_chunking(int n_rows, int problems, int ctas_per_sm, int* chunk_rows,
   return 0;
 }
 
-int launch_gram_tc(const void* X_hi, const void* X_lo, int problems, int n_rows, int D, float* partial,
-                   double* gram, double* colsum, int* status, cudaStream_t st) {
-  GramParams prm;
-  prm.partial = partial; prm.status = status; prm.n_rows = n_rows; prm.has_lo = X_lo ? 1 : 0;
-  const int tile = kRows * D * 2 * (X_lo ? 2 : 1);
-  prm.stages = (200 * 1024 - 4096) / tile;
-  if (prm.stages > 6) prm.stages = 6;
-  // one part per tile (32 KB at d = 128): three stages, so that two CTAs share an SM and one's
-  // start-up and epilogue overlap the other's streaming (video480: 0.36 -> 0.34 ms for the step's
-  // three launches)
-  if (!X_lo && prm.stages > 3) prm.stages = 3;
+int launch_gram_tc(const void* X, int problems, int n_rows, int D, float* partial, double* gram, double* colsum,
+                   int* status, cudaStream_t st) {
+  GramParams prm{};
+  prm.partial = partial; prm.status = status; prm.n_rows = n_rows;
+  const int tile = kRows * D * 2;
+  // three stages, so that two CTAs share an SM and one's start-up and epilogue overlap the other's
+  // streaming (video480: 0.36 -> 0.34 ms for the step's three launches)
+  prm.stages = 3;
+  const size_t smem = 1024 + (size_t)prm.stages * tile + 2048 + 8 * (2 * prm.stages + 1) + 64;
   {
-    const size_t smem_cta = 1024 + (size_t)prm.stages * tile + 2048 + 8 * (2 * prm.stages + 1) + 64 + 1024;
-    int per_sm = (int)((227 * 1024) / smem_cta);
+    int per_sm = (int)((227 * 1024) / (smem + 1024));
     const int by_tmem = 512 / ((D + 16 <= 128) ? 128 : 256);
     if (per_sm > by_tmem) per_sm = by_tmem;
     gram_tc_chunking(n_rows, problems, per_sm, &prm.chunk_rows, &prm.n_chunks);
   }
-  CUtensorMap mh, ml;
-  if (!map_3d(&mh, X_hi, problems, n_rows, D, 2, 64, kRows)) return CA_ERR_CUDA;
-  if (!map_3d(&ml, X_lo ? X_lo : X_hi, problems, n_rows, D, 2, 64, kRows)) return CA_ERR_CUDA;
-  const size_t smem = 1024 + (size_t)prm.stages * tile + 2048 + 8 * (2 * prm.stages + 1) + 64;
-  dim3 grid(prm.n_chunks, problems);
-  if (D == 64) {
-    auto k = gram_tc_kernel<64>;
-    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, kLinThreads, smem, st>>>(mh, ml, prm);
-  } else {
-    auto k = gram_tc_kernel<128>;
-    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, kLinThreads, smem, st>>>(mh, ml, prm);
-  }
+  CUtensorMap mx;
+  if (!map_3d(&mx, X, problems, n_rows, D, 2, 64, kRows)) return CA_ERR_CUDA;
+  auto k = D == 64 ? gram_tc_kernel<64> : gram_tc_kernel<128>;
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<dim3(prm.n_chunks, problems), kLinThreads, smem, st>>>(mx, prm);
   CA_LAUNCH_CHECK();
   return launch_gram_finalize(partial, problems, prm.n_chunks, D, gram, colsum, st);
 }
 
-int launch_transform_tc(const void* X_hi, const void* X_lo, int problems, int n_rows, int D, const float* W,
-                        const float* bias, int normalize, float* out, void* out_hi, void* out_lo,
-                        void* wt_hi, void* wt_lo, int* status, cudaStream_t st, float* out_t, bool weights_ready) {
-  if (!weights_ready) {               // otherwise the kernel that produced W has laid it out
-    weight_prep_kernel<<<dim3(ceil_div(D * D, 256), problems), 256, 0, st>>>(
-        W, D, static_cast<__nv_bfloat16*>(wt_hi), static_cast<__nv_bfloat16*>(wt_lo));
-    CA_LAUNCH_CHECK();
-  }
-  LinParams prm;
-  prm.bias = bias; prm.out_t = out ? out_t : nullptr; prm.status = status; prm.n_rows = n_rows; prm.has_lo = X_lo ? 1 : 0;
-  prm.normalize = normalize; prm.out_split = out ? 0 : 1;
-  const int tile = kRows * D * 2 * (X_lo ? 2 : 1);
+template <int D>
+static int launch_rep_gram(const void* X, int problems, int n_rows, int normalize, float* partial, double* gram,
+                           double* colsum, const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st) {
+  using C = RepCfg<D>;
+  GramParams prm{};
+  prm.partial = partial; prm.status = status; prm.n_rows = n_rows; prm.normalize = normalize;
+  gram_tc_chunking(n_rows, problems, C::CTAS_PER_SM, &prm.chunk_rows, &prm.n_chunks);
+  CUtensorMap mx, mwh, mwl;
+  if (!map_3d(&mx, X, problems, n_rows, D, 2, 64, kRows) || !map_2d(&mwh, wt_hi, (size_t)problems * D, D, D) ||
+      !map_2d(&mwl, wt_lo, (size_t)problems * D, D, D))
+    return CA_ERR_CUDA;
+  auto k = rep_gram_tc_kernel<D>;
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+  k<<<dim3(prm.n_chunks, problems), kLinThreads, C::SMEM, st>>>(mx, mwh, mwl, prm);
+  CA_LAUNCH_CHECK();
+  return launch_gram_finalize(partial, problems, prm.n_chunks, D, gram, colsum, st);
+}
+
+int launch_rep_gram_tc(const void* X, int problems, int n_rows, int D, int normalize, float* partial, double* gram,
+                       double* colsum, const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st) {
+  return D == 64 ? launch_rep_gram<64>(X, problems, n_rows, normalize, partial, gram, colsum, wt_hi, wt_lo, status, st)
+                 : launch_rep_gram<128>(X, problems, n_rows, normalize, partial, gram, colsum, wt_hi, wt_lo, status, st);
+}
+
+int launch_transform_tc(const void* X, int problems, int n_rows, int D, const float* bias, int normalize, float* out,
+                        const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st, float* out_t) {
+  LinParams prm{};
+  prm.bias = bias; prm.out_t = out_t; prm.status = status; prm.n_rows = n_rows; prm.normalize = normalize;
+  const int tile = kRows * D * 2;
   const int fixed = 2 * D * D * 2 + kRows * D * 4 + 4096;
   prm.stages = (200 * 1024 - fixed) / tile;
   if (prm.stages > 4) prm.stages = 4;
@@ -538,24 +705,14 @@ int launch_transform_tc(const void* X_hi, const void* X_lo, int problems, int n_
   if (ctas < 1) ctas = 1;
   prm.tiles_per_cta = ceil_div(total_tiles, ctas);
   if (prm.tiles_per_cta < 2) prm.tiles_per_cta = 2;
-  CUtensorMap mxh, mxl, mwh, mwl, mo, mol;
-  bool ok = map_3d(&mxh, X_hi, problems, n_rows, D, 2, 64, kRows) &&
-            map_3d(&mxl, X_lo ? X_lo : X_hi, problems, n_rows, D, 2, 64, kRows) &&
-            map_2d(&mwh, wt_hi, (size_t)problems * D, D, D) && map_2d(&mwl, wt_lo, (size_t)problems * D, D, D);
-  if (out) ok = ok && map_3d(&mo, out, problems, n_rows, D, 4, 32, kRows) && map_3d(&mol, out, problems, n_rows, D, 4, 32, kRows);
-  else ok = ok && map_3d(&mo, out_hi, problems, n_rows, D, 2, 64, kRows) && map_3d(&mol, out_lo, problems, n_rows, D, 2, 64, kRows);
-  if (!ok) return CA_ERR_CUDA;
+  CUtensorMap mx, mwh, mwl, mo;
+  if (!map_3d(&mx, X, problems, n_rows, D, 2, 64, kRows) || !map_2d(&mwh, wt_hi, (size_t)problems * D, D, D) ||
+      !map_2d(&mwl, wt_lo, (size_t)problems * D, D, D) || !map_3d(&mo, out, problems, n_rows, D, 4, 32, kRows))
+    return CA_ERR_CUDA;
   const size_t smem = 1024 + (size_t)fixed + (size_t)prm.stages * tile + D * 4;
-  dim3 grid(ceil_div(total_tiles, prm.tiles_per_cta), problems);
-  if (D == 64) {
-    auto k = transform_tc_kernel<64>;
-    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, kLinThreads, smem, st>>>(mxh, mxl, mwh, mwl, mo, mol, prm);
-  } else {
-    auto k = transform_tc_kernel<128>;
-    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, kLinThreads, smem, st>>>(mxh, mxl, mwh, mwl, mo, mol, prm);
-  }
+  auto k = D == 64 ? transform_tc_kernel<64> : transform_tc_kernel<128>;
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k<<<dim3(ceil_div(total_tiles, prm.tiles_per_cta), problems), kLinThreads, smem, st>>>(mx, mwh, mwl, mo, prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
