@@ -76,13 +76,14 @@ struct ClusterWs {
   size_t bytes;
 };
 
-// A level of the splitter reads one coordinate of every row of a set, rows scattered: from the
-// row-major coordinates that costs a 128-byte DRAM line per row and level.  A coordinate-major copy
-// makes it a 4-byte read inside an L2-resident column, at the price of writing the coordinates a
-// second time (4 d bytes per row): worth it when levels x 128 > 1.5 x 4 d (long sequences, d = 64).
-static bool use_yt(const ca_problem_t* p, int n, int c) {
-  const bool tc = p->dtype == CA_DTYPE_BF16 && (p->head_dim == 64 || p->head_dim == 128);
-  return tc && !(p->flags & CA_Y_IN) && split_top_levels_for(n, c) * 128 >= 6 * p->head_dim;
+// A level of the splitter reads one coordinate of every row of a set, rows in ascending order: from the
+// row-major coordinates a line per row, from a coordinate-major copy neighbouring rows of the set
+// share lines, and a column stays in L2.  The coordinates are in order of variance and a split
+// removes most of the variance of its coordinate in both parts, so a tree of ten levels splits along the first
+// ten or so: the copy holds kSplitCols coordinates (64 bytes per row), any other is read
+// row-major.  (All d coordinates cost as much to write as the coordinates themselves.)
+static bool use_yt(const ca_problem_t* p) {
+  return p->dtype == CA_DTYPE_BF16 && !(p->flags & CA_Y_IN);
 }
 
 ClusterWs carve_cluster(const ca_problem_t* p, void* base, bool need_yq, bool need_yk) {
@@ -115,9 +116,9 @@ ClusterWs carve_cluster(const ca_problem_t* p, void* base, bool need_yq, bool ne
     w.wt2_lo = c.take<__nv_bfloat16>(P * DD);
     if (need_yq) w.Yq = c.take<float>(P * (size_t)p->n_q * D);
     if (need_yk) w.Yk = c.take<float>(P * (size_t)p->n_k * D);
-    // coordinate-major copies of the split coordinates, where they pay (use_yt)
-    if (use_yt(p, p->n_q, p->cluster_q)) w.Ytq = c.take<float>(P * (size_t)p->n_q * D);
-    if (use_yt(p, p->n_k, p->cluster_k)) w.Ytk = c.take<float>(P * (size_t)p->n_k * D);
+    // coordinate-major copies of the first split coordinates (use_yt)
+    if (use_yt(p)) w.Ytq = c.take<float>(P * (size_t)p->n_q * kSplitCols);
+    if (use_yt(p)) w.Ytk = c.take<float>(P * (size_t)p->n_k * kSplitCols);
   }
   w.perm_q_tmp = c.take<int32_t>(P * (size_t)p->n_q);
   w.perm_k_tmp = c.take<int32_t>(P * (size_t)p->n_k);

@@ -60,9 +60,9 @@ int launch_cholesky_factor(const double* gram, const double* sum, double n, doub
                            double* out64, float* out32, void* wt_hi, void* wt_lo, cudaStream_t st);
 
 // split.cu
+// Coordinates that the tensor-core transform also writes coordinate-major for the splitter
+constexpr int kSplitCols = 16;
 int split_levels_for(int n, int c);
-// levels that run as per-level launches over whole sets (the rest is finished per subtree)
-int split_top_levels_for(int n, int c);
 int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q, int n_k, int c_q,
                  int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp, int32_t* perm_k_out,
                  int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k, int sides, cudaStream_t st,

@@ -119,83 +119,114 @@ __device__ __forceinline__ pair2 add_pair(pair2 a, pair2 b) {
   return d;
 }
 
-// The same estimate for `ng` subsets at once, the sample rows read straight from the coordinates
-// in global memory.  `sub` holds the sample rows residue-major: sub[gi * D + r * (D / 8) + k] is
-// the row of sample r + 8 k of subset gi, -1 beyond its m rows.  Same operations in the same order
-// as staged_variances, hence the same bits; what differs is the parallelism: every (subset,
-// residue, coordinate) is a thread's task, so a round of many small subsets keeps all warps busy
-// between two barriers, and a task's loads (one per sample row of its residue) are in flight four
-// at a time.  The stage is bound by the instructions it issues, so a subset with all D sample rows
-// (every subset that still splits when the cluster size is at least D) runs without a test per
-// row; a missing row otherwise reads as 0 in the pass of the sums and as the mean in the pass of
-// the squares, which adds an exact zero.
-template <int D, typename RowsOf>
-__device__ __forceinline__ void gathered_variances(const float* __restrict__ Y, const int* sub, int ng, RowsOf rows_of,
-                                                   float* part, float* out, int tid, int nt) {
-  constexpr int PER = D / 8;                       // sample rows of a residue
-  constexpr int Q4 = D / 4;                        // 16-byte vectors of a row
-  constexpr int B = 4;                             // loads in flight per task
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int task = tid; task < ng * 8 * Q4; task += nt) {
-      const int gi = task / (8 * Q4), r = (task / Q4) % 8, t4 = task % Q4;
-      const int m = rows_of(gi);
-      float4 mean = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (pass == 1) mean = *reinterpret_cast<const float4*>(out + gi * D + 4 * t4);
-      pair2 acc_a = pair(0.f, 0.f), acc_b = acc_a;
-      float4 sq = make_float4(0.f, 0.f, 0.f, 0.f);
-      const pair2 nmean_a = pair(-mean.x, -mean.y), nmean_b = pair(-mean.z, -mean.w);
-      const int4* idx = reinterpret_cast<const int4*>(sub + gi * D + r * PER);
-      const float4* Yv = reinterpret_cast<const float4*>(Y) + t4;
-      const bool full = m == D;                    // all PER rows of the residue are there
+// The same estimate for one block of 4 V coordinates of one subset, by one warp: lane = 4 r + q
+// takes the sample rows r, r + 8, ... of V consecutive coordinates.  The eight residues are combined by
+// a butterfly over the lanes, which adds in the order of staged_variances, hence the same bits; a
+// row is read once and kept in registers for the squares, and no barrier is needed.  Writes the largest
+// variance of the block, and its coordinate (the lowest on ties) with that coordinate's mean.
+template <int D, int V, bool full>          // full: the subset has at least D rows
+__device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const int32_t* rows, int sz, int block, int lane,
+                                              float* best_out, int2* arg_out) {
+  constexpr int PER = D / 8;                         // sample rows of a residue
+  const int r = lane >> 2, t = (block * 4 + (lane & 3)) * V;
+  const int m = full ? D : sz;
+  // sample j stands at position floor(j sz / m): j itself where the sample is the whole subset; a
+  // row beyond the sample is loaded as the last one and counts as zero
+  pair2 x[PER][V / 2];
 #pragma unroll
-      for (int k0 = 0; k0 < PER; k0 += B) {
-        const int4 ri = idx[k0 / B];
-        const int row[B] = {ri.x, ri.y, ri.z, ri.w};
-        float4 x[B];
-        if (full) {
-#pragma unroll
-          for (int k = 0; k < B; ++k) x[k] = __ldg(Yv + (size_t)row[k] * Q4);
-        } else {
-#pragma unroll
-          for (int k = 0; k < B; ++k) x[k] = row[k] >= 0 ? __ldg(Yv + (size_t)row[k] * Q4) : mean;
-        }
-        // Sums and differences two values per instruction (each half rounded on its own: the bits
-        // of two scalar additions).  The squares and their sums stay scalar operations that are
-        // never contracted: a two-value multiply followed by a two-value add is merged into one
-        // fused multiply-add by the assembler, which rounds once where the definition rounds twice.
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          const pair2 xa = pair(x[k].x, x[k].y), xb = pair(x[k].z, x[k].w);
-          if (pass == 0) {
-            acc_a = add_pair(acc_a, xa);
-            acc_b = add_pair(acc_b, xb);
-          } else {
-            float dx, dy, dz, dw;
-            unpair(add_pair(xa, nmean_a), dx, dy);                                // x - mean
-            unpair(add_pair(xb, nmean_b), dz, dw);
-            sq.x = __fadd_rn(sq.x, __fmul_rn(dx, dx)); sq.y = __fadd_rn(sq.y, __fmul_rn(dy, dy));
-            sq.z = __fadd_rn(sq.z, __fmul_rn(dz, dz)); sq.w = __fadd_rn(sq.w, __fmul_rn(dw, dw));
-          }
-        }
-      }
-      float4 acc = sq;
-      if (pass == 0) {
-        unpair(acc_a, acc.x, acc.y);
-        unpair(acc_b, acc.z, acc.w);
-      }
-      *reinterpret_cast<float4*>(part + (gi * 8 + r) * D + 4 * t4) = acc;
+  for (int k = 0; k < PER; ++k) {
+    const unsigned j = r + 8 * k;
+    const int pos = full ? (int)(j * (unsigned)sz / D) : min((int)j, m - 1);
+    const float* src = Y + (size_t)rows[pos] * D + t;
+    if constexpr (V == 4) {
+      const float4 w = __ldg(reinterpret_cast<const float4*>(src));
+      x[k][0] = pair(w.x, w.y);
+      x[k][V / 2 - 1] = pair(w.z, w.w);
+    } else {
+      const float2 w = __ldg(reinterpret_cast<const float2*>(src));
+      x[k][0] = pair(w.x, w.y);
     }
-    __syncthreads();
-    for (int task = tid; task < ng * D; task += nt) {
-      const int gi = task / D, t = task % D;
-      const float* p = part + gi * 8 * D + t;
-      const float tot = __fadd_rn(__fadd_rn(__fadd_rn(p[0], p[D]), __fadd_rn(p[2 * D], p[3 * D])),
-                                  __fadd_rn(__fadd_rn(p[4 * D], p[5 * D]), __fadd_rn(p[6 * D], p[7 * D])));
-      const int m = rows_of(gi);
-      out[task] = m > 0 ? __fdiv_rn(tot, (float)m) : -1.0f;
-    }
-    __syncthreads();
   }
+  if (!full) {
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+#pragma unroll
+      for (int h = 0; h < V / 2; ++h) x[k][h] = r + 8 * k < m ? x[k][h] : 0ull;
+  }
+  // D is a power of two: the product with 1 / D rounds as the division does.  For a partial sample
+  // a lane divides the value of its residue's number and the lanes of a coordinate exchange them.
+  auto divide = [&](float (&v)[V]) {
+    if (full) {
+#pragma unroll
+      for (int i = 0; i < V; ++i) v[i] = __fmul_rn(v[i], 1.0f / D);
+    } else {
+      float q = v[0];
+#pragma unroll
+      for (int i = 1; i < V; ++i) q = (r & (V - 1)) == i ? v[i] : q;
+      q = __fdiv_rn(q, (float)m);
+#pragma unroll
+      for (int i = 0; i < V; ++i) v[i] = __shfl_sync(0xffffffffu, q, 4 * i + (lane & 3));
+    }
+  };
+  float mean[V], var[V];
+#pragma unroll
+  for (int h = 0; h < V / 2; ++h) {
+    pair2 acc = pair(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) acc = add_pair(acc, x[k][h]);
+    unpair(acc, mean[2 * h], mean[2 * h + 1]);
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+    for (int v = 0; v < V; ++v) mean[v] = __fadd_rn(mean[v], __shfl_xor_sync(0xffffffffu, mean[v], o));
+  divide(mean);
+  // Sums and differences two values per instruction (each half rounded on its own: the bits
+  // of two scalar additions).  The squares and their sums stay scalar operations that are
+  // never contracted: a two-value multiply followed by a two-value add is merged into one
+  // fused multiply-add by the assembler, which rounds once where the definition rounds twice.
+#pragma unroll
+  for (int h = 0; h < V / 2; ++h) {
+    const pair2 neg = pair(-mean[2 * h], -mean[2 * h + 1]);
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      float d0, d1;
+      unpair(add_pair(x[k][h], neg), d0, d1);
+      if (!full && r + 8 * k >= m) d0 = d1 = 0.f;    // a missing row adds an exact zero
+      s0 = __fadd_rn(s0, __fmul_rn(d0, d0));
+      s1 = __fadd_rn(s1, __fmul_rn(d1, d1));
+    }
+    var[2 * h] = s0;
+    var[2 * h + 1] = s1;
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+    for (int v = 0; v < V; ++v) var[v] = __fadd_rn(var[v], __shfl_xor_sync(0xffffffffu, var[v], o));
+  divide(var);
+  float best = var[0], best_mean = mean[0];
+  int arg = t;
+#pragma unroll
+  for (int v = 1; v < V; ++v)
+    if (var[v] > best) { best = var[v]; arg = t + v; best_mean = mean[v]; }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+    const float om = __shfl_xor_sync(0xffffffffu, best_mean, o);
+    if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; best_mean = om; }
+  }
+  if (lane == 0) {
+    *best_out = best;
+    *arg_out = make_int2(arg, __float_as_int(best_mean));
+  }
+}
+// Out of line: only subsets of fewer than D rows take it, which split only where the cluster size is below D.
+template <int D, int V>
+__device__ __noinline__ void unit_variance_small(const float* __restrict__ Y, const int32_t* rows, int sz, int block, int lane,
+                                                 float* best_out, int2* arg_out) {
+  unit_variance<D, V, false>(Y, rows, sz, block, lane, best_out, arg_out);
 }
 
 // 16-byte asynchronous copy global -> shared (no registers held while in flight)
@@ -203,11 +234,15 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 struct SplitSide {
   const float* Y;          // [P][n][D]
-  const float* Yt;         // [P][D][n] the same coordinates, coordinate-major, or null
+  const float* Yt;         // [P][kSplitCols][n] the first coordinates once more, coordinate-major, or null
   const int32_t* perm_in;  // [P][n] or null (identity)
   int32_t* perm_out;       // [P][n]
   uint32_t* keybuf;        // [P][n] staging for sets larger than the shared-memory windows
@@ -253,7 +288,6 @@ __global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitP
   if (!seg.active) return;
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const float* Y = sd.Y + (size_t)p * sd.n * D;
-  const float* Yt = sd.Yt ? sd.Yt + (size_t)p * sd.n * D : nullptr;
   const int32_t* pin = sd.perm_in ? sd.perm_in + (size_t)p * sd.n : nullptr;
   int32_t* pout = sd.perm_out + (size_t)p * sd.n;
   const int lo = seg.lo, s = seg.size;
@@ -318,6 +352,9 @@ __global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitP
   } else {
   // gathers in batches of eight: the row indices first, then the coordinates, so that the
   // memory latencies of a batch overlap
+  const bool column = sd.Yt && coord < kSplitCols;
+  const float* Yc = column ? sd.Yt + ((size_t)p * kSplitCols + coord) * sd.n : Y + coord;
+  const int row_stride = column ? 1 : D;
   for (int i0 = tid; i0 < cs; i0 += 8 * nt) {
     int row[8];
     float val[8];
@@ -327,7 +364,7 @@ __global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitP
       row[u] = (i < cs) ? (pin ? __ldg(pin + lo + c0 + i) : lo + c0 + i) : 0;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) val[u] = Yt ? __ldg(Yt + (size_t)coord * sd.n + row[u]) : __ldg(Y + (size_t)row[u] * D + coord);
+    for (int u = 0; u < 8; ++u) val[u] = __ldg(Yc + (size_t)row[u] * row_stride);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * nt;
@@ -492,191 +529,123 @@ __global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitP
 // ---------------------------------------------------------------------------
 // Subtree of a set of at most kTailRowsMax rows, finished by one CTA.
 // ---------------------------------------------------------------------------
+constexpr int kTailList = 64;            // candidates of a subset that a warp ranks
+
 struct TailSmem {
   int32_t rows[2][kTailRowsMax];
-  uint32_t keys[kTailRowsMax];
-  uint32_t scan[kTailRowsMax];            // inclusive (less | equal << 16) counts over positions
-  int hist[kTailSegs][256];
-  int seg_lo[2][2 * kTailSegs + 2];       // start of each subset (relative), +1 sentinel
-  int seg_coord[kTailSegs], seg_digit[kTailSegs], seg_rem[kTailSegs], seg_L[kTailSegs];
-  int seg_cand[kTailSegs];                // candidates left after the first two digits; -1: threshold found
-  int overflow;                           // some subset has more candidates than a warp takes
-  uint32_t seg_prefix[kTailSegs];
-  float vpart[4 * 8 * 64];                // partial sums of the variance stage ([ng][8][D])
-  float vout[4 * 64];
-  int sub_rows[4 * 64];                    // subsample rows of the subsets being staged                     // means / variances ([ng][D])
-  float best[kTailSegs][4];
-  int arg[kTailSegs][4];
+  uint32_t keys[kTailRowsMax];           // by position: first the value, then its key
+  uint16_t state[kTailRowsMax];          // by position: subset << 8 | bin
+  uint32_t hist[kTailSegs][128];         // counts of 256 bins, two to a word
+  unsigned long long list[kTailSegs][kTailList];   // (key, position) of the rows in the threshold's bin
+  int4 seg[kTailSegs];                   // coordinate, L (0: final), start, index of the first child
+  float2 seg_map[kTailSegs];             // bin of a value x = x . x + y
+  int2 seg_pick[kTailSegs];              // the threshold's bin (-1: found digit by digit), its 1-based rank in the bin
+  unsigned long long seg_thr[kTailSegs]; // the last (key, position) that goes down
+  int seg_base[kTailSegs];               // rows that go down in the subsets before this one
+  int seg_cand[kTailSegs];               // entries of the list
+  uint32_t seg_prefix[kTailSegs];        // digits found so far, and the rank that is left
+  int seg_rem[kTailSegs];
+  int seg_lo[2][kTailSegs + 1];          // start of each subset (relative), +1 sentinel
+  float unit_best[kTailSegs][20];        // per block of coordinates: largest variance, then (coordinate, mean) of it
+  int2 unit_arg[kTailSegs][17];
   int warp_tot[32];
-  int nseg[2];
-  int more;
+  unsigned crowded;                      // subsets whose bin has more rows than the list holds
+  int nseg, more;
 };
 
-// Selection and partition of one level of a subtree, all of its subsets side by side: radix
-// selection of every subset's threshold key (seg_L, seg_rem, seg_prefix set up by the caller), then
-// the stable partition into rows_next.  A thread owns the four consecutive positions 4 tid .. 4 tid + 3
-// (my_seg: subset of a position, -1 - g in a final subset, INT_MIN past the end; my_key: its key).
-template <typename Smem>
-__device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_seg)[kTailRowsMax / kSplitThreads],
-                                                      const uint32_t (&my_key)[kTailRowsMax / kSplitThreads],
-                                                      int nseg, const int* slo, const int32_t* rows,
-                                                      int32_t* rows_next, int tid, int* hist, uint32_t* scan) {
-  constexpr int nt = kSplitThreads;
-  constexpr int PT = kTailRowsMax / kSplitThreads;
-  const int lane = tid & 31, warp = tid >> 5;
-  // ---- radix selection, all subsets side by side: two digits of eight bits by counting; then the
-  // keys that share those sixteen bits with the threshold are few (a handful per subset unless keys
-  // repeat), and a warp ranks them directly.  A subset with more than 32 of them goes on with the two
-  // remaining digits.  (The digit counts are cleared once per level: the warp that picks a subset's
-  // digit clears the counts it has read, ready for the next pass.)
-  uint32_t mask = 0;
-  for (int e = tid; e < nseg * 256; e += nt) hist[e] = 0;
-  if (tid < nseg) sm.seg_cand[tid] = 0;
-  if (tid == 0) sm.overflow = 0;
-  __syncthreads();
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    uint32_t pre[PT];                               // read ahead of the atomics, which order memory accesses
+// The bin of one subset that holds its `rank`-th row (1-based), the rank inside it and its rows, in
+// the one lane that finds it (false elsewhere); clears the counts for their next use.
+__device__ __forceinline__ bool pick_bin(uint32_t* hist, int rank, int lane, int& bin, int& rank_in, int& rows_in) {
+  uint4* h4 = reinterpret_cast<uint4*>(hist) + lane;
+  const uint4 h = *h4;
+  *h4 = make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t pairs = (h.x + h.y) + (h.z + h.w);      // at most 4,096 rows: the halves do not overflow
+  const int sum = (int)((pairs & 0xffffu) + (pairs >> 16));
+  int incl = sum;
 #pragma unroll
-    for (int u = 0; u < PT; ++u) pre[u] = sm.seg_prefix[my_seg[u] >= 0 ? my_seg[u] : 0];
-    if (shift == 8) {
-      // candidates of every subset into its list (the scan array is free until the partition)
-#pragma unroll
-      for (int u = 0; u < PT; ++u) {
-        const int g = my_seg[u];
-        if (g >= 0 && (my_key[u] & mask) == pre[u]) {
-          const int slot = atomicAdd(&sm.seg_cand[g], 1);
-          if (slot < 32) scan[g * 32 + slot] = my_key[u];
-        }
-      }
-      __syncthreads();
-      for (int g = warp; g < nseg; g += nt / 32) {
-        if (sm.seg_L[g] == 0) continue;             // warp-uniform
-        const int n = sm.seg_cand[g];
-        if (n > 32) {
-          if (lane == 0) sm.overflow = 1;
-          continue;
-        }
-        const int remaining = sm.seg_rem[g];        // 1 <= remaining <= n
-        const uint32_t key = lane < n ? scan[g * 32 + lane] : 0xffffffffu;
-        int less = 0, eq_before = 0;
-        for (int j = 0; j < n; ++j) {
-          const uint32_t kj = __shfl_sync(0xffffffffu, key, j);
-          less += kj < key ? 1 : 0;
-          eq_before += (kj == key && j < lane) ? 1 : 0;
-        }
-        if (lane < n && less + eq_before == remaining - 1) {   // exactly one lane
-          sm.seg_prefix[g] = key;
-          sm.seg_rem[g] = remaining - less;          // how many of the keys equal to the threshold go down
-          sm.seg_cand[g] = -1;
-        }
-      }
-      __syncthreads();
-      if (!sm.overflow) break;                      // uniform: every threshold is found
-#pragma unroll
-      for (int u = 0; u < PT; ++u) pre[u] = sm.seg_prefix[my_seg[u] >= 0 ? my_seg[u] : 0];
-    }
-#pragma unroll
-    for (int u = 0; u < PT; ++u) {
-      const int g = my_seg[u];
-      const bool live = g >= 0;
-      const uint32_t k = my_key[u];
-      if (live && ((k & mask) == pre[u])) atomicAdd(&hist[(g << 8) | (int)((k >> shift) & 255u)], 1);
-    }
-    __syncthreads();
-    for (int g = warp; g < nseg; g += nt / 32) {
-      const int remaining = sm.seg_rem[g];
-      if (sm.seg_L[g] == 0) continue;               // warp-uniform
-      int local[8]; int sum = 0;
-      {
-        int4* h4 = reinterpret_cast<int4*>(&hist[g * 256 + lane * 8]);
-        const int4 h0 = h4[0], h1 = h4[1];
-        h4[0] = make_int4(0, 0, 0, 0);
-        h4[1] = make_int4(0, 0, 0, 0);
-        local[0] = h0.x; local[1] = h0.y; local[2] = h0.z; local[3] = h0.w;
-        local[4] = h1.x; local[5] = h1.y; local[6] = h1.z; local[7] = h1.w;
-      }
-      if (sm.seg_cand[g] < 0) continue;             // found by the direct ranking (its keys were still counted)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) sum += local[j];
-      int incl = sum;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int before = incl - sum;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (before < remaining && remaining <= before + local[j]) {
-          sm.seg_digit[g] = lane * 8 + j;
-          sm.seg_rem[g] = remaining - before;
-        }
-        before += local[j];
-      }
-      __syncwarp();
-      if (lane == 0) sm.seg_prefix[g] |= (uint32_t)sm.seg_digit[g] << shift;
-    }
-    mask |= 255u << shift;
-    __syncthreads();
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
   }
+  if (!(incl - sum < rank && rank <= incl)) return false;
+  rank_in = rank - (incl - sum);
+  bin = lane * 8;
+  const uint32_t w[4] = {h.x, h.y, h.z, h.w};
+  bool found = false;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int n = (int)((w[j / 2] >> (16 * (j & 1))) & 0xffffu);
+    if (found) continue;
+    if (rank_in <= n) { found = true; rows_in = n; }
+    else { rank_in -= n; ++bin; }
+  }
+  return true;
+}
 
-  // ---- 3. stable partition of every subset: one scan of (less | equal << 16) over all positions
-  // (a thread's four, then the warp, then the warps' totals by warp 0)
-  uint32_t my_scan[PT];
-  {
-    int run = 0;
-#pragma unroll
-    for (int u = 0; u < PT; ++u) {
-      if (my_seg[u] >= 0) {
-        const uint32_t k = my_key[u], thr = sm.seg_prefix[my_seg[u]];
-        run += (k < thr ? 1 : 0) | (k == thr ? 1 << 16 : 0);
-      }
-      my_scan[u] = (uint32_t)run;
-    }
-    int incl = run;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) sm.warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      const int v = sm.warp_tot[lane];                 // nt / 32 == 32 warps
-      int wi = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, wi, o);
-        if (lane >= o) wi += x;
-      }
-      sm.warp_tot[lane] = wi - v;                      // totals of the warps before this one
+// The thresholds of the crowded subsets by radix selection, eight bits a pass; keys that are equal in
+// all digits go down in order of position.  Out of line: rarely needed.
+template <int nt>
+__device__ __noinline__ void tail_thresholds_by_digits(TailSmem& sm, unsigned crowded, int s0, int nseg, const int* slo, int tid) {
+  const int lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = nt / 32;
+#pragma unroll 1
+  for (int shift = 24; shift >= 0; shift -= 8) {
+#pragma unroll 1
+    for (int i = tid; i < s0; i += nt) {
+      const int g = sm.state[i] >> 8;
+      const uint32_t key = sm.keys[i];
+      if (!((crowded >> g) & 1) || (shift < 24 && (key >> (shift + 8)) != sm.seg_prefix[g])) continue;
+      const int digit = (key >> shift) & 255;
+      atomicAdd(&sm.hist[g][digit >> 1], 1u << (16 * (digit & 1)));
     }
     __syncthreads();
-    const uint32_t before = (uint32_t)(sm.warp_tot[warp] + incl - run);
-#pragma unroll
-    for (int u = 0; u < PT; ++u) my_scan[u] += before;
-    *reinterpret_cast<uint4*>(&scan[PT * tid]) = make_uint4(my_scan[0], my_scan[1], my_scan[2], my_scan[3]);
+#pragma unroll 1
+    for (int g = warp; g < nseg; g += NW) {
+      if (!((crowded >> g) & 1)) continue;
+      int digit, rank, rows_in;
+      const int want = shift == 24 ? sm.seg[g].y : sm.seg_rem[g];
+      __syncwarp();
+      if (pick_bin(sm.hist[g], want, lane, digit, rank, rows_in)) {
+        sm.seg_prefix[g] = shift == 24 ? digit : (sm.seg_prefix[g] << 8 | digit);
+        sm.seg_rem[g] = rank;
+      }
+    }
     __syncthreads();
   }
-#pragma unroll
-  for (int u = 0; u < PT; ++u) {
-    const int i = PT * tid + u;
-    const int g = my_seg[u];
-    if (g == INT_MIN) continue;
-    if (g < 0) { rows_next[i] = rows[i]; continue; }
-    const int a = slo[g];
-    const uint32_t base = a > 0 ? scan[a - 1] : 0u;
-    const uint32_t k = my_key[u], thr = sm.seg_prefix[g];
-    const int is_less = k < thr, is_eq = k == thr;
-    const uint32_t excl = my_scan[u] - base - (uint32_t)(is_less | (is_eq << 16));
-    const int less_here = (int)(excl & 0xffffu), eq_here = (int)(excl >> 16);
-    const int eq_left = sm.seg_rem[g], L = sm.seg_L[g];
-    const bool down = is_less || (is_eq && eq_here < eq_left);
-    const int down_before = less_here + min(eq_here, eq_left);
-    const int dst = down ? a + down_before : a + L + (i - a - down_before);
-    rows_next[dst] = rows[i];
+#pragma unroll 1
+  for (int g = warp; g < nseg; g += NW) {
+    if (!((crowded >> g) & 1)) continue;
+    const uint32_t thr = sm.seg_prefix[g];
+    int left = sm.seg_rem[g];                            // of the keys equal to the threshold go down
+    for (int i0 = slo[g]; i0 < slo[g + 1]; i0 += 32) {
+      const bool eq = i0 + lane < slo[g + 1] && sm.keys[i0 + lane] == thr;
+      const unsigned b = __ballot_sync(0xffffffffu, eq);
+      if (left <= __popc(b)) {
+        if (eq && __popc(b & ((1u << lane) - 1u)) == left - 1)
+          sm.seg_thr[g] = ((unsigned long long)thr << 32) | (unsigned)(i0 + lane);
+        break;
+      }
+      left -= __popc(b);
+    }
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kSplitThreads) split_tail_kernel(const SplitParams prm) {
+// Subtree of a set of at most kTailRowsMax rows, finished by one CTA.  A level is a chain of short
+// stages between barriers (at most 32 subsets side by side), so its time is latency: loads from L2,
+// shuffles, barriers, and the instruction fetch of a long loop body, which has to stay well below the
+// 32 KB that the SM keeps: the position loops are rolled and their state lives in shared memory.  Per level:
+// sample variances by independent warps (unit_variance); values gathered by asynchronous copies; the
+// bin of every value between mean - 2 s and mean + 2 s of the sample in 256 steps; the bin that holds
+// the L-th value; the rows in that bin, ranked by one warp; the partition from ballots, where the
+// rows that go down before a subset are known beforehand (the L of the subsets to its left).  A bin with
+// more than 64 rows (values repeat, or far outliers stretch s) is resolved digit by digit.
+// Two CTAs of 512 threads share an SM; where all CTAs of both sides fit the SMs one each, 1,024 threads
+// (12 heads of 1,370 rows, d = 64: 43 -> 35 us a side).  With the earlier form (samples read twice between
+// barriers, two digits of counting, one CTA of 1,024 threads an SM) 12 x 1,370 rows took 52 us, 12 x
+// 16,385 rows 90 and now 47.  At d = 128 the sample rows are read from HBM (40 heads of 32,760 rows, 0.65 GB in
+// pieces of one row: 356 -> 315 us).
+template <int D, int nt>
+__global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(const SplitParams prm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TailSmem& sm = *reinterpret_cast<TailSmem*>(smem_raw);
   const int which = blockIdx.y / prm.problems;
@@ -687,128 +656,190 @@ __global__ void __launch_bounds__(kSplitThreads) split_tail_kernel(const SplitPa
   const SegmentRef root = locate_segment(sd.n, sd.c, level, blockIdx.x);
   if (!root.active) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int nt = kSplitThreads;
+  constexpr int NW = nt / 32;
+  constexpr int V = D == 64 ? 4 : 2;                     // coordinates of a lane in unit_variance: D V / 8 = 32 registers
+  constexpr int UNITS = D / (4 * V);
   const int c = sd.c;
   const float* Y = sd.Y + (size_t)p * sd.n * D;
-  const float* Yt = sd.Yt ? sd.Yt + (size_t)p * sd.n * D : nullptr;
+  const float* Yt = sd.Yt ? sd.Yt + (size_t)p * sd.n * kSplitCols : nullptr;
   const int32_t* pin = sd.perm_in ? sd.perm_in + (size_t)p * sd.n : nullptr;
   int32_t* pout = sd.perm_out + (size_t)p * sd.n;
   const int lo = root.lo, s0 = root.size;
+  // a warp owns consecutive positions, 32 at a time
+  const int span = 32 * (((s0 + 31) / 32 + NW - 1) / NW);
+  const int w0 = warp * span, w1 = min(s0, w0 + span);
 
-  for (int i = tid; i < s0; i += nt) sm.rows[0][i] = pin ? pin[lo + i] : lo + i;
-  if (tid == 0) { sm.seg_lo[0][0] = 0; sm.seg_lo[0][1] = s0; sm.nseg[0] = 1; sm.more = s0 > c; }
+#pragma unroll 1
+  for (int i = tid; i < s0; i += nt) {
+    sm.rows[0][i] = pin ? pin[lo + i] : lo + i;
+    sm.state[i] = 0;
+  }
+#pragma unroll 1
+  for (int e = tid; e < kTailSegs * 32; e += nt) reinterpret_cast<uint4*>(&sm.hist[0][0])[e] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) { sm.seg_lo[0][0] = 0; sm.seg_lo[0][1] = s0; sm.nseg = 1; sm.more = s0 > c; }
   __syncthreads();
 
   int cur = 0;
-  constexpr int wps = D / 32;                            // warps per (subset, all coordinates)
   while (sm.more) {
-    const int nseg = sm.nseg[cur];
+    const int nseg = sm.nseg;
     const int* slo = sm.seg_lo[cur];
     const int32_t* rows = sm.rows[cur];
     int32_t* rows_next = sm.rows[cur ^ 1];
 
-    // ---- 1. coordinate of largest subsample variance for every subset that still splits.
-    // Rounds of up to 1024 / D subsets: their sample rows are located (one division per row), then
-    // every (subset, residue, coordinate) is a thread's task that reads its sample values straight
-    // from the coordinates; partial sums, means and variances live in the 64 KB that keys, scan and
-    // hist occupy later in the level.
-    {
-      float* part = reinterpret_cast<float*>(sm.keys);                 // [G][8][D]
-      constexpr int G = 1024 / D;
-      float* vout = part + G * 8 * D;                                  // [G][D] means, then variances
-      int* sub_rows = reinterpret_cast<int*>(vout + G * D);            // [G][D]
-      for (int g0 = 0; g0 < nseg; g0 += G) {
-        const int ng = min(G, nseg - g0);
-        for (int e = tid; e < ng * D; e += nt) {
-          const int gi = e / D, j = e % D;
-          const int a = slo[g0 + gi], sz = slo[g0 + gi + 1] - a;
-          const int m = min(D, sz);
-          // residue-major: sample j sits at (j % 8) * (D / 8) + j / 8 of its subset's D entries
-          sub_rows[gi * D + (j & 7) * (D / 8) + (j >> 3)] =
-              (sz > c && j < m) ? rows[a + (int)(((unsigned)j * (unsigned)sz) / (unsigned)m)] : -1;
-        }
-        __syncthreads();
-        gathered_variances<D>(Y, sub_rows, ng,
-                              [&](int gi) { const int sz = slo[g0 + gi + 1] - slo[g0 + gi]; return sz > c ? min(D, sz) : 0; },
-                              part, vout, tid, nt);
-        for (int task = tid; task < ng * D; task += nt) {
-          const int gi = task / D, t = task % D, g = g0 + gi;
-          float v = vout[task];                        // -1 for a subset that is already final
-          // argmax inside the warp (32 consecutive coordinates), lowest coordinate on ties
-          int at = t;
-          for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-            const int oa = __shfl_xor_sync(0xffffffffu, at, o);
-            if (ov > v || (ov == v && oa < at)) { v = ov; at = oa; }
-          }
-          if (lane == 0) { sm.best[g][(t / 32)] = v; sm.arg[g][(t / 32)] = at; }
-        }
-        __syncthreads();
-      }
+    // ---- 1. coordinate of largest subsample variance for every subset that still splits
+#pragma unroll 1
+    for (int unit = warp; unit < nseg * UNITS; unit += NW) {
+      const int g = unit / UNITS, block = unit % UNITS;
+      const int a = slo[g], sz = slo[g + 1] - a;
+      if (sz <= c) continue;
+      if (sz >= D) unit_variance<D, V, true>(Y, rows + a, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
+      else unit_variance_small<D, V>(Y, rows + a, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
     }
-    if (tid < nseg) {
-      const int a = slo[tid], sz = slo[tid + 1] - a;
-      float v = sm.best[tid][0]; int at = sm.arg[tid][0];
-      for (int w = 1; w < wps; ++w)
-        if (sm.best[tid][w] > v) { v = sm.best[tid][w]; at = sm.arg[tid][w]; }   // later warps hold higher coordinates
-      sm.seg_coord[tid] = at;
-      sm.seg_L[tid] = sz > c ? c * ((sz + c) / (2 * c)) : 0;
-      sm.seg_prefix[tid] = 0u;
-      sm.seg_rem[tid] = sm.seg_L[tid];
+    __syncthreads();
+    if (warp == 0) {
+      const bool live = lane < nseg;
+      const int a = live ? slo[lane] : 0, sz = live ? slo[lane + 1] - a : 0;
+      const bool splits = sz > c;
+      const int L = splits ? c * ((sz + c) / (2 * c)) : 0;
+      const unsigned ballot = __ballot_sync(0xffffffffu, splits);
+      const int child = lane + __popc(ballot & ((1u << lane) - 1u));
+      int coord = 0;
+      if (splits) {
+        float v = sm.unit_best[lane][0];
+        int at = 0;
+#pragma unroll
+        for (int b = 1; b < UNITS; ++b) {
+          const float q = sm.unit_best[lane][b];
+          if (q > v) { v = q; at = b; }                  // later blocks hold higher coordinates
+        }
+        const int2 am = sm.unit_arg[lane][at];
+        coord = am.x;
+        const float scale = 64.f * rsqrtf(v), shift = fmaf(-__int_as_float(am.y), scale, 128.f);
+        const bool usable = v > 0.f && scale < 1e30f && fabsf(shift) < 1e30f;     // also false for NaN
+        sm.seg_map[lane] = usable ? make_float2(scale, shift) : make_float2(0.f, 128.f);
+      }
+      int before = L;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += x;
+      }
+      if (live) {
+        sm.seg[lane] = make_int4(coord, L, a, child);
+        sm.seg_base[lane] = before - L;
+        sm.seg_cand[lane] = 0;
+        int* nlo = sm.seg_lo[cur ^ 1];
+        nlo[child] = a;
+        if (splits) nlo[child + 1] = a + L;
+      }
+      const bool more = __any_sync(0xffffffffu, splits && (L > c || sz - L > c));
+      if (lane == 0) {
+        sm.nseg = nseg + __popc(ballot);
+        sm.seg_lo[cur ^ 1][nseg + __popc(ballot)] = s0;
+        sm.more = more;
+        sm.crowded = 0u;
+      }
     }
     __syncthreads();
 
-    // ---- 2. keys.  A thread owns four consecutive positions for the rest of the level (their
-    // keys stay in registers); the first finds its subset by bisection of the start offsets, the
-    // others walk on from there.
-    constexpr int PT = kTailRowsMax / kSplitThreads;     // positions per thread
-    static_assert(PT == 4 && kSplitThreads == 1024, "the scan below stores four counts per thread and scans 32 warp totals");
-    int my_seg[PT];
-    uint32_t my_key[PT];
-    {
-      const int i0 = PT * tid;
-      int g = 0;
-      if (i0 < s0) {
-        int hi = nseg;                                  // slo[g] <= i0 < slo[g+1]
-        while (hi - g > 1) { const int mid = (g + hi) >> 1; if (slo[mid] <= i0) g = mid; else hi = mid; }
-      }
-#pragma unroll
-      for (int u = 0; u < PT; ++u) {
-        const int i = i0 + u;
-        my_key[u] = 0u;
-        if (i < s0) {
-          while (slo[g + 1] <= i) ++g;
-          const bool splits = slo[g + 1] - slo[g] > c;
-          if (splits) my_key[u] = order_key(Yt ? __ldg(Yt + (size_t)sm.seg_coord[g] * sd.n + rows[i])
-                                               : __ldg(Y + (size_t)rows[i] * D + sm.seg_coord[g]));
-          my_seg[u] = splits ? g : -1 - g;              // final subset: carried over unchanged
-        } else {
-          my_seg[u] = INT_MIN;
-        }
+    // ---- 2. values, keys and bins
+#pragma unroll 2
+    for (int i = w0 + lane; i < w1; i += 32) {
+      const int4 sg = sm.seg[sm.state[i] >> 8];
+      const int row = rows[i];
+      const bool column = Yt && sg.x < kSplitCols;
+      if (sg.y > 0) cp_async4(&sm.keys[i], column ? Yt + (size_t)sg.x * sd.n + row : Y + (size_t)row * D + sg.x);
+    }
+    cp_async_wait_all();
+#pragma unroll 1
+    for (int i = w0 + lane; i < w1; i += 32) {
+      const int g = sm.state[i] >> 8;
+      if (sm.seg[g].y == 0) continue;
+      const float x = __uint_as_float(sm.keys[i]);
+      const uint32_t key = order_key(x);
+      // the bin grows with the key for every value: infinities land at the ends (the scale is positive
+      // and finite, or zero and all bins equal), NaNs are put where their keys stand
+      const float2 map = sm.seg_map[g];
+      int bin = (int)fminf(fmaxf(fmaf(x, map.x, map.y), 0.f), 255.f);
+      if (x != x) bin = (int)key < 0 ? 255 : 0;
+      if (map.x == 0.f) bin = 0;
+      sm.keys[i] = key;
+      sm.state[i] = (uint16_t)(g << 8 | bin);
+      atomicAdd(&sm.hist[g][bin >> 1], 1u << (16 * (bin & 1)));
+    }
+    __syncthreads();
+
+    // ---- 3. the bin with the L-th value
+#pragma unroll 1
+    for (int g = warp; g < nseg; g += NW) {
+      const int L = sm.seg[g].y;
+      if (L == 0) continue;                              // warp-uniform
+      int bin, rank, rows_in;
+      if (pick_bin(sm.hist[g], L, lane, bin, rank, rows_in)) {
+        if (rows_in > kTailList) { atomicOr(&sm.crowded, 1u << g); bin = -1; }
+        sm.seg_pick[g] = make_int2(bin, rank);
       }
     }
+    __syncthreads();
+    const unsigned crowded = sm.crowded;
+    if (crowded) tail_thresholds_by_digits<nt>(sm, crowded, s0, nseg, slo, tid);
 
-    tail_select_partition(sm, my_seg, my_key, nseg, slo, rows, rows_next, tid, &sm.hist[0][0], sm.scan);
-    // ---- next level's subsets
-    if (tid == 0) {
-      int* nlo = sm.seg_lo[cur ^ 1];
-      int n2 = 0, more = 0;
-      for (int g = 0; g < nseg; ++g) {
-        const int a = slo[g], sz = slo[g + 1] - a;
-        nlo[n2++] = a;
-        if (sz > c) {
-          const int L = sm.seg_L[g];
-          nlo[n2++] = a + L;
-          more |= (L > c) | (sz - L > c);
-        }
+    // ---- 4. the rows of that bin, ranked by (key, position)
+#pragma unroll 2
+    for (int i = w0 + lane; i < w1; i += 32) {
+      const int st = sm.state[i], g = st >> 8;
+      if (sm.seg[g].y > 0 && (st & 255) == sm.seg_pick[g].x)
+        sm.list[g][atomicAdd(&sm.seg_cand[g], 1)] = ((unsigned long long)sm.keys[i] << 32) | (unsigned)i;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int g = warp; g < nseg; g += NW) {
+      if (sm.seg[g].y == 0) continue;
+      const int n = sm.seg_cand[g], rank = sm.seg_pick[g].y - 1;
+      const unsigned long long e0 = sm.list[g][lane], e1 = sm.list[g][32 + lane];   // beyond n: not used
+      int r0 = 0, r1 = 0;
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) {
+        const unsigned long long v = sm.list[g][j];
+        r0 += v < e0 ? 1 : 0;
+        r1 += v < e1 ? 1 : 0;
       }
-      nlo[n2] = s0;
-      sm.nseg[cur ^ 1] = n2;
-      sm.more = more;
+      if (lane < n && r0 == rank) sm.seg_thr[g] = e0;                              // exactly one lane
+      if (32 + lane < n && r1 == rank) sm.seg_thr[g] = e1;
+    }
+    __syncthreads();
+
+    // ---- 5. stable partition
+    auto goes_down = [&](int i) {
+      const int g = sm.state[i] >> 8;
+      return sm.seg[g].y > 0 && (((unsigned long long)sm.keys[i] << 32) | (unsigned)i) <= sm.seg_thr[g];
+    };
+    int total = 0;
+#pragma unroll 2
+    for (int i = w0 + lane; i - lane < w1; i += 32)
+      total += __popc(__ballot_sync(0xffffffffu, i < w1 && goes_down(i)));
+    if (lane == 0) sm.warp_tot[warp] = total;
+    __syncthreads();
+    int below = (int)__reduce_add_sync(0xffffffffu, lane < warp ? sm.warp_tot[lane & (NW - 1)] : 0);
+#pragma unroll 1
+    for (int i = w0 + lane; i - lane < w1; i += 32) {
+      const bool down = i < w1 && goes_down(i);
+      const unsigned b = __ballot_sync(0xffffffffu, down);
+      if (i < w1) {
+        const int g = sm.state[i] >> 8;
+        const int4 sg = sm.seg[g];
+        const int mine = below + __popc(b & ((1u << lane) - 1u)) - sm.seg_base[g];
+        const int dst = sg.y == 0 ? i : (down ? sg.z + mine : i + sg.y - mine);
+        rows_next[dst] = rows[i];
+        // the subsets of the next level stand at known positions
+        sm.state[i] = (uint16_t)((sg.w + (sg.y > 0 && i - sg.z >= sg.y ? 1 : 0)) << 8);
+      }
+      below += __popc(b);
     }
     __syncthreads();
     cur ^= 1;
   }
+#pragma unroll 1
   for (int i = tid; i < s0; i += nt) pout[lo + i] = sm.rows[cur][i];
 }
 
@@ -844,18 +875,13 @@ static int tail_level_for(int n, int c) {
   return level;
 }
 
-int split_top_levels_for(int n, int c) { return tail_level_for(n, c); }
-
 int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q, int n_k, int c_q,
                  int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp, int32_t* perm_k_out,
                  int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k, int sides, cudaStream_t st,
                  const float* Ytq, const float* Ytk) {
   // sides: bit 0 = queries, bit 1 = keys
   auto level_kernel = D == 64 ? split_level_kernel<64> : split_level_kernel<128>;
-  auto tail_kernel = D == 64 ? split_tail_kernel<64> : split_tail_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRowsMax * 8));
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(TailSmem)));
   const bool do_q = (sides & 1) != 0, do_k = (sides & 2) != 0;
   const int tail_q = tail_level_for(n_q, c_q), tail_k = tail_level_for(n_k, c_k);
   const int top_q = do_q ? tail_q : 0, top_k = do_k ? tail_k : 0;
@@ -919,7 +945,12 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   prm.level = top_levels;
   prm.smem_rows = 0;
   const int slots = 1 << ((do_q ? tail_q : 0) > (do_k ? tail_k : 0) ? (do_q ? tail_q : 0) : (do_k ? tail_k : 0));
-  tail_kernel<<<dim3(slots, 2 * problems), kSplitThreads, sizeof(TailSmem), st>>>(prm);
+  const bool one_wave = 2 * slots * problems <= 148;      // both sides run at the same time
+  const int threads = one_wave ? 1024 : 512;
+  auto tail_kernel = D == 64 ? (one_wave ? split_tail_kernel<64, 1024> : split_tail_kernel<64, 512>)
+                             : (one_wave ? split_tail_kernel<128, 1024> : split_tail_kernel<128, 512>);
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TailSmem)));
+  tail_kernel<<<dim3(slots, 2 * problems), threads, sizeof(TailSmem), st>>>(prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -1097,6 +1128,169 @@ __global__ void __launch_bounds__(256) basic_keys_kernel(const BasicParams prm) 
 }
 
 // ---------------------------------------------------------------------------
+// Selection and partition of one level of a subtree, all of its subsets side by side: radix
+// selection of every subset's threshold key (seg_L, seg_rem, seg_prefix set up by the caller), then
+// the stable partition into rows_next.  A thread owns the four consecutive positions 4 tid .. 4 tid + 3
+// (my_seg: subset of a position, -1 - g in a final subset, INT_MIN past the end; my_key: its key).
+template <typename Smem>
+__device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_seg)[kTailRowsMax / kSplitThreads],
+                                                      const uint32_t (&my_key)[kTailRowsMax / kSplitThreads],
+                                                      int nseg, const int* slo, const int32_t* rows,
+                                                      int32_t* rows_next, int tid, int* hist, uint32_t* scan) {
+  constexpr int nt = kSplitThreads;
+  constexpr int PT = kTailRowsMax / kSplitThreads;
+  const int lane = tid & 31, warp = tid >> 5;
+  // ---- radix selection, all subsets side by side: two digits of eight bits by counting; then the
+  // keys that share those sixteen bits with the threshold are few (a handful per subset unless keys
+  // repeat), and a warp ranks them directly.  A subset with more than 32 of them goes on with the two
+  // remaining digits.  (The digit counts are cleared once per level: the warp that picks a subset's
+  // digit clears the counts it has read, ready for the next pass.)
+  uint32_t mask = 0;
+  for (int e = tid; e < nseg * 256; e += nt) hist[e] = 0;
+  if (tid < nseg) sm.seg_cand[tid] = 0;
+  if (tid == 0) sm.overflow = 0;
+  __syncthreads();
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    uint32_t pre[PT];                               // read ahead of the atomics, which order memory accesses
+#pragma unroll
+    for (int u = 0; u < PT; ++u) pre[u] = sm.seg_prefix[my_seg[u] >= 0 ? my_seg[u] : 0];
+    if (shift == 8) {
+      // candidates of every subset into its list (the scan array is free until the partition)
+#pragma unroll
+      for (int u = 0; u < PT; ++u) {
+        const int g = my_seg[u];
+        if (g >= 0 && (my_key[u] & mask) == pre[u]) {
+          const int slot = atomicAdd(&sm.seg_cand[g], 1);
+          if (slot < 32) scan[g * 32 + slot] = my_key[u];
+        }
+      }
+      __syncthreads();
+      for (int g = warp; g < nseg; g += nt / 32) {
+        if (sm.seg_L[g] == 0) continue;             // warp-uniform
+        const int n = sm.seg_cand[g];
+        if (n > 32) {
+          if (lane == 0) sm.overflow = 1;
+          continue;
+        }
+        const int remaining = sm.seg_rem[g];        // 1 <= remaining <= n
+        const uint32_t key = lane < n ? scan[g * 32 + lane] : 0xffffffffu;
+        int less = 0, eq_before = 0;
+        for (int j = 0; j < n; ++j) {
+          const uint32_t kj = __shfl_sync(0xffffffffu, key, j);
+          less += kj < key ? 1 : 0;
+          eq_before += (kj == key && j < lane) ? 1 : 0;
+        }
+        if (lane < n && less + eq_before == remaining - 1) {   // exactly one lane
+          sm.seg_prefix[g] = key;
+          sm.seg_rem[g] = remaining - less;          // how many of the keys equal to the threshold go down
+          sm.seg_cand[g] = -1;
+        }
+      }
+      __syncthreads();
+      if (!sm.overflow) break;                      // uniform: every threshold is found
+#pragma unroll
+      for (int u = 0; u < PT; ++u) pre[u] = sm.seg_prefix[my_seg[u] >= 0 ? my_seg[u] : 0];
+    }
+#pragma unroll
+    for (int u = 0; u < PT; ++u) {
+      const int g = my_seg[u];
+      const bool live = g >= 0;
+      const uint32_t k = my_key[u];
+      if (live && ((k & mask) == pre[u])) atomicAdd(&hist[(g << 8) | (int)((k >> shift) & 255u)], 1);
+    }
+    __syncthreads();
+    for (int g = warp; g < nseg; g += nt / 32) {
+      const int remaining = sm.seg_rem[g];
+      if (sm.seg_L[g] == 0) continue;               // warp-uniform
+      int local[8]; int sum = 0;
+      {
+        int4* h4 = reinterpret_cast<int4*>(&hist[g * 256 + lane * 8]);
+        const int4 h0 = h4[0], h1 = h4[1];
+        h4[0] = make_int4(0, 0, 0, 0);
+        h4[1] = make_int4(0, 0, 0, 0);
+        local[0] = h0.x; local[1] = h0.y; local[2] = h0.z; local[3] = h0.w;
+        local[4] = h1.x; local[5] = h1.y; local[6] = h1.z; local[7] = h1.w;
+      }
+      if (sm.seg_cand[g] < 0) continue;             // found by the direct ranking (its keys were still counted)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum += local[j];
+      int incl = sum;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      int before = incl - sum;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (before < remaining && remaining <= before + local[j]) {
+          sm.seg_digit[g] = lane * 8 + j;
+          sm.seg_rem[g] = remaining - before;
+        }
+        before += local[j];
+      }
+      __syncwarp();
+      if (lane == 0) sm.seg_prefix[g] |= (uint32_t)sm.seg_digit[g] << shift;
+    }
+    mask |= 255u << shift;
+    __syncthreads();
+  }
+
+  // ---- 3. stable partition of every subset: one scan of (less | equal << 16) over all positions
+  // (a thread's four, then the warp, then the warps' totals by warp 0)
+  uint32_t my_scan[PT];
+  {
+    int run = 0;
+#pragma unroll
+    for (int u = 0; u < PT; ++u) {
+      if (my_seg[u] >= 0) {
+        const uint32_t k = my_key[u], thr = sm.seg_prefix[my_seg[u]];
+        run += (k < thr ? 1 : 0) | (k == thr ? 1 << 16 : 0);
+      }
+      my_scan[u] = (uint32_t)run;
+    }
+    int incl = run;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) sm.warp_tot[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const int v = sm.warp_tot[lane];                 // nt / 32 == 32 warps
+      int wi = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, wi, o);
+        if (lane >= o) wi += x;
+      }
+      sm.warp_tot[lane] = wi - v;                      // totals of the warps before this one
+    }
+    __syncthreads();
+    const uint32_t before = (uint32_t)(sm.warp_tot[warp] + incl - run);
+#pragma unroll
+    for (int u = 0; u < PT; ++u) my_scan[u] += before;
+    *reinterpret_cast<uint4*>(&scan[PT * tid]) = make_uint4(my_scan[0], my_scan[1], my_scan[2], my_scan[3]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int u = 0; u < PT; ++u) {
+    const int i = PT * tid + u;
+    const int g = my_seg[u];
+    if (g == INT_MIN) continue;
+    if (g < 0) { rows_next[i] = rows[i]; continue; }
+    const int a = slo[g];
+    const uint32_t base = a > 0 ? scan[a - 1] : 0u;
+    const uint32_t k = my_key[u], thr = sm.seg_prefix[g];
+    const int is_less = k < thr, is_eq = k == thr;
+    const uint32_t excl = my_scan[u] - base - (uint32_t)(is_less | (is_eq << 16));
+    const int less_here = (int)(excl & 0xffffu), eq_here = (int)(excl >> 16);
+    const int eq_left = sm.seg_rem[g], L = sm.seg_L[g];
+    const bool down = is_less || (is_eq && eq_here < eq_left);
+    const int down_before = less_here + min(eq_here, eq_left);
+    const int dst = down ? a + down_before : a + L + (i - a - down_before);
+    rows_next[dst] = rows[i];
+  }
+}
+
 // Subtree of the basic variant: a set of at most kTailRowsMax rows finished by one CTA, so that
 // the deepest levels are one launch instead of three per level.  Per level: the directions of all
 // subsets that still split (a team of D threads per subset; the operations of

@@ -182,7 +182,7 @@ struct LinCfg {
 
 struct LinParams {
   const float* bias;      // [P][D] or null
-  float* out_t;           // [P][D][n_rows] or null: the fp32 result once more, coordinate-major
+  float* out_t;           // [P][kSplitCols][n_rows] or null: the first coordinates once more, coordinate-major
   int* status;
   int n_rows, tiles_per_cta, stages, normalize;       // normalize: rows are divided by their norm before the bias
 };
@@ -315,15 +315,13 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         for (int j = 0; j < D; ++j) v[j] += s_bias[j];
       }
       if (prm.out_t) {
-        // coordinate-major copy: for one coordinate the 128 threads of the tile write 512
-        // consecutive bytes.  The splitter gathers one coordinate of scattered rows per level; from
-        // this layout that is a 4-byte read inside an L2-resident column instead of one DRAM line
-        // per row of the row-major result.
+        // coordinate-major copy of the coordinates that the splitter reads one at a time: for one
+        // coordinate the 128 threads of the tile write 512 consecutive bytes
         const int grow = (t_begin + t) * kRows + row;
         if (grow < prm.n_rows) {
-          float* dst = prm.out_t + (size_t)p * D * prm.n_rows + grow;
+          float* dst = prm.out_t + (size_t)p * kSplitCols * prm.n_rows + grow;
 #pragma unroll
-          for (int j = 0; j < D; ++j) dst[(size_t)j * prm.n_rows] = v[j];
+          for (int j = 0; j < kSplitCols; ++j) dst[(size_t)j * prm.n_rows] = v[j];
         }
       }
       // the previous tile's stores must have finished reading the staging buffer

@@ -1,0 +1,67 @@
+"""The subtree kernel of the splitter where its selection changes path, bit for bit against the oracle: bins
+that hold more rows than a list takes (far outliers, repeated values, infinities), subsets of fewer rows
+than a full sample, subtrees of exactly and just above the largest size, one wave of CTAs or several;
+and split coordinates beyond those that are kept coordinate-major."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import clusterattn_oracle as orc
+from paper_2608_26965_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _coordinates(kind, heads, n, d, seed):
+    r = np.random.default_rng(seed)
+    Y = r.standard_normal((heads, n, d)).astype(np.float32)
+    if kind == "outliers":
+        Y *= np.where(r.random((heads, n, 1)) < 0.01, 1e4, 1.0).astype(np.float32)
+    elif kind == "repeated":
+        Y[r.random((heads, n)) < 0.9] = 0.0
+    elif kind == "two values":
+        Y = np.where(Y > 0.3, np.float32(2.0), np.float32(-1.0))
+    elif kind == "huge":
+        Y[:, 5::7] *= np.float32(1e25)
+        Y[:, 3::4] *= np.float32(1e-30)
+    return Y
+
+
+@pytest.mark.parametrize("kind,heads,n,d,c", [
+    ("normal", 1, 4096, 64, 128), ("normal", 1, 4097, 128, 128), ("normal", 40, 4096, 128, 128),
+    ("normal", 90, 515, 64, 16), ("normal", 2, 513, 128, 16),
+    ("outliers", 1, 4096, 128, 256), ("outliers", 80, 1030, 64, 64), ("outliers", 40, 2000, 128, 64),
+    ("repeated", 2, 4095, 64, 128), ("repeated", 80, 700, 128, 32),
+    ("two values", 1, 4096, 64, 128), ("huge", 1, 2049, 64, 64), ("huge", 80, 600, 128, 64),
+])
+def test_subtrees_match_the_oracle(kind, heads, n, d, c):
+    Y = _coordinates(kind, heads, n, d, n + d)
+    p = binding.make_problem(1, heads, n, n, d, "bf16", c, c, 1, flags=binding.CA_Y_IN)
+    plan = binding.Plan(p, DEV)
+    X = torch.zeros((1, heads, n, d), dtype=torch.bfloat16, device=DEV)
+    Yd = torch.from_numpy(Y[None]).to(DEV)
+    plan.cluster_qk(X, X, X, Yq=Yd, Yk=Yd)
+    torch.cuda.synchronize()
+    assert all(v == 0 for v in plan.last_status().values())
+    for h in sorted({0, heads // 2, heads - 1}):
+        ref = orc.recursive_split_f32(Y[h], c)
+        assert np.array_equal(plan.perm_q[0, h].cpu().numpy(), ref), f"queries, head {h}"
+        assert np.array_equal(plan.perm_k[0, h].cpu().numpy(), ref), f"keys, head {h}"
+
+
+@pytest.mark.parametrize("heads,n,d,c", [(2, 3000, 64, 16), (40, 6000, 128, 32), (1, 20000, 64, 16)])
+def test_split_coordinates_beyond_the_coordinate_major_ones(heads, n, d, c):
+    """Isotropic rows: small subsets split along any of the d coordinates."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n)
+    X = torch.randn((3, 1, heads, n, d), generator=g, device=DEV).to(torch.bfloat16)
+    plan = binding.Plan(binding.make_problem(1, heads, n, n, d, "bf16", c, c, 1), DEV)
+    Yq = torch.empty((1, heads, n, d), device=DEV)
+    Yk = torch.empty((1, heads, n, d), device=DEV)
+    plan.cluster_qk(X[0], X[1], X[2], Yq=Yq, Yk=Yk)
+    torch.cuda.synchronize()
+    assert all(v == 0 for v in plan.last_status().values())
+    for h in sorted({0, heads - 1}):
+        assert np.array_equal(plan.perm_q[0, h].cpu().numpy(), orc.recursive_split_f32(Yq[0, h].cpu().numpy(), c))
+        assert np.array_equal(plan.perm_k[0, h].cpu().numpy(), orc.recursive_split_f32(Yk[0, h].cpu().numpy(), c))
