@@ -5,8 +5,8 @@
 //   1. takes m = min(d, s) rows at positions floor(j*s/m), estimates the variance
 //      of each coordinate over them in float32 with a fixed operation order and
 //      picks the coordinate of largest variance, lowest index on exact ties;
-//   2. finds, by radix selection on order-preserving 32-bit keys, the L-th
-//      smallest (value, row) along it, L = c * floor((s + c) / (2c));
+//   2. finds, by counting into bins and ranking one bin, the L-th smallest
+//      (value, row) along it, L = c * floor((s + c) / (2c));
 //   3. moves the L smallest rows to [lo, lo+L) and the others to [lo+L, lo+s),
 //      both sides keeping their order (stable partition by prefix sums).
 // Nothing depends on floating-point rounding except step 1, whose operation
@@ -31,10 +31,11 @@ namespace ca {
 
 namespace cg = cooperative_groups;
 
-constexpr int kSplitThreads = 1024;
+constexpr int kSplitThreads = 1024;      // subtree kernel of the basic variant
 constexpr int kSmemRowsMax = 24576;      // rows a CTA stages (8 bytes each)
 constexpr int kMaxCluster = 8;
-constexpr int kLevelListMax = 1024;      // candidates that the level kernel ranks from a list after two digits
+constexpr int kLevelBins = 1024;
+constexpr int kLevelList = 512;          // candidates that the level kernel ranks from a list
 constexpr int kTailRowsMax = 4096;
 constexpr int kTailSegs = 32;            // subsets a tail CTA splits side by side
 
@@ -63,45 +64,6 @@ __device__ __forceinline__ uint32_t order_key(float x) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Variances of all coordinates over subsamples staged in shared memory, `ng` tiles of
-// tile[j*D + t], j < m_g.  The estimate only feeds an argmax, so it is taken in float32 with
-// a fixed operation order (reproducible bit for bit; every operation rounded on its own, no
-// fused multiply-add): eight partial sums over the rows j = r, r+8, ... taken row after row,
-// combined as ((p0+p1)+(p2+p3)) + ((p4+p5)+(p6+p7)); first the mean, then the squared
-// deviations.  part: [ng][8][D] floats, out: [ng][D] floats.  Called by all threads of the CTA.
-template <int D, typename RowsOf>
-__device__ __forceinline__ void staged_variances(const float* tiles, int ng, RowsOf rows_of,
-                                                 float* part, float* out, int tid, int nt) {
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int task = tid; task < ng * 8 * D; task += nt) {
-      const int gi = task / (8 * D), r = (task / D) % 8, t = task % D;
-      const int m = rows_of(gi);
-      const float* tile = tiles + gi * D * D;
-      float acc = 0.f;
-      if (pass == 0) {
-        for (int j = r; j < m; j += 8) acc = __fadd_rn(acc, tile[j * D + t]);
-      } else {
-        const float mean = out[gi * D + t];
-        for (int j = r; j < m; j += 8) {
-          const float dev = __fsub_rn(tile[j * D + t], mean);
-          acc = __fadd_rn(acc, __fmul_rn(dev, dev));
-        }
-      }
-      part[(gi * 8 + r) * D + t] = acc;
-    }
-    __syncthreads();
-    for (int task = tid; task < ng * D; task += nt) {
-      const int gi = task / D, t = task % D;
-      const float* p = part + gi * 8 * D + t;
-      const float tot = __fadd_rn(__fadd_rn(__fadd_rn(p[0], p[D]), __fadd_rn(p[2 * D], p[3 * D])),
-                                  __fadd_rn(__fadd_rn(p[4 * D], p[5 * D]), __fadd_rn(p[6 * D], p[7 * D])));
-      const int m = rows_of(gi);
-      out[task] = m > 0 ? __fdiv_rn(tot, (float)m) : -1.0f;
-    }
-    __syncthreads();
-  }
-}
-
 // Two fp32 values in one 64-bit register and the instructions that work on both halves at once
 // (each half rounded to nearest on its own: the same bits as two scalar operations).
 typedef unsigned long long pair2;
@@ -119,14 +81,18 @@ __device__ __forceinline__ pair2 add_pair(pair2 a, pair2 b) {
   return d;
 }
 
-// The same estimate for one block of 4 V coordinates of one subset, by one warp: lane = 4 r + q
-// takes the sample rows r, r + 8, ... of V consecutive coordinates.  The eight residues are combined by
-// a butterfly over the lanes, which adds in the order of staged_variances, hence the same bits; a
-// row is read once and kept in registers for the squares, and no barrier is needed.  Writes the largest
-// variance of the block, and its coordinate (the lowest on ties) with that coordinate's mean.
-template <int D, int V, bool full>          // full: the subset has at least D rows
-__device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const int32_t* rows, int sz, int block, int lane,
-                                              float* best_out, int2* arg_out) {
+// Largest variance over the subsample of one block of 4 V coordinates of one subset, by one warp.  The estimate
+// only feeds an argmax, so it is taken in float32 with a fixed operation order (reproducible bit for
+// bit; every operation rounded on its own, no fused multiply-add): eight partial sums over the rows
+// j = r, r+8, ... taken row after row, combined as ((p0+p1)+(p2+p3)) + ((p4+p5)+(p6+p7)); first the
+// mean, then the squared deviations.  Lane 4 r + q takes the rows of residue r and V consecutive
+// coordinates, and a butterfly over the lanes adds the residues in that order; a row is read once
+// and kept in registers for the squares, and no barrier is needed.  Writes the largest variance of the
+// block, and its coordinate (the lowest on ties) with that coordinate's mean.
+// rows: the subset's rows, in shared memory, or (global) in global memory or null, then first, first + 1, ...
+template <int D, int V, bool full, bool global>      // full: the subset has at least D rows
+__device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const int32_t* rows, int first, int sz, int block,
+                                              int lane, float* best_out, int2* arg_out) {
   constexpr int PER = D / 8;                         // sample rows of a residue
   const int r = lane >> 2, t = (block * 4 + (lane & 3)) * V;
   const int m = full ? D : sz;
@@ -137,7 +103,7 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
   for (int k = 0; k < PER; ++k) {
     const unsigned j = r + 8 * k;
     const int pos = full ? (int)(j * (unsigned)sz / D) : min((int)j, m - 1);
-    const float* src = Y + (size_t)rows[pos] * D + t;
+    const float* src = Y + (size_t)(global ? (rows ? __ldg(rows + pos) : first + pos) : rows[pos]) * D + t;
     if constexpr (V == 4) {
       const float4 w = __ldg(reinterpret_cast<const float4*>(src));
       x[k][0] = pair(w.x, w.y);
@@ -223,17 +189,13 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
   }
 }
 // Out of line: only subsets of fewer than D rows take it, which split only where the cluster size is below D.
-template <int D, int V>
-__device__ __noinline__ void unit_variance_small(const float* __restrict__ Y, const int32_t* rows, int sz, int block, int lane,
-                                                 float* best_out, int2* arg_out) {
-  unit_variance<D, V, false>(Y, rows, sz, block, lane, best_out, arg_out);
+template <int D, int V, bool global>
+__device__ __noinline__ void unit_variance_small(const float* __restrict__ Y, const int32_t* rows, int first, int sz,
+                                                 int block, int lane, float* best_out, int2* arg_out) {
+  unit_variance<D, V, false, global>(Y, rows, first, sz, block, lane, best_out, arg_out);
 }
 
-// 16-byte asynchronous copy global -> shared (no registers held while in flight)
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
-}
+// 4-byte asynchronous copy global -> shared (no register held while in flight)
 __device__ __forceinline__ void cp_async4(void* smem_dst, const void* gmem_src) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(gmem_src) : "memory");
@@ -253,32 +215,60 @@ struct SplitSide {
 struct SplitParams {
   SplitSide side[2];
   int D, level, problems, smem_rows;
-  int keys_in;             // the keys of this level are already in keybuf (basic variant): no coordinate choice, no gather
 };
+
+// Scale and offset of the bins of one coordinate: `half` bins to either side of the sample's mean for two
+// standard deviations; scale 0 (all rows in one bin) where that cannot be had.
+__device__ __forceinline__ float2 bin_map(float variance, float mean, float half) {
+  const float scale = 0.5f * half * rsqrtf(variance), shift = fmaf(-mean, scale, half);
+  const bool usable = variance > 0.f && scale < 1e30f && fabsf(shift) < 1e30f;     // also false for NaN
+  return usable ? make_float2(scale, shift) : make_float2(0.f, half);
+}
+// The bin of a value among `bins`.  It grows with the key for every value: infinities land at the ends
+// (the scale is positive and finite, or zero and all bins equal), NaNs are put where their keys stand.
+__device__ __forceinline__ int bin_of(float x, uint32_t key, float2 map, int bins) {
+  const float last = (float)(bins - 1);
+  int bin = (int)fminf(fmaxf(fmaf(x, map.x, map.y), 0.f), last);
+  if (x != x) bin = (int)key < 0 ? bins - 1 : 0;
+  return map.x == 0.f ? 0 : bin;
+}
+__device__ __forceinline__ float key_value(uint32_t key) {               // inverse of order_key
+  return __uint_as_float((key & 0x80000000u) ? key & 0x7fffffffu : ~key);
+}
 
 // ---------------------------------------------------------------------------
 // One level of the large sets.  grid.x = slots * cluster size.
 // ---------------------------------------------------------------------------
-template <int D>
-__global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitParams prm) {
+// A cluster per set, a slice of up to 8,192 rows per CTA where eight CTAs can hold the set that way.  A CTA is
+// a chain of short sweeps over its slice between barriers, bound by their latencies: two CTAs
+// share an SM and small sets take more CTAs while the SMs are not all taken.  The L-th value is found from
+// one count into 1,024 bins between mean - 2 s and mean + 2 s of the sample, the rows of its bin are
+// collected in the first CTA's list and every CTA ranks a copy.  Where the bin holds more rows than the
+// list (values repeat, far outliers) and for keys computed elsewhere (keys_in, the basic variant) the
+// digits of the key are counted eight bits a pass until the candidates fit the list, or are all equal.
+// Levels of both sides, against one CTA of 1,024 threads per 16,384 rows that counted two digits: 12 heads of
+// 16,385 rows, d = 64: 151 -> 103 us; 8 heads of 1,531 x 23,117 rows: 66 -> 44; 8 heads of 16,384 x 131,072 rows: 191
+// -> 160; 40 heads of 32,760 rows, d = 128: 214 -> 184.
+template <int D, int nt, bool keys_in>
+__global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_level_kernel(const SplitParams prm) {
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks();
   const int crank = (int)cluster.block_rank();
+  constexpr int NW = nt / 32;
+  constexpr int V = D == 64 ? 4 : 2, UNITS = D / (4 * V);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(smem_raw);                  // [smem_rows]
   int32_t* s_rows = reinterpret_cast<int32_t*>(s_keys + prm.smem_rows);      // [smem_rows]
-  __shared__ int s_hist2[2][256];  // digit counts of this slice, two in rotation over the passes
-  __shared__ int s_total[256];
-  __shared__ float s_var[128];
-  __shared__ float s_part[8 * 128];
-  __shared__ int s_sub[128];
-  __shared__ int s_warp[2 * 32];
-  __shared__ int s_scalar[4];      // 0: coordinate, 1: digit, 2: remaining rank, 3: chunk total
-  __shared__ int s_counts[2];      // this CTA's (less, equal) totals
-  __shared__ uint32_t s_list[kLevelListMax];   // the keys that share the first two digits with the threshold
-  __shared__ int s_list_n;         // entries of the list (counted in the cluster's first CTA)
-  __shared__ int s_ncand;          // keys in the digit that the last pass chose
-  int* const s_hist = s_hist2[1];  // scratch of the partition (the last pass counts in the other array)
+  __shared__ __align__(8) int s_hist[kLevelBins];        // bins, or 256 digits for each of four passes
+  __shared__ unsigned long long s_list[kLevelList];      // (key, position in the set)
+  __shared__ int s_list_n;                               // counted in the cluster's first CTA
+  __shared__ float s_best[UNITS];
+  __shared__ int2 s_arg[UNITS];
+  __shared__ float2 s_map;
+  __shared__ int s_coord, s_pick[3];                     // bin, 1-based rank inside it, its rows
+  __shared__ int s_warp[NW];
+  __shared__ int s_total;                                // of this CTA, read by its peers
+  __shared__ unsigned long long s_thr;                   // the last (key, position) that goes down
 
   const int which = blockIdx.y / prm.problems;
   const int p = blockIdx.y % prm.problems;
@@ -286,242 +276,254 @@ __global__ void __launch_bounds__(kSplitThreads) split_level_kernel(const SplitP
   if (!sd.active || prm.level >= sd.tail_level) return;   // uniform over the cluster
   const SegmentRef seg = locate_segment(sd.n, sd.c, prm.level, blockIdx.x / csize);
   if (!seg.active) return;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* Y = sd.Y + (size_t)p * sd.n * D;
   const int32_t* pin = sd.perm_in ? sd.perm_in + (size_t)p * sd.n : nullptr;
   int32_t* pout = sd.perm_out + (size_t)p * sd.n;
   const int lo = seg.lo, s = seg.size;
+  auto row_at = [pin, lo](int i) { return pin ? __ldg(pin + lo + i) : lo + i; };
+  auto sync_all = [&]() {
+    if (csize > 1) cluster.sync();
+    else __syncthreads();
+  };
 
   if (s <= sd.c) {                                   // final set: carry over
     if (crank == 0)
-      for (int i = tid; i < s; i += nt) pout[lo + i] = pin ? pin[lo + i] : lo + i;
+#pragma unroll 1
+      for (int i = tid; i < s; i += nt) pout[lo + i] = row_at(i);
     return;
   }
 
   // ---- 1. coordinate of largest subsample variance (every CTA of the cluster computes it)
-  const int m = min(D, s);
-  int coord = 0;
-  if (!prm.keys_in) {
-  if (tid < m) {
-    const int pos = lo + (int)(((long long)tid * s) / m);
-    s_sub[tid] = pin ? pin[pos] : pos;
-  }
-  __syncthreads();
-  {
-    // the subsample rows are staged by all threads (16-byte loads in flight together)
-    float4* stage4 = reinterpret_cast<float4*>(smem_raw);
-    constexpr int q = D / 4;
-    for (int e = tid; e < m * q; e += nt)
-      cp_async16(stage4 + e, reinterpret_cast<const float4*>(Y + (size_t)s_sub[e / q] * D) + (e % q));
-    cp_async_wait_all();
-  }
-  __syncthreads();
-  staged_variances<D>(reinterpret_cast<const float*>(smem_raw), 1, [&](int) { return m; }, s_part, s_var, tid, nt);
-  if (warp == 0) {
-    float best = -1.0f; int arg = 0;
-    for (int t = lane; t < D; t += 32) {
-      const float v = s_var[t];
-      if (v > best) { best = v; arg = t; }
+  if (tid < kLevelBins / 2) reinterpret_cast<int2*>(s_hist)[tid] = make_int2(0, 0);
+  if (tid == 0) s_list_n = 0;
+  if constexpr (!keys_in) {
+#pragma unroll 1
+    for (int unit = warp; unit < UNITS; unit += NW) {
+      const int32_t* set = pin ? pin + lo : nullptr;
+      if (s >= D) unit_variance<D, V, true, true>(Y, set, lo, s, unit, lane, &s_best[unit], &s_arg[unit]);
+      else unit_variance_small<D, V, true>(Y, set, lo, s, unit, lane, &s_best[unit], &s_arg[unit]);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-      if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; }
+    __syncthreads();
+    if (warp == 0) {
+      float v = s_best[lane % UNITS];
+      int at = lane % UNITS;
+#pragma unroll
+      for (int o = 1; o < UNITS; o <<= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int oa = __shfl_xor_sync(0xffffffffu, at, o);
+        if (ov > v || (ov == v && oa < at)) { v = ov; at = oa; }       // later blocks hold higher coordinates
+      }
+      if (lane == 0) {
+        const int2 am = s_arg[at];
+        s_coord = am.x;
+        s_map = bin_map(v, __int_as_float(am.y), kLevelBins / 2);
+      }
     }
-    if (lane == 0) s_scalar[0] = arg;
   }
   __syncthreads();
-  coord = s_scalar[0];
-  }
 
-  // ---- 2. keys of this CTA's slice [c0, c1) of the set
+  // ---- 2. keys of this CTA's slice [c0, c1) of the set, and their bins
   const int chunk = (s + csize - 1) / csize;
   const int c0 = min(s, crank * chunk), c1 = min(s, c0 + chunk);
   const int cs = c1 - c0;
   const bool in_smem = cs <= prm.smem_rows;
-  uint32_t* keys = in_smem ? s_keys : sd.keybuf + (size_t)p * sd.n + lo + c0;
-  if (prm.keys_in) {
+  uint32_t* g_keys = sd.keybuf + (size_t)p * sd.n + lo + c0;
+  auto key_at = [&](int i) { return in_smem ? s_keys[i] : g_keys[i]; };
+  float2 map = make_float2(0.f, 0.f);
+  if constexpr (keys_in) {
     // the projections of this level were turned into keys by another kernel, position by position
     if (in_smem) {
-      const uint32_t* kin = sd.keybuf + (size_t)p * sd.n + lo + c0;
+#pragma unroll 4
       for (int i = tid; i < cs; i += nt) {
-        s_keys[i] = kin[i];
-        s_rows[i] = pin ? pin[lo + c0 + i] : lo + c0 + i;
+        s_keys[i] = g_keys[i];
+        s_rows[i] = row_at(c0 + i);
       }
     }
   } else {
-  // gathers in batches of eight: the row indices first, then the coordinates, so that the
-  // memory latencies of a batch overlap
-  const bool column = sd.Yt && coord < kSplitCols;
-  const float* Yc = column ? sd.Yt + ((size_t)p * kSplitCols + coord) * sd.n : Y + coord;
-  const int row_stride = column ? 1 : D;
-  for (int i0 = tid; i0 < cs; i0 += 8 * nt) {
-    int row[8];
-    float val[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * nt;
-      row[u] = (i < cs) ? (pin ? __ldg(pin + lo + c0 + i) : lo + c0 + i) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) val[u] = __ldg(Yc + (size_t)row[u] * row_stride);
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * nt;
-      if (i < cs) {
-        keys[i] = order_key(val[u]);
-        if (in_smem) s_rows[i] = row[u];
-      }
-    }
-  }
-  }
-  for (int b = tid; b < 256; b += nt) s_hist2[1][b] = 0;      // the first pass (shift 24) counts here
-  if (tid == 0) s_list_n = 0;
-  __syncthreads();
-
-  // ---- radix selection of the L-th smallest key of the whole set (8 bits per pass).  The slices'
-  // counts alternate between two arrays: a peer may still be adding up one pass's counts while
-  // this CTA counts the next pass, and an array is cleared only after the cluster barrier of the
-  // pass after the one that used it, when every peer has finished reading it.
-  // After two digits the keys that share them with the threshold are usually few: if they fit the
-  // list, every slice appends its candidates to the list of the cluster's first CTA (one more
-  // cluster barrier), every CTA takes a copy, and the last two digits are counted over that list
-  // alone, with no sweep over the slice, no cluster barrier and no sums over the peers.
-  const int L = sd.c * ((s + sd.c) / (2 * sd.c));
-  uint32_t prefix = 0, mask = 0;
-  int remaining = L;                                // 1-based rank among the candidates
-  bool listed = false;
-  int n_list = 0;
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    int* const hist = s_hist2[(shift >> 3) & 1];
-    int* const hist_next = s_hist2[((shift >> 3) & 1) ^ 1];
-    if (shift == 8 && s_ncand <= kLevelListMax) {   // uniform over the cluster: every CTA holds the same totals
-      listed = true;
-      n_list = s_ncand;
-      uint32_t* const list0 = csize > 1 ? cluster.map_shared_rank(s_list, 0) : s_list;
-      int* const count0 = csize > 1 ? cluster.map_shared_rank(&s_list_n, 0) : &s_list_n;
-      for (int i = tid; i < cs; i += nt) {
-        const uint32_t k = keys[i];
-        if ((k & mask) == prefix) list0[atomicAdd(count0, 1)] = k;   // n_list such keys in the whole set
-      }
-      if (csize > 1) {
-        cluster.sync();                              // the list is complete (and every peer is past the second pass)
-        if (crank != 0)
-          for (int i = tid; i < n_list; i += nt) s_list[i] = list0[i];
-      }
-      __syncthreads();
-    }
-    if (!listed) {
-      for (int i0 = 0; i0 < cs; i0 += nt) {
-        const int i = i0 + tid;
-        const bool ok = i < cs;
-        const uint32_t k = ok ? keys[i] : 0u;
-        // one atomic per candidate key, also for the leading digit with its few distinct values:
-        // a sweep of plain atomics costs the same whatever the digit's spread, and a warp match per
-        // position to merge equal digits costs three times as much
-        if (ok && ((k & mask) == prefix)) atomicAdd(&hist[(k >> shift) & 255u], 1);
-      }
-      if (csize > 1) {
-        cluster.sync();                              // every slice has counted
-        for (int b = tid; b < 256; b += nt) {
-          int sum = 0;
-          for (int r = 0; r < csize; ++r) sum += cluster.map_shared_rank(hist, r)[b];
-          s_total[b] = sum;
-        }
+    map = s_map;
+    const int coord = s_coord;
+    const bool column = sd.Yt && coord < kSplitCols;
+    const float* Yc = column ? sd.Yt + ((size_t)p * kSplitCols + coord) * sd.n : Y + coord;
+    const int row_stride = column ? 1 : D;
+    if (in_smem) {
+      // asynchronous copies: the rows, then their values in place of the keys.  (The loops are rolled: a
+      // launch runs this code once, so an unrolled sweep costs more in instruction fetch than it saves.)
+      if (pin) {
+#pragma unroll 1
+        for (int i = tid; i < cs; i += nt) cp_async4(&s_rows[i], pin + lo + c0 + i);
+        cp_async_wait_all();
       } else {
-        __syncthreads();
-        for (int b = tid; b < 256; b += nt) s_total[b] = hist[b];
+#pragma unroll 1
+        for (int i = tid; i < cs; i += nt) s_rows[i] = lo + c0 + i;
       }
-    } else {
-      for (int i = tid; i < n_list; i += nt) {
-        const uint32_t k = s_list[i];
-        if ((k & mask) == prefix) atomicAdd(&hist[(k >> shift) & 255u], 1);
-      }
-      __syncthreads();
-      for (int b = tid; b < 256; b += nt) s_total[b] = hist[b];
+#pragma unroll 1
+      for (int i = tid; i < cs; i += nt) cp_async4(&s_keys[i], Yc + (size_t)s_rows[i] * row_stride);
+      cp_async_wait_all();
     }
-    for (int b = tid; b < 256; b += nt) hist_next[b] = 0;
-    __syncthreads();
-    if (warp == 0) {
-      int local[8]; int sum = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { local[j] = s_total[lane * 8 + j]; sum += local[j]; }
-      int incl = sum;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int before = incl - sum;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        if (before < remaining && remaining <= before + local[j]) {
-          s_scalar[1] = lane * 8 + j;
-          s_scalar[2] = remaining - before;
-          s_ncand = local[j];
-        }
-        before += local[j];
-      }
+#pragma unroll 1
+    for (int i = tid; i < cs; i += nt) {
+      const float x = in_smem ? __uint_as_float(s_keys[i]) : __ldg(Yc + (size_t)row_at(c0 + i) * row_stride);
+      const uint32_t key = order_key(x);
+      if (in_smem) s_keys[i] = key;
+      else g_keys[i] = key;
+      atomicAdd(&s_hist[bin_of(x, key, map, kLevelBins)], 1);
     }
-    __syncthreads();
-    prefix |= (uint32_t)s_scalar[1] << shift;
-    mask |= 255u << shift;
-    remaining = s_scalar[2];
-    // (s_scalar is written again only after the next pass's barriers)
   }
-  const uint32_t thr = prefix;
-  const int eq_left = remaining;        // how many rows equal to the threshold go down
 
-  // ---- 3. stable two-sided partition.  Every warp owns a contiguous run of the slice and walks
+  // ---- 3. the threshold.  Counts of bins [first, first + 2 w) summed over the cluster; the bin that holds the
+  // row of rank `rank`.  A peer may still be reading counts after this returns, so they are
+  // cleared or counted again only beyond another cluster barrier.
+  auto pick = [&](int first, int w, int rank) {
+    sync_all();                                        // every slice has counted
+    int n0 = 0, n1 = 0;
+    if (tid < w) {
+#pragma unroll 1
+      for (int r = 0; r < csize; ++r) {
+        const int* h = csize > 1 ? cluster.map_shared_rank(s_hist, r) : s_hist;
+        const int2 n = *reinterpret_cast<const int2*>(h + first + 2 * tid);
+        n0 += n.x;
+        n1 += n.y;
+      }
+    }
+    int incl = n0 + n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    const int left = rank - (int)__reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane & (NW - 1)] : 0) - (incl - n0 - n1);
+    if (left >= 1 && left <= n0 + n1) {                // exactly one thread
+      const bool second = left > n0;
+      s_pick[0] = 2 * tid + (second ? 1 : 0);
+      s_pick[1] = second ? left - n0 : left;
+      s_pick[2] = second ? n1 : n0;
+    }
+    __syncthreads();
+  };
+  const int L = sd.c * ((s + sd.c) / (2 * sd.c));
+  int rank = L, shift = 32, n_list = 0;                 // shift: digits known down to this bit
+  uint32_t prefix = 0;
+  bool listed = false;
+  if constexpr (!keys_in) {
+    pick(0, kLevelBins / 2, rank);
+    n_list = s_pick[2];
+    listed = n_list <= kLevelList;                     // uniform over the cluster: every CTA holds the same totals
+    if (!listed) {
+      sync_all();
+      if (tid < kLevelBins / 2) reinterpret_cast<int2*>(s_hist)[tid] = make_int2(0, 0);
+    } else {
+      prefix = (uint32_t)s_pick[0];
+      rank = s_pick[1];
+    }
+  }
+  if (!listed) {
+    __syncthreads();
+#pragma unroll 1
+    while (shift > 0 && !listed) {
+      const int first = 256 * (shift / 8 - 1);
+#pragma unroll 4
+      for (int i = tid; i < cs; i += nt) {
+        const uint32_t k = key_at(i);
+        if (shift == 32 || (k >> shift) == prefix) atomicAdd(&s_hist[first + ((k >> (shift - 8)) & 255u)], 1);
+      }
+      shift -= 8;
+      pick(first, 128, rank);
+      prefix = prefix << 8 | (uint32_t)s_pick[0];
+      rank = s_pick[1];
+      n_list = s_pick[2];
+      listed = n_list <= kLevelList;
+    }
+  }
+  if (listed) {
+    unsigned long long* const list0 = csize > 1 ? cluster.map_shared_rank(s_list, 0) : s_list;
+    int* const count0 = csize > 1 ? cluster.map_shared_rank(&s_list_n, 0) : &s_list_n;
+    const bool digits = keys_in || shift < 32;
+#pragma unroll 1
+    for (int i = tid; i < cs; i += nt) {
+      const uint32_t k = key_at(i);
+      const uint32_t mine = digits ? k >> shift : (uint32_t)bin_of(key_value(k), k, map, kLevelBins);
+      if (mine == prefix) list0[atomicAdd(count0, 1)] = ((unsigned long long)k << 32) | (unsigned)(c0 + i);
+    }
+    sync_all();                                        // the list is complete
+    if (crank != 0) {
+#pragma unroll 1
+      for (int i = tid; i < n_list; i += nt) s_list[i] = list0[i];
+      __syncthreads();
+    }
+#pragma unroll 1
+    for (int i = tid; i < n_list; i += nt) {
+      const unsigned long long e = s_list[i];
+      int less = 0;
+#pragma unroll 4
+      for (int j = 0; j < n_list; ++j) less += s_list[j] < e ? 1 : 0;
+      if (less == rank - 1) s_thr = e;                 // exactly one thread
+    }
+    __syncthreads();
+  } else {
+    // more rows than the list holds are equal to the threshold: the one of rank `rank` in order of position
+    int equal = 0;
+#pragma unroll 1
+    for (int i = tid; i < cs; i += nt) equal += key_at(i) == prefix ? 1 : 0;
+    equal = (int)__reduce_add_sync(0xffffffffu, equal);
+    if (lane == 0) s_warp[warp] = equal;
+    __syncthreads();
+    equal = (int)__reduce_add_sync(0xffffffffu, lane < NW ? s_warp[lane & (NW - 1)] : 0);
+    if (tid == 0) s_total = equal;
+    sync_all();
+#pragma unroll 1
+    for (int r = 0; r < crank; ++r) rank -= *cluster.map_shared_rank(&s_total, r);
+    if (warp == 0 && rank >= 1 && rank <= equal) {     // in one CTA of the cluster
+#pragma unroll 1
+      for (int i0 = 0; i0 < cs; i0 += 32) {
+        const bool eq = i0 + lane < cs && key_at(i0 + lane) == prefix;
+        const unsigned b = __ballot_sync(0xffffffffu, eq);
+        if (rank <= __popc(b)) {
+          if (eq && __popc(b & ((1u << lane) - 1u)) == rank - 1)
+            for (int r = 0; r < csize; ++r)
+              *(csize > 1 ? cluster.map_shared_rank(&s_thr, r) : &s_thr) = ((unsigned long long)prefix << 32) | (unsigned)(c0 + i0 + lane);
+          break;
+        }
+        rank -= __popc(b);
+      }
+    }
+    sync_all();
+  }
+  const unsigned long long thr = s_thr;
+
+  // ---- 4. stable two-sided partition.  Every warp owns a contiguous run of the slice and walks
   // it 32 positions at a time with ballots; offsets = totals of the earlier slices and warps.
-  const int nwarps = nt >> 5;
-  const int run = ((cs + nwarps - 1) / nwarps + 31) & ~31;       // positions per warp (multiple of 32)
+  const int run = ((cs + NW - 1) / NW + 31) & ~31;               // positions per warp (multiple of 32)
   const int w0 = min(cs, warp * run), w1 = min(cs, w0 + run);
-  int nl = 0, ne = 0;
+  int below = 0;
+#pragma unroll 1
   for (int i0 = w0; i0 < w1; i0 += 32) {
     const int i = i0 + lane;
-    const uint32_t k = (i < w1) ? keys[i] : 0xffffffffu;
-    nl += __popc(__ballot_sync(0xffffffffu, i < w1 && k < thr));
-    ne += __popc(__ballot_sync(0xffffffffu, i < w1 && k == thr));
+    const bool down = i < w1 && (((unsigned long long)key_at(i) << 32) | (unsigned)(c0 + i)) <= thr;
+    below += __popc(__ballot_sync(0xffffffffu, down));
   }
-  if (lane == 0) s_warp[warp] = nl | (ne << 16);       // a warp run holds fewer than 65536 positions
+  if (lane == 0) s_warp[warp] = below;
   __syncthreads();
-  if (warp == 0) {
-    const int v = (lane < nwarps) ? s_warp[lane] : 0;
-    int vl = v & 0xffff, ve = v >> 16;
-    int il = vl, ie = ve;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int a = __shfl_up_sync(0xffffffffu, il, o), b = __shfl_up_sync(0xffffffffu, ie, o);
-      if (lane >= o) { il += a; ie += b; }
-    }
-    s_hist[lane] = il - vl;                            // exclusive offsets per warp (s_hist is free now)
-    s_hist[32 + lane] = ie - ve;
-    if (lane == 31) { s_counts[0] = il; s_counts[1] = ie; }
+  const int mine = lane < NW ? s_warp[lane & (NW - 1)] : 0;
+  below = (int)__reduce_add_sync(0xffffffffu, lane < warp ? mine : 0);
+  if (csize > 1) {
+    const int total = (int)__reduce_add_sync(0xffffffffu, mine);
+    if (tid == 0) s_total = total;
+    cluster.sync();
+    const int earlier = lane < crank ? *cluster.map_shared_rank(&s_total, lane) : 0;
+    below += (int)__reduce_add_sync(0xffffffffu, earlier);
   }
-  if (csize > 1) cluster.sync(); else __syncthreads();
-  int less_before = s_hist[warp], eq_before = s_hist[32 + warp];
-  for (int r = 0; r < crank; ++r) {                     // totals of the earlier slices of the cluster
-    const int* rc = cluster.map_shared_rank(s_counts, r);
-    less_before += rc[0];
-    eq_before += rc[1];
-  }
-  const unsigned lt_mask = (1u << lane) - 1u;
+#pragma unroll 1
   for (int i0 = w0; i0 < w1; i0 += 32) {
     const int i = i0 + lane;
     const bool ok = i < w1;
-    const uint32_t k = ok ? keys[i] : 0xffffffffu;
-    const bool is_less = ok && k < thr, is_eq = ok && k == thr;
-    const unsigned bl = __ballot_sync(0xffffffffu, is_less), be = __ballot_sync(0xffffffffu, is_eq);
-    if (ok) {
-      const int less_here = less_before + __popc(bl & lt_mask);
-      const int eq_here = eq_before + __popc(be & lt_mask);
-      const bool down = is_less || (is_eq && eq_here < eq_left);
-      const int down_before = less_here + min(eq_here, eq_left);
-      const int row = in_smem ? s_rows[i] : (pin ? pin[lo + c0 + i] : lo + c0 + i);
-      const int dst = down ? lo + down_before : lo + L + (c0 + i - down_before);
-      pout[dst] = row;
-    }
-    less_before += __popc(bl);
-    eq_before += __popc(be);
+    const bool down = ok && (((unsigned long long)key_at(i) << 32) | (unsigned)(c0 + i)) <= thr;
+    const unsigned b = __ballot_sync(0xffffffffu, down);
+    const int before = below + __popc(b & ((1u << lane) - 1u));
+    if (ok) pout[down ? lo + before : lo + L + (c0 + i - before)] = in_smem ? s_rows[i] : row_at(c0 + i);
+    below += __popc(b);
   }
   if (csize > 1) cluster.sync();                     // keep shared memory alive for the peers' reads
 }
@@ -692,8 +694,8 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(cons
       const int g = unit / UNITS, block = unit % UNITS;
       const int a = slo[g], sz = slo[g + 1] - a;
       if (sz <= c) continue;
-      if (sz >= D) unit_variance<D, V, true>(Y, rows + a, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
-      else unit_variance_small<D, V>(Y, rows + a, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
+      if (sz >= D) unit_variance<D, V, true, false>(Y, rows + a, 0, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
+      else unit_variance_small<D, V, false>(Y, rows + a, 0, sz, block, lane, &sm.unit_best[g][block], &sm.unit_arg[g][block]);
     }
     __syncthreads();
     if (warp == 0) {
@@ -714,9 +716,7 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(cons
         }
         const int2 am = sm.unit_arg[lane][at];
         coord = am.x;
-        const float scale = 64.f * rsqrtf(v), shift = fmaf(-__int_as_float(am.y), scale, 128.f);
-        const bool usable = v > 0.f && scale < 1e30f && fabsf(shift) < 1e30f;     // also false for NaN
-        sm.seg_map[lane] = usable ? make_float2(scale, shift) : make_float2(0.f, 128.f);
+        sm.seg_map[lane] = bin_map(v, __int_as_float(am.y), 128.f);
       }
       int before = L;
 #pragma unroll
@@ -757,12 +757,7 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(cons
       if (sm.seg[g].y == 0) continue;
       const float x = __uint_as_float(sm.keys[i]);
       const uint32_t key = order_key(x);
-      // the bin grows with the key for every value: infinities land at the ends (the scale is positive
-      // and finite, or zero and all bins equal), NaNs are put where their keys stand
-      const float2 map = sm.seg_map[g];
-      int bin = (int)fminf(fmaxf(fmaf(x, map.x, map.y), 0.f), 255.f);
-      if (x != x) bin = (int)key < 0 ? 255 : 0;
-      if (map.x == 0.f) bin = 0;
+      const int bin = bin_of(x, key, sm.seg_map[g], 256);
       sm.keys[i] = key;
       sm.state[i] = (uint16_t)(g << 8 | bin);
       atomicAdd(&sm.hist[g][bin >> 1], 1u << (16 * (bin & 1)));
@@ -875,19 +870,44 @@ static int tail_level_for(int n, int c) {
   return level;
 }
 
+// One launch of the per-level kernel: the cluster size (see the kernel) and the slice it stages.
+static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, cudaStream_t st) {
+  const long long sets = (long long)prm.problems * 2 << level;             // of both sides
+  int csize = 1;
+  while (csize < kMaxCluster && (max_seg > csize * 8192 || (max_seg > csize * 2048 && sets * csize * 2 <= 296))) csize *= 2;
+  const int per_cta = ceil_div(max_seg, csize);
+  const bool wide = per_cta > 8192;
+  auto kernel = keys_in ? (wide ? split_level_kernel<64, 1024, true> : split_level_kernel<64, 512, true>)
+                : prm.D == 64 ? (wide ? split_level_kernel<64, 1024, false> : split_level_kernel<64, 512, false>)
+                              : (wide ? split_level_kernel<128, 1024, false> : split_level_kernel<128, 512, false>);
+  prm.level = level;
+  prm.smem_rows = per_cta < kSmemRowsMax ? per_cta : kSmemRowsMax;
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRowsMax * 8));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((1u << level) * csize, 2 * prm.problems);
+  cfg.blockDim = dim3(wide ? 1024 : 512);
+  cfg.dynamicSmemBytes = (size_t)prm.smem_rows * 8;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  CA_RETURN_IF_CUDA(cudaLaunchKernelEx(&cfg, kernel, prm));
+  CA_LAUNCH_CHECK();
+  return CA_OK;
+}
+
 int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q, int n_k, int c_q,
                  int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp, int32_t* perm_k_out,
                  int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k, int sides, cudaStream_t st,
                  const float* Ytq, const float* Ytk) {
   // sides: bit 0 = queries, bit 1 = keys
-  auto level_kernel = D == 64 ? split_level_kernel<64> : split_level_kernel<128>;
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRowsMax * 8));
   const bool do_q = (sides & 1) != 0, do_k = (sides & 2) != 0;
   const int tail_q = tail_level_for(n_q, c_q), tail_k = tail_level_for(n_k, c_k);
   const int top_q = do_q ? tail_q : 0, top_k = do_k ? tail_k : 0;
   const int top_levels = top_q > top_k ? top_q : top_k;
   SplitParams prm;
-  prm.D = D; prm.problems = problems; prm.keys_in = 0;
+  prm.D = D; prm.problems = problems;
   // per-level launches write alternately to tmp/out so that the tail kernel, which runs last,
   // reads the buffer that is not the output
   auto fill = [&](int level) {
@@ -918,26 +938,11 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   if (top_levels > 0 && prof_enabled()) prof_mark(kProfSplitLevels, st, true);
   for (int level = 0; level < top_levels; ++level) {
     fill(level);
-    prm.level = level;
     int max_seg = 1;
     if (level < top_q) max_seg = max_segment_at_level(n_q, c_q, level);
     if (level < top_k) { const int ms = max_segment_at_level(n_k, c_k, level); if (ms > max_seg) max_seg = ms; }
-    int csize = 1;
-    while (csize < kMaxCluster && max_seg > csize * 16384) csize *= 2;
-    const int per_cta = (max_seg + csize - 1) / csize;
-    prm.smem_rows = per_cta < kSmemRowsMax ? per_cta : kSmemRowsMax;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((1u << level) * csize, 2 * problems);
-    cfg.blockDim = dim3(kSplitThreads);
-    // keys + rows of the slice; the same space first stages the d x d subsample tile
-    cfg.dynamicSmemBytes = (size_t)prm.smem_rows * 8 > (size_t)D * D * 4 ? (size_t)prm.smem_rows * 8 : (size_t)D * D * 4;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    CA_RETURN_IF_CUDA(cudaLaunchKernelEx(&cfg, level_kernel, prm));
-    CA_LAUNCH_CHECK();
+    const int rc = launch_level(prm, false, level, max_seg, st);
+    if (rc != CA_OK) return rc;
   }
   if (top_levels > 0 && prof_enabled()) prof_mark(kProfSplitLevels, st, false);
   ProfScope ps(kProfSplitTail, st);
@@ -1586,8 +1591,6 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
                                 int D, int n_q, int n_k, int c_q, int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp,
                                 int32_t* perm_k_out, int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k,
                                 cudaStream_t st) {
-  auto level_kernel = D == 64 ? split_level_kernel<64> : split_level_kernel<128>;
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRowsMax * 8));
   const int lev_q = split_levels_for(n_q, c_q), lev_k = split_levels_for(n_k, c_k);
   // Sets of more than kTailRowsMax rows take three launches per level (directions, projections,
   // select + partition); the subtree kernel finishes the rest.  Per-level launches write alternately
@@ -1597,7 +1600,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
   BasicParams bp;
   bp.problems = problems; bp.iterations = iterations;
   SplitParams prm;
-  prm.D = D; prm.problems = problems; prm.keys_in = 1;
+  prm.D = D; prm.problems = problems;
   auto fill = [&](int level) {
     for (int w = 0; w < 2; ++w) {
       const int tail = w == 0 ? tail_q : tail_k;
@@ -1632,7 +1635,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
   };
   for (int level = 0; level < top; ++level) {
     fill(level);
-    bp.level = level; prm.level = level;
+    bp.level = level;
     const size_t dsmem = (size_t)D * (D + 1) * sizeof(float);
     if (D == 64) {
       auto dk = basic_direction_kernel<T, 64>;
@@ -1651,23 +1654,8 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
     int max_seg = 1;
     if (level < tail_q) max_seg = max_segment_at_level(n_q, c_q, level);
     if (level < tail_k) { const int ms = max_segment_at_level(n_k, c_k, level); if (ms > max_seg) max_seg = ms; }
-    int csize = 1;
-    while (csize < kMaxCluster && max_seg > csize * 16384) csize *= 2;
-    const int per_cta = (max_seg + csize - 1) / csize;
-    prm.smem_rows = per_cta < kSmemRowsMax ? per_cta : kSmemRowsMax;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((1u << level) * csize, 2 * problems);
-    int threads = 128;
-    while (threads < kSplitThreads && threads * 4 < per_cta) threads *= 2;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = (size_t)prm.smem_rows * 8 > 16 ? (size_t)prm.smem_rows * 8 : 16;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    CA_RETURN_IF_CUDA(cudaLaunchKernelEx(&cfg, level_kernel, prm));
-    CA_LAUNCH_CHECK();
+    const int rc = launch_level(prm, true, level, max_seg, st);
+    if (rc != CA_OK) return rc;
   }
   fill(top);
   bp.level = top; prm.level = top;

@@ -65,3 +65,16 @@ def test_split_coordinates_beyond_the_coordinate_major_ones(heads, n, d, c):
     for h in sorted({0, heads - 1}):
         assert np.array_equal(plan.perm_q[0, h].cpu().numpy(), orc.recursive_split_f32(Yq[0, h].cpu().numpy(), c))
         assert np.array_equal(plan.perm_k[0, h].cpu().numpy(), orc.recursive_split_f32(Yk[0, h].cpu().numpy(), c))
+
+
+@pytest.mark.parametrize("kind,heads,n,d,c", [
+    ("normal", 1, 4097, 64, 64), ("normal", 20, 8193, 128, 128), ("normal", 2, 65537, 64, 128),
+    ("normal", 1, 140000, 64, 128),                       # slices of more than 8,192 rows
+    ("outliers", 2, 30000, 64, 128), ("repeated", 2, 30000, 64, 128), ("repeated", 1, 4200, 128, 128),
+    ("two values", 1, 70000, 64, 256), ("two values", 40, 4500, 64, 128),
+    ("normal", 1, 200003, 64, 256), ("repeated", 1, 200003, 64, 256),   # slices beyond shared memory
+])
+def test_levels_of_large_sets_match_the_oracle(kind, heads, n, d, c):
+    """The same through the per-level kernel: one CTA per set up to eight, thresholds from a bin, from
+    the digits, and among equal keys whose positions lie in several CTAs."""
+    test_subtrees_match_the_oracle(kind, heads, n, d, c)
