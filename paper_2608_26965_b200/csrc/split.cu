@@ -81,6 +81,12 @@ __device__ __forceinline__ pair2 add_pair(pair2 a, pair2 b) {
   return d;
 }
 
+__device__ __forceinline__ pair2 fma_pair(pair2 a, pair2 b, pair2 c) {
+  pair2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
 // Largest variance over the subsample of one block of 4 V coordinates of one subset, by one warp.  The estimate
 // only feeds an argmax, so it is taken in float32 with a fixed operation order (reproducible bit for
 // bit; every operation rounded on its own, no fused multiply-add): eight partial sums over the rows
@@ -99,18 +105,19 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
   // sample j stands at position floor(j sz / m): j itself where the sample is the whole subset; a
   // row beyond the sample is loaded as the last one and counts as zero
   pair2 x[PER][V / 2];
+  const float* Yq = Y + t;
+  unsigned scaled = (unsigned)r * (unsigned)sz;      // j sz for j = r, r + 8, ...
 #pragma unroll
-  for (int k = 0; k < PER; ++k) {
-    const unsigned j = r + 8 * k;
-    const int pos = full ? (int)(j * (unsigned)sz / D) : min((int)j, m - 1);
-    const float* src = Y + (size_t)(global ? (rows ? __ldg(rows + pos) : first + pos) : rows[pos]) * D + t;
+  for (int k = 0; k < PER; ++k, scaled += 8u * (unsigned)sz) {
+    const int pos = full ? (int)(scaled / D) : min(r + 8 * k, m - 1);
+    const unsigned row = (unsigned)(global ? (rows ? __ldg(rows + pos) : first + pos) : rows[pos]);
+    const float* src = Yq + (size_t)row * D;
     if constexpr (V == 4) {
-      const float4 w = __ldg(reinterpret_cast<const float4*>(src));
-      x[k][0] = pair(w.x, w.y);
-      x[k][V / 2 - 1] = pair(w.z, w.w);
+      const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(src));
+      x[k][0] = w.x;
+      x[k][V / 2 - 1] = w.y;
     } else {
-      const float2 w = __ldg(reinterpret_cast<const float2*>(src));
-      x[k][0] = pair(w.x, w.y);
+      x[k][0] = __ldg(reinterpret_cast<const unsigned long long*>(src));
     }
   }
   if (!full) {
@@ -147,24 +154,23 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
 #pragma unroll
     for (int v = 0; v < V; ++v) mean[v] = __fadd_rn(mean[v], __shfl_xor_sync(0xffffffffu, mean[v], o));
   divide(mean);
-  // Sums and differences two values per instruction (each half rounded on its own: the bits
-  // of two scalar additions).  The squares and their sums stay scalar operations that are
-  // never contracted: a two-value multiply followed by a two-value add is merged into one
-  // fused multiply-add by the assembler, which rounds once where the definition rounds twice.
+  // All operations on two values per instruction (each half rounded on its own: the bits of two
+  // scalar operations).  A multiply followed by an add would be merged into one fused multiply-add, which
+  // rounds once where the definition rounds twice; the square is a fused multiply-add of its own, with
+  // an addend of -0 that only the launch knows (gridDim.z is 1).
+  const float minus_zero = __uint_as_float(gridDim.z << 31);
+  const pair2 addend = pair(minus_zero, minus_zero);
 #pragma unroll
   for (int h = 0; h < V / 2; ++h) {
     const pair2 neg = pair(-mean[2 * h], -mean[2 * h + 1]);
-    float s0 = 0.f, s1 = 0.f;
+    pair2 acc = pair(0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-      float d0, d1;
-      unpair(add_pair(x[k][h], neg), d0, d1);
-      if (!full && r + 8 * k >= m) d0 = d1 = 0.f;    // a missing row adds an exact zero
-      s0 = __fadd_rn(s0, __fmul_rn(d0, d0));
-      s1 = __fadd_rn(s1, __fmul_rn(d1, d1));
+      pair2 dev = add_pair(x[k][h], neg);
+      if (!full && r + 8 * k >= m) dev = 0ull;       // a missing row adds an exact zero
+      acc = add_pair(acc, fma_pair(dev, dev, addend));
     }
-    var[2 * h] = s0;
-    var[2 * h + 1] = s1;
+    unpair(acc, var[2 * h], var[2 * h + 1]);
   }
 #pragma unroll
   for (int o = 4; o < 32; o <<= 1)
@@ -209,12 +215,12 @@ struct SplitSide {
   int32_t* perm_out;       // [P][n]
   uint32_t* keybuf;        // [P][n] staging for sets larger than the shared-memory windows
   int n, c, levels, tail_level;
-  int active;              // 0: this launch leaves the side alone (the two sides can run on different streams)
 };
 
 struct SplitParams {
   SplitSide side[2];
   int D, level, problems, smem_rows;
+  int first_side, sides;   // the sides of this launch: queries 0, keys 1 (they can run on different streams)
 };
 
 // Scale and offset of the bins of one coordinate: `half` bins to either side of the sample's mean for two
@@ -270,10 +276,10 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_level_kernel(con
   __shared__ int s_total;                                // of this CTA, read by its peers
   __shared__ unsigned long long s_thr;                   // the last (key, position) that goes down
 
-  const int which = blockIdx.y / prm.problems;
+  const int which = prm.first_side + blockIdx.y / prm.problems;
   const int p = blockIdx.y % prm.problems;
   const SplitSide sd = prm.side[which];
-  if (!sd.active || prm.level >= sd.tail_level) return;   // uniform over the cluster
+  if (prm.level >= sd.tail_level) return;             // uniform over the cluster
   const SegmentRef seg = locate_segment(sd.n, sd.c, prm.level, blockIdx.x / csize);
   if (!seg.active) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -650,11 +656,11 @@ template <int D, int nt>
 __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(const SplitParams prm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TailSmem& sm = *reinterpret_cast<TailSmem*>(smem_raw);
-  const int which = blockIdx.y / prm.problems;
+  const int which = prm.first_side + blockIdx.y / prm.problems;
   const int p = blockIdx.y % prm.problems;
   const SplitSide sd = prm.side[which];
   const int level = sd.tail_level;
-  if (!sd.active || (int)blockIdx.x >= (1 << level)) return;
+  if ((int)blockIdx.x >= (1 << level)) return;
   const SegmentRef root = locate_segment(sd.n, sd.c, level, blockIdx.x);
   if (!root.active) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -884,7 +890,7 @@ static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, 
   prm.smem_rows = per_cta < kSmemRowsMax ? per_cta : kSmemRowsMax;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemRowsMax * 8));
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((1u << level) * csize, 2 * prm.problems);
+  cfg.gridDim = dim3((1u << level) * csize, prm.sides * prm.problems);
   cfg.blockDim = dim3(wide ? 1024 : 512);
   cfg.dynamicSmemBytes = (size_t)prm.smem_rows * 8;
   cfg.stream = st;
@@ -908,6 +914,7 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   const int top_levels = top_q > top_k ? top_q : top_k;
   SplitParams prm;
   prm.D = D; prm.problems = problems;
+  prm.first_side = do_q ? 0 : 1; prm.sides = do_q && do_k ? 2 : 1;
   // per-level launches write alternately to tmp/out so that the tail kernel, which runs last,
   // reads the buffer that is not the output
   auto fill = [&](int level) {
@@ -922,7 +929,6 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
       sd.n = w == 0 ? n_q : n_k; sd.c = w == 0 ? c_q : c_k;
       sd.levels = split_levels_for(sd.n, sd.c);
       sd.tail_level = tail;
-      sd.active = (w == 0 ? do_q : do_k) ? 1 : 0;
       // level l of this side (l < tail) writes tmp if (tail - 1 - l) is even, else out;
       // the tail kernel (level == tail) reads what level tail-1 wrote and writes out
       const bool to_tmp = ((tail - 1 - level) % 2) == 0;
@@ -955,7 +961,7 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   auto tail_kernel = D == 64 ? (one_wave ? split_tail_kernel<64, 1024> : split_tail_kernel<64, 512>)
                              : (one_wave ? split_tail_kernel<128, 1024> : split_tail_kernel<128, 512>);
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TailSmem)));
-  tail_kernel<<<dim3(slots, 2 * problems), threads, sizeof(TailSmem), st>>>(prm);
+  tail_kernel<<<dim3(slots, prm.sides * problems), threads, sizeof(TailSmem), st>>>(prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -1354,7 +1360,7 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
   const BasicSide bs = prm.side[which];
   const SplitSide sd = sp.side[which];
   const int level0 = sd.tail_level;
-  if (!sd.active || (int)blockIdx.x >= (1 << level0)) return;
+  if ((int)blockIdx.x >= (1 << level0)) return;
   const SegmentRef root = locate_segment(sd.n, sd.c, level0, blockIdx.x);
   if (!root.active) return;
   const int tid = threadIdx.x;
@@ -1601,6 +1607,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
   bp.problems = problems; bp.iterations = iterations;
   SplitParams prm;
   prm.D = D; prm.problems = problems;
+  prm.first_side = 0; prm.sides = 2;
   auto fill = [&](int level) {
     for (int w = 0; w < 2; ++w) {
       const int tail = w == 0 ? tail_q : tail_k;
@@ -1613,7 +1620,6 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
       sd.n = w == 0 ? n_q : n_k; sd.c = w == 0 ? c_q : c_k;
       sd.levels = w == 0 ? lev_q : lev_k;
       sd.tail_level = tail;
-      sd.active = 1;
       const bool to_tmp = ((tail - 1 - level) % 2) == 0;
       if (level < tail) {
         sd.perm_out = to_tmp ? tmp : out;
