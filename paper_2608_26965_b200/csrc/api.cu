@@ -248,10 +248,10 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     // symmetric roots: any factor yields the same principal-component coordinates).  The
     // un-normalised query representation (Appendix B.1) takes the root of K_c^T K_c / n_k, the
     // normalised one is indifferent to the scale and keeps the scatter matrix as it is.
-    // F_q comes from Q on the caller's stream and leads into the key side; F_k comes from K on the
-    // side stream and leads into the query side: the fork is at the very start, and the key side
-    // only waits for the Gram matrix and column sums of K (event `mid`), from which its
-    // principal-component kernel forms C_K itself.
+    // F_k comes from K and leads into the query side, F_q comes from Q and leads into the key side: the fork
+    // is at the very start, and the key side only waits for the Gram matrix and column sums of K
+    // (event `mid`), from which its principal-component kernel forms C_K itself.  K comes first: both
+    // sides need its Gram matrix.
     const bool unnormalized = (p->flags & CA_QUERY_UNNORMALIZED) != 0;
     const double ck_scale = unnormalized ? 1.0 / (double)p->n_k : 1.0;
     double* Fq = w.roots;
@@ -262,29 +262,33 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     // while the per-kernel timers are on, both sides run on the caller's stream, one kernel after
     // the other, so that every kernel group is timed alone
     const bool serial = prof_enabled();
-    cudaStream_t sq = serial ? st : side->stream;
+    // The longer chain runs on the caller's stream, which the other joins: the query side, whose
+    // covariance takes a pass over the rows, unless the keys (and values) are far more.
+    const bool keys_longer = p->n_k > 2LL * p->n_q;
+    cudaStream_t aside = serial ? st : side->stream;
+    cudaStream_t sq = keys_longer ? aside : st, sk = keys_longer ? st : aside;
     if (!serial) {
       CA_RETURN_IF_CUDA(cudaEventRecord(side->fork, st));
-      CA_RETURN_IF_CUDA(cudaStreamWaitEvent(sq, side->fork, 0));
+      CA_RETURN_IF_CUDA(cudaStreamWaitEvent(aside, side->fork, 0));
     }
     {
       ProfScope ps(kProfGram, st);
       if (tc) {
-        CA_TRY(launch_gram_tc(Q, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, st));
         CA_TRY(launch_gram_tc(K, P, p->n_k, D, w.partial2, w.gramK, w.sumK, w.status, sq));
+        CA_TRY(launch_gram_tc(Q, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, w.status, sk));
       } else {
-        CA_TRY(launch_moments(Q, p->dtype, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, st));
         CA_TRY(launch_moments(K, p->dtype, P, p->n_k, D, w.partial2, w.gramK, w.sumK, sq));
+        CA_TRY(launch_moments(Q, p->dtype, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, sk));
       }
     }
     if (!serial) CA_RETURN_IF_CUDA(cudaEventRecord(side->mid, sq));
     {
       ProfScope ps(kProfFactor, st);
-      CA_TRY(launch_cholesky_factor(w.gramQ, nullptr, 1.0, 1.0 / (double)p->n_q, P, D, Fq, w.roots32, nullptr, nullptr, st));
       CA_TRY(launch_cholesky_factor(w.gramK, w.sumK, (double)p->n_k, ck_scale, P, D, Fk, w.roots32 + (size_t)P * DD,
                                     tc ? w.wt2_hi : nullptr, tc ? w.wt2_lo : nullptr, sq));
+      CA_TRY(launch_cholesky_factor(w.gramQ, nullptr, 1.0, 1.0 / (double)p->n_q, P, D, Fq, w.roots32, nullptr, nullptr, sk));
     }
-    // ---- query side (side stream)
+    // ---- query side
     // query representation r(q) = F_k^T q / |F_k^T q|, its covariance and principal components E_Q
     // (one kernel), the coordinates Y = (r(q) - mean) E_Q.  fp32 storage keeps r(q); bf16 storage
     // sums its moments without storing it and projects from Q once more: E_Q is orthogonal, so
@@ -331,13 +335,12 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
       ProfScope ps(kProfPermute, sq);
       CA_TRY(launch_permute_centroid(Q, p->dtype, perm_q, P, p->n_q, D, p->cluster_q, Qp, cq, count_q, sq));
     }
-    if (!serial) CA_RETURN_IF_CUDA(cudaEventRecord(side->join, sq));
-    // ---- key side on the caller's stream: covariance of the transformed keys K F_q
+    // ---- key side: covariance of the transformed keys K F_q
     // (F_q^T C_K F_q / n_k, d x d algebra), its principal components E_K and the projection
     // W = F_q E_K with its bias in one kernel; Y = (K - kbar) W
-    if (!serial) CA_RETURN_IF_CUDA(cudaStreamWaitEvent(st, side->mid, 0));
+    if (!serial) CA_RETURN_IF_CUDA(cudaStreamWaitEvent(sk, side->mid, 0));
     {
-      ProfScope ps(kProfPca, st);
+      ProfScope ps(kProfPca, sk);
       PcaArgs a{};
       a.mode = kPcaKeys;
       a.gram = w.gramK; a.sum = w.sumK; a.n = (double)p->n_k; a.c_scale = ck_scale;
@@ -346,22 +349,23 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
       a.mean_sum = w.sumK; a.mean_n = (double)p->n_k;
       a.W32 = w.WK32; a.bias = w.biasK;
       a.wt_hi = tc ? w.wt_hi : nullptr; a.wt_lo = tc ? w.wt_lo : nullptr;
-      CA_TRY(launch_pca(a, P, D, st));
+      CA_TRY(launch_pca(a, P, D, sk));
     }
     {
-      ProfScope ps(kProfTransform, st);
+      ProfScope ps(kProfTransform, sk);
       if (tc) {
-        CA_TRY(launch_transform_tc(K, P, p->n_k, D, w.biasK, 0, yk_out, w.wt_hi, w.wt_lo, w.status, st, w.Ytk));
+        CA_TRY(launch_transform_tc(K, P, p->n_k, D, w.biasK, 0, yk_out, w.wt_hi, w.wt_lo, w.status, sk, w.Ytk));
       } else {
-        CA_TRY(launch_transform_rows(K, p->dtype, P, p->n_k, D, w.WK32, w.biasK, 0, yk_out, st));
+        CA_TRY(launch_transform_rows(K, p->dtype, P, p->n_k, D, w.WK32, w.biasK, 0, yk_out, sk));
       }
     }
     CA_TRY(launch_split(nullptr, yk_out, P, D, p->n_q, p->n_k, p->cluster_q, p->cluster_k, perm_q, w.perm_q_tmp,
-                        perm_k, w.perm_k_tmp, w.keybuf_q, w.keybuf_k, 2, st, nullptr, w.Ytk));
+                        perm_k, w.perm_k_tmp, w.keybuf_q, w.keybuf_k, 2, sk, nullptr, w.Ytk));
     {
-      ProfScope ps(kProfPermute, st);
-      CA_TRY(launch_permute_centroid(K, p->dtype, perm_k, P, p->n_k, D, p->cluster_k, Kp, ck, count_k, st, V, Vp, cv));
+      ProfScope ps(kProfPermute, sk);
+      CA_TRY(launch_permute_centroid(K, p->dtype, perm_k, P, p->n_k, D, p->cluster_k, Kp, ck, count_k, sk, V, Vp, cv));
     }
+    if (!serial) CA_RETURN_IF_CUDA(cudaEventRecord(side->join, aside));
     // ---- join
     if (!serial) CA_RETURN_IF_CUDA(cudaStreamWaitEvent(st, side->join, 0));
     return CA_OK;
