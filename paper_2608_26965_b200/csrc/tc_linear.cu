@@ -50,10 +50,9 @@ struct GramParams {
   int n_rows, chunk_rows, n_chunks, stages, normalize;    // normalize: of the representation
 };
 
-// One of the four epilogue warps writes its rows of the accumulated Gram matrix and column sums.
+// One of the four epilogue warps writes its rows of the accumulated Gram matrix.
 template <int D>
-__device__ __forceinline__ void write_gram(uint32_t tmem_acc, uint32_t tmem_sum, int quarter, int lane, bool any,
-                                           float* __restrict__ out) {
+__device__ __forceinline__ void write_gram(uint32_t tmem_acc, int quarter, int lane, bool any, float* __restrict__ out) {
   // accumulator row m sits in lane m (D = 128) or in lane (m % 16) + 32 (m / 16) (D = 64)
   const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
   const int m = D == 128 ? quarter * 32 + lane : quarter * 16 + lane;
@@ -71,9 +70,6 @@ __device__ __forceinline__ void write_gram(uint32_t tmem_acc, uint32_t tmem_sum,
                              __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
     }
   }
-  const uint32_t sum = tmem_ld1(tmem_sum + lane_addr);     // one of 16 identical sums
-  tmem_wait_ld();
-  if (live) out[D * D + m] = __uint_as_float(sum);
 }
 
 template <int D>
@@ -158,8 +154,12 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const GramParams prm) {
     const bool ok = __all_sync(0xffffffffu, mbar_wait(b_done, 0, abort_flag, prm.status));
     tc_fence_after();
     if (ok) {
-      write_gram<D>(tmem_acc, tmem_sum, quarter, lane, n_tiles > 0,
-                    prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D));
+      float* out = prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D);
+      write_gram<D>(tmem_acc, quarter, lane, n_tiles > 0, out);
+      const uint32_t sum = tmem_ld1(tmem_sum + ((uint32_t)(quarter * 32) << 16));     // one of 16 identical sums
+      tmem_wait_ld();
+      if (n_tiles > 0 && (D == 128 || lane < 16))
+        out[D * D + (D == 128 ? quarter * 32 + lane : quarter * 16 + lane)] = __uint_as_float(sum);
     }
   }
   tc_fence_before();
@@ -371,17 +371,19 @@ struct RepCfg {
   static constexpr int STAGES = D == 64 ? 3 : 2;
   static constexpr int OFF_X = 2 * W_BYTES;
   static constexpr int OFF_R = OFF_X + STAGES * TILE_BYTES;             // hi tile, 2 lo tile
-  static constexpr int OFF_ONES = OFF_R + 2 * TILE_BYTES;               // 2 KB of bf16 1.0, 2 KB of 0.5
-  static constexpr int OFF_BAR = OFF_ONES + 4096;
-  static constexpr int NUM_BARS = 2 + 2 * STAGES + 4 + 2;               // weights, done; x full/empty; acc full/empty x 2; r full/empty
+  static constexpr int GROUPS = D / 64;                                 // epilogue warps per 32 rows: 64 columns each
+  static constexpr int THREADS = 64 + 128 * GROUPS;
+  static constexpr int OFF_NORM = OFF_R + 2 * TILE_BYTES;               // [2][GROUPS][128 rows] partial squared norms
+  static constexpr int OFF_BAR = OFF_NORM + 2 * GROUPS * kRows * 4;
+  static constexpr int NUM_BARS = 2 + 2 * STAGES + 4 + 3;               // weights, done; x full/empty; acc full/empty x 2; r full/empty; norms
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
   static constexpr int SMEM = 1024 + OFF_MISC + 16;
-  static constexpr uint32_t TMEM_COLS = D == 64 ? 256 : 512;            // two T accumulators, G, sums
+  static constexpr uint32_t TMEM_COLS = D == 64 ? 256 : 512;            // two T accumulators, G
   static constexpr int CTAS_PER_SM = D == 64 ? 2 : 1;
 };
 
 template <int D>
-__global__ void __launch_bounds__(kLinThreads, 1)
+__global__ void __launch_bounds__(RepCfg<D>::THREADS, RepCfg<D>::CTAS_PER_SM)
 rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_whi,
                    const __grid_constant__ CUtensorMap tm_wlo, const GramParams prm) {
   using C = RepCfg<D>;
@@ -389,7 +391,7 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
   const uint32_t s_base = smem_u32(smem);
-  const uint32_t s_w = s_base, s_x = s_base + C::OFF_X, s_r = s_base + C::OFF_R, s_ones = s_base + C::OFF_ONES;
+  const uint32_t s_w = s_base, s_x = s_base + C::OFF_X, s_r = s_base + C::OFF_R;
   unsigned char* r_ptr = smem + C::OFF_R;
   const uint32_t bar0 = s_base + C::OFF_BAR;
   const uint32_t b_w = bar0, b_done = bar0 + 8;
@@ -397,7 +399,7 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
   auto b_empty = [&](int s) { return bar0 + 16 + 8 * (C::STAGES + s); };
   auto b_acc_full = [&](int a) { return bar0 + 16 + 8 * (2 * C::STAGES + a); };
   auto b_acc_empty = [&](int a) { return bar0 + 16 + 8 * (2 * C::STAGES + 2 + a); };
-  const uint32_t b_r_full = bar0 + 16 + 8 * (2 * C::STAGES + 4), b_r_empty = b_r_full + 8;
+  const uint32_t b_r_full = bar0 + 16 + 8 * (2 * C::STAGES + 4), b_r_empty = b_r_full + 8, b_norm = b_r_full + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
 
@@ -411,20 +413,18 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     mbar_init(b_w, 1);
     mbar_init(b_done, 1);
     for (int s = 0; s < C::STAGES; ++s) { mbar_init(b_full(s), 1); mbar_init(b_empty(s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(b_acc_full(a), 1); mbar_init(b_acc_empty(a), 4); }
-    mbar_init(b_r_full, 4);
+    for (int a = 0; a < 2; ++a) { mbar_init(b_acc_full(a), 1); mbar_init(b_acc_empty(a), 4 * C::GROUPS); }
+    mbar_init(b_r_full, 4 * C::GROUPS);
     mbar_init(b_r_empty, 1);
+    mbar_init(b_norm, 4 * C::GROUPS);
     *abort_flag = 0;
     fence_mbar_init();
   }
-  for (int e = tid; e < 2048; e += kLinThreads)
-    reinterpret_cast<__nv_bfloat16*>(smem + C::OFF_ONES)[e] = __float2bfloat16_rn(e < 1024 ? 1.0f : 0.5f);
-  fence_proxy_async();                 // the ones are read by the tensor core (async proxy)
   if (warp == 1) { tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_t = *tmem_slot, tmem_g = tmem_t + 2 * D, tmem_sum = tmem_g + D;
+  const uint32_t tmem_t = *tmem_slot, tmem_g = tmem_t + 2 * D;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -447,7 +447,6 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
     if (lane == 0) {
       constexpr uint32_t idesc_t = idesc_bf16_f32(kRows, D, 0, 0);     // X (K-major) times W^T (K-major)
       constexpr uint32_t idesc_g = idesc_bf16_f32(D, D, 1, 1);         // R^T R: both operands MN-major
-      constexpr uint32_t idesc_s = idesc_bf16_f32(D, 16, 1, 1);
       bool ok = mbar_wait(b_w, 0, abort_flag, prm.status);
       auto product_t = [&](int t) {
         const int s = t % C::STAGES, a = t & 1;
@@ -472,8 +471,6 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
         if (ok) ok = mbar_wait(b_r_full, t & 1, abort_flag, prm.status);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t ones = smem_desc_sw128(s_ones, C::PANEL_BYTES, 1024);
-        const uint64_t halves = smem_desc_sw128(s_ones + 2048, C::PANEL_BYTES, 1024);
 #pragma unroll
         for (int ks = 0; ks < kRows / 16; ++ks) {
           // 16 rows (the contraction index) per step = 2048 bytes; 64-column panels along M and N
@@ -482,34 +479,37 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
           const uint32_t acc = (t > 0 || ks > 0) ? 1u : 0u;
           mma_ss(tmem_g, dh, dh, idesc_g, acc);
           mma_ss(tmem_g, dh, dl, idesc_g, 1u);
-          mma_ss(tmem_sum, dh, ones, idesc_s, acc);
-          mma_ss(tmem_sum, dl, halves, idesc_s, 1u);
         }
         mma_commit(b_r_empty);
       }
       mma_commit(b_done);
     }
   } else {
-    const int quarter = warp & 3;
+    const int quarter = warp & 3, group = (warp - 2) >> 2;
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    float* s_norm = reinterpret_cast<float*>(smem + C::OFF_NORM);
     auto wait = [&](uint32_t bar, uint32_t parity) {
       return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, prm.status));
     };
+    float sum[64];                                     // of this thread's row of every tile
+#pragma unroll
+    for (int j = 0; j < 64; ++j) sum[j] = 0.f;
     bool ok = true;
+#pragma unroll 1
     for (int t = 0; t < n_tiles && ok; ++t) {
       const int a = t & 1;
       ok = wait(b_acc_full(a), (t >> 1) & 1);
       if (!ok) break;
       tc_fence_after();
-      float v[D];
-#pragma unroll
-      for (int c4 = 0; c4 < D / 32; ++c4) {
-        uint32_t r[32];
-        tmem_ld32(tmem_t + a * D + lane_addr + c4 * 32, r);
+      float v[64];
+      {
+        uint32_t r0[32], r1[32];
+        tmem_ld32(tmem_t + a * D + group * 64 + lane_addr, r0);
+        tmem_ld32(tmem_t + a * D + group * 64 + 32 + lane_addr, r1);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[c4 * 32 + j] = __uint_as_float(r[j]);
+        for (int j = 0; j < 32; ++j) { v[j] = __uint_as_float(r0[j]); v[32 + j] = __uint_as_float(r1[j]); }
       }
       tc_fence_before();
       __syncwarp();
@@ -517,40 +517,65 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       if (prm.normalize) {
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
-        for (int j = 0; j < D; j += 4) {
+        for (int j = 0; j < 64; j += 4) {
           s0 = fmaf(v[j], v[j], s0); s1 = fmaf(v[j + 1], v[j + 1], s1);
           s2 = fmaf(v[j + 2], v[j + 2], s2); s3 = fmaf(v[j + 3], v[j + 3], s3);
         }
-        const float nrm = sqrtf((s0 + s1) + (s2 + s3));
+        float ss = (s0 + s1) + (s2 + s3);
+        if constexpr (C::GROUPS > 1) {                 // the other half of the row is another warp's
+          float* norms = s_norm + a * C::GROUPS * kRows + row;
+          norms[group * kRows] = ss;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_norm);
+          ok = wait(b_norm, t & 1);
+          if (!ok) break;
+          ss = norms[0] + norms[kRows];
+        }
+        const float nrm = sqrtf(ss);
         const float inv = nrm >= 1e-30f ? 1.f / nrm : 0.f;
 #pragma unroll
-        for (int j = 0; j < D; ++j) v[j] *= inv;
+        for (int j = 0; j < 64; ++j) v[j] *= inv;
+      }
+      uint32_t hi[32], lo[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const float x0 = v[2 * j], x1 = v[2 * j + 1];
+        sum[2 * j] += x0;
+        sum[2 * j + 1] += x1;
+        hi[j] = pack_bf16x2(x0, x1);
+        lo[j] = pack_bf16x2(2.f * (x0 - __uint_as_float(hi[j] << 16)), 2.f * (x1 - __uint_as_float(hi[j] & 0xffff0000u)));
       }
       if (t > 0) ok = wait(b_r_empty, (t - 1) & 1);
       if (!ok) break;
 #pragma unroll
-      for (int pn = 0; pn < D / 64; ++pn)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint32_t h[4], l[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float x0 = v[pn * 64 + 8 * c + 2 * j], x1 = v[pn * 64 + 8 * c + 2 * j + 1];
-            h[j] = pack_bf16x2(x0, x1);
-            l[j] = pack_bf16x2(2.f * (x0 - __uint_as_float(h[j] << 16)), 2.f * (x1 - __uint_as_float(h[j] & 0xffff0000u)));
-          }
-          const int off = pn * C::PANEL_BYTES + row * 128 + ((c ^ (row & 7)) * 16);
-          *reinterpret_cast<uint4*>(r_ptr + off) = make_uint4(h[0], h[1], h[2], h[3]);
-          *reinterpret_cast<uint4*>(r_ptr + C::TILE_BYTES + off) = make_uint4(l[0], l[1], l[2], l[3]);
-        }
+      for (int c = 0; c < 8; ++c) {
+        const int off = group * C::PANEL_BYTES + row * 128 + ((c ^ (row & 7)) * 16);
+        *reinterpret_cast<uint4*>(r_ptr + off) = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
+        *reinterpret_cast<uint4*>(r_ptr + C::TILE_BYTES + off) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
+      }
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(b_r_full);
     }
     if (ok) ok = wait(b_done, 0);
     tc_fence_after();
-    if (ok) write_gram<D>(tmem_g, tmem_sum, quarter, lane, n_tiles > 0,
-                          prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D));
+    float* out = prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D);
+    if (ok && group == 0) write_gram<D>(tmem_g, quarter, lane, n_tiles > 0, out);
+    // the tensor core is done with R: its space takes the sums per row, [D / 64][128 rows][64 columns]
+    if (ok) {
+      float* mine = reinterpret_cast<float*>(r_ptr) + (group * kRows + row) * 64;
+#pragma unroll
+      for (int j = 0; j < 64; j += 4)
+        *reinterpret_cast<float4*>(mine + (j ^ (4 * (lane & 7)))) = make_float4(sum[j], sum[j + 1], sum[j + 2], sum[j + 3]);
+    }
+  }
+  __syncthreads();
+  if (tid < D && !*abort_flag) {
+    const float* rows = reinterpret_cast<const float*>(r_ptr) + (tid >> 6) * kRows * 64;
+    float total = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < kRows; ++r) total += rows[r * 64 + ((tid & 63) ^ (4 * (r & 7)))];
+    prm.partial[((size_t)p * prm.n_chunks + chunk) * (D * D + D) + D * D + tid] = total;
   }
   tc_fence_before();
   __syncthreads();
@@ -678,7 +703,7 @@ static int launch_rep_gram(const void* X, int problems, int n_rows, int normaliz
     return CA_ERR_CUDA;
   auto k = rep_gram_tc_kernel<D>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-  k<<<dim3(prm.n_chunks, problems), kLinThreads, C::SMEM, st>>>(mx, mwh, mwl, prm);
+  k<<<dim3(prm.n_chunks, problems), C::THREADS, C::SMEM, st>>>(mx, mwh, mwl, prm);
   CA_LAUNCH_CHECK();
   return launch_gram_finalize(partial, problems, prm.n_chunks, D, gram, colsum, st);
 }
