@@ -386,14 +386,13 @@ int select_blocks(const ca_problem_t* p, const float* cq, const float* ck, int32
     return CA_ERR_INVALID_ARG;
   if (!ws || ws_bytes < kStatusBytes) return CA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
   const int P = p->batch * p->heads;
   // room behind the status block holds tiles of scores when there are many key clusters
   float* score_ws = reinterpret_cast<float*>(static_cast<char*>(ws) + kStatusBytes);
   const size_t score_floats = aligned16(ws) ? (ws_bytes - kStatusBytes) / sizeof(float) : 0;
   ProfScope ps(kProfSelect, st);
   return launch_score_select(cq, ck, P, ceil_div(p->n_q, p->cluster_q), ceil_div(p->n_k, p->cluster_k),
-                             p->head_dim, p->keep, block_idx, score_ws, score_floats, st);
+                             p->head_dim, p->keep, block_idx, score_ws, score_floats, static_cast<int*>(ws), st);
 }
 
 int cluster_attention_fwd(const ca_problem_t* p, const void* Qp, const void* Kp, const void* Vp,
@@ -409,7 +408,8 @@ int cluster_attention_fwd(const ca_problem_t* p, const void* Qp, const void* Kp,
   const size_t need = tensor_cores ? attn_tc_workspace_bytes(*p) : kStatusBytes;
   if (!ws || !aligned16(ws) || ws_bytes < need) return CA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusClearBytes, st));
+  // with compensation the tensor-core path clears the status block in the kernel that prepares the centroids
+  if (!tensor_cores || !p->compensate) CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusClearBytes, st));
   const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->head_dim);
   if (tensor_cores)
     return launch_attn_tc(*p, Qp, Kp, Vp, ck, cv, count_k, block_idx, nullptr, p->keep, perm_q, scale, O, lse,
@@ -428,14 +428,13 @@ int select_blocks_adaptive(const ca_problem_t* p, const float* cq, const float* 
   if (!(recall > 0.f) || min_count < 1) return CA_ERR_INVALID_ARG;
   if (!ws || ws_bytes < kStatusBytes) return CA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
   const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->head_dim);
   float* score_ws = reinterpret_cast<float*>(static_cast<char*>(ws) + kStatusBytes);
   const size_t score_floats = aligned16(ws) ? (ws_bytes - kStatusBytes) / sizeof(float) : 0;
   ProfScope ps(kProfSelect, st);
   return launch_select_adaptive(cq, ck, count_k, p->batch * p->heads, ceil_div(p->n_q, p->cluster_q),
                                 ceil_div(p->n_k, p->cluster_k), p->head_dim, scale, recall, min_count,
-                                block_idx, keep_count, score_ws, score_floats, st);
+                                block_idx, keep_count, score_ws, score_floats, static_cast<int*>(ws), st);
 }
 
 int cluster_attention_fwd_ragged(const ca_problem_t* p, const void* Qp, const void* Kp, const void* Vp,
@@ -453,7 +452,8 @@ int cluster_attention_fwd_ragged(const ca_problem_t* p, const void* Qp, const vo
   const size_t need = tensor_cores ? attn_tc_workspace_bytes(*p) : kStatusBytes;
   if (!ws || !aligned16(ws) || ws_bytes < need) return CA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusClearBytes, st));
+  // with compensation the tensor-core path clears the status block in the kernel that prepares the centroids
+  if (!tensor_cores || !p->compensate) CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusClearBytes, st));
   const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->head_dim);
   if (tensor_cores)
     return launch_attn_tc(*p, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, scale,

@@ -834,11 +834,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // ---------------------------------------------------------------------------
 // Centroids for the tensor-core path, 64 per tile: key tile = 64 rows of bf16 hi
 // parts followed by 64 rows of lo parts; value centroids as bf16.  Rows beyond
-// the last centroid are zero.
+// the last centroid are zero.  The first CTA clears the status block (the kernels before the attention
+// kernel write no status).
 // ---------------------------------------------------------------------------
 __global__ void centroid_prep_kernel(const float* __restrict__ ck, const float* __restrict__ cv, int n_kc,
                                      int cen_tiles, int D, __nv_bfloat16* __restrict__ kmix,
-                                     __nv_bfloat16* __restrict__ vb) {
+                                     __nv_bfloat16* __restrict__ vb, int* __restrict__ status) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusClearBytes / sizeof(int)) status[threadIdx.x] = 0;
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= cen_tiles * kCen * D) return;
@@ -969,7 +971,7 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   if (pr.compensate) {
     ProfScope ps(kProfAttnPrep, st);
     centroid_prep_kernel<<<dim3(ceil_div(cen_tiles * kCen * D, 256), P), 256, 0, st>>>(ck, cv, n_kc, cen_tiles, D,
-                                                                                        kmix, vb);
+                                                                                        kmix, vb, status);
     CA_LAUNCH_CHECK();
   }
   CUtensorMap maps[5];

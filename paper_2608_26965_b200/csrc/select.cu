@@ -22,13 +22,19 @@ __device__ __forceinline__ uint32_t score_key(float s) {
   return (u >> 31) ? ~u : (u | 0x80000000u);
 }
 
+// The selection records no errors: its kernels clear the status block themselves, one launch less.
+__device__ __forceinline__ void clear_status(int* status) {
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(int)) status[threadIdx.x] = 0;
+}
+
 // QT query clusters per CTA: 4 when the CTA computes the scores itself (the key centroids are read
 // once for the four), 1 when the scores come from memory (less shared memory, more CTAs per SM).
 template <int D, int QT>
 __global__ void __launch_bounds__(kSelectThreads)
 score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, int n_qc, int n_kc,
                     int keep, int32_t* __restrict__ block_idx, const float* __restrict__ scores, int row0,
-                    int chunk_rows) {
+                    int chunk_rows, int* __restrict__ status) {
+  clear_status(status);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);                       // [QT][n_kc]
   float* qs = reinterpret_cast<float*>(keys + (size_t)QT * n_kc);        // [QT][D]
@@ -286,7 +292,7 @@ static int launch_score_tiles(const float* cq, const float* ck, int P, int n_qc,
 }
 
 int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n_kc, int D, int keep,
-                        int32_t* block_idx, float* score_ws, size_t score_floats, cudaStream_t st) {
+                        int32_t* block_idx, float* score_ws, size_t score_floats, int* status, cudaStream_t st) {
   const int chunk = select_chunk_rows(P, n_qc, n_kc, score_ws ? score_floats : 0);
   if (chunk == 0) {
     const size_t smem = select_smem_bytes(n_kc, D, kSelectQT);
@@ -295,11 +301,11 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     if (D == 64) {
       auto k = score_select_kernel<64, kSelectQT>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc);
+      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
     } else {
       auto k = score_select_kernel<128, kSelectQT>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc);
+      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
     }
     CA_LAUNCH_CHECK();
     return CA_OK;
@@ -315,8 +321,8 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     if (D == 64) { int rc = launch_score_tiles<64>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
     else { int rc = launch_score_tiles<128>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
     dim3 grid(rows, P);
-    if (D == 64) k64<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk);
-    else k128<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk);
+    if (D == 64) k64<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
+    else k128<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
     CA_LAUNCH_CHECK();
   }
   return CA_OK;
@@ -355,7 +361,8 @@ select_adaptive_kernel(const float* __restrict__ cq, const float* __restrict__ c
                        const int32_t* __restrict__ count_k, int n_qc, int n_kc, int n_pad, float c_log2,
                        float recall, int min_count, int32_t* __restrict__ block_idx,
                        int32_t* __restrict__ keep_count, const float* __restrict__ scores, int row0,
-                       int chunk_rows) {
+                       int chunk_rows, int* __restrict__ status) {
+  clear_status(status);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);   // [n_pad] (mass, ~index)
   float* score = reinterpret_cast<float*>(keys + n_pad);                         // [n_kc]
@@ -469,7 +476,7 @@ select_adaptive_kernel(const float* __restrict__ cq, const float* __restrict__ c
 
 int launch_select_adaptive(const float* cq, const float* ck, const int32_t* count_k, int P, int n_qc, int n_kc,
                            int D, float scale, float recall, int min_count, int32_t* block_idx,
-                           int32_t* keep_count, float* score_ws, size_t score_floats, cudaStream_t st) {
+                           int32_t* keep_count, float* score_ws, size_t score_floats, int* status, cudaStream_t st) {
   int n_pad = 1;
   while (n_pad < n_kc) n_pad <<= 1;
   const size_t smem = (size_t)n_pad * 8 + (size_t)n_kc * 4 + (size_t)D * 4;
@@ -493,10 +500,10 @@ int launch_select_adaptive(const float* cq, const float* ck, const int32_t* coun
     dim3 grid(rows, P);
     if (D == 64)
       k64<<<grid, 256, smem, st>>>(cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
-                                   keep_count, scores, row0, step);
+                                   keep_count, scores, row0, step, status);
     else
       k128<<<grid, 256, smem, st>>>(cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
-                                    keep_count, scores, row0, step);
+                                    keep_count, scores, row0, step, status);
     CA_LAUNCH_CHECK();
   }
   return CA_OK;
