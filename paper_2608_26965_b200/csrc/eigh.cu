@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
   double* pivots = G + kPanel * D;            // [D]
   __shared__ double s_tol;
   constexpr double kDrop = 1e-12;             // share of the largest diagonal entry below which a pivot drops out
+  wait_for_previous();
   const int tid = threadIdx.x, w = tid >> 5, q = tid & 31;
   const double* A = gram + (size_t)blockIdx.x * D * D;
   const double* sm = sum ? sum + (size_t)blockIdx.x * D : nullptr;
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
       }
     }
   }
+  let_next_start();
   __syncthreads();
   if (tid < D) pivots[tid] = pivots[tid] > 0.0 ? rsqrt(pivots[tid]) : 0.0;
   __syncthreads();
@@ -171,13 +173,13 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
 }
 
 int launch_cholesky_factor(const double* gram, const double* sum, double n, double scale, int count, int D,
-                           double* out64, float* out32, void* wt_hi, void* wt_lo, cudaStream_t st) {
+                           double* out64, float* out32, void* wt_hi, void* wt_lo, LaunchStream st) {
   __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(wt_hi);
   __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(wt_lo);
   const size_t smem = sizeof(double) * ((size_t)D * (D + 1) + kPanel * D + D);
   auto k = D == 64 ? cholesky_factor_kernel<64> : cholesky_factor_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<count, 4 * D, smem, st>>>(gram, sum, n, scale, out64, out32, hi, lo);
+  launch_chained(k, count, 4 * D, smem, st, gram, sum, n, scale, out64, out32, hi, lo);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -203,14 +205,14 @@ __global__ void cast_f64_f32_kernel(const double* __restrict__ src, float* __res
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) dst[i] = (float)src[i];
 }
-int launch_cast_f64_f32(const double* src, float* dst, size_t count, cudaStream_t st) {
+int launch_cast_f64_f32(const double* src, float* dst, size_t count, LaunchStream st) {
   cast_f64_f32_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(src, dst, count);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 int launch_metric(const double* gramQ, const double* gramK, const double* sumK, int P, int D, int n_q,
-                  int n_k, double ck_scale, double* M, double* CK, cudaStream_t st) {
+                  int n_k, double ck_scale, double* M, double* CK, LaunchStream st) {
   metric_kernel<<<dim3(ceil_div(D * D, 256), P), 256, 0, st>>>(gramQ, gramK, sumK, D, (double)n_q,
                                                                 (double)n_k, ck_scale, M, CK);
   CA_LAUNCH_CHECK();

@@ -552,6 +552,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
 
 template <int D>
 __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
+  wait_for_previous();
   constexpr int NT = kThreads, LDA = D + 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* A = reinterpret_cast<float*>(smem_raw);       // [D][LDA]
@@ -927,6 +928,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
         for (int y = 0; y < 4; ++y) A[(4 * tile_i + x) * LDA + tile_j + (D / 4) * y] = acc[x][y];
     }
   }
+  let_next_start();
   // ---- order, sign, bias
   double* lam = reinterpret_cast<double*>(xbuf);             // [D] doubles over xbuf's 2D floats
   int* rank_of = reinterpret_cast<int*>(pbuf);
@@ -979,11 +981,11 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
   }
 }
 
-int launch_pca(const PcaArgs& args, int count, int D, cudaStream_t st) {
+int launch_pca(const PcaArgs& args, int count, int D, LaunchStream st) {
   const size_t smem = sizeof(float) * ((size_t)3 * D * (D + 4) + 8 * D + 18 * D);
   auto k = D == 64 ? eigh_tql_kernel<64> : eigh_tql_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<count, kThreads, smem, st>>>(args);
+  launch_chained(k, count, kThreads, smem, st, args);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }

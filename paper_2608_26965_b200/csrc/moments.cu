@@ -14,6 +14,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256) gram_chunk_kernel(const T* __restrict__ X, int n_rows,
                                                          int chunk_rows, int n_chunks,
                                                          float* __restrict__ partial) {
+  wait_for_previous();
   constexpr int TR = 32;            // rows staged per step
   constexpr int TM = D / 16;        // 4 (D=64) or 8 (D=128)
   __shared__ __align__(16) float xs[TR][D + 4];
@@ -62,6 +63,7 @@ __global__ void __launch_bounds__(256) gram_chunk_kernel(const T* __restrict__ X
     }
     __syncthreads();
   }
+  let_next_start();
   float* out = partial + ((size_t)p * n_chunks + chunk) * (D * D + D);
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -74,6 +76,8 @@ __global__ void __launch_bounds__(256) gram_chunk_kernel(const T* __restrict__ X
 __global__ void gram_finalize_kernel(const float* __restrict__ partial, int n_chunks, int elems,
                                      double* __restrict__ gram, double* __restrict__ colsum,
                                      int dd) {
+  wait_for_previous();
+  let_next_start();
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= elems) return;
@@ -97,28 +101,28 @@ int moments_chunking(int n_rows, int problems, int* chunk_rows, int* n_chunks) {
 }
 
 int launch_gram_finalize(const float* partial, int problems, int n_chunks, int D, double* gram,
-                         double* colsum, cudaStream_t st) {
+                         double* colsum, LaunchStream st) {
   const int elems = D * D + D;
-  gram_finalize_kernel<<<dim3(ceil_div(elems, 256), problems), 256, 0, st>>>(partial, n_chunks, elems, gram,
-                                                                              colsum, D * D);
+  launch_chained(gram_finalize_kernel, dim3(ceil_div(elems, 256), problems), 256, 0, st, partial, n_chunks, elems, gram,
+                 colsum, D * D);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 template <typename T>
 static int launch_moments_t(const T* X, int problems, int n_rows, int D, float* partial,
-                            double* gram, double* colsum, cudaStream_t st) {
+                            double* gram, double* colsum, LaunchStream st) {
   int chunk_rows, n_chunks;
   moments_chunking(n_rows, problems, &chunk_rows, &n_chunks);
   dim3 grid(n_chunks, problems);
-  if (D == 64) gram_chunk_kernel<T, 64><<<grid, 256, 0, st>>>(X, n_rows, chunk_rows, n_chunks, partial);
-  else gram_chunk_kernel<T, 128><<<grid, 256, 0, st>>>(X, n_rows, chunk_rows, n_chunks, partial);
+  auto k = D == 64 ? gram_chunk_kernel<T, 64> : gram_chunk_kernel<T, 128>;
+  launch_chained(k, grid, 256, 0, st, X, n_rows, chunk_rows, n_chunks, partial);
   CA_LAUNCH_CHECK();
   return launch_gram_finalize(partial, problems, n_chunks, D, gram, colsum, st);
 }
 
 int launch_moments(const void* X, int dtype, int problems, int n_rows, int D, float* partial,
-                   double* gram, double* colsum, cudaStream_t st) {
+                   double* gram, double* colsum, LaunchStream st) {
   if (dtype == CA_DTYPE_BF16)
     return launch_moments_t(static_cast<const __nv_bfloat16*>(X), problems, n_rows, D, partial, gram, colsum, st);
   return launch_moments_t(static_cast<const float*>(X), problems, n_rows, D, partial, gram, colsum, st);
@@ -144,6 +148,7 @@ __global__ void __launch_bounds__(256) transform_rows_kernel(const T* __restrict
   float* Ws = smem;                       // [D][D]
   float* xs = Ws + D * D;                 // [TR][LD]  rows, then results
   __shared__ float inv_norm[TR];
+  wait_for_previous();
   const int p = blockIdx.y;
   const int r0 = blockIdx.x * TR;
   const int nr = min(TR, n_rows - r0);
@@ -219,24 +224,24 @@ __global__ void __launch_bounds__(256) transform_rows_kernel(const T* __restrict
 
 template <typename T>
 static int launch_transform_t(const T* X, int problems, int n_rows, int D, const float* W,
-                              const float* bias, int normalize, float* out, cudaStream_t st) {
+                              const float* bias, int normalize, float* out, LaunchStream st) {
   dim3 grid(ceil_div(n_rows, 64), problems);
   size_t smem = (size_t)(D * D + 64 * (D + 4)) * sizeof(float);
   if (D == 64) {
     auto k = transform_rows_kernel<T, 64>;
     CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, 256, smem, st>>>(X, n_rows, W, bias, normalize, out);
+    launch_chained(k, grid, 256, smem, st, X, n_rows, W, bias, normalize, out);
   } else {
     auto k = transform_rows_kernel<T, 128>;
     CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k<<<grid, 256, smem, st>>>(X, n_rows, W, bias, normalize, out);
+    launch_chained(k, grid, 256, smem, st, X, n_rows, W, bias, normalize, out);
   }
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 int launch_transform_rows(const void* X, int dtype, int problems, int n_rows, int D, const float* W,
-                          const float* bias, int normalize, float* out, cudaStream_t st) {
+                          const float* bias, int normalize, float* out, LaunchStream st) {
   if (dtype == CA_DTYPE_BF16)
     return launch_transform_t(static_cast<const __nv_bfloat16*>(X), problems, n_rows, D, W, bias, normalize, out, st);
   return launch_transform_t(static_cast<const float*>(X), problems, n_rows, D, W, bias, normalize, out, st);

@@ -17,6 +17,8 @@ __global__ void __launch_bounds__(128) permute_centroid_kernel(const T* __restri
                                                                float* __restrict__ centroid0,
                                                                float* __restrict__ centroid1,
                                                                int32_t* __restrict__ count0) {
+  wait_for_previous();
+  let_next_start();
   const T* X = blockIdx.z ? X1 : X0;
   T* Xp = blockIdx.z ? Xp1 : Xp0;
   float* centroid = blockIdx.z ? centroid1 : centroid0;
@@ -58,19 +60,17 @@ __global__ void __launch_bounds__(128) permute_centroid_kernel(const T* __restri
 
 template <typename T>
 static int launch_t(const T* X, const T* X2, const int32_t* perm, int P, int n, int D, int c, T* Xp, T* Xp2,
-                    float* cen, float* cen2, int32_t* count, cudaStream_t st) {
+                    float* cen, float* cen2, int32_t* count, LaunchStream st) {
   const int n_c = ceil_div(n, c);
   dim3 grid(n_c, P, X2 ? 2 : 1);
-  if (D == 64)
-    permute_centroid_kernel<T, 64><<<grid, 128, 0, st>>>(X, X2, perm, n, c, n_c, Xp, Xp2, cen, cen2, count);
-  else
-    permute_centroid_kernel<T, 128><<<grid, 128, 0, st>>>(X, X2, perm, n, c, n_c, Xp, Xp2, cen, cen2, count);
+  auto k = D == 64 ? permute_centroid_kernel<T, 64> : permute_centroid_kernel<T, 128>;
+  launch_chained(k, grid, 128, 0, st, X, X2, perm, n, c, n_c, Xp, Xp2, cen, cen2, count);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 int launch_permute_centroid(const void* X, int dtype, const int32_t* perm, int P, int n, int D, int c,
-                            void* Xp, float* cen, int32_t* count, cudaStream_t st, const void* X2, void* Xp2,
+                            void* Xp, float* cen, int32_t* count, LaunchStream st, const void* X2, void* Xp2,
                             float* cen2) {
   if (dtype == CA_DTYPE_BF16)
     return launch_t(static_cast<const __nv_bfloat16*>(X), static_cast<const __nv_bfloat16*>(X2), perm, P, n, D, c,

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const __nv_bfloat16*
 // + one scale per run of 64.
 int launch_quantize_qk(const void* Qp, const void* Kp, const float* ck, int P, int n_qc, int c_q, int n_kc, int c_k,
                        int cen_tiles, int D, unsigned char* q8, float* sq, unsigned char* k8, float* sk,
-                       unsigned char* c8, float* sc, cudaStream_t st) {
+                       unsigned char* c8, float* sc, LaunchStream st) {
   if (D != 128) return CA_ERR_UNSUPPORTED;
   const size_t q_rows = (size_t)P * n_qc * c_q;
   quantize_rows_kernel<128><<<(unsigned)((q_rows + 15) / 16), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(Qp), q_rows, q8, sq);

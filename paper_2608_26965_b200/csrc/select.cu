@@ -34,6 +34,8 @@ __global__ void __launch_bounds__(kSelectThreads)
 score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, int n_qc, int n_kc,
                     int keep, int32_t* __restrict__ block_idx, const float* __restrict__ scores, int row0,
                     int chunk_rows, int* __restrict__ status) {
+  wait_for_previous();
+  let_next_start();
   clear_status(status);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);                       // [QT][n_kc]
@@ -207,6 +209,8 @@ template <int D>
 __global__ void __launch_bounds__(256)
 score_tile_kernel(const float* __restrict__ cq, const float* __restrict__ ck, int n_qc, int n_kc, int row0,
                   int chunk_rows, float* __restrict__ scores) {
+  wait_for_previous();
+  let_next_start();
   extern __shared__ __align__(16) float tile_smem[];
   float* As = tile_smem;                 // [D][64]  As[k][i]
   float* Bs = tile_smem + D * 64;        // [D][64]  Bs[k][j]
@@ -281,18 +285,18 @@ size_t select_score_floats(int P, int n_qc, int n_kc) {
 
 template <int D>
 static int launch_score_tiles(const float* cq, const float* ck, int P, int n_qc, int n_kc, int row0, int chunk_rows,
-                              float* scores, cudaStream_t st) {
+                              float* scores, LaunchStream st) {
   auto k = score_tile_kernel<D>;
   const size_t smem = (size_t)2 * D * 64 * sizeof(float);
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int rows = min(chunk_rows, n_qc - row0);
-  k<<<dim3(ceil_div(n_kc, 64), ceil_div(rows, 64), P), 256, smem, st>>>(cq, ck, n_qc, n_kc, row0, chunk_rows, scores);
+  launch_chained(k, dim3(ceil_div(n_kc, 64), ceil_div(rows, 64), P), 256, smem, st, cq, ck, n_qc, n_kc, row0, chunk_rows, scores);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n_kc, int D, int keep,
-                        int32_t* block_idx, float* score_ws, size_t score_floats, int* status, cudaStream_t st) {
+                        int32_t* block_idx, float* score_ws, size_t score_floats, int* status, LaunchStream st) {
   const int chunk = select_chunk_rows(P, n_qc, n_kc, score_ws ? score_floats : 0);
   if (chunk == 0) {
     const size_t smem = select_smem_bytes(n_kc, D, kSelectQT);
@@ -301,11 +305,11 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     if (D == 64) {
       auto k = score_select_kernel<64, kSelectQT>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
+      launch_chained(k, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
     } else {
       auto k = score_select_kernel<128, kSelectQT>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      k<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
+      launch_chained(k, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, nullptr, 0, n_qc, status);
     }
     CA_LAUNCH_CHECK();
     return CA_OK;
@@ -321,8 +325,8 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     if (D == 64) { int rc = launch_score_tiles<64>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
     else { int rc = launch_score_tiles<128>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
     dim3 grid(rows, P);
-    if (D == 64) k64<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
-    else k128<<<grid, kSelectThreads, smem, st>>>(cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
+    if (D == 64) launch_chained(k64, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
+    else launch_chained(k128, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
     CA_LAUNCH_CHECK();
   }
   return CA_OK;
@@ -362,6 +366,8 @@ select_adaptive_kernel(const float* __restrict__ cq, const float* __restrict__ c
                        float recall, int min_count, int32_t* __restrict__ block_idx,
                        int32_t* __restrict__ keep_count, const float* __restrict__ scores, int row0,
                        int chunk_rows, int* __restrict__ status) {
+  wait_for_previous();
+  let_next_start();
   clear_status(status);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);   // [n_pad] (mass, ~index)
@@ -476,7 +482,7 @@ select_adaptive_kernel(const float* __restrict__ cq, const float* __restrict__ c
 
 int launch_select_adaptive(const float* cq, const float* ck, const int32_t* count_k, int P, int n_qc, int n_kc,
                            int D, float scale, float recall, int min_count, int32_t* block_idx,
-                           int32_t* keep_count, float* score_ws, size_t score_floats, int* status, cudaStream_t st) {
+                           int32_t* keep_count, float* score_ws, size_t score_floats, int* status, LaunchStream st) {
   int n_pad = 1;
   while (n_pad < n_kc) n_pad <<= 1;
   const size_t smem = (size_t)n_pad * 8 + (size_t)n_kc * 4 + (size_t)D * 4;
@@ -499,10 +505,10 @@ int launch_select_adaptive(const float* cq, const float* ck, const int32_t* coun
     }
     dim3 grid(rows, P);
     if (D == 64)
-      k64<<<grid, 256, smem, st>>>(cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
+      launch_chained(k64, grid, 256, smem, st, cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
                                    keep_count, scores, row0, step, status);
     else
-      k128<<<grid, 256, smem, st>>>(cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
+      launch_chained(k128, grid, 256, smem, st, cq, ck, count_k, n_qc, n_kc, n_pad, c_log2, recall, min_count, block_idx,
                                     keep_count, scores, row0, step, status);
     CA_LAUNCH_CHECK();
   }

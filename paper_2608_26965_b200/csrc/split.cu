@@ -257,6 +257,7 @@ __device__ __forceinline__ float key_value(uint32_t key) {               // inve
 // -> 160; 40 heads of 32,760 rows, d = 128: 214 -> 184.
 template <int D, int nt, bool keys_in>
 __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_level_kernel(const SplitParams prm) {
+  wait_for_previous();
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks();
   const int crank = (int)cluster.block_rank();
@@ -499,6 +500,7 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_level_kernel(con
   }
   const unsigned long long thr = s_thr;
 
+  let_next_start();
   // ---- 4. stable two-sided partition.  Every warp owns a contiguous run of the slice and walks
   // it 32 positions at a time with ballots; offsets = totals of the earlier slices and warps.
   const int run = ((cs + NW - 1) / NW + 31) & ~31;               // positions per warp (multiple of 32)
@@ -654,6 +656,7 @@ __device__ __noinline__ void tail_thresholds_by_digits(TailSmem& sm, unsigned cr
 // pieces of one row: 356 -> 315 us).
 template <int D, int nt>
 __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(const SplitParams prm) {
+  wait_for_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TailSmem& sm = *reinterpret_cast<TailSmem*>(smem_raw);
   const int which = prm.first_side + blockIdx.y / prm.problems;
@@ -840,6 +843,7 @@ __global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(cons
     __syncthreads();
     cur ^= 1;
   }
+  let_next_start();
 #pragma unroll 1
   for (int i = tid; i < s0; i += nt) pout[lo + i] = sm.rows[cur][i];
 }
@@ -877,7 +881,7 @@ static int tail_level_for(int n, int c) {
 }
 
 // One launch of the per-level kernel: the cluster size (see the kernel) and the slice it stages.
-static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, cudaStream_t st) {
+static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, LaunchStream st) {
   const long long sets = (long long)prm.problems * 2 << level;             // of both sides
   int csize = 1;
   while (csize < kMaxCluster && (max_seg > csize * 8192 || (max_seg > csize * 2048 && sets * csize * 2 <= 296))) csize *= 2;
@@ -894,10 +898,12 @@ static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, 
   cfg.blockDim = dim3(wide ? 1024 : 512);
   cfg.dynamicSmemBytes = (size_t)prm.smem_rows * 8;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = st.chained ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = 2;
   CA_RETURN_IF_CUDA(cudaLaunchKernelEx(&cfg, kernel, prm));
   CA_LAUNCH_CHECK();
   return CA_OK;
@@ -905,7 +911,7 @@ static int launch_level(SplitParams& prm, bool keys_in, int level, int max_seg, 
 
 int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q, int n_k, int c_q,
                  int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp, int32_t* perm_k_out,
-                 int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k, int sides, cudaStream_t st,
+                 int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k, int sides, LaunchStream st,
                  const float* Ytq, const float* Ytk) {
   // sides: bit 0 = queries, bit 1 = keys
   const bool do_q = (sides & 1) != 0, do_k = (sides & 2) != 0;
@@ -961,7 +967,7 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   auto tail_kernel = D == 64 ? (one_wave ? split_tail_kernel<64, 1024> : split_tail_kernel<64, 512>)
                              : (one_wave ? split_tail_kernel<128, 1024> : split_tail_kernel<128, 512>);
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TailSmem)));
-  tail_kernel<<<dim3(slots, prm.sides * problems), threads, sizeof(TailSmem), st>>>(prm);
+  launch_chained(tail_kernel, dim3(slots, prm.sides * problems), threads, sizeof(TailSmem), st, prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -1596,7 +1602,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
                                 const float* noise_k, float* dirs_q, float* dirs_k, int iterations, int problems,
                                 int D, int n_q, int n_k, int c_q, int c_k, int32_t* perm_q_out, int32_t* perm_q_tmp,
                                 int32_t* perm_k_out, int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k,
-                                cudaStream_t st) {
+                                LaunchStream st) {
   const int lev_q = split_levels_for(n_q, c_q), lev_k = split_levels_for(n_k, c_k);
   // Sets of more than kTailRowsMax rows take three launches per level (directions, projections,
   // select + partition); the subtree kernel finishes the rest.  Per-level launches write alternately
@@ -1683,7 +1689,7 @@ int launch_split_basic(const void* Q, const void* K, int dtype, const float* A_q
                        const float* noise_q, const float* noise_k, float* dirs_q, float* dirs_k, int iterations,
                        int problems, int D, int n_q, int n_k, int c_q, int c_k, int32_t* perm_q_out,
                        int32_t* perm_q_tmp, int32_t* perm_k_out, int32_t* perm_k_tmp, uint32_t* keybuf_q,
-                       uint32_t* keybuf_k, cudaStream_t st) {
+                       uint32_t* keybuf_k, LaunchStream st) {
   if (dtype == CA_DTYPE_BF16)
     return launch_split_basic_t(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), A_q, A_k,
                                 noise_q, noise_k, dirs_q, dirs_k, iterations, problems, D, n_q, n_k, c_q, c_k,

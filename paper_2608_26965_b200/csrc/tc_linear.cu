@@ -75,6 +75,7 @@ __device__ __forceinline__ void write_gram(uint32_t tmem_acc, int quarter, int l
 template <int D>
 __global__ void __launch_bounds__(kLinThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const GramParams prm) {
+  wait_for_previous();
   using C = GramCfg<D>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -152,6 +153,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const GramParams prm) {
   } else {
     const int quarter = warp & 3;
     const bool ok = __all_sync(0xffffffffu, mbar_wait(b_done, 0, abort_flag, prm.status));
+    if (warp == 2) let_next_start();
     tc_fence_after();
     if (ok) {
       float* out = prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D);
@@ -192,6 +194,7 @@ __global__ void __launch_bounds__(kLinThreads, 1)
 transform_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_whi,
                     const __grid_constant__ CUtensorMap tm_wlo, const __grid_constant__ CUtensorMap tm_out,
                     const LinParams prm) {
+  wait_for_previous();
   using C = LinCfg<D>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -343,6 +346,7 @@ transform_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         tma_store_commit();
       }
     }
+    let_next_start();
     if (st == 0) tma_store_wait_all();
   }
   tc_fence_before();
@@ -386,6 +390,7 @@ template <int D>
 __global__ void __launch_bounds__(RepCfg<D>::THREADS, RepCfg<D>::CTAS_PER_SM)
 rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_whi,
                    const __grid_constant__ CUtensorMap tm_wlo, const GramParams prm) {
+  wait_for_previous();
   using C = RepCfg<D>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -557,6 +562,7 @@ rep_gram_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_consta
       __syncwarp();
       if (lane == 0) mbar_arrive(b_r_full);
     }
+    if (warp == 2) let_next_start();
     if (ok) ok = wait(b_done, 0);
     tc_fence_after();
     float* out = prm.partial + ((size_t)p * prm.n_chunks + chunk) * (D * D + D);
@@ -667,7 +673,7 @@ int gram_tc_chunking(int n_rows, int problems, int ctas_per_sm, int* chunk_rows,
 }
 
 int launch_gram_tc(const void* X, int problems, int n_rows, int D, float* partial, double* gram, double* colsum,
-                   int* status, cudaStream_t st) {
+                   int* status, LaunchStream st) {
   GramParams prm{};
   prm.partial = partial; prm.status = status; prm.n_rows = n_rows;
   const int tile = kRows * D * 2;
@@ -685,14 +691,14 @@ int launch_gram_tc(const void* X, int problems, int n_rows, int D, float* partia
   if (!map_3d(&mx, X, problems, n_rows, D, 2, 64, kRows)) return CA_ERR_CUDA;
   auto k = D == 64 ? gram_tc_kernel<64> : gram_tc_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<dim3(prm.n_chunks, problems), kLinThreads, smem, st>>>(mx, prm);
+  launch_chained(k, dim3(prm.n_chunks, problems), kLinThreads, smem, st, mx, prm);
   CA_LAUNCH_CHECK();
   return launch_gram_finalize(partial, problems, prm.n_chunks, D, gram, colsum, st);
 }
 
 template <int D>
 static int launch_rep_gram(const void* X, int problems, int n_rows, int normalize, float* partial, double* gram,
-                           double* colsum, const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st) {
+                           double* colsum, const void* wt_hi, const void* wt_lo, int* status, LaunchStream st) {
   using C = RepCfg<D>;
   GramParams prm{};
   prm.partial = partial; prm.status = status; prm.n_rows = n_rows; prm.normalize = normalize;
@@ -703,19 +709,19 @@ static int launch_rep_gram(const void* X, int problems, int n_rows, int normaliz
     return CA_ERR_CUDA;
   auto k = rep_gram_tc_kernel<D>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-  k<<<dim3(prm.n_chunks, problems), C::THREADS, C::SMEM, st>>>(mx, mwh, mwl, prm);
+  launch_chained(k, dim3(prm.n_chunks, problems), C::THREADS, C::SMEM, st, mx, mwh, mwl, prm);
   CA_LAUNCH_CHECK();
   return launch_gram_finalize(partial, problems, prm.n_chunks, D, gram, colsum, st);
 }
 
 int launch_rep_gram_tc(const void* X, int problems, int n_rows, int D, int normalize, float* partial, double* gram,
-                       double* colsum, const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st) {
+                       double* colsum, const void* wt_hi, const void* wt_lo, int* status, LaunchStream st) {
   return D == 64 ? launch_rep_gram<64>(X, problems, n_rows, normalize, partial, gram, colsum, wt_hi, wt_lo, status, st)
                  : launch_rep_gram<128>(X, problems, n_rows, normalize, partial, gram, colsum, wt_hi, wt_lo, status, st);
 }
 
 int launch_transform_tc(const void* X, int problems, int n_rows, int D, const float* bias, int normalize, float* out,
-                        const void* wt_hi, const void* wt_lo, int* status, cudaStream_t st, float* out_t) {
+                        const void* wt_hi, const void* wt_lo, int* status, LaunchStream st, float* out_t) {
   LinParams prm{};
   prm.bias = bias; prm.out_t = out_t; prm.status = status; prm.n_rows = n_rows; prm.normalize = normalize;
   const int tile = kRows * D * 2;
@@ -735,7 +741,7 @@ int launch_transform_tc(const void* X, int problems, int n_rows, int D, const fl
   const size_t smem = 1024 + (size_t)fixed + (size_t)prm.stages * tile + D * 4;
   auto k = D == 64 ? transform_tc_kernel<64> : transform_tc_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k<<<dim3(ceil_div(total_tiles, prm.tiles_per_cta), problems), kLinThreads, smem, st>>>(mx, mwh, mwl, mo, prm);
+  launch_chained(k, dim3(ceil_div(total_tiles, prm.tiles_per_cta), problems), kLinThreads, smem, st, mx, mwh, mwl, mo, prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
