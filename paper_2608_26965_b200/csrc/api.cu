@@ -292,6 +292,9 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
                                     tc ? w.wt2_hi : nullptr, tc ? w.wt2_lo : nullptr, sq));
       CA_TRY(launch_cholesky_factor(w.gramQ, nullptr, 1.0, 1.0 / (double)p->n_q, P, D, Fq, w.roots32, nullptr, nullptr, sk));
     }
+    // The launches of both sides are enqueued in the order in which they can start (a call's 21 launches take
+    // the host 0.11 ms; with one side after the other the second side's principal components, in small calls,
+    // waited 30 us for their launch).
     // ---- query side
     // query representation r(q) = F_k^T q / |F_k^T q|, its covariance and principal components E_Q
     // (one kernel), the coordinates Y = (r(q) - mean) E_Q.  fp32 storage keeps r(q); bf16 storage
@@ -313,6 +316,23 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
         CA_TRY(launch_moments(w.Qprime, CA_DTYPE_FP32, P, p->n_q, D, w.partial2, w.gramQp, w.sumQp, sq));
       }
     }
+    // ---- key side: covariance of the transformed keys K F_q
+    // (F_q^T C_K F_q / n_k, d x d algebra), its principal components E_K and the projection
+    // W = F_q E_K with its bias in one kernel; Y = (K - kbar) W
+    if (!serial) CA_RETURN_IF_CUDA(cudaStreamWaitEvent(sk, side->mid, 0));
+    {
+      ProfScope ps(kProfPca, sk);
+      PcaArgs a{};
+      a.mode = kPcaKeys;
+      a.gram = w.gramK; a.sum = w.sumK; a.n = (double)p->n_k; a.c_scale = ck_scale;
+      a.alpha = unnormalized ? 1.0 : 1.0 / (double)p->n_k;
+      a.lift = Fq; a.out_lifted = 1;
+      a.mean_sum = w.sumK; a.mean_n = (double)p->n_k;
+      a.W32 = w.WK32; a.bias = w.biasK;
+      a.wt_hi = tc ? w.wt_hi : nullptr; a.wt_lo = tc ? w.wt_lo : nullptr;
+      CA_TRY(launch_pca(a, P, D, sk));
+    }
+    // ---- query side: principal components of r(q); then both sides side by side
     {
       ProfScope ps(kProfPca, sq);
       PcaArgs a{};
@@ -333,28 +353,6 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
         CA_TRY(launch_transform_rows(w.Qprime, CA_DTYPE_FP32, P, p->n_q, D, EQ32, w.biasQ, 0, yq_out, sq));
       }
     }
-    CA_TRY(launch_split(yq_out, nullptr, P, D, p->n_q, p->n_k, p->cluster_q, p->cluster_k, perm_q, w.perm_q_tmp,
-                        perm_k, w.perm_k_tmp, w.keybuf_q, w.keybuf_k, 1, sq, w.Ytq, nullptr));
-    {
-      ProfScope ps(kProfPermute, sq);
-      CA_TRY(launch_permute_centroid(Q, p->dtype, perm_q, P, p->n_q, D, p->cluster_q, Qp, cq, count_q, sq));
-    }
-    // ---- key side: covariance of the transformed keys K F_q
-    // (F_q^T C_K F_q / n_k, d x d algebra), its principal components E_K and the projection
-    // W = F_q E_K with its bias in one kernel; Y = (K - kbar) W
-    if (!serial) CA_RETURN_IF_CUDA(cudaStreamWaitEvent(sk, side->mid, 0));
-    {
-      ProfScope ps(kProfPca, sk);
-      PcaArgs a{};
-      a.mode = kPcaKeys;
-      a.gram = w.gramK; a.sum = w.sumK; a.n = (double)p->n_k; a.c_scale = ck_scale;
-      a.alpha = unnormalized ? 1.0 : 1.0 / (double)p->n_k;
-      a.lift = Fq; a.out_lifted = 1;
-      a.mean_sum = w.sumK; a.mean_n = (double)p->n_k;
-      a.W32 = w.WK32; a.bias = w.biasK;
-      a.wt_hi = tc ? w.wt_hi : nullptr; a.wt_lo = tc ? w.wt_lo : nullptr;
-      CA_TRY(launch_pca(a, P, D, sk));
-    }
     {
       ProfScope ps(kProfTransform, sk);
       if (tc) {
@@ -363,8 +361,14 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
         CA_TRY(launch_transform_rows(K, p->dtype, P, p->n_k, D, w.WK32, w.biasK, 0, yk_out, sk));
       }
     }
+    CA_TRY(launch_split(yq_out, nullptr, P, D, p->n_q, p->n_k, p->cluster_q, p->cluster_k, perm_q, w.perm_q_tmp,
+                        perm_k, w.perm_k_tmp, w.keybuf_q, w.keybuf_k, 1, sq, w.Ytq, nullptr));
     CA_TRY(launch_split(nullptr, yk_out, P, D, p->n_q, p->n_k, p->cluster_q, p->cluster_k, perm_q, w.perm_q_tmp,
                         perm_k, w.perm_k_tmp, w.keybuf_q, w.keybuf_k, 2, sk, nullptr, w.Ytk));
+    {
+      ProfScope ps(kProfPermute, sq);
+      CA_TRY(launch_permute_centroid(Q, p->dtype, perm_q, P, p->n_q, D, p->cluster_q, Qp, cq, count_q, sq));
+    }
     {
       ProfScope ps(kProfPermute, sk);
       CA_TRY(launch_permute_centroid(K, p->dtype, perm_k, P, p->n_k, D, p->cluster_k, Kp, ck, count_k, sk, V, Vp, cv));

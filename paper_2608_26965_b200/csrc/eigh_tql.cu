@@ -572,19 +572,28 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
   constexpr int TILES = D * D / 16;                    // d x d x d products: 4 x 4 tiles
 
   // ---- prologue: the matrix to decompose, in A
-  if (a.lift) {
-    const double* F = a.lift + mat;
-    for (int e = tid; e < D * D; e += NT) L[(e / D) * LDA + e % D] = (float)F[e];
-  }
+  // (16-byte loads, several in flight: the launch starts with nothing else to do)
+  auto load_factor = [&]() {
+    const double2* F = reinterpret_cast<const double2*>(a.lift + mat);
+#pragma unroll 4
+    for (int e = tid; e < D * D / 2; e += NT) {
+      const double2 f = F[e];
+      *reinterpret_cast<float2*>(&L[(2 * e / D) * LDA + 2 * e % D]) = make_float2((float)f.x, (float)f.y);
+    }
+  };
+  if (a.lift) load_factor();
   if (a.mode == kPcaKeys) {
     // C = (gram - s s^T / n) c_scale, the centred scatter of the keys; then alpha F^T C F
     // (double-precision operations are scarce on this part: no division per element)
     const double* G = a.gram + mat;
     const double* sm = a.sum + (size_t)blockIdx.x * D;
     const double cs = a.c_scale, cn = a.c_scale / a.n;
-    for (int e = tid; e < D * D; e += NT) {
-      const int i = e / D, j = e % D;
-      A[i * LDA + j] = (float)fma(-cn * sm[i], sm[j], G[e] * cs);
+#pragma unroll 4
+    for (int e = tid; e < D * D / 2; e += NT) {
+      const int i = 2 * e / D, j = 2 * e % D;
+      const double2 g = reinterpret_cast<const double2*>(G)[e];
+      const double si = -cn * sm[i];
+      *reinterpret_cast<float2*>(&A[i * LDA + j]) = make_float2((float)fma(si, sm[j], g.x * cs), (float)fma(si, sm[j + 1], g.y * cs));
     }
     __syncthreads();
     float acc[4][4];
@@ -612,9 +621,12 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     const double* G = a.gram + mat;
     const double* sm = a.sum + (size_t)blockIdx.x * D;
     const double inv_n = 1.0 / a.n, inv_n2 = inv_n * inv_n;
-    for (int e = tid; e < D * D; e += NT) {
-      const int i = e / D, j = e % D;
-      A[i * LDA + j] = (float)fma(-inv_n2 * sm[i], sm[j], G[e] * inv_n);
+#pragma unroll 4
+    for (int e = tid; e < D * D / 2; e += NT) {
+      const int i = 2 * e / D, j = 2 * e % D;
+      const double2 g = reinterpret_cast<const double2*>(G)[e];
+      const double si = -inv_n2 * sm[i];
+      *reinterpret_cast<float2*>(&A[i * LDA + j]) = make_float2((float)fma(si, sm[j], g.x * inv_n), (float)fma(si, sm[j + 1], g.y * inv_n));
     }
   } else {
     const double* Ain = a.A_in + mat;
@@ -909,10 +921,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
   }
   __syncthreads();
   // the factor of the sign rule (its space served the prologue, the merges and the reflectors)
-  if (a.lift) {
-    const double* F = a.lift + mat;
-    for (int e = tid; e < D * D; e += NT) L[(e / D) * LDA + e % D] = (float)F[e];
-  }
+  if (a.lift) load_factor();
   __syncthreads();
 
   // ---- the map from the original space, W = F E (W[i][j] = sum_k F[i][k] Qt[j][k]), into A
@@ -964,13 +973,15 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     if (a.evals) a.evals[(size_t)blockIdx.x * D + rank] = mine;
   }
   __syncthreads();
-  // projection matrix [in i][out rank(j)], fp32, and its transpose as bf16 hi + lo parts
-  for (int e = tid; e < D * D; e += NT) {
-    const int i = e / D, j = e % D;
-    const float v = sign_of[j] * (lifted_out ? A[i * LDA + j] : Qt[j * LDA + i]);
-    a.W32[mat + (size_t)i * D + rank_of[j]] = v;
-  }
-  if (a.wt_hi) {
+  // projection matrix [in i][out rank(j)] in fp32, or its transpose as bf16 hi + lo parts
+  if (!a.wt_hi) {
+    for (int e = tid; e < D * D; e += NT) {
+      const int i = e / D, j = e % D;
+      const float v = sign_of[j] * (lifted_out ? A[i * LDA + j] : Qt[j * LDA + i]);
+      a.W32[mat + (size_t)i * D + rank_of[j]] = v;
+    }
+  } else {
+#pragma unroll 4
     for (int e = tid; e < D * D; e += NT) {
       const int j = e / D, i = e % D;
       const float v = sign_of[j] * (lifted_out ? A[i * LDA + j] : Qt[j * LDA + i]);

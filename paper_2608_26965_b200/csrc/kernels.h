@@ -44,7 +44,7 @@ struct PcaArgs {
   const double* mean_sum;   // [P][D] column sums of the rows, and their count (null: zero bias):
   double mean_n;            //   bias = -(mean_sum / mean_n) . F E,
   int mean_lifted;          //   or . E where the sums are of transformed rows
-  float* W32;               // [P][D in][D out] projection matrix
+  float* W32;               // [P][D in][D out] projection matrix (scratch where wt_hi is given)
   float* bias;              // [P][D] or null
   __nv_bfloat16* wt_hi;     // [P][D out][D in] transposed projection as bf16 hi + lo parts, or null
   __nv_bfloat16* wt_lo;
