@@ -305,10 +305,11 @@ def stage_rooflines(w, heads, group_ms, hbm_gbs, peak_kind):
     top_k, tail_k = split_level_counts(nk, c)
     sub = lambda nodes: nodes * d * d * 4                      # subsample rows read by `nodes` sets
     algo = {
-        # Gram matrices of Q, K and of the query representation r(q) (stored as two bf16 halves / fp32)
-        "gram": heads * ((nq + nk) * d * b + nq * d * 4),
-        # Q -> r(q) (4 bytes per element out), r(q) -> Y_q, K -> Y_k (fp32 coordinates out)
-        "transform": heads * (nq * d * (b + 4) + nq * d * 8 + nk * d * (b + 4)),
+        # Gram matrices of Q, K and of the query representation r(q): bf16 reads Q once more, fp32 reads
+        # the stored representation
+        "gram": heads * ((nq + nk) * d * b + nq * d * b),
+        # Q -> Y_q, K -> Y_k (fp32 coordinates out); fp32 also writes r(q) and reads it instead of Q
+        "transform": heads * ((nq + nk) * d * (b + 4) + (nq * d * 8 if b == 4 else 0)),
         # per level and side: a key and a row index read, a row index written, plus the subsample tiles
         "split_levels": heads * (12 * (nq * top_q + nk * top_k) + sub((1 << top_q) - 1) + sub((1 << top_k) - 1)),
         "split_tail": heads * (12 * (nq * tail_q + nk * tail_k)

@@ -279,16 +279,16 @@ int ca_last_status(const void* ws);
  * second pass of the attention calls on this workspace has recomputed with the fp32 kernel, summed
  * over all calls since the caller zero-filled the workspace (the calls only add to the counter,
  * the last word of the 256-byte status block).  The tensor-core kernel keeps the reference of its
- * online softmax (Section 3.1: exact softmax over the kept blocks) one half-step behind; a query
- * cluster whose scores climb by more than 2^96 within 64 keys leaves its range and is recomputed.
+ * online softmax (Section 3.1: exact softmax over the kept blocks) a few steps of 128 keys behind; a
+ * query cluster whose scores climb by more than 2^96 in between leaves its range and is recomputed.
  * Returns the count (>= 0), or minus an error code. */
 int ca_attn_recomputed(const void* ws);
 
 /* Diagnostic hook for tests of the failure path (process-wide, not thread-safe; affects the
  * attention calls issued after it).  wait_limit_cycles: SM cycles after which a device-side wait
  * of the tensor-core attention kernel gives up (<= 0 restores the default of about two seconds).
- * skip_key_load: the loader leaves out the key rows of this half-step (64 keys) of every query
- * tile, so that the waits for them run out: the kernel records CA_ERR_TIMEOUT, releases its tensor
+ * skip_key_load: counted in half-steps of 64 keys; the loader leaves out the key rows of the step of
+ * 128 keys that holds this one, in every query tile, so that the waits for them run out: the kernel records CA_ERR_TIMEOUT, releases its tensor
  * memory and returns, and the output of the call is undefined; -1 restores normal operation. */
 void ca_debug_attn_wait(long long wait_limit_cycles, int skip_key_load);
 

@@ -1019,7 +1019,8 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   if (rc != CA_OK) return rc;
   ProfScope ps(kProfAttnSecond, st);
   // second pass: query tiles whose scores left the range of the fast softmax (a climb of more than
-  // 2^96 within 64 keys) are recomputed by the fp32 kernel; its CTAs return at once for the others
+  // 2^96 within the steps that the reference lags behind) are recomputed by the fp32 kernel; its CTAs
+  // return at once for the others
   return launch_attn_ref(pr, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, scale, O, lse,
                          status, st, redo, tiles_per_qc, status + kRecomputedWord);
 }

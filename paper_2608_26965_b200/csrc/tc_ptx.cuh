@@ -66,7 +66,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-// The same bounded wait for a warp with time to spare (the loader runs a whole half-step ahead): it
+// The same bounded wait for a warp with time to spare (the loaders run ahead): it
 // sleeps between polls, so that it does not take issue slots from the warps that share its
 // sub-core.
 __device__ __forceinline__ bool mbar_wait_relaxed(uint32_t bar, uint32_t parity, volatile int* abort_flag,
