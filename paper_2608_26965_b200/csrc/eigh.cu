@@ -191,7 +191,9 @@ int launch_cholesky_factor(const double* gram, const double* sum, double n, doub
 __global__ void metric_kernel(const double* __restrict__ gramQ, const double* __restrict__ gramK,
                               const double* __restrict__ sumK, int D, double n_q, double n_k,
                               double ck_scale, double* __restrict__ M, double* __restrict__ CK) {
-  // either output may be left out (null): the two come from different streams in cluster_qk
+  wait_for_previous();
+  let_next_start();
+  // either output may be left out (null)
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= D * D) return;
@@ -202,19 +204,21 @@ __global__ void metric_kernel(const double* __restrict__ gramQ, const double* __
 }
 
 __global__ void cast_f64_f32_kernel(const double* __restrict__ src, float* __restrict__ dst, size_t count) {
+  wait_for_previous();
+  let_next_start();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) dst[i] = (float)src[i];
 }
 int launch_cast_f64_f32(const double* src, float* dst, size_t count, LaunchStream st) {
-  cast_f64_f32_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(src, dst, count);
+  launch_chained(cast_f64_f32_kernel, (unsigned)((count + 255) / 256), 256, 0, st, src, dst, count);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
 
 int launch_metric(const double* gramQ, const double* gramK, const double* sumK, int P, int D, int n_q,
                   int n_k, double ck_scale, double* M, double* CK, LaunchStream st) {
-  metric_kernel<<<dim3(ceil_div(D * D, 256), P), 256, 0, st>>>(gramQ, gramK, sumK, D, (double)n_q,
-                                                                (double)n_k, ck_scale, M, CK);
+  launch_chained(metric_kernel, dim3(ceil_div(D * D, 256), P), 256, 0, st, gramQ, gramK, sumK, D, (double)n_q,
+                 (double)n_k, ck_scale, M, CK);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }

@@ -1015,6 +1015,7 @@ __device__ __forceinline__ float seq_norm(const float* v, int d) {
 // One CTA of D threads per (slot, side, head).
 template <typename T, int D>
 __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams prm) {
+  wait_for_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* z = reinterpret_cast<float*>(smem_raw);       // [m][D + 1]
   __shared__ float u[D], v[D], w[D], y[D], g[D];
@@ -1096,12 +1097,15 @@ __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams pr
     if (nrm > 0.f && isfinite(nrm)) u[tid] = __fdiv_rn(y[tid], nrm);
     __syncthreads();
   }
+  let_next_start();
   sd.dirs[((size_t)p * sd.nodes + node) * D + tid] = u[tid];
 }
 
 // Keys of one level: one thread per position; the set of a position follows from the size rule.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) basic_keys_kernel(const BasicParams prm) {
+  wait_for_previous();
+  let_next_start();
   const int which = blockIdx.y / prm.problems, p = blockIdx.y % prm.problems;
   const BasicSide sd = prm.side[which];
   if (prm.level >= sd.levels) return;
@@ -1349,6 +1353,7 @@ __device__ __forceinline__ float stored_value<__nv_bfloat16>(const __nv_bfloat16
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicParams prm, const SplitParams sp) {
+  wait_for_previous();
   using Sm = BasicTailSmem<D>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Sm& sm = *reinterpret_cast<Sm*>(smem_raw);
@@ -1594,6 +1599,7 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
     cur ^= 1;
     ++level;
   }
+  let_next_start();
   for (int i = tid; i < s0; i += nt) pout[lo + i] = sm.rows[cur][i];
 }
 
@@ -1652,16 +1658,16 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
     if (D == 64) {
       auto dk = basic_direction_kernel<T, 64>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
-      dk<<<dim3(1u << level, 2 * problems), 64, dsmem, st>>>(bp);
+      launch_chained(dk, dim3(1u << level, 2 * problems), 64, dsmem, st, bp);
     } else {
       auto dk = basic_direction_kernel<T, 128>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
-      dk<<<dim3(1u << level, 2 * problems), 128, dsmem, st>>>(bp);
+      launch_chained(dk, dim3(1u << level, 2 * problems), 128, dsmem, st, bp);
     }
     CA_LAUNCH_CHECK();
     const int n_max = n_q > n_k ? n_q : n_k;
-    if (D == 64) basic_keys_kernel<T, 64><<<dim3(ceil_div(n_max, 256), 2 * problems), 256, 0, st>>>(bp);
-    else basic_keys_kernel<T, 128><<<dim3(ceil_div(n_max, 256), 2 * problems), 256, 0, st>>>(bp);
+    launch_chained(D == 64 ? basic_keys_kernel<T, 64> : basic_keys_kernel<T, 128>, dim3(ceil_div(n_max, 256), 2 * problems), 256,
+                   0, st, bp);
     CA_LAUNCH_CHECK();
     int max_seg = 1;
     if (level < tail_q) max_seg = max_segment_at_level(n_q, c_q, level);
@@ -1675,11 +1681,11 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
   if (D == 64) {
     auto tk = basic_tail_kernel<T, 64>;
     CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BasicTailSmem<64>)));
-    tk<<<dim3(slots, 2 * problems), kSplitThreads, sizeof(BasicTailSmem<64>), st>>>(bp, prm);
+    launch_chained(tk, dim3(slots, 2 * problems), kSplitThreads, sizeof(BasicTailSmem<64>), st, bp, prm);
   } else {
     auto tk = basic_tail_kernel<T, 128>;
     CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BasicTailSmem<128>)));
-    tk<<<dim3(slots, 2 * problems), kSplitThreads, sizeof(BasicTailSmem<128>), st>>>(bp, prm);
+    launch_chained(tk, dim3(slots, 2 * problems), kSplitThreads, sizeof(BasicTailSmem<128>), st, bp, prm);
   }
   CA_LAUNCH_CHECK();
   return CA_OK;
