@@ -185,6 +185,47 @@ def root_split_agreement(Y_dev, Y_orc, c):
     return out
 
 
+def split_partings(Y_dev, Y_orc, c):
+    """The sets of the split tree at which two clusterings part, walked from the root while both agree
+    (float32 coordinate choices on either side).  Per set: its size, the coordinates chosen, the relative gap of the two
+    variances (oracle) where the choices differ, otherwise the rows that change sides, how far the farthest of
+    them lies from the oracle's threshold and by how much the two key columns differ at most, both in spreads of the key."""
+    Y_dev, Y_orc = np.asarray(Y_dev), np.asarray(Y_orc)
+    perm = np.arange(Y_orc.shape[0])
+    out, work = [], [(0, Y_orc.shape[0])]
+    while work:
+        nxt = []
+        for lo, hi in work:
+            s = hi - lo
+            if s <= c:
+                continue
+            rows = perm[lo:hi].copy()
+            sub = rows[orc.subsample_positions(s, min(Y_orc.shape[1], s))]
+            t, _ = orc.choose_coordinate_f32(Y_dev[sub])
+            t_orc, var = orc.choose_coordinate_f32(Y_orc[sub])
+            if t != t_orc:
+                out.append(dict(size=s, t_dev=t, t_orc=t_orc, gap=float((var[t_orc] - var[t]) / var[t_orc])))
+                continue
+            L = orc.split_point(s, c)
+            below = []
+            for Y in (Y_dev, Y_orc):
+                b = np.zeros(s, bool)
+                b[np.lexsort((rows, Y[rows, t]))[:L]] = True
+                below.append(b)
+            changed = below[0] != below[1]
+            if changed.any():
+                keys = Y_orc[rows, t].astype(np.float64)
+                thr, spread = np.partition(keys, L - 1)[L - 1], keys.std()
+                out.append(dict(size=s, t_dev=t, t_orc=t, rows=int(changed.sum()),
+                                distance=float(np.abs(keys[changed] - thr).max() / spread),
+                                key_difference=float(np.abs(Y_dev[rows, t].astype(np.float64) - keys).max() / spread)))
+                continue
+            perm[lo:hi] = np.concatenate([rows[below[0]], rows[~below[0]]])
+            nxt += [(lo, lo + L), (lo + L, hi)]
+        work = nxt
+    return out
+
+
 def within_cluster_scatter(Y, perm, c):
     """Mean squared distance of the rows to their cluster's mean, in the coordinates Y."""
     Y = np.asarray(Y, np.float64)
