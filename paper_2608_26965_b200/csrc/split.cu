@@ -26,6 +26,7 @@
 #include <cooperative_groups.h>
 
 #include "kernels.h"
+#include "sample_position.h"
 
 namespace ca {
 
@@ -106,10 +107,9 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
   // row beyond the sample is loaded as the last one and counts as zero
   pair2 x[PER][V / 2];
   const float* Yq = Y + t;
-  unsigned scaled = (unsigned)r * (unsigned)sz;      // j sz for j = r, r + 8, ...
 #pragma unroll
-  for (int k = 0; k < PER; ++k, scaled += 8u * (unsigned)sz) {
-    const int pos = full ? (int)(scaled / D) : min(r + 8 * k, m - 1);
+  for (int k = 0; k < PER; ++k) {
+    const int pos = full ? sample_position<D>(r + 8 * k, sz) : min(r + 8 * k, m - 1);
     const unsigned row = (unsigned)(global ? (rows ? __ldg(rows + pos) : first + pos) : rows[pos]);
     const float* src = Yq + (size_t)row * D;
     if constexpr (V == 4) {
