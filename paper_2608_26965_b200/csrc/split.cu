@@ -177,6 +177,9 @@ __device__ __forceinline__ void unit_variance(const float* __restrict__ Y, const
 #pragma unroll
     for (int v = 0; v < V; ++v) var[v] = __fadd_rn(var[v], __shfl_xor_sync(0xffffffffu, var[v], o));
   divide(var);
+  // a variance that is not a number (an infinity among the samples) loses against every other
+#pragma unroll
+  for (int v = 0; v < V; ++v) var[v] = fmaxf(var[v], -1.f);
   float best = var[0], best_mean = mean[0];
   int arg = t;
 #pragma unroll

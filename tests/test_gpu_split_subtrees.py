@@ -1,7 +1,7 @@
 """The subtree kernel of the splitter where its selection changes path, bit for bit against the oracle: bins
-that hold more rows than a list takes (far outliers, repeated values, infinities), subsets of fewer rows
+that hold more rows than a list takes (far outliers, repeated values, infinite variances), subsets of fewer rows
 than a full sample, subtrees of exactly and just above the largest size, one wave of CTAs or several;
-and split coordinates beyond those that are kept coordinate-major."""
+split coordinates beyond those that are kept coordinate-major, and infinite coordinates."""
 import numpy as np
 import pytest
 import torch
@@ -78,3 +78,35 @@ def test_levels_of_large_sets_match_the_oracle(kind, heads, n, d, c):
     """The same through the per-level kernel: one CTA per set up to eight, thresholds from a bin, from
     the digits, and among equal keys whose positions lie in several CTAs."""
     test_subtrees_match_the_oracle(kind, heads, n, d, c)
+
+
+def _choose_among_numbers(sub):
+    """The float32 choice with a variance that is not a number below every other."""
+    _, var = orc.choose_coordinate_f32(sub)
+    return int(np.argmax(np.where(np.isnan(var), np.float32(-1.0), var))), var
+
+
+@pytest.mark.parametrize("heads,n,d,c,columns", [
+    (2, 4096, 64, 64, [0, 5, 18, 40]), (2, 1500, 128, 16, [1, 2, 64, 127]), (40, 2000, 128, 64, [0, 8, 31, 90]),
+    (1, 30000, 64, 128, [3, 16, 33, 63]), (1, 20000, 128, 64, [0, 1, 70]), (2, 5000, 64, 32, range(64)),
+])
+@pytest.mark.filterwarnings("ignore:invalid value")
+def test_coordinates_with_infinities(heads, n, d, c, columns):
+    """Infinite coordinates give variances that are not numbers, beside ones that are: those columns are not
+    chosen (the first column where no variance is a number), whichever lanes hold them."""
+    r = np.random.default_rng(n + d)
+    Y = (r.standard_normal((heads, n, d)) * r.uniform(0.5, 2.0, d)).astype(np.float32)
+    for t in columns:
+        rows = r.random((heads, n)) < 0.2
+        Y[:, :, t][rows] = np.where(r.random(int(rows.sum())) < 0.5, np.inf, -np.inf)
+    p = binding.make_problem(1, heads, n, n, d, "bf16", c, c, 1, flags=binding.CA_Y_IN)
+    plan = binding.Plan(p, DEV)
+    X = torch.zeros((1, heads, n, d), dtype=torch.bfloat16, device=DEV)
+    Yd = torch.from_numpy(Y[None]).to(DEV)
+    plan.cluster_qk(X, X, X, Yq=Yd, Yk=Yd)
+    torch.cuda.synchronize()
+    assert all(v == 0 for v in plan.last_status().values())
+    for h in sorted({0, heads - 1}):
+        ref = orc.recursive_split(Y[h], c, choose=_choose_among_numbers)
+        assert np.array_equal(plan.perm_q[0, h].cpu().numpy(), ref), f"queries, head {h}"
+        assert np.array_equal(plan.perm_k[0, h].cpu().numpy(), ref), f"keys, head {h}"
