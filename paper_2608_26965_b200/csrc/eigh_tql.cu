@@ -58,6 +58,10 @@ constexpr int kThreads = 512;
 constexpr int kBaseLog = 2, kBase = 1 << kBaseLog;   // rows of a base block of the divide and conquer
 constexpr int kMaxQlIterations = 64;
 
+// Eigenvalues that are not numbers (the covariance of rows with infinities, or whose sums overflow) stand as +inf: the
+// rank of a pole among the others is then a permutation for every input, and indexes stay in range.
+__device__ __forceinline__ float pole_value(float x) { return fminf(x, INFINITY); }
+
 // ---- implicit-shift QL on rows [l0, l0 + kBase) of a tridiagonal matrix (de[i] = (diagonal i, coupling of
 // i and i + 1); the coupling behind the last row is not part of the block), by one warp: the search
 // for a negligible sub-diagonal entry uses all lanes, the rotation chase is one dependent chain on
@@ -148,6 +152,7 @@ __device__ __forceinline__ void ql_block(float2* de, int l0, float2* rt, float* 
     }
   }
   if (lane < kBase) {
+    de[l0 + lane].x = pole_value(de[l0 + lane].x);
 #pragma unroll
     for (int i = 0; i < kBase; ++i) Qt[(l0 + i) * lda + l0 + lane] = z[i];
   }
@@ -278,7 +283,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
       zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
     }
     const float tol = 8.f * 6e-8f * fmaxf(dmax, zmax);
-    const bool skip = rho2 * zmax <= tol;                  // the blocks do not couple: nothing to merge
+    const bool skip = !(rho2 * zmax > tol);                // the blocks do not couple, or not by a number: nothing to merge
     int K = 0, ng = 0, nd = 0;
     if (!skip) {
       // negligible weights, a pole per lane
@@ -485,7 +490,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
   // eigenvector i over the kept poles, normalised, as row b0 + i of A
   {
     const int i = live ? gi : 0;
-    const float d0 = kd[korg[i]], mu = kmu[i];
+    const float d0 = K > 0 ? kd[korg[i]] : 0.f, mu = kmu[i];     // (without a kept pole there is no root, and no korg)
     float nrm = 0.f;
 #pragma unroll 2
     for (int j = sub; j < K; j += T) {
@@ -546,7 +551,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
 #pragma unroll 1
   for (int e = lt; e < nd * NB; e += GT)
     L[(b0 + K + (e >> lg)) * LDA + b0 + (e & (NB - 1))] = Qt[defl_row[e >> lg] * LDA + b0 + (e & (NB - 1))];
-  if (lt < NB) de[b0 + lt].x = lt < K ? kd[korg[lt]] + kmu[lt] : defl_d[lt - K];
+  if (lt < NB) de[b0 + lt].x = pole_value(lt < K ? kd[korg[lt]] + kmu[lt] : defl_d[lt - K]);
   sync();
 }
 
