@@ -398,9 +398,12 @@ int select_blocks(const ca_problem_t* p, const float* cq, const float* ck, int32
   // room behind the status block holds tiles of scores when there are many key clusters
   float* score_ws = reinterpret_cast<float*>(static_cast<char*>(ws) + kStatusBytes);
   const size_t score_floats = aligned16(ws) ? (ws_bytes - kStatusBytes) / sizeof(float) : 0;
+  // the kernels clear the status block; at any other address a memset does
+  int* status = aligned16(ws) ? static_cast<int*>(ws) : nullptr;
+  if (!status) CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
   ProfScope ps(kProfSelect, st);
   return launch_score_select(cq, ck, P, ceil_div(p->n_q, p->cluster_q), ceil_div(p->n_k, p->cluster_k),
-                             p->head_dim, p->keep, block_idx, score_ws, score_floats, static_cast<int*>(ws), st);
+                             p->head_dim, p->keep, block_idx, score_ws, score_floats, status, st);
 }
 
 int cluster_attention_fwd(const ca_problem_t* p, const void* Qp, const void* Kp, const void* Vp,
@@ -439,10 +442,13 @@ int select_blocks_adaptive(const ca_problem_t* p, const float* cq, const float* 
   const float scale = p->softmax_scale > 0.f ? p->softmax_scale : 1.0f / sqrtf((float)p->head_dim);
   float* score_ws = reinterpret_cast<float*>(static_cast<char*>(ws) + kStatusBytes);
   const size_t score_floats = aligned16(ws) ? (ws_bytes - kStatusBytes) / sizeof(float) : 0;
+  // the kernels clear the status block; at any other address a memset does
+  int* status = aligned16(ws) ? static_cast<int*>(ws) : nullptr;
+  if (!status) CA_RETURN_IF_CUDA(cudaMemsetAsync(ws, 0, kStatusBytes, st));
   ProfScope ps(kProfSelect, st);
   return launch_select_adaptive(cq, ck, count_k, p->batch * p->heads, ceil_div(p->n_q, p->cluster_q),
                                 ceil_div(p->n_k, p->cluster_k), p->head_dim, scale, recall, min_count,
-                                block_idx, keep_count, score_ws, score_floats, static_cast<int*>(ws), st);
+                                block_idx, keep_count, score_ws, score_floats, status, st);
 }
 
 int cluster_attention_fwd_ragged(const ca_problem_t* p, const void* Qp, const void* Kp, const void* Vp,

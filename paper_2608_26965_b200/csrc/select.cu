@@ -22,9 +22,10 @@ __device__ __forceinline__ uint32_t score_key(float s) {
   return (u >> 31) ? ~u : (u | 0x80000000u);
 }
 
-// The selection records no errors: its kernels clear the status block themselves, one launch less.
+// The selection records no errors: its kernels clear the status block themselves, one launch less (null: cleared
+// by the caller, for a workspace that 4-byte stores cannot reach).
 __device__ __forceinline__ void clear_status(int* status) {
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(int)) status[threadIdx.x] = 0;
+  if (status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(int)) status[threadIdx.x] = 0;
 }
 
 // QT query clusters per CTA: 4 when the CTA computes the scores itself (the key centroids are read

@@ -339,3 +339,36 @@ def test_two_host_threads_on_two_streams_give_the_sequential_results():
         got = (plans[i].O, plans[i].lse, plans[i].perm_q, plans[i].perm_k, plans[i].block_idx)
         for a, b in zip(got, alone[i]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n_kc", [40, 300])                                  # fused, and tiled where the workspace allows it
+def test_selection_with_a_workspace_at_any_address(n_kc):
+    """The selection takes a workspace at any address (without room for score tiles unless it is aligned): the same lists,
+    the status block cleared and nothing behind it touched."""
+    lib = binding.load_library()
+    c, n_qc, d = 16, 37, 64
+    p = binding.make_problem(1, 2, n_qc * c, n_kc * c, d, "bf16", c, c, 5)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(n_kc)
+    cq, ck = (torch.randn((1, 2, n, d), generator=g, device=DEV) for n in (n_qc, n_kc))
+    plan = binding.Plan(p, DEV)
+    want = plan.select_blocks(cq, ck).clone()
+    count = torch.full((1, 2, n_kc), c, dtype=torch.int32, device=DEV)
+    want_ragged, want_count = (t.clone() for t in plan.select_blocks_adaptive(0.5, 3, cq, ck, count))
+    for offset in (1, 4, 7):
+        ws = torch.full((512,), 0x5a, dtype=torch.uint8, device=DEV)
+        ptr = lambda t: ctypes.c_void_p(t.data_ptr())
+        at, size = ctypes.c_void_p(ws.data_ptr() + offset), ctypes.c_size_t(256)
+        plan.block_idx.zero_()
+        assert lib.select_blocks(ctypes.byref(p), ptr(cq), ptr(ck), ptr(plan.block_idx), at, size, None) == binding.CA_OK
+        torch.cuda.synchronize()
+        assert torch.equal(plan.block_idx, want)
+        for step in range(2):
+            assert bool((ws[offset:offset + 256] == 0).all())
+            assert bool((ws[:offset] == 0x5a).all()) and bool((ws[offset + 256:] == 0x5a).all())
+            if step == 0:
+                ws[offset:offset + 256] = 1
+                assert lib.select_blocks_adaptive(ctypes.byref(p), ptr(cq), ptr(ck), ptr(count), 0.5, 3, ptr(plan.block_idx_ragged),
+                                                  ptr(plan.keep_count), at, size, None) == binding.CA_OK
+                torch.cuda.synchronize()
+        assert torch.equal(plan.block_idx_ragged, want_ragged) and torch.equal(plan.keep_count, want_count)
