@@ -5,20 +5,23 @@
 // Serves fp32 storage, unusual cluster sizes, and as an on-device cross-check of
 // the tensor-core kernel.  Flash-style online softmax, fp32 throughout.
 //
-// Bound by the fp32 pipe and by what feeds it from shared memory: 16 threads share four query
-// rows, a thread computes 4 x 2 scores and 4 x D / 16 outputs, so that eight 16-byte loads feed 64 (scores)
+// Bound by the fp32 pipe and by what feeds it from shared memory: 16 threads share RY = 4 query
+// rows, a thread computes 4 x 2 scores and 4 x D / 16 outputs, so that six 16-byte loads feed 32 (scores)
 // and 12 feed 128 (outputs) multiply-adds; the rows of the next tile of keys are fetched from global memory
 // while a tile is computed.  4 heads of 5,003 rows, d = 128, 5 of 40 clusters of 128 kept: 0.80 ->
 // 0.36 ms; 2 heads of 1,024 rows, d = 64: 49 -> 26 us (before: 16 query rows per CTA, scalar loads).
-// A CTA takes 64 query rows where that still gives every SM one, otherwise 32.
+// A CTA takes 64 query rows where that still gives every SM one, otherwise 32; of a query cluster of 16
+// rows it takes those, with RY = 2: in a tile of 32 half of the threads computed nothing, and calls with such
+// clusters took up to 1.4 times as long as with the scalar kernel (60 shapes: 1.00 of its speed in the mean, 0.71 at worst; with the narrow
+// tile 1.37 and 0.99, with RY = 4 in it 1.35 and 0.94).
 #include "kernels.h"
 
 namespace ca {
 
 constexpr int kRefKT = 32;       // keys per staged tile
 
-template <typename T, int D, int QR>
-__global__ void __launch_bounds__(4 * QR)
+template <typename T, int D, int QR, int RY>
+__global__ void __launch_bounds__(16 * QR / RY)
 attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __restrict__ Vp,
                 const float* __restrict__ ck, const float* __restrict__ cv,
                 const int32_t* __restrict__ count_k, const int32_t* __restrict__ block_idx,
@@ -28,7 +31,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
                 int* __restrict__ status, const int32_t* __restrict__ redo, int redo_tiles,
                 int* __restrict__ redo_count, int per_cta, int n_clusters) {
   wait_for_previous();
-  constexpr int NT = 4 * QR;             // threads: 16 per four query rows
+  constexpr int NT = 16 * QR / RY;       // threads: 16 per RY query rows
   constexpr int LD = D + 4;              // row pitch: rows of eight threads in distinct banks
   constexpr int LP = kRefKT + 4;
   constexpr int CG = D / 64;             // groups of four output columns per thread
@@ -105,9 +108,9 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       *reinterpret_cast<float4*>(&qs[r * LD + col]) = v;
     }
 
-    float m_run[4], l_run[4], acc[4][CG][4];
+    float m_run[RY], l_run[RY], acc[RY][CG][4];
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
+    for (int y = 0; y < RY; ++y) {
       m_run[y] = -INFINITY;
       l_run[y] = 0.f;
 #pragma unroll
@@ -173,21 +176,21 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       else rows = max(0, min(kRefKT, n_kc - t0));
       if (rows > 0) fetch();
 
-      // scores of rows 4 tr + y, keys tc + 16 i
-      float s[4][KI];
+      // scores of rows RY tr + y, keys tc + 16 i
+      float s[RY][KI];
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
+      for (int y = 0; y < RY; ++y)
 #pragma unroll
         for (int i = 0; i < KI; ++i) s[y][i] = 0.f;
 #pragma unroll 4
       for (int k = 0; k < D; k += 4) {
-        float4 q4[4], k4[KI];
+        float4 q4[RY], k4[KI];
 #pragma unroll
-        for (int y = 0; y < 4; ++y) q4[y] = *reinterpret_cast<const float4*>(&qs[(4 * tr + y) * LD + k]);
+        for (int y = 0; y < RY; ++y) q4[y] = *reinterpret_cast<const float4*>(&qs[(RY * tr + y) * LD + k]);
 #pragma unroll
         for (int i = 0; i < KI; ++i) k4[i] = *reinterpret_cast<const float4*>(&ks[(tc + 16 * i) * LD + k]);
 #pragma unroll
-        for (int y = 0; y < 4; ++y)
+        for (int y = 0; y < RY; ++y)
 #pragma unroll
           for (int i = 0; i < KI; ++i) {
             s[y][i] = fmaf(q4[y].x, k4[i].x, s[y][i]); s[y][i] = fmaf(q4[y].y, k4[i].y, s[y][i]);
@@ -195,9 +198,9 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
           }
       }
       // online softmax: the 16 threads of a row are half a warp
-      float tmax[4];
+      float tmax[RY];
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
+      for (int y = 0; y < RY; ++y) {
         tmax[y] = -INFINITY;
 #pragma unroll
         for (int i = 0; i < KI; ++i) {
@@ -208,10 +211,10 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
 #pragma unroll
       for (int o = 1; o < 16; o <<= 1)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) tmax[y] = fmaxf(tmax[y], __shfl_xor_sync(0xffffffffu, tmax[y], o));
-      float psum[4], alpha[4];
+        for (int y = 0; y < RY; ++y) tmax[y] = fmaxf(tmax[y], __shfl_xor_sync(0xffffffffu, tmax[y], o));
+      float psum[RY], alpha[RY];
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
+      for (int y = 0; y < RY; ++y) {
         const float m_new = fmaxf(m_run[y], tmax[y]);
         const bool any = m_new > -INFINITY;
         alpha[y] = any ? expf(m_run[y] - m_new) : 1.f;
@@ -219,7 +222,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
 #pragma unroll
         for (int i = 0; i < KI; ++i) {
           const float pv = any ? expf(s[y][i] - m_new) : 0.f;
-          ps[(4 * tr + y) * LP + tc + 16 * i] = pv;
+          ps[(RY * tr + y) * LP + tc + 16 * i] = pv;
           psum[y] += pv;
         }
         m_run[y] = m_new;
@@ -227,9 +230,9 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
 #pragma unroll
       for (int o = 1; o < 16; o <<= 1)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) psum[y] += __shfl_xor_sync(0xffffffffu, psum[y], o);
+        for (int y = 0; y < RY; ++y) psum[y] += __shfl_xor_sync(0xffffffffu, psum[y], o);
 #pragma unroll
-      for (int y = 0; y < 4; ++y) {
+      for (int y = 0; y < RY; ++y) {
         l_run[y] = l_run[y] * alpha[y] + psum[y];
 #pragma unroll
         for (int g = 0; g < CG; ++g)
@@ -239,16 +242,16 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       __syncwarp();
 #pragma unroll 2
       for (int key = 0; key < kRefKT; key += 4) {
-        float4 p4[4];
+        float4 p4[RY];
 #pragma unroll
-        for (int y = 0; y < 4; ++y) p4[y] = *reinterpret_cast<const float4*>(&ps[(4 * tr + y) * LP + key]);
+        for (int y = 0; y < RY; ++y) p4[y] = *reinterpret_cast<const float4*>(&ps[(RY * tr + y) * LP + key]);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
 #pragma unroll
           for (int g = 0; g < CG; ++g) {
             const float4 v4 = *reinterpret_cast<const float4*>(&vs[(key + kk) * LD + 64 * g + 4 * tc]);
 #pragma unroll
-            for (int y = 0; y < 4; ++y) {
+            for (int y = 0; y < RY; ++y) {
               const float pv = kk == 0 ? p4[y].x : kk == 1 ? p4[y].y : kk == 2 ? p4[y].z : p4[y].w;
               acc[y][g][0] = fmaf(pv, v4.x, acc[y][g][0]); acc[y][g][1] = fmaf(pv, v4.y, acc[y][g][1]);
               acc[y][g][2] = fmaf(pv, v4.z, acc[y][g][2]); acc[y][g][3] = fmaf(pv, v4.w, acc[y][g][3]);
@@ -258,8 +261,8 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
     }
 
 #pragma unroll
-    for (int y = 0; y < 4; ++y) {
-      const int row = r0 + 4 * tr + y, pos = qc * c_q + row;
+    for (int y = 0; y < RY; ++y) {
+      const int row = r0 + RY * tr + y, pos = qc * c_q + row;
       if (row >= c_q || pos >= n_q) continue;
       const int orig = perm_q[(size_t)p * n_q + pos];
       if (orig < 0 || orig >= n_q) {
@@ -279,7 +282,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   }   // clusters of the CTA
 }
 
-template <typename T, int D, int QR>
+template <typename T, int D, int QR, int RY = 4>
 static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* Vp, const float* ck,
                        const float* cv, const int32_t* count_k, const int32_t* block_idx,
                        const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
@@ -290,12 +293,13 @@ static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T
                       sizeof(unsigned) * ((n_kc + 31) / 32);
   // second pass: some 600 CTAs that look at their share of the marks (10,240 CTAs that each looked at one took 18 us)
   const int n_clusters = pr.batch * pr.heads * n_qc;
-  const int per_cta = redo ? (ceil_div(n_clusters, 592) < 4 * QR ? ceil_div(n_clusters, 592) : 4 * QR) : 1;
+  constexpr int NT = 16 * QR / RY;
+  const int per_cta = redo ? (ceil_div(n_clusters, 592) < NT ? ceil_div(n_clusters, 592) : NT) : 1;
   const dim3 grid = redo ? dim3(ceil_div(n_clusters, per_cta))
                          : dim3(n_qc * ceil_div(pr.cluster_q, QR), pr.batch * pr.heads);
-  auto k = attn_ref_kernel<T, D, QR>;
+  auto k = attn_ref_kernel<T, D, QR, RY>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  launch_chained(k, grid, 4 * QR, smem, st, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
+  launch_chained(k, grid, NT, smem, st, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
                                 pr.cluster_q, pr.cluster_k, pr.keep, pr.compensate, scale, O, lse, status, redo,
                                 redo_tiles, redo_count, per_cta, n_clusters);
   CA_LAUNCH_CHECK();
@@ -315,8 +319,9 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
     return launch(pr, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, scale, O, lse, status, st,
                   redo, redo_tiles, redo_count);
   };
-  if (pr.head_dim == 64) return wide ? go(launch_rows<T, 64, 64>) : go(launch_rows<T, 64, 32>);
-  return wide ? go(launch_rows<T, 128, 64>) : go(launch_rows<T, 128, 32>);
+  const bool narrow = pr.cluster_q < 32;       // (never a second pass: the tensor-core kernel takes 64 rows and more)
+  if (pr.head_dim == 64) return narrow ? go(launch_rows<T, 64, 16, 2>) : wide ? go(launch_rows<T, 64, 64>) : go(launch_rows<T, 64, 32>);
+  return narrow ? go(launch_rows<T, 128, 16, 2>) : wide ? go(launch_rows<T, 128, 64>) : go(launch_rows<T, 128, 32>);
 }
 
 int launch_attn_ref(const ca_problem_t& pr, const void* Qp, const void* Kp, const void* Vp,

@@ -1,7 +1,7 @@
 """The tensor-core attention kernel at the edges of its walk over tiles and steps: tiles of one to four
 steps (fewer than its softmax groups, and one more), several tiles per CTA, lists without a key, key
 clusters of every size against query clusters of every size, short last clusters.  Compared with the
-library's fp32 kernel on the same clustering."""
+library's fp32 kernel on the same clustering, which itself is compared with float64 sums at each of its tile widths."""
 import pytest
 import torch
 
@@ -65,3 +65,47 @@ def test_tiles_of_few_steps_and_many_tiles(d, c_q, c_k, heads, n_q, n_k, compens
     assert (O - o_ref).norm() <= 1e-2 * o_ref.norm()
     assert (O - o_ref).abs().max() <= 5e-2
     assert (lse - lse_ref)[~empty].abs().max() <= 2e-3
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("d,c_q,c_k,heads,n_q,n_k,compensate", [
+    (64, 16, 32, 3, 16 * 9 - 5, 32 * 6 - 7, True), (128, 16, 16, 2, 16 * 5, 16 * 20 - 3, False),      # tiles of 16 rows
+    (128, 16, 256, 1, 33, 700, True),
+    (64, 32, 64, 2, 32 * 4 - 31, 64 * 5, True), (128, 32, 32, 1, 100, 32 * 9 - 1, False),             # of 32
+    (64, 256, 64, 1, 300, 64 * 4 - 9, True),
+    (128, 64, 128, 5, 64 * 30 - 3, 128 * 3 - 60, True), (64, 128, 32, 3, 128 * 26, 32 * 8, False),    # of 64: from 148 tiles on
+])
+def test_fp32_kernel_against_float64(d, c_q, c_k, heads, n_q, n_k, compensate, dtype):
+    Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, c_q, c_k, d + c_q + c_k + n_q)
+    if dtype == "fp32":
+        Qp, Kp, Vp = Qp.float(), Kp.float(), Vp.float()
+    n_qc, n_kc = lists.shape[2:]
+    keep = torch.arange(heads * n_qc, device=DEV).remainder(5).reshape(1, heads, n_qc).clamp(max=n_kc).int().contiguous()
+    rows = torch.arange(n_kc, device=DEV)
+    idx = torch.where(rows < keep[..., None], lists, n_kc + 1).sort(-1).values
+    idx = torch.where(rows < keep[..., None], idx, -1).int().contiguous()
+    plan = binding.Plan(binding.make_problem(1, heads, n_q, n_k, d, dtype, c_q, c_k, 1, compensate, flags=binding.CA_ATTN_FP32), DEV)
+    O, lse = plan.cluster_attention_fwd_ragged(idx, keep, Qp, Kp, Vp, ck, cv, count, perm)
+    torch.cuda.synchronize()
+    assert plan.last_status()["attn"] == 0
+    # every key and every centroid as columns, masked per query cluster
+    kept = torch.zeros((heads, n_qc, n_kc + 2), dtype=torch.bool, device=DEV).scatter_(2, torch.where(idx[0] < 0, n_kc, idx[0]).long(), True)
+    kept = kept[:, :, :n_kc]
+    pos = torch.arange(n_kc * c_k, device=DEV)
+    member = kept[:, :, pos // c_k] & (pos < n_k)
+    cluster = torch.arange(n_qc * c_q, device=DEV) // c_q
+    scale = 1.0 / d ** 0.5
+    x = torch.cat([Qp[0].double() @ Kp[0].double().mT, Qp[0].double() @ ck[0].double().mT], dim=2) * scale
+    x[:, :, n_kc * c_k:] += count[0, :, None].double().log()
+    live = torch.cat([member[:, cluster], ~kept[:, cluster] & compensate], dim=2)
+    x = x.masked_fill(~live, -torch.inf)
+    want_lse = x.logsumexp(2)[:, :n_q]
+    w = (x - x.logsumexp(2, keepdim=True)).exp().nan_to_num(0.0)
+    want = (w @ torch.cat([Vp[0], cv[0]], dim=1).double())[:, :n_q]
+    back = perm[0].long()
+    got, got_lse = O[0].double().gather(1, back[..., None].expand(-1, -1, d)), lse[0].double().gather(1, back)
+    empty = torch.isneginf(want_lse)
+    assert torch.equal(torch.isneginf(got_lse), empty) and bool((got[empty] == 0).all())
+    # float32 sums of up to d products and of all columns; results rounded to 2^-9 in bf16 storage
+    assert (got - want).norm() <= (1e-5 if dtype == "fp32" else 4e-3) * want.norm()
+    assert (got_lse - want_lse)[~empty].abs().max() <= 2e-5
