@@ -19,8 +19,12 @@
 namespace ca {
 
 constexpr int kRefKT = 32;       // keys per staged tile
+// Key clusters that the bitmap of the selected ones covers at a time (128 KB, beside the widest tile), so that their number
+// has no bound in shared memory.  With more of them (`many`, an instance of its own: moving the window costs the others
+// registers) the bitmap is set anew per window; a second pass never has as many (the tensor-core kernel takes an eighth).
+constexpr int kRefWindow = 1 << 20;
 
-template <typename T, int D, int QR, int RY>
+template <typename T, int D, int QR, int RY, bool many>
 __global__ void __launch_bounds__(16 * QR / RY)
 attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __restrict__ Vp,
                 const float* __restrict__ ck, const float* __restrict__ cv,
@@ -43,7 +47,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   float* vs = ks + kRefKT * LD;          // [KT][LD]
   float* ps = vs + kRefKT * LD;          // [QR][LP]
   float* bias = ps + QR * LP;            // [KT] per-key additive term (ln|c| or -inf)
-  unsigned* selected = reinterpret_cast<unsigned*>(bias + kRefKT);   // bitmap over key clusters
+  unsigned* selected = reinterpret_cast<unsigned*>(bias + kRefKT);   // bitmap over a window of key clusters
 
   const int n_qc = (n_q + c_q - 1) / c_q, n_kc = (n_k + c_k - 1) / c_k;
   const int tiles_per_cluster = (c_q + QR - 1) / QR;
@@ -90,14 +94,17 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   }
   const int32_t* cnt = count_k + (size_t)p * n_kc;
 
-  const int words = (n_kc + 31) / 32;
-  for (int w = tid; w < words; w += NT) selected[w] = 0u;
-  __syncthreads();
-  for (int t = tid; t < keep; t += NT) {
-    const int j = sel[t];
-    if (j < 0 || j >= n_kc) atomicCAS(status, 0, 6);
-    else atomicOr(&selected[j >> 5], 1u << (j & 31));
-  }
+  auto mark = [&](int first) {             // the selected ones among the clusters [first, first + kRefWindow)
+    const int words = many ? kRefWindow / 32 : (n_kc + 31) / 32;
+    for (int w = tid; w < words; w += NT) selected[w] = 0u;
+    __syncthreads();
+    for (int t = tid; t < keep; t += NT) {
+      const int j = sel[t];
+      if (j < 0 || j >= n_kc) atomicCAS(status, 0, 6);
+      else if (!many || (j >= first && j - first < kRefWindow)) atomicOr(&selected[(j - first) >> 5], 1u << (j & 31));
+    }
+  };
+  mark(0);
 
   for (int r0 = r0_first; r0 < r0_end; r0 += QR) {
     __syncthreads();                       // the previous tile's readers are done with the staged rows
@@ -151,7 +158,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         bool use = tid < rows;
         if (cen && use) {
           const int j = t0 + tid;
-          use = !((selected[j >> 5] >> (j & 31)) & 1u);
+          use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
           next_bias = use ? logf((float)cnt[j]) : -INFINITY;
         } else {
           next_bias = use ? 0.f : -INFINITY;
@@ -174,6 +181,13 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       rows = 0;
       if (t < keep) settle();
       else rows = max(0, min(kRefKT, n_kc - t0));
+      if constexpr (many) {
+        if (rows > 0 && t >= keep && t0 > 0 && t0 % kRefWindow == 0) {
+          __syncthreads();                 // the window before has been read
+          mark(t0);
+          __syncthreads();
+        }
+      }
       if (rows > 0) fetch();
 
       // scores of rows RY tr + y, keys tc + 16 i
@@ -282,7 +296,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   }   // clusters of the CTA
 }
 
-template <typename T, int D, int QR, int RY = 4>
+template <typename T, int D, int QR, int RY = 4, bool many = false>
 static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* Vp, const float* ck,
                        const float* cv, const int32_t* count_k, const int32_t* block_idx,
                        const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
@@ -290,14 +304,14 @@ static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T
                        int* redo_count) {
   const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
   const size_t smem = sizeof(float) * ((size_t)(QR + 2 * kRefKT) * (D + 4) + QR * (kRefKT + 4) + kRefKT) +
-                      sizeof(unsigned) * ((n_kc + 31) / 32);
+                      sizeof(unsigned) * (((n_kc < kRefWindow ? n_kc : kRefWindow) + 31) / 32);
   // second pass: some 600 CTAs that look at their share of the marks (10,240 CTAs that each looked at one took 18 us)
   const int n_clusters = pr.batch * pr.heads * n_qc;
   constexpr int NT = 16 * QR / RY;
   const int per_cta = redo ? (ceil_div(n_clusters, 592) < NT ? ceil_div(n_clusters, 592) : NT) : 1;
   const dim3 grid = redo ? dim3(ceil_div(n_clusters, per_cta))
                          : dim3(n_qc * ceil_div(pr.cluster_q, QR), pr.batch * pr.heads);
-  auto k = attn_ref_kernel<T, D, QR, RY>;
+  auto k = attn_ref_kernel<T, D, QR, RY, many>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, grid, NT, smem, st, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
                                 pr.cluster_q, pr.cluster_k, pr.keep, pr.compensate, scale, O, lse, status, redo,
@@ -313,6 +327,7 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
                     float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                     int* redo_count) {
   // 64 query rows per CTA read every key half as often as 32; 32 where 64 would leave SMs without a CTA
+  const int n_kc = ceil_div(pr.n_k, pr.cluster_k);
   const long long ctas = (long long)pr.batch * pr.heads * ceil_div(pr.n_q, 64);
   const bool wide = !redo && pr.cluster_q >= 64 && ctas >= 148;
   auto go = [&](auto launch) {
@@ -320,6 +335,7 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
                   redo, redo_tiles, redo_count);
   };
   const bool narrow = pr.cluster_q < 32;       // (never a second pass: the tensor-core kernel takes 64 rows and more)
+  if (n_kc > kRefWindow) return pr.head_dim == 64 ? go(launch_rows<T, 64, 32, 4, true>) : go(launch_rows<T, 128, 32, 4, true>);
   if (pr.head_dim == 64) return narrow ? go(launch_rows<T, 64, 16, 2>) : wide ? go(launch_rows<T, 64, 64>) : go(launch_rows<T, 64, 32>);
   return narrow ? go(launch_rows<T, 128, 16, 2>) : wide ? go(launch_rows<T, 128, 64>) : go(launch_rows<T, 128, 32>);
 }

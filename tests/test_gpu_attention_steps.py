@@ -2,6 +2,8 @@
 steps (fewer than its softmax groups, and one more), several tiles per CTA, lists without a key, key
 clusters of every size against query clusters of every size, short last clusters.  Compared with the
 library's fp32 kernel on the same clustering, which itself is compared with float64 sums at each of its tile widths."""
+import ctypes
+
 import pytest
 import torch
 
@@ -109,3 +111,40 @@ def test_fp32_kernel_against_float64(d, c_q, c_k, heads, n_q, n_k, compensate, d
     # float32 sums of up to d products and of all columns; results rounded to 2^-9 in bf16 storage
     assert (got - want).norm() <= (1e-5 if dtype == "fp32" else 4e-3) * want.norm()
     assert (got_lse - want_lse)[~empty].abs().max() <= 2e-5
+
+
+@pytest.mark.parametrize("n_kc,c_q", [(2 ** 20 + 37, 16), (1_640_000, 64)])
+def test_fp32_kernel_with_very_many_key_clusters(n_kc, c_q):
+    """More key clusters than the bitmap of the selected ones covers at a time, with selected ones at the edges of its windows."""
+    d, c_k, n_q = 64, 16, 61
+    g = torch.Generator(device=DEV)
+    g.manual_seed(c_q)
+    n_qc = -(-n_q // c_q)
+    Qp = torch.zeros((n_qc * c_q, d), dtype=torch.bfloat16, device=DEV)
+    Qp[:n_q] = torch.randn((n_q, d), generator=g, device=DEV).to(torch.bfloat16)
+    Kp, Vp = (torch.randn((n_kc * c_k, d), generator=g, device=DEV, dtype=torch.bfloat16) for _ in range(2))
+    ck, cv = (torch.randn((n_kc, d), generator=g, device=DEV) for _ in range(2))
+    count = torch.full((n_kc,), c_k, dtype=torch.int32, device=DEV)
+    picked = [0, 31, 2 ** 20 - 1, 2 ** 20, 2 ** 20 + 32, n_kc - 1]
+    idx = torch.tensor(picked, dtype=torch.int32, device=DEV).expand(n_qc, -1).contiguous()
+    perm = torch.randperm(n_q, generator=g, device=DEV).int()
+    O = torch.empty((n_q, d), dtype=torch.bfloat16, device=DEV)
+    lse = torch.empty((n_q,), device=DEV)
+    ws = torch.zeros((256,), dtype=torch.uint8, device=DEV)
+    p = binding.make_problem(1, 1, n_q, n_kc * c_k, d, "bf16", c_q, c_k, len(picked), True)
+    rc = binding.load_library().cluster_attention_fwd(
+        ctypes.byref(p), *[ctypes.c_void_p(t.data_ptr()) for t in (Qp, Kp, Vp, ck, cv, count, idx, perm, O, lse, ws)], 256, None)
+    assert rc == binding.CA_OK
+    torch.cuda.synchronize()
+    assert binding.load_library().ca_last_status(ctypes.c_void_p(ws.data_ptr())) == 0
+    q = Qp[:n_q].double()
+    rows = (idx[0].long()[:, None] * c_k + torch.arange(c_k, device=DEV)).flatten()
+    cen = (q @ ck.double().mT) / d ** 0.5 + count.double().log()
+    cen[:, idx[0].long()] = -torch.inf
+    x = torch.cat([(q @ Kp[rows].double().mT) / d ** 0.5, cen], dim=1)
+    want_lse = x.logsumexp(1)
+    want = (x - want_lse[:, None]).exp() @ torch.cat([Vp[rows].double(), cv.double()])
+    got, got_lse = O.double()[perm.long()], lse.double()[perm.long()]
+    # results rounded to 2^-9; float32 sums of up to 1.6 million terms, 32 at a time
+    assert (got - want).norm() <= 4e-3 * want.norm()
+    assert (got_lse - want_lse).abs().max() <= 1e-3
