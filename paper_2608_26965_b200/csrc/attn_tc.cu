@@ -775,7 +775,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
       if (!got) break;
       // a row without a single live entry (an empty list without compensation): zeros, lse = -inf
-      const bool lost = !(l_all < INFINITY);            // left the range: the second pass computes it
       const bool empty = !(l_all > 0.f);
       const float inv = empty ? 0.f : 1.f / l_all;
       __nv_bfloat16* out = prm.O + ((size_t)tl.x * prm.n_q + orig) * D;
@@ -794,6 +793,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             if (!got) break;
 #pragma unroll
             for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(fmaf(merge[j], inv_other, __uint_as_float(o[j])));
+            // 0 x inf, an infinite value among the other half's keys: for the second pass
+            float any = 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) any += __uint_as_float(o[j]);
+            if (any != any) l_all = any;
             __syncwarp();
             if (lane == 0) mbar_arrive(b_m_empty(pair));
           }
@@ -818,8 +822,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (lane == 0) mbar_arrive(b_o_empty);
       if (write && prm.lse)
         prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_all + log2f(l_all)) * 0.6931471805599453f;
-      // one word per tile, written on every launch by the last of its four warps: 1 = recompute
-      const bool redo = __any_sync(0xffffffffu, lost && !(twice && half == 1));
+      // one word per tile, written on every launch by the last of its four warps: 1 = recompute (a row left the range)
+      const bool redo = __any_sync(0xffffffffu, !(l_all < INFINITY) && !(twice && half == 1));
       if (lane == 0) {
         int* acc = &redo_acc[tl.w & 3];
         if ((atomicAdd(acc, redo ? 257 : 1) & 255) == 3) prm.redo[tl.z] = atomicExch(acc, 0) >= 256 ? 1 : 0;

@@ -148,3 +148,30 @@ def test_fp32_kernel_with_very_many_key_clusters(n_kc, c_q):
     # results rounded to 2^-9; float32 sums of up to 1.6 million terms, 32 at a time
     assert (got - want).norm() <= 4e-3 * want.norm()
     assert (got_lse - want_lse).abs().max() <= 1e-3
+
+
+@pytest.mark.parametrize("compensate", [False, True])
+@pytest.mark.parametrize("d,c_q,c_k,keep", [(64, 64, 64, 3), (128, 64, 128, 2), (128, 64, 256, 1), (64, 64, 16, 9),
+                                            (64, 128, 64, 4), (128, 256, 128, 3)])
+def test_values_with_infinities(d, c_q, c_k, keep, compensate):
+    """An infinite value makes the outputs that attend to it infinite (NaN where both signs meet), and those that do
+    not stay as they are: as from the fp32 kernel."""
+    heads, n_q, n_k = 2, c_q * 5 - 3, c_k * 12 - 5
+    Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, c_q, c_k, d + c_q + c_k)
+    n_kc = lists.shape[3]
+    idx = lists[..., :keep].sort(-1).values.contiguous()
+    Vp[0, 0, 3 * c_k + 5, 7] = torch.inf                 # in clusters 3 and 8 of head 0
+    Vp[0, 0, 8 * c_k + c_k - 1, 7] = -torch.inf
+    Vp[0, 0, 8 * c_k, d - 1] = -torch.inf
+    out = []
+    for flags in (0, binding.CA_ATTN_FP32):
+        plan = binding.Plan(binding.make_problem(1, heads, n_q, n_k, d, "bf16", c_q, c_k, keep, compensate, flags=flags), DEV)
+        out.append(plan.cluster_attention_fwd(Qp, Kp, Vp, ck, cv, count, idx, perm)[0].float())
+        torch.cuda.synchronize()
+        assert plan.last_status()["attn"] == 0
+    (O, want) = out
+    assert bool(torch.isinf(want).any()) and bool(torch.isfinite(want[0, 1]).all())
+    for mask in (torch.isnan, torch.isposinf, torch.isneginf):
+        assert torch.equal(mask(O), mask(want)), mask.__name__
+    fine = torch.isfinite(want)
+    assert (O - want)[fine].norm() <= 1e-2 * want[fine].norm()
