@@ -284,14 +284,28 @@ size_t select_score_floats(int P, int n_qc, int n_kc) {
   return (take + 63) / 64 * 64;
 }
 
+// Shared memory per CTA such that an SM takes no more CTAs than its share of the grid.  A launch that overlaps the one before
+// it is brought onto whichever SMs have room first, so that a grid of less than a wave was packed onto some of them:
+// 8 heads of 128 x 1,024 clusters took 34 us and take 21 (with launches one after the other 24), 552 x 4,688 60 -> 46 (47),
+// mass-recall lists of 586 x 2,344 333 -> 282 (287).  From eight CTAs of 256 threads on an SM is full anyway.
+static size_t spread_smem(size_t smem, size_t fixed, long long ctas) {
+  int sms = 0, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return smem;
+  const long long per_sm = (ctas + sms - 1) / sms;
+  if (per_sm >= 8) return smem;
+  const size_t share = (size_t)(228 * 1024 / per_sm - 1024 - fixed) / 128 * 128;   // 1 KB per CTA is the system's
+  return share > smem ? share : smem;
+}
+
 template <int D>
 static int launch_score_tiles(const float* cq, const float* ck, int P, int n_qc, int n_kc, int row0, int chunk_rows,
                               float* scores, LaunchStream st) {
   auto k = score_tile_kernel<D>;
-  const size_t smem = (size_t)2 * D * 64 * sizeof(float);
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int rows = min(chunk_rows, n_qc - row0);
-  launch_chained(k, dim3(ceil_div(n_kc, 64), ceil_div(rows, 64), P), 256, smem, st, cq, ck, n_qc, n_kc, row0, chunk_rows, scores);
+  const dim3 grid(ceil_div(n_kc, 64), ceil_div(rows, 64), P);
+  const size_t smem = spread_smem((size_t)2 * D * 64 * sizeof(float), 0, (long long)grid.x * grid.y * grid.z);
+  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  launch_chained(k, grid, 256, smem, st, cq, ck, n_qc, n_kc, row0, chunk_rows, scores);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -315,8 +329,9 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     CA_LAUNCH_CHECK();
     return CA_OK;
   }
-  const size_t smem = select_smem_bytes(n_kc, D, 1);
+  size_t smem = select_smem_bytes(n_kc, D, 1);
   if (smem > 200 * 1024) return CA_ERR_UNSUPPORTED;
+  smem = spread_smem(smem, 2048, (long long)min(chunk, n_qc) * P);
   auto k64 = score_select_kernel<64, 1>;
   auto k128 = score_select_kernel<128, 1>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -486,15 +501,16 @@ int launch_select_adaptive(const float* cq, const float* ck, const int32_t* coun
                            int32_t* keep_count, float* score_ws, size_t score_floats, int* status, LaunchStream st) {
   int n_pad = 1;
   while (n_pad < n_kc) n_pad <<= 1;
-  const size_t smem = (size_t)n_pad * 8 + (size_t)n_kc * 4 + (size_t)D * 4;
+  size_t smem = (size_t)n_pad * 8 + (size_t)n_kc * 4 + (size_t)D * 4;
   if (smem > 200 * 1024) return CA_ERR_UNSUPPORTED;
+  const int chunk = select_chunk_rows(P, n_qc, n_kc, score_ws ? score_floats : 0);
+  const int step = chunk == 0 ? n_qc : chunk;
+  smem = spread_smem(smem, 512, (long long)min(step, n_qc) * P);
   const float c_log2 = scale * 1.4426950408889634f;      // one float32 product, as in the definition
   auto k64 = select_adaptive_kernel<64>;
   auto k128 = select_adaptive_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int chunk = select_chunk_rows(P, n_qc, n_kc, score_ws ? score_floats : 0);
-  const int step = chunk == 0 ? n_qc : chunk;
   for (int row0 = 0; row0 < n_qc; row0 += step) {
     const int rows = min(step, n_qc - row0);
     const float* scores = nullptr;
