@@ -794,9 +794,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
             for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(fmaf(merge[j], inv_other, __uint_as_float(o[j])));
             // 0 x inf, an infinite value among the other half's keys: for the second pass
-            float any = 0.f;
+            f32x2 any2 = pack2(0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) any += __uint_as_float(o[j]);
+            for (int j = 0; j < 16; j += 2) any2 = add2(any2, pack2(__uint_as_float(o[j]), __uint_as_float(o[j + 1])));
+            float any, any_odd;
+            unpack2(any2, any, any_odd);
+            any += any_odd;
             if (any != any) l_all = any;
             __syncwarp();
             if (lane == 0) mbar_arrive(b_m_empty(pair));
