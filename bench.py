@@ -692,7 +692,7 @@ def run_ours(args, w):
                     "peak_source": "148 SMs x 128 FMA lanes x 2 x 1.965 GHz", "unit": "TFLOP/s",
                     "frac": attn_tflops / FP32_ALU_TFLOPS, "traffic": None}
     if w.dtype == "bf16" and w.head_dim == 64:
-        # At d = 64 the exponentials bound the kernel before the tensor pipe does: a half-step of 64 keys
+        # At d = 64 the exponentials bound the kernel before the tensor pipe does: a query tile against 64 keys
         # is 2 x (128 x 64 x 64) multiply-adds = 2^21 flops of tensor work per query tile and
         # 128 x 64 = 8192 exponentials, which the special-function unit of an SM takes 512 cycles for
         # (16 per cycle: 4 sub-cores x 1 warp instruction per 8 cycles): at most 4096 flops per cycle

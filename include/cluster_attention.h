@@ -104,11 +104,11 @@ int ca_workspace_bytes(const ca_problem_t* p, size_t* cluster_ws, size_t* select
  *   Yq [B,H,n_q,d], Yk [B,H,n_k,d] fp32 split coordinates: input when
  *        p->flags has CA_Y_IN, otherwise output (may be NULL: kept in ws).
  * The chain from Q to the key side (metric, its factor, key projection, key split)
- * and the chain from K to the query side need each other only through C_K: the
- * second one is enqueued on a side stream of the library (a pool of four per
- * device, taken in turn, created together with their events at the first call on
- * that device) that forks from `stream` at the start of the call and joins it
- * again before the call returns.  Nothing waits on the host; a capture of `stream`
+ * and the chain from K to the query side need each other only through C_K: one of
+ * them (the query side where n_k > 2 n_q, otherwise the key side) is enqueued on a
+ * side stream of the library (a pool of four per device, taken in turn, created
+ * together with their events at the first call on that device) that forks from
+ * `stream` at the start of the call and joins it again before the call returns.  Nothing waits on the host; a capture of `stream`
  * records the side stream as a parallel branch (make the first call on a device
  * before capturing).  The calls of this library may be issued from several host
  * threads; ca_profile, ca_debug_attn_wait and the workspaces themselves are not
@@ -159,7 +159,7 @@ int cluster_qk_basic(const ca_problem_t* p, const void* Q, const void* K, const 
  * clusters); for each query cluster the `keep` best key clusters, ties to the
  * lower index, written in ascending index order.
  *   block_idx [B,H,n_qc,keep] int32.
- * With 2048 key clusters or more and a workspace as large as ca_workspace_bytes
+ * With 128 key clusters or more and a workspace as large as ca_workspace_bytes
  * reports, the scores are first computed in tiles into the workspace (same
  * operation order, same bits); a workspace of 256 bytes selects the fused kernel.
  */
@@ -280,16 +280,18 @@ int ca_last_status(const void* ws);
  * over all calls since the caller zero-filled the workspace (the calls only add to the counter,
  * the last word of the 256-byte status block).  The tensor-core kernel keeps the reference of its
  * online softmax (Section 3.1: exact softmax over the kept blocks) a few steps of 128 keys behind; a
- * query cluster whose scores climb by more than 2^96 in between leaves its range and is recomputed.
+ * query cluster whose scores climb by more than 2^96 in between leaves its range and is recomputed;
+ * so is one of 64 rows whose output would not be a number (infinite values among its keys).
  * Returns the count (>= 0), or minus an error code. */
 int ca_attn_recomputed(const void* ws);
 
 /* Diagnostic hook for tests of the failure path (process-wide, not thread-safe; affects the
  * attention calls issued after it).  wait_limit_cycles: SM cycles after which a device-side wait
  * of the tensor-core attention kernel gives up (<= 0 restores the default of about two seconds).
- * skip_key_load: counted in half-steps of 64 keys; the loader leaves out the key rows of the step of
- * 128 keys that holds this one, in every query tile, so that the waits for them run out: the kernel records CA_ERR_TIMEOUT, releases its tensor
- * memory and returns, and the output of the call is undefined; -1 restores normal operation. */
+ * skip_key_load: counted in 64 keys from the start of a CTA's walk over its query tiles; the loader
+ * of every CTA leaves out the key rows of the step of 128 keys that holds these, so that the waits for
+ * them run out: the kernel records CA_ERR_TIMEOUT, releases its tensor memory and returns, and the
+ * output of the call is undefined; -1 restores normal operation. */
 void ca_debug_attn_wait(long long wait_limit_cycles, int skip_key_load);
 
 /* Diagnostic: the symmetric eigen-decomposition that cluster_qk uses for the principal components

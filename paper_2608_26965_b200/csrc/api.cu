@@ -78,10 +78,11 @@ struct ClusterWs {
 
 // A level of the splitter reads one coordinate of every row of a set, rows in ascending order: from the
 // row-major coordinates a line per row, from a coordinate-major copy neighbouring rows of the set
-// share lines, and a column stays in L2.  The coordinates are in order of variance and a split
-// removes most of the variance of its coordinate in both parts, so a tree of ten levels splits along the first
-// ten or so: the copy holds kSplitCols coordinates (64 bytes per row), any other is read
-// row-major.  (All d coordinates cost as much to write as the coordinates themselves.)
+// share lines, and a column stays in L2.  The coordinates are in order of variance, and a split
+// removes most of the variance of its coordinate in both parts: the copy holds the first kSplitCols (64
+// bytes per row), any other is read row-major.  A choice: rows of 16 groups split along no other;
+// rows of 32 groups, 8 heads of 131,072 keys at d = 64, reach coordinate 38 (3 % of the reads, 7 % of the subtree kernel's), 64
+// groups at d = 128 coordinate 48 (9 and 13 %).  All d coordinates cost as much to write as the coordinates themselves.
 static bool use_yt(const ca_problem_t* p) {
   return p->dtype == CA_DTYPE_BF16 && !(p->flags & CA_Y_IN);
 }
@@ -266,9 +267,9 @@ int cluster_qk(const ca_problem_t* p, const void* Q, const void* K, const void* 
     // covariance takes a pass over the rows, unless the keys (and values) are far more.
     const bool keys_longer = p->n_k > 2LL * p->n_q;
     cudaStream_t aside = serial ? st : side->stream;
-    // Overlapping launches save 25 us of a call (8 heads of 16,384 x 131,072 rows, d = 64: 1,446 -> 1,419); where the kernels
-    // of each side fill the GPU by themselves, the CTAs that wait keep the other side's from running
-    // (40 heads of 32,760 rows, d = 128: 4,650 -> 4,750).
+    // Overlapping launches save 25 us of a call (8 heads of 16,384 x 131,072 rows, d = 64, 7.5e7 elements: 1,446 ->
+    // 1,419); where the kernels of each side fill the GPU by themselves, the CTAs that wait keep the other side's from
+    // running (40 heads of 32,760 rows, d = 128, 3.4e8: 4,650 -> 4,750).  The line lies between the two, not where they cross.
     const bool chained = (double)P * ((double)p->n_q + p->n_k) * D < 1.5e8;
     const LaunchStream sq(keys_longer ? aside : st, chained), sk(keys_longer ? st : aside, chained);
     if (!serial) {

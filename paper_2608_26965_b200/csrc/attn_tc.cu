@@ -23,15 +23,17 @@
 // upper half takes keys 0-63 of every step and the lower half keys 64-127 (the other
 // probabilities of a row are stored as zeros), so that all four softmax warps of a group
 // work and each on half of the columns; the two halves are independent rows with sums,
-// references and outputs of their own, merged at the end of the tile.
+// references and outputs of their own, merged at the end of the tile.  (0 x inf is NaN: where
+// a kept cluster holds an infinite value the merged outputs send the tile to the second pass.)
 // All roles run at the same time on one SM and have to fit its instruction cache
 // together: with the loops of the single-warp roles unrolled (105 KB of code) the same
 // kernel took 1.40 ms where it now takes 0.73 (2 x 16 heads of 20,000 rows, d = 128, 10
 // clusters of 256 kept), so loops stay rolled unless a step is shorter for it.
-// What bounds it: at d = 128 every step brings 64 KB through L2, which delivers 43 bytes
-// per cycle and SM (1,520 cycles; a step takes 1,850), since the lists of two query
-// clusters share nothing; at d = 64 the exponentials (1,024 of 1,340 cycles per step)
-// and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
+// What bounds it: at d = 128 no unit by itself.  A step brings 64 KB through L2, since every tile
+// loads its lists for itself, and takes 0.96 us (1,850 cycles of 1.92 GHz): 10.0 TB/s over the SMs of the
+// 14.6 that plain bulk loads of L2-resident data reach (51 bytes per cycle and SM, 0.66 us),
+// with the tensor pipe 62 % and the exponentials 61 % busy; the rest are hand-offs.  At d = 64 the
+// exponentials (1,024 of 1,340 cycles per step) and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
 // four at d = 64, half-steps of 64 keys in one chain per CTA): 40 heads of 32,760 rows,
 // d = 128, 32 of 256 clusters kept 2.91 -> 2.44 ms; 8 heads of 16,384 x 131,072, d = 64,
 // 128 of 1,024 kept 0.88 -> 0.82; 12 heads of 16,385 in clusters of 64 0.373 -> 0.356.
@@ -130,7 +132,7 @@ struct TcParams {
   const float* k_scale;
   const float* c_scale;
   long long wait_limit;           // SM cycles after which a barrier wait gives up (CA_ERR_TIMEOUT)
-  int skip_key_load;              // diagnostic hook: the loader leaves out the keys of this half-step (-1: none)
+  int skip_key_load;              // diagnostic hook: the loader leaves out the keys of the step with these 64 (-1: none)
 };
 
 constexpr int kErrBadIndex = 6;   // CA_ERR_BAD_INDEX
@@ -912,7 +914,7 @@ bool attn_tc_supported(const ca_problem_t& pr) {
 }
 
 // quantised Q K^T: head dimension 128 (one 128-byte panel row of codes), key clusters of at least
-// 64 rows (one scale per half-step)
+// 64 rows (one scale per 64 columns)
 bool attn_tc_fp8_supported(const ca_problem_t& pr) {
   return attn_tc_supported(pr) && pr.head_dim == 128 && pr.cluster_k >= kCen;
 }

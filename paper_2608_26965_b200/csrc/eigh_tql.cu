@@ -38,10 +38,11 @@
 // the original space to the coordinates is F E; component t is oriented so that
 // the entry of largest magnitude (lowest row on ties) of column t of F E is
 // positive -- a rule that gives the same signs whatever root of the metric F is.
-// Written out: the projection matrix (F E for the keys, which are projected
-// straight from K; E for the queries, whose representation is already stored),
-// its bias -mean . W, and W^T as bf16 hi + lo parts for the tensor-core
-// projection.
+// Written out: the projection matrix W (F E where rows are projected from the original
+// space, the keys always and the queries of bf16 storage; E for the queries of fp32
+// storage, whose representation is kept) or W^T as bf16 hi + lo parts for the
+// tensor-core projection, and its bias -mean . F E, or . E where the mean is one of
+// transformed rows.
 #include <type_traits>
 
 #include "kernels.h"
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
             make_float4(al * acc[x][0], al * acc[x][1], al * acc[x][2], al * acc[x][3]);
     }
   } else if (a.mode == kPcaQueries) {
-    // covariance of the stored representation: gram / n - mean mean^T
+    // covariance of the representation from its moments: gram / n - mean mean^T
     const double* G = a.gram + mat;
     const double* sm = a.sum + (size_t)blockIdx.x * D;
     const double inv_n = 1.0 / a.n, inv_n2 = inv_n * inv_n;

@@ -105,14 +105,14 @@ def _bf16_round(a):
 
 @pytest.mark.parametrize("d,c_q,c_k,compensate", [(64, 128, 128, False), (64, 128, 32, True), (128, 128, 128, True),
                                                   (128, 128, 32, False), (64, 128, 64, True),
-                                                  (64, 256, 128, True),      # two CTAs per query cluster
-                                                  (128, 64, 128, False)])    # half-filled query tile
+                                                  (64, 256, 128, True),      # two tiles per query cluster
+                                                  (128, 64, 128, False)])    # both halves of a tile hold the same query cluster
 def test_attention_scores_that_rise_along_the_list(d, c_q, c_k, compensate):
     """Key blocks listed in an order in which the scores of a row climb by tens and by hundreds of
     binary orders of magnitude from one block to the next, and fall by as much for other rows: the
     running reference of the online softmax (Section 3.1: exact softmax over the kept blocks) has
     to follow without overflow, whatever it was before.  With 32-row key clusters the climb happens
-    in the middle of a 64-column half-step."""
+    in the middle of a step."""
     r = np.random.default_rng(31 + d + c_k)
     H, n_q = 1, 300 if c_q < 256 else 700
     gains = np.array([0.0, 2.0, 4.0, 60.0, 62.0, 30.0, 600.0, 610.0, 100.0, 1200.0, 1.0, 3.0])
@@ -271,7 +271,7 @@ def test_ragged_list_lengths_of_zero_and_beyond_the_row(dtype, compensate):
 @pytest.mark.parametrize("d", [64, 128])
 def test_a_wait_that_runs_out_ends_the_kernel_with_a_status(d):
     """The loader of the tensor-core attention kernel is told (diagnostic hook) to leave out the key
-    rows of one half-step, with the limit of the device-side waits set to about a millisecond: the
+    rows of one step, with the limit of the device-side waits set to about a millisecond: the
     waits for those rows run out, the kernel records CA_ERR_TIMEOUT, releases its tensor memory and
     returns.  With the hook cleared the next call on the same workspace is correct again."""
     lib = binding.load_library()

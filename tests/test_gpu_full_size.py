@@ -148,7 +148,7 @@ def test_sweep_full_size_one_eighth():
                                                          (256, 1 / 32, False), (256, 1 / 2, True)])
 def test_sweep_full_size_other_cluster_sizes(cluster, fraction, compensate):
     """The sweep workload at 131,072 tokens with 64-row clusters (2,048 clusters per side: the tiled
-    selection, half-filled query tiles) and 256-row clusters (two CTAs per query cluster), at the
+    selection, query tiles that hold a cluster twice) and 256-row clusters (two tiles per query cluster), at the
     lowest and the highest density of the sweep, with and without compensation."""
     n_kc = inputs.WORKLOADS["sweep"].n_k // cluster
     check_workload("sweep", sample_heads=[3], clusters_per_head=3, split_heads=[3], cluster=cluster,
@@ -158,7 +158,7 @@ def test_sweep_full_size_other_cluster_sizes(cluster, fraction, compensate):
 def test_long_sequence_half_a_million_tokens():
     """One head of 524,288 tokens (d = 64, 128-row clusters, 64 kept blocks, compensation on), the
     regime of the token-count sweep in which the 4,096 centroid columns per query outweigh the kept
-    blocks: 12 split levels, selection in score tiles, attention with 64 half-steps of centroids."""
+    blocks: 12 split levels, selection in score tiles, attention with 64 steps of centroids."""
     check_workload("tabular", sample_heads=[0], clusters_per_head=3, split_heads=[0], keep=64,
                    heads=1, n_q=524288, n_k=524288)
 

@@ -304,7 +304,7 @@ def bf16_close(O, o_ref):
     ("video480", 1000, 1000, 2, True, 0), ("sweep", 2048, 2048, 16, True, 0),
     ("tabular", 512, 2048, 4, True, binding.CA_ATTN_FP32),
     ("sweep64", 1100, 3000, 9, True, 0),          # 64-row clusters on both sides, short last clusters
-    ("sweep256", 1024, 2100, 3, True, 0),         # 256-row clusters: two CTAs per query cluster
+    ("sweep256", 1024, 2100, 3, True, 0),         # 256-row clusters: two tiles per query cluster
     ("sweep32k", 640, 1000, 11, False, 0),        # 32-row key clusters packed four to a tile
     ("sweep64x128", 1100, 3000, 5, True, 0),      # 64 query rows x 128 key rows: the paper's block shape
 ])
@@ -329,9 +329,9 @@ def test_attention_bf16(name, n_q, n_k, keep, compensate, flags):
 @pytest.mark.parametrize("name,n_q,n_k,c_q,c_k,keep,compensate,perm_seed", [
     ("video480", 1000, 1000, 128, 128, 2, True, None),     # short last clusters, centroid columns
     ("sweep", 2048, 2048, 128, 128, 16, True, None),       # all blocks kept but none short
-    ("sweep", 1100, 3000, 64, 64, 9, True, 5),             # 64-row clusters: one key scale per half-step
+    ("sweep", 1100, 3000, 64, 64, 9, True, 5),             # 64-row clusters: two key scales per step
     ("sweep", 1100, 3000, 64, 128, 5, False, None),        # the paper's block shape, no compensation
-    ("sweep", 1024, 2100, 256, 256, 3, True, 6),           # two CTAs per query cluster, two tiles per key cluster
+    ("sweep", 1024, 2100, 256, 256, 3, True, 6),           # two tiles per query cluster, two steps per key cluster
 ])
 def test_attention_with_quantised_qk(name, n_q, n_k, c_q, c_k, keep, compensate, perm_seed):
     """CA_ATTN_FP8_QK: Q K^T on E4M3 codes with a scale per query row, per key cluster and per run
