@@ -9,29 +9,28 @@
 // the representation r(q) from its Gram matrix and column sums.
 //
 // Decomposition (d = 64, 128; float32: the bases only feed fp32 coordinates), in three parts.
-// 1. Householder reduction to tridiagonal form.  For k = 0 .. d-3 the reflector H_k = I - beta v v^T
-// annihilates A[k+2.., k]; the trailing block is updated as A - v w^T - w v^T with p = beta A v,
-// w = p - (beta/2)(v.p) v.  A step is a chain of latencies (two barriers, shuffles, a root), so
-// what counts is how short the chain is and how few instructions stand in it: a few threads per
-// row keep the matrix in registers, the owners of the next row only publish it, and every thread
-// derives the reflector from it for itself; rows and columns that are done drop out.  The
-// reflectors are stored, not accumulated.
+// 1. Householder reduction to tridiagonal form.  For k = 0 .. d-3 the reflector H = I - beta v v^T of row k,
+// v = x - alpha e_{k+1}, x the row right of the diagonal, takes A to H A H.  A step is a chain of latencies
+// (barrier, shuffles, root), so what counts is how short the chain is and how few instructions stand in it.  With
+// y = A x, row k + 1 of H A H right of its diagonal is H y / alpha: every thread forms the next x for itself from the
+// published y, one barrier per step and two sums over the threads of a row, and the update of A (A - v p^T - u v^T
+// with p = beta A v = beta (y - alpha A e_{k+1}), u = p - beta (v.p) v) is off the chain.  (Before: two barriers
+// and three sums, the next row published behind the update; 58 k and 184 k cycles for d = 64 / 128, now 47 k and
+// 160 k by itself.)  The warps that the reduction does not use apply the reflectors, a block behind, to the
+// rows of the factor F (another 3 k and 25 k cycles of the reduction's time, against 12 k and 52 k for applying them to the
+// eigenvectors of the tridiagonal matrix at the end, by all warps).
 // 2. Divide and conquer.  The tridiagonal matrix is cut into blocks of kBase rows (a cut writes
-// T = diag(T1, T2) + rho u u^T), each diagonalised by one warp with the implicit-shift QL iteration
-// (the rotation chase is one dependent chain on lane 0, the lanes apply its rotations to the columns
-// that they keep in registers), then merged pairwise up to the whole.  A merge solves
+// T = diag(T1, T2) + rho u u^T), each diagonalised by one lane with Jacobi rotations, then merged pairwise up to
+// the whole.  A merge solves
 // diag(d) + rho z z^T, z the eigenvectors' components at the cut: poles sorted, negligible weights and
 // coinciding poles deflated, the roots of the secular equation by an iteration that treats the
 // nearest pole exactly (a few threads per root; offsets from that pole keep the differences
 // d_j - x accurate), the weights recomputed from the roots (Gu and Eisenstat, 1994) so that the
-// eigenvectors stay orthogonal to rounding, and one product with the blocks' eigenvectors.
-// 3. The stored reflectors are applied to the eigenvectors of T, a few threads per vector, without a barrier.
-// Two launches (keys, queries) one after the other: 8 heads, d = 64 0.27 ms and 40 heads, d = 128 0.86 ms
-// with the transform accumulated during the reduction (eight threads per row, the next reflector
-// built by one warp, branches around finished chunks), quarters as base blocks and bisected roots;
-// now 0.185 and 0.53 ms.  SM cycles of a launch (d = 64 / d = 128): covariance 8-25 k / 12-80 k,
-// reduction 58 k / 180 k (62 / 126 steps), base blocks 8 k / 15 k, merges 56-65 k / 120-135 k, reflectors
-// 13 k / 55 k, map and output 9 k / 45 k.
+// eigenvectors stay orthogonal to rounding, and one product with the blocks' eigenvectors, which leaves out their zeros.
+// 3. W = (F Q) S, Q the product of the reflectors and S the eigenvectors of T.
+// SM cycles of a launch (12 heads, d = 64 / 40 heads, d = 128; queries): covariance 2.5 k / 11 k (keys 11 k / 60 k),
+// reduction 51 k / 187 k, base blocks 5 k / 10 k, merges 50 k / 103 k, map 4.5 k / 26 k, output 4.5 k / 11 k;
+// in all 120 k / 352 k, where it took 152 k / 437 k.
 //
 // Epilogue.  Components in order of descending eigenvalue.  With E the
 // eigenvectors and F the factor that produced the transformed rows, the map from
@@ -46,181 +45,173 @@
 #include <type_traits>
 
 #include "kernels.h"
+#include "tc_ptx.cuh"
 
 namespace ca {
 
+using namespace ptx;
+
 namespace {
+
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
+  return lo + hi;
+}
 
 __device__ __forceinline__ void named_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
+__device__ __forceinline__ void named_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
 
 constexpr int kThreads = 512;
 constexpr int kBaseLog = 2, kBase = 1 << kBaseLog;   // rows of a base block of the divide and conquer
-constexpr int kMaxQlIterations = 64;
+constexpr int kMaxSweeps = 12;
 
 // Eigenvalues that are not numbers (the covariance of rows with infinities, or whose sums overflow) stand as +inf: the
 // rank of a pole among the others is then a permutation for every input, and indexes stay in range.
 __device__ __forceinline__ float pole_value(float x) { return fminf(x, INFINITY); }
 
-// ---- implicit-shift QL on rows [l0, l0 + kBase) of a tridiagonal matrix (de[i] = (diagonal i, coupling of
-// i and i + 1); the coupling behind the last row is not part of the block), by one warp: the search
-// for a negligible sub-diagonal entry uses all lanes, the rotation chase is one dependent chain on
-// lane 0, and lane t applies the rotations of a chase (rt, in shared memory) to column t of the
-// block's eigenvectors, which start as the identity and end as rows of Qt.
-__device__ __forceinline__ void ql_block(float2* de, int l0, float2* rt, float* Qt, int lda, int lane) {
-  const float eps = 6e-8f;
-  const int l1 = l0 + kBase;
-  float z[kBase];
+// ---- eigen-decomposition of the 4 x 4 blocks on the diagonal of a tridiagonal matrix (de[i] = (diagonal i, coupling of
+// i and i + 1); the coupling behind a block's last row is not part of it), a block per lane of one warp:
+// cyclic Jacobi rotations in registers, two disjoint ones at a time.  Four sweeps or so of three rounds, against one
+// dependent chain of rotations per eigenvalue with the implicit-shift QL iteration (a warp per block): 2.5 k
+// cycles where that took 8-9 k at d = 64 and 14-15 k at d = 128.  Eigenvectors become rows of Qt.
+__device__ __forceinline__ void jacobi_blocks(float2* de, int blocks, float* Qt, int lda, int lane) {
+  static_assert(kBase == 4, "rounds of a 4 x 4 matrix");
+  const bool mine = lane < blocks;
+  float m[4][4], v[4][4];
 #pragma unroll
-  for (int i = 0; i < kBase; ++i) z[i] = i == lane ? 1.f : 0.f;
-#pragma unroll 1
-  for (int l = l0; l < l1; ++l) {
-#pragma unroll 1
-    for (int iter = 0; iter < kMaxQlIterations; ++iter) {
-      // first m >= l whose sub-diagonal entry is negligible (m = l1 - 1 if none)
-      const int idx = l + lane;
-      bool small = false;
-      if (idx < l1 - 1) {
-        const float2 a = de[idx];
-        small = fabsf(a.y) <= eps * (fabsf(a.x) + fabsf(de[idx + 1].x));
-      }
-      const unsigned bal = __ballot_sync(0xffffffffu, small);
-      const int m = bal ? l + __ffs(bal) - 1 : l1 - 1;
-      if (m == l) break;
-      int lo = l;
-      if (lane == 0) {
-        const float2 top = de[l];
-        // the shift only steers the convergence (the rotations are formed from the matrix itself), so
-        // approximate division and root are enough for it
-        float g = __fdividef(de[l + 1].x - top.x, 2.f * top.y);
-        float rr;
-        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rr) : "f"(fmaf(g, g, 1.f)));
-        g = de[m].x - top.x + __fdividef(top.y, g + (g >= 0.f ? rr : -rr));
-        float s = 1.f, c = 1.f, p = 0.f;
-        bool under = false;
-        int i = m - 1;
-        float2 cur = de[i];              // (d_i, e_i)
-        float d_i1 = de[i + 1].x;
-#pragma unroll 1
-        for (; i >= l; --i) {
-          // operands of the next rotation, fetched ahead of the dependent chain
-          const float2 nxt = de[i > l ? i - 1 : l];
-          const float f = s * cur.y, bb = c * cur.y;
-          const float r2 = fmaf(f, f, g * g);
-          float rinv;
-          asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rinv) : "f"(r2));
-          const float p_old = p, d_old = d_i1;
-          s = f * rinv;
-          c = g * rinv;
-          g = d_i1 - p;
-          rr = fmaf(c, bb + bb, (cur.x - g) * s);
-          p = s * rr;
-          de[i + 1] = make_float2(g + p, r2 * rinv);       // new d_{i+1}; e_{i+1} = hypot(f, g)
-          g = fmaf(c, rr, -bb);
-          rt[i - l0] = make_float2(c, s);
-          // The chase has died out (f = g = 0): deflate here.  Tested after the rotation has been
-          // formed so that the test is off the dependent chain; its results are discarded.
-          if (r2 < 1e-36f) {
-            de[i + 1] = make_float2(d_old - p_old, 0.f);
-            de[m].y = 0.f;
-            under = true;
-            break;
-          }
-          d_i1 = cur.x;          // d_i is the next step's d_{i+1}; it has not been modified yet
-          cur = nxt;
-        }
-        if (!under) {
-          de[l] = make_float2(top.x - p, g);
-          de[m].y = 0.f;
-        } else {
-          lo = i + 1;
-        }
-      }
-      lo = __shfl_sync(0xffffffffu, lo, 0);
-      __syncwarp();
+  for (int i = 0; i < 4; ++i) {
+    const float2 d = mine ? de[4 * lane + i] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int i = kBase - 2; i >= 0; --i) {
-        // (no branch: a rotation outside the chase is the identity)
-        const bool in = l0 + i < m && l0 + i >= lo;
-        const float2 cs = rt[i];
-        const float c = in ? cs.x : 1.f, sn = in ? cs.y : 0.f;
-        const float zi = z[i], zn = z[i + 1];
-        z[i + 1] = fmaf(sn, zi, c * zn);
-        z[i] = fmaf(c, zi, -sn * zn);
-      }
-      __syncwarp();
-    }
+    for (int j = 0; j < 4; ++j) v[i][j] = i == j ? 1.f : 0.f;
+#pragma unroll
+    for (int j = i + 1; j < 4; ++j) m[i][j] = m[j][i] = j == i + 1 ? d.y : 0.f;
+    m[i][i] = d.x;
   }
-  if (lane < kBase) {
-    de[l0 + lane].x = pole_value(de[l0 + lane].x);
+  // zero to rounding: of the two diagonal entries, or of the whole matrix, whose largest diagonal entry is 1
+  auto negligible = [&](int p, int q) { return !(fabsf(m[p][q]) > fmaxf(1e-8f * (fabsf(m[p][p]) + fabsf(m[q][q])), 1e-15f)); };
+  auto rotate = [&](int p, int q) {
+    const float x = m[p][q], d = m[q][q] - m[p][p];
+    float root, inv;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"(fmaf(d, d, 4.f * x * x)));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(fabsf(d) + root));
+    const float t = negligible(p, q) ? 0.f : copysignf(2.f * inv, d) * x;          // tangent of the angle
+    const float n = fmaf(t, t, 1.f);
+    float c;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(n));
+    c = c * fmaf(-0.5f * n, c * c, 1.5f);
+    const float sn = t * c;
+    m[p][p] = fmaf(-t, x, m[p][p]);
+    m[q][q] = fmaf(t, x, m[q][q]);
+    m[p][q] = m[q][p] = t == 0.f ? x : 0.f;
 #pragma unroll
-    for (int i = 0; i < kBase; ++i) Qt[(l0 + i) * lda + l0 + lane] = z[i];
+    for (int k = 0; k < 4; ++k) {
+      if (k != p && k != q) {
+        const float a = m[k][p], b = m[k][q];
+        m[k][p] = m[p][k] = fmaf(c, a, -sn * b);
+        m[k][q] = m[q][k] = fmaf(sn, a, c * b);
+      }
+      const float a = v[k][p], b = v[k][q];
+      v[k][p] = fmaf(c, a, -sn * b);
+      v[k][q] = fmaf(sn, a, c * b);
+    }
+  };
+#pragma unroll 1
+  for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+    const bool done = negligible(0, 1) && negligible(0, 2) && negligible(0, 3) && negligible(1, 2) && negligible(1, 3) && negligible(2, 3);
+    if (__all_sync(0xffffffffu, done)) break;
+    rotate(0, 1); rotate(2, 3);
+    rotate(0, 2); rotate(1, 3);
+    rotate(0, 3); rotate(1, 2);
+  }
+  if (mine) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      de[4 * lane + i].x = pole_value(m[i][i]);
+      *reinterpret_cast<float4*>(&Qt[(4 * lane + i) * lda + 4 * lane]) = make_float4(v[0][i], v[1][i], v[2][i], v[3][i]);
+    }
   }
 }
 
 }  // namespace
 
-// d x d x d products in shared memory, a 4 x 4 tile of the result per thread (the first d^2 / 16
-// threads; every shared-memory load feeds four or sixteen multiply-adds, and the lanes of a
-// quarter-warp read distinct banks).  Terms are added for k = 0, 1, ... in that order.
-//   XT = false: acc[a][b] = sum_k X[(4 ti + a) lda + k] Y[k lda + 4 tj + b]
-//   XT = true:  acc[a][b] = sum_k X[k lda + 4 ti + a]   Y[k lda + 4 tj + b]
+// d x d x d products in shared memory, a tile of 8 x TJ of the result per thread (128 threads of 8 x 4 at d = 64, 256 of
+// 8 x 8 at d = 128): a 16-byte load costs four cycles of shared memory whether its lanes read one address or eight, so
+// that what counts is how many multiply-adds it feeds.  With 4 x 4 tiles the products took 4.1 k (d = 64) and
+// 26-30 k cycles, all of it shared memory.  The lanes of a quarter-warp read distinct banks.
+template <int D>
+struct Tile {
+  static constexpr int TI = 8, TJ = D == 64 ? 4 : 8, NUMBER = D * D / (TI * TJ), COLS = D / TJ;
+  static_assert(NUMBER <= kThreads, "a tile per thread");
+  int i, j;                                            // rows 8 i .., columns 4 j + (D / 2) c .. or j + COLS c
+  bool live;
+  __device__ __forceinline__ explicit Tile(int tid) : i(tid / COLS), j(tid % COLS), live(tid < NUMBER) {}
+};
+
+// Terms are added for k = 0, 1, ... in that order; column b of a tile is 4 tj + b (b < 4) or d / 2 + 4 tj + b - 4.
+//   XT = false: acc[a][b] = sum_k X[(8 ti + a) lda + k] Y[k lda + column b]
+//   XT = true:  acc[a][b] = sum_k X[k lda + 8 ti + a]   Y[k lda + column b]
 template <int D, bool XT>
-__device__ __forceinline__ void tile_product(const float* __restrict__ X, const float* __restrict__ Y, int lda,
-                                             int ti, int tj, float (&acc)[4][4]) {
+__device__ __forceinline__ void tile_product(const float* __restrict__ X, const float* __restrict__ Y, int lda, const Tile<D>& t,
+                                             float (&acc)[Tile<D>::TI][Tile<D>::TJ]) {
+  constexpr int TI = Tile<D>::TI, TJ = Tile<D>::TJ;
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < TI; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-#pragma unroll 2
+    for (int y = 0; y < TJ; ++y) acc[x][y] = 0.f;
+#pragma unroll 1
   for (int k0 = 0; k0 < D; k0 += 4) {
-    float xa[4][4];                                    // [row][k]
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
+      float y[TJ], x[TI];
+#pragma unroll
+      for (int c = 0; c < TJ; c += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&Y[(k0 + e) * lda + 4 * t.j + (D / 8) * c]);
+        y[c] = v.x; y[c + 1] = v.y; y[c + 2] = v.z; y[c + 3] = v.w;
+      }
       if (XT) {
-        const float4 v = *reinterpret_cast<const float4*>(&X[(k0 + e) * lda + 4 * ti]);
-        xa[0][e] = v.x; xa[1][e] = v.y; xa[2][e] = v.z; xa[3][e] = v.w;
+#pragma unroll
+        for (int r = 0; r < TI; r += 4) {
+          const float4 v = *reinterpret_cast<const float4*>(&X[(k0 + e) * lda + TI * t.i + r]);
+          x[r] = v.x; x[r + 1] = v.y; x[r + 2] = v.z; x[r + 3] = v.w;
+        }
       } else {
-        const float4 v = *reinterpret_cast<const float4*>(&X[(4 * ti + e) * lda + k0]);
-        xa[e][0] = v.x; xa[e][1] = v.y; xa[e][2] = v.z; xa[e][3] = v.w;
-      }
-    }
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const float4 y = *reinterpret_cast<const float4*>(&Y[(k0 + kk) * lda + 4 * tj]);
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        acc[x][0] = fmaf(xa[x][kk], y.x, acc[x][0]); acc[x][1] = fmaf(xa[x][kk], y.y, acc[x][1]);
-        acc[x][2] = fmaf(xa[x][kk], y.z, acc[x][2]); acc[x][3] = fmaf(xa[x][kk], y.w, acc[x][3]);
+        for (int r = 0; r < TI; ++r) x[r] = X[(TI * t.i + r) * lda + k0 + e];
       }
+#pragma unroll
+      for (int r = 0; r < TI; ++r)
+#pragma unroll
+        for (int c = 0; c < TJ; ++c) acc[r][c] = fmaf(x[r], y[c], acc[r][c]);
     }
   }
 }
 
-// acc[a][c] = sum_k X[(4 ti + a) lda + k] Yr[(tj + (D / 4) c) lda + k]   (both operands by rows)
+// acc[a][c] = sum_k X[(8 ti + a) lda + k] Yr[(tj + COLS c) lda + k]   (both operands by rows, terms in order)
 template <int D>
-__device__ __forceinline__ void tile_product_rows(const float* __restrict__ X, const float* __restrict__ Yr, int lda,
-                                                  int ti, int tj, float (&acc)[4][4]) {
+__device__ __forceinline__ void tile_product_rows(const float* __restrict__ X, const float* __restrict__ Yr, int lda, const Tile<D>& t,
+                                                  float (&acc)[Tile<D>::TI][Tile<D>::TJ]) {
+  constexpr int TI = Tile<D>::TI, TJ = Tile<D>::TJ;
 #pragma unroll
-  for (int x = 0; x < 4; ++x)
+  for (int x = 0; x < TI; ++x)
 #pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-#pragma unroll 2
+    for (int y = 0; y < TJ; ++y) acc[x][y] = 0.f;
+#pragma unroll 1
   for (int k0 = 0; k0 < D; k0 += 4) {
-    float4 xv[4], yv[4];
+    float4 y[TJ];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      xv[e] = *reinterpret_cast<const float4*>(&X[(4 * ti + e) * lda + k0]);
-      yv[e] = *reinterpret_cast<const float4*>(&Yr[(tj + (D / 4) * e) * lda + k0]);
+    for (int c = 0; c < TJ; ++c) y[c] = *reinterpret_cast<const float4*>(&Yr[(t.j + Tile<D>::COLS * c) * lda + k0]);
+#pragma unroll
+    for (int r = 0; r < TI; ++r) {
+      const float4 v = *reinterpret_cast<const float4*>(&X[(TI * t.i + r) * lda + k0]);
+#pragma unroll
+      for (int c = 0; c < TJ; ++c)
+        acc[r][c] = fmaf(v.w, y[c].w, fmaf(v.z, y[c].z, fmaf(v.y, y[c].y, fmaf(v.x, y[c].x, acc[r][c]))));
     }
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-      for (int y = 0; y < 4; ++y) {
-        acc[x][y] = fmaf(xv[x].x, yv[y].x, acc[x][y]); acc[x][y] = fmaf(xv[x].y, yv[y].y, acc[x][y]);
-        acc[x][y] = fmaf(xv[x].z, yv[y].z, acc[x][y]); acc[x][y] = fmaf(xv[x].w, yv[y].w, acc[x][y]);
-      }
   }
 }
 
@@ -258,31 +249,43 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
   int* gb = ga + D;
   int* defl_row = gb + D;                                  // deflated: row of Qt, eigenvalue
   float* defl_d = reinterpret_cast<float*>(defl_row + D);
-  float* kz2 = defl_d + D;                                 // squared weights of the kept poles
-  int* counts = reinterpret_cast<int*>(scratch + 16 * D) + 8 * grp;   // kept, rotations, deflated, skip
-  float* z2sum = reinterpret_cast<float*>(counts + 4);
+  int* counts = reinterpret_cast<int*>(scratch + 15 * D) + 8 * grp;   // kept, rotations, deflated, skip, left, right
+  // The rows of the two blocks are zero in the other block's columns (but for those that a rotation has mixed): the
+  // columns of the left half take the terms of one list of kept poles, those of the right half of another, which
+  // grows downwards from position NB + 3, each filled up to a multiple of four.  (A rotation takes a pole away for every
+  // row that it mixes, so that both fit.)
+  int* place = reinterpret_cast<int*>(scratch + 16 * D) + b0;         // kept pole -> positions in the lists (16 bits each, 0xffff: none)
+  int* at_row = reinterpret_cast<int*>(scratch + 17 * D) + b0 + 4 * grp;   // position -> row of Qt
+  float2* pole = reinterpret_cast<float2*>(scratch + 19 * D) + b0;    // kept pole, squared weight
+  int* side = reinterpret_cast<int*>(kzh);                            // kept pole -> halves of its row that are not zero
   const float rho2 = 2.f * rho;
-  if (lt < NB) {
-    const float mine = de[b0 + lt].x;
+  {
+    // rank of a pole among the others, T threads to a pole
+    const int i = lt / T;
+    const float mine = de[b0 + i].x;
+    const int cut = b0 + NB / 2;
+    const float z = i < NB / 2 ? Qt[(b0 + i) * LDA + cut - 1] : theta * Qt[(b0 + i) * LDA + cut];
     int rank = 0;
 #pragma unroll 4
-    for (int k = 0; k < NB; ++k) {
+    for (int k = lt % T; k < NB; k += T) {
       const float other = de[b0 + k].x;
-      rank += (other < mine) || (other == mine && k < lt);
+      rank += (other < mine) || (other == mine && k < i);
     }
-    const int cut = b0 + NB / 2;
-    ord[rank] = b0 + lt;
-    ds[rank] = mine;
-    zs[rank] = 0.70710678f * (lt < NB / 2 ? Qt[(b0 + lt) * LDA + cut - 1] : theta * Qt[(b0 + lt) * LDA + cut]);
+#pragma unroll
+    for (int o = 1; o < T; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+    if (lt % T == 0) {
+      ord[rank] = b0 + i;
+      ds[rank] = mine;
+      zs[rank] = 0.70710678f * z;
+    }
   }
   sync();
   if (lt < 32) {
     float dmax = 0.f, zmax = 0.f;
     for (int j = lane; j < NB; j += 32) { dmax = fmaxf(dmax, fabsf(ds[j])); zmax = fmaxf(zmax, fabsf(zs[j])); }
-    for (int o = 16; o > 0; o >>= 1) {
-      dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-    }
+    // (the bits of floats that are not negative are in their order)
+    dmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dmax)));
+    zmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(zmax)));
     const float tol = 8.f * 6e-8f * fmaxf(dmax, zmax);
     const bool skip = !(rho2 * zmax > tol);                // the blocks do not couple, or not by a number: nothing to merge
     int K = 0, ng = 0, nd = 0;
@@ -299,6 +302,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
         if (keep) {
           const int at = K + __popc(mk & below);
           keep_row[at] = ord[j]; kd[at] = dj; kz[at] = zj;
+          side[at] = ord[j] < b0 + NB / 2 ? 1 : 2;
         } else if (in) {
           const int at = nd + __popc(md & below);
           defl_row[at] = ord[j]; defl_d[at] = dj;
@@ -334,18 +338,31 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
               int j = 32 * c + __ffs(m) - 1;
               m &= m - 1;
               // (a pair already taken in, or parted by the rotation before, fails the test)
+              float dp = kd[j - 1], zp = kz[j - 1];
+              int rp = keep_row[j - 1], both = side[j - 1];
+              float dj = kd[j], zj = kz[j];
 #pragma unroll 1
-              for (; j < K && coincide(j); ++j) {
-                const float d_prev = kd[j - 1], dj = kd[j];
-                float sn = kz[j - 1], cs = kz[j];
-                const float tau = sqrtf(fmaf(cs, cs, sn * sn));
-                cs = __fdividef(cs, tau);
-                sn = -__fdividef(sn, tau);
-                gc[ng] = cs; gs[ng] = sn; ga[ng] = keep_row[j - 1]; gb[ng] = keep_row[j]; ++ng;
-                kd[j] = d_prev * sn * sn + dj * cs * cs;
-                kz[j] = tau;
-                defl_row[nd] = keep_row[j - 1]; defl_d[nd] = d_prev * cs * cs + dj * sn * sn; ++nd;
+              for (; j < K; ++j) {
+                const float n2 = fmaf(zj, zj, zp * zp);
+                if (zp == 0.f || !(fabsf((dj - dp) * zj * zp) <= tol * n2)) break;
+                float r;
+                asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(n2));
+                r = r * fmaf(-0.5f * n2 * r, r, 1.5f);
+                const int rj = keep_row[j];
+                both |= side[j];
+                side[j] = both;
+                const float d_next = kd[j + 1], z_next = kz[j + 1];   // (within scratch; not used behind the last pole)
+                const float cs = zj * r, sn = -zp * r, cc = cs * cs, ss = sn * sn;
+                gc[ng] = cs; gs[ng] = sn; ga[ng] = rp; gb[ng] = rj; ++ng;
+                defl_row[nd] = rp; defl_d[nd] = fmaf(dj, ss, dp * cc); ++nd;
                 kz[j - 1] = 0.f;                           // mark of a pole that has given way
+                dp = fmaf(dj, cc, dp * ss);
+                zp = n2 * r;
+                rp = rj;
+                kd[j] = dp;
+                kz[j] = zp;
+                dj = d_next;
+                zj = z_next;
               }
             }
           }
@@ -356,11 +373,11 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
         for (int base = 0; base < K; base += 32) {
           const int j = base + lane;
           const float dj = j < K ? kd[j] : 0.f, zj = j < K ? kz[j] : 0.f;
-          const int rj = j < K ? keep_row[j] : 0;
+          const int rj = j < K ? keep_row[j] : 0, sj = j < K ? side[j] : 0;
           const unsigned mk = __ballot_sync(0xffffffffu, zj != 0.f);
           if (zj != 0.f) {
             const int at = kept + __popc(mk & ((1u << lane) - 1u));
-            keep_row[at] = rj; kd[at] = dj; kz[at] = zj;
+            keep_row[at] = rj; kd[at] = dj; kz[at] = zj; side[at] = sj;
           }
           kept += __popc(mk);
           __syncwarp();
@@ -369,15 +386,30 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
         ng = __shfl_sync(0xffffffffu, ng, 0);
         nd = __shfl_sync(0xffffffffu, nd, 0);
       }
-      // squared weights of the kept poles and their sum (the last root's bracket)
-      float z2 = 0.f;
-      for (int j = lane; j < NB; j += 32) {
-        const float w = j < K ? kz[j] * kz[j] : 0.f;
-        kz2[j] = w;
-        z2 += w;
+      // squared weights of the kept poles; the two lists
+      int nl = 0, nr = 0;
+      const unsigned below = (1u << lane) - 1u;
+#pragma unroll 1
+      for (int base = 0; base < K; base += 32) {
+        const int j = base + lane;
+        const int sj = j < K ? side[j] : 0;
+        const unsigned ml = __ballot_sync(0xffffffffu, sj & 1), mr = __ballot_sync(0xffffffffu, sj & 2);
+        const int at = nl + __popc(ml & below), at_r = NB + 3 - nr - __popc(mr & below);
+        if (j < K) {
+          const float zj = kz[j];
+          const int row = keep_row[j];
+          pole[j] = make_float2(kd[j], zj * zj);
+          place[j] = (sj & 1 ? at : 0xffff) | (sj & 2 ? at_r : 0xffff) << 16;
+          if (sj & 1) at_row[at] = row;
+          if (sj & 2) at_row[at_r] = row;
+        }
+        nl += __popc(ml);
+        nr += __popc(mr);
       }
-      for (int o = 16; o > 0; o >>= 1) z2 += __shfl_xor_sync(0xffffffffu, z2, o);
-      if (lane == 0) *z2sum = z2;
+      // (any row where a list is filled up: its factor is zero)
+      if (lane < (-nl & 3)) at_row[nl + lane] = b0;
+      if (lane < (-nr & 3)) at_row[NB + 3 - nr - lane] = b0;
+      if (lane == 0) { counts[4] = (nl + 3) & ~3; counts[5] = (nr + 3) & ~3; }
     }
     if (lane == 0) { counts[0] = K; counts[1] = ng; counts[2] = nd; counts[3] = skip; }
   }
@@ -390,7 +422,7 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
     sync();
     return;
   }
-  const int K = counts[0], ng = counts[1], nd = counts[2];
+  const int K = counts[0], ng = counts[1], nd = counts[2], nl = counts[4], nr = counts[5];
   // rotations of the deflation on the rows of Qt (one column per thread, in the order recorded)
   if (ng > 0) {
     if (lt < NB) {
@@ -415,22 +447,23 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
   const bool live = gi < K;
   {
     const int i = live ? gi : 0;
-    // the last root lies in (d_{K-1}, d_{K-1} + rho2 |z|^2); every other one between two poles, and the
-    // sign of the function half-way says next to which
+    // the last root lies in (d_{K-1}, d_{K-1} + rho2 |z|^2), |z| = 1 to rounding; every other one between two
+    // poles, and the sign of the function half-way says next to which
     const bool last = i >= K - 1;
-    const float width = last ? rho2 * *z2sum : kd[i + 1] - kd[i];
+    const float width = last ? 1.0001f * rho2 : kd[i + 1] - kd[i];
     const float mid = 0.5f * width, d0 = kd[i];
     float acc = 0.f;
 #pragma unroll 4
     for (int j = sub; j < K; j += T) {
+      const float2 pj = pole[j];
       float inv;                                            // one special-function operation, no rounding fix-up
-      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"((kd[j] - d0) - mid));
-      acc = fmaf(kz2[j], inv, acc);
+      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"((pj.x - d0) - mid));
+      acc = fmaf(pj.y, inv, acc);
     }
     const float f_mid = fmaf(rho2, sum_t(acc), 1.f);
     const bool right = !last && f_mid < 0.f;
     const int org = right ? i + 1 : i;
-    const float w_org = rho2 * kz2[org], d_org = kd[org];
+    const float w_org = rho2 * pole[org].y, d_org = kd[org];
     // f(m) = 1 - w_org / m + r(m), r the sum over the other poles: smooth around the root, so it is
     // replaced by its tangent and the pole is kept as it is: the root of b m^2 + a m - w_org = 0 on the
     // origin's side.  Safeguarded by the bracket; a root that has not settled after kSteps is bisected.
@@ -443,9 +476,10 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
       float r0 = 0.f, r1 = 0.f;
 #pragma unroll 4
       for (int j = sub; j < K; j += T) {
+        const float2 pj = pole[j];
         float inv;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"((kd[j] - d_org) - m));
-        const float x = j == org ? 0.f : kz2[j] * inv;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"((pj.x - d_org) - m));
+        const float x = j == org ? 0.f : pj.y * inv;
         r0 += x;
         r1 = fmaf(x, inv, r1);
       }
@@ -456,13 +490,15 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
       const float ca = fmaf(-r1, m, 1.f + r0);
       float disc;
       asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(disc) : "f"(fmaf(ca, ca, 4.f * r1 * w_org)));
-      float next;
-      if (!right) next = ca >= 0.f ? __fdividef(2.f * w_org, ca + disc) : __fdividef(disc - ca, 2.f * r1);
-      else next = ca <= 0.f ? -__fdividef(2.f * w_org, disc - ca) : -__fdividef(ca + disc, 2.f * r1);
-      // settled: convergence is quadratic, so behind a step of 1e-5 nothing but rounding is left (and the
-      // sign of f, which moves the bracket, is rounding too: such a step may leave it)
-      bool still = fabsf(next - m) <= 1e-5f * fabsf(m);
-      if (!still && (it >= kSteps || !(next > lo_m && next < hi_m))) {
+      const float cs = right ? -ca : ca;                   // (one expression for both sides: no branches)
+      const float mag = __fdividef(cs >= 0.f ? 2.f * w_org : disc - cs, cs >= 0.f ? cs + disc : 2.f * r1);
+      float next = right ? -mag : mag;
+      // settled: convergence is quadratic, so behind a step of 1e-4 nothing but rounding is left.  The sign of f,
+      // which moves the bracket, is rounding too by then: a short step that leaves the bracket ends the search (bisecting a bracket
+      // whose other end is still far away starts it again: up to 58 rounds, 14 k cycles of a merge).
+      const bool inside = next > lo_m && next < hi_m;
+      bool still = fabsf(next - m) <= (inside ? 1e-4f : 1e-3f) * fabsf(m);
+      if (!still && (it >= kSteps || !inside)) {
         next = 0.5f * (lo_m + hi_m);
         still = next == lo_m || next == hi_m;
       }
@@ -497,27 +533,39 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
     for (int j = sub; j < K; j += T) {
       const float v = __fdividef(kzh[j], (kd[j] - d0) - mu);
       nrm = fmaf(v, v, nrm);
-      if (live) A[(b0 + gi) * LDA + j] = v;
     }
     const float inv = rsqrtf(sum_t(nrm));
-    if (live)
-      for (int j = sub; j < K; j += T) A[(b0 + gi) * LDA + j] *= inv;
+    if (live) {
+      float* row = A + (b0 + gi) * LDA;
+      if (sub < 4) {                                        // what fills the lists up
+        if (nl > sub) row[nl - 1 - sub] = 0.f;
+        if (nr > sub) row[NB + 4 - nr + sub] = 0.f;
+      }
+      __syncwarp(((1u << T) - 1u) << (lane & ~(T - 1)));
+#pragma unroll 2
+      for (int j = sub; j < K; j += T) {
+        const float v = inv * __fdividef(kzh[j], (kd[j] - d0) - mu);
+        const unsigned at = place[j];
+        if ((at & 0xffffu) != 0xffffu) row[at & 0xffffu] = v;
+        if ((at >> 16) != 0xffffu) row[at >> 16] = v;
+      }
+    }
   }
   sync();
-  // rows of the merged basis into L: row b0 + i = sum_j A[b0 + i][j] Qt[keep_row[j]] (i < K), then
+  // rows of the merged basis into L: row b0 + i = sum_j A[b0 + i][place of j] Qt[keep_row[j]] (i < K), then
   // the deflated rows (a 4 x 4 tile per thread, terms in the order of j)
 #pragma unroll 1
   for (int tile = lt; tile < NB * NB / 16; tile += GT) {
-    const int i0 = 4 * (tile >> (lg - 2)), c0 = b0 + 4 * (tile & (NB / 4 - 1));
+    const int i0 = 4 * (tile >> (lg - 2)), c = 4 * (tile & (NB / 4 - 1)), c0 = b0 + c;
     if (i0 >= K) break;
+    const int first = c < NB / 2 ? 0 : NB + 4 - nr, end = c < NB / 2 ? nl : NB + 4;
     float acc[4][4];
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-    int j = 0;
 #pragma unroll 1
-    for (; j + 4 <= K; j += 4) {
+    for (int j = first; j < end; j += 4) {
       float xa[4][4];
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
@@ -526,22 +574,12 @@ __device__ __noinline__ void merge_blocks(float* __restrict__ Qt, float* __restr
       }
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        const float4 y = *reinterpret_cast<const float4*>(&Qt[keep_row[j + kk] * LDA + c0]);
+        const float4 y = *reinterpret_cast<const float4*>(&Qt[at_row[j + kk] * LDA + c0]);
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
           acc[x][0] = fmaf(xa[x][kk], y.x, acc[x][0]); acc[x][1] = fmaf(xa[x][kk], y.y, acc[x][1]);
           acc[x][2] = fmaf(xa[x][kk], y.z, acc[x][2]); acc[x][3] = fmaf(xa[x][kk], y.w, acc[x][3]);
         }
-      }
-    }
-#pragma unroll 1
-    for (; j < K; ++j) {
-      const float4 y = *reinterpret_cast<const float4*>(&Qt[keep_row[j] * LDA + c0]);
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const float xv = A[(b0 + i0 + x) * LDA + j];
-        acc[x][0] = fmaf(xv, y.x, acc[x][0]); acc[x][1] = fmaf(xv, y.y, acc[x][1]);
-        acc[x][2] = fmaf(xv, y.z, acc[x][2]); acc[x][3] = fmaf(xv, y.w, acc[x][3]);
       }
     }
 #pragma unroll
@@ -564,18 +602,22 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
   float* A = reinterpret_cast<float*>(smem_raw);       // [D][LDA]
   float* Qt = A + D * LDA;                             // [D][LDA]   rows become the eigenvectors
   float* L = Qt + D * LDA;                             // [D][LDA]   the factor F (prologue, sign rule); merged bases and reflectors in between
-  float* xbuf = A + 3 * D * LDA;                       // [2][D]     the next row of the reduction
-  float* pbuf = xbuf + 2 * D;                          // [D]
-  float2* de = reinterpret_cast<float2*>(pbuf + D);    // [D]        (diagonal i, sub-diagonal coupling i and i+1)
-  float* beta = pbuf + 3 * D;                          // [D]        factors of the reflectors
-  float* rot = beta + D;                               // [2 D]      rotations of a chase, (c, s) per row
-  float* scratch = rot + 2 * D;                        // [18 D]     arrays of the merge
+  float* refl = A;                                     // rows: the reflectors as they come
+  float* ybuf = A + 3 * D * LDA;                       // [2][D]     A times the row to be reflected
+  float* abuf = ybuf + 2 * D;                          // [2][D]     the row after it
+  float2* de = reinterpret_cast<float2*>(abuf + 2 * D);   // [D]     (diagonal i, sub-diagonal coupling i and i+1)
+  float* beta = abuf + 4 * D;                          // [D]        factors of the reflectors
+  float* mean = beta + D;                              // [D]
+  float* scratch = mean + D;                           // [21 D]     arrays of the merge
+  // what is multiplied by the reduction's Q on the way: the factor F, or the identity where E itself is asked for
+  const bool need_e = !(a.lift && a.out_lifted);
   __shared__ double s_scale;
   __shared__ float s_rho[D / kBase], s_theta[D / kBase];   // cut before row i kBase
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t mat = (size_t)blockIdx.x * D * D;
-  constexpr int TILES = D * D / 16;                    // d x d x d products: 4 x 4 tiles
+  constexpr int TI = Tile<D>::TI, TJ = Tile<D>::TJ;
+  const Tile<D> tile(tid);
 
   // ---- prologue: the matrix to decompose, in A
   // (16-byte loads, several in flight: the launch starts with nothing else to do)
@@ -602,25 +644,23 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
       *reinterpret_cast<float2*>(&A[i * LDA + j]) = make_float2((float)fma(si, sm[j], g.x * cs), (float)fma(si, sm[j + 1], g.y * cs));
     }
     __syncthreads();
-    float acc[4][4];
-#pragma unroll 1
-    for (int tile = tid; tile < TILES; tile += NT) {
-      const int tile_i = tile / (D / 4), tile_j = tile % (D / 4);
-      tile_product<D, true>(L, A, LDA, tile_i, tile_j, acc);                              // F^T C
+    float acc[TI][TJ];
+    auto put_tile = [&](float* out, float f) {
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
-        *reinterpret_cast<float4*>(&Qt[(4 * tile_i + x) * LDA + 4 * tile_j]) = make_float4(acc[x][0], acc[x][1], acc[x][2], acc[x][3]);
+      for (int x = 0; x < TI; ++x)
+#pragma unroll
+        for (int c = 0; c < TJ; c += 4)
+          *reinterpret_cast<float4*>(&out[(TI * tile.i + x) * LDA + 4 * tile.j + (D / 8) * c]) =
+              make_float4(f * acc[x][c], f * acc[x][c + 1], f * acc[x][c + 2], f * acc[x][c + 3]);
+    };
+    if (tile.live) {
+      tile_product<D, true>(L, A, LDA, tile, acc);                                        // F^T C
+      put_tile(Qt, 1.f);
     }
     __syncthreads();
-    const float al = (float)a.alpha;
-#pragma unroll 1
-    for (int tile = tid; tile < TILES; tile += NT) {
-      const int tile_i = tile / (D / 4), tile_j = tile % (D / 4);
-      tile_product<D, false>(Qt, L, LDA, tile_i, tile_j, acc);                            // (F^T C) F
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-        *reinterpret_cast<float4*>(&A[(4 * tile_i + x) * LDA + 4 * tile_j]) =
-            make_float4(al * acc[x][0], al * acc[x][1], al * acc[x][2], al * acc[x][3]);
+    if (tile.live) {
+      tile_product<D, false>(Qt, L, LDA, tile, acc);                                      // (F^T C) F
+      put_tile(A, (float)a.alpha);
     }
   } else if (a.mode == kPcaQueries) {
     // covariance of the representation from its moments: gram / n - mean mean^T
@@ -646,173 +686,331 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (tid == 0) s_scale = mx > 0.f ? (double)mx : 1.0;
   }
-  // zero outside the blocks of the divide and conquer, in both buffers
-  for (int e = tid; e < D * LDA; e += NT) { Qt[e] = 0.f; L[e] = 0.f; }
   __syncthreads();
   const double a_scale = s_scale;
 
   // ---- 1. reduction to tridiagonal form
-  // A thread keeps RW rows by D / TR columns.  The vectors that a step reads back (v, then p) cost shared-memory
-  // bandwidth -- every thread reads its columns -- and every halving of the columns costs another
-  // shuffle in each of the three sums: one row by 32 columns at d = 64, two rows by 16 at d = 128.
-  constexpr int RW = D == 64 ? 1 : 2, TR = D == 64 ? 2 : 8;
+  // By the first warps: one per sub-core at d = 64, two at d = 128.  A thread keeps RW rows by D / TR columns of the
+  // matrix, and its columns of the row to be reflected.
+  constexpr int RW = D == 64 ? 2 : 4, TR = D == 64 ? 4 : 8;
   constexpr int CH = D / (4 * TR), CW = 4 * TR;        // float4 chunks of a row per thread; columns of a chunk
-  constexpr int SEG = CH / 4;                          // chunks per segment
-  if (tid < TR * D / RW) {
-    constexpr int kParties = TR * D / RW;
+  constexpr int kParties = TR * D / RW, kHelpers = NT - kParties;
+  // the other warps take the reflectors over in blocks, each behind a barrier of its own
+  constexpr int kBlock = D / 8, kBlockBar = 2, kHelperBar = 10;
+  static_assert(CH == 4 && kParties % 128 == 0, "division of the reduction");
+  if (tid < kParties) {
     const int r = RW * (tid / TR), q = tid % TR;       // first of this thread's rows
     const int warp_last = (32 * RW / TR) * (warp + 1) - 1;   // last row of this warp
-    float areg[RW][CH][4];
+    const bool publisher = warp == kParties / 32 - 1, publish = publisher && lane < TR;   // the last warp lives to the end
+    float v0_prev = 0.f;
+    f32x2 areg[RW][CH][2], x[CH][2];
+    float d_cur;
     {
       const float inv = (float)(1.0 / a_scale);
-#pragma unroll
-      for (int x = 0; x < RW; ++x)
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int j = 4 * (q + TR * t) + c;
-            areg[x][t][c] = 0.5f * (A[(r + x) * LDA + j] + A[j * LDA + r + x]) * inv;
-          }
-    }
-    if (r == 0) {
+      auto entry = [&](int i, int j) { return 0.5f * (A[i * LDA + j] + A[j * LDA + i]) * inv; };
 #pragma unroll
       for (int t = 0; t < CH; ++t)
-        *reinterpret_cast<float4*>(&xbuf[4 * (q + TR * t)]) = make_float4(areg[0][t][0], areg[0][t][1], areg[0][t][2], areg[0][t][3]);
-    }
-    auto sum_row = [](float x) {
 #pragma unroll
-      for (int o = 1; o < TR; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      return x;
+        for (int h = 0; h < 2; ++h) {
+          const int j = 4 * (q + TR * t) + 2 * h;
+#pragma unroll
+          for (int y = 0; y < RW; ++y) areg[y][t][h] = pack2(entry(r + y, j), entry(r + y, j + 1));
+          x[t][h] = pack2(j > 0 ? entry(0, j) : 0.f, entry(0, j + 1));
+        }
+      d_cur = entry(0, 0);
+    }
+    // row k of `refl` takes the reflector of step k
+    auto put_row = [&](float* row, const f32x2 (&val)[CH][2], int t0) {
+#pragma unroll
+      for (int t = 0; t < CH; ++t) {
+        ulonglong2 w = make_ulonglong2(0ull, 0ull);
+        if (t >= t0) w = make_ulonglong2(val[t][0], val[t][1]);
+        *reinterpret_cast<ulonglong2*>(&row[4 * (q + TR * t)]) = w;
+      }
     };
+    named_sync(1, kParties);                           // (the matrix has been read)
+    if (publish) put_row(refl, x, 0);
     // Columns below T0 chunks are done in a segment: its chunks are left out without a branch per chunk
     // (a taken branch costs some 20 cycles and keeps the loads of the chunks from overlapping).
     auto segment = [&](auto t0c) {
       constexpr int T0 = decltype(t0c)::value;
-      constexpr int k_first = T0 > 0 ? CW * T0 - 1 : 0, k_end = T0 + SEG < CH ? CW * (T0 + SEG) - 1 : D - 2;
+      constexpr int k_first = T0 > 0 ? CW * T0 - 1 : 0, k_end = T0 + 1 < CH ? CW * (T0 + 1) - 1 : D - 2;
 #pragma unroll 1
       for (int k = k_first; k < k_end; ++k) {
         const int m0 = k + 1;
-        const float* x = xbuf + (k & 1) * D;
-        named_sync(1, kParties);                       // row k has been published
-        if (warp_last < k) {                           // rows that are done: only the barriers
+        float* yk = ybuf + (k & 1) * D;
+        float* ak = abuf + (k & 1) * D;
+        if (warp_last < m0) {                          // rows that are done: only the barrier
           named_sync(1, kParties);
           continue;
         }
-        // reflector of row k, the same in every thread group
-        float v[CH][4];
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        const float x0 = x[m0], x_k = x[k];
-        float x_r[RW];
-#pragma unroll
-        for (int y = 0; y < RW; ++y) x_r[y] = x[r + y];
-#pragma unroll
-        for (int t = T0; t < CH; ++t) {
-          const float4 xx = *reinterpret_cast<const float4*>(&x[4 * (q + TR * t)]);
-          v[t][0] = xx.x; v[t][1] = xx.y; v[t][2] = xx.z; v[t][3] = xx.w;
-        }
-#pragma unroll
-        for (int t = T0; t < CH; ++t) {
-          if (t <= T0 + SEG) {                         // chunks that can hold column m0
-            const int j0 = 4 * (q + TR * t);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[t][c] = j0 + c >= m0 ? v[t][c] : 0.f;
-          }
-          s0 = fmaf(v[t][0], v[t][0], s0); s1 = fmaf(v[t][1], v[t][1], s1);
-          s2 = fmaf(v[t][2], v[t][2], s2); s3 = fmaf(v[t][3], v[t][3], s3);
-        }
-        const float sig = sum_row((s0 + s1) + (s2 + s3));
-        // already tridiagonal in this column otherwise (uniform: every group has added the same numbers);
-        // beta = 0 then makes the step do nothing
-        const bool reflect = sig - x0 * x0 > 1e-30f;
-        // approximate root and reciprocal (a unit in the last place or two): the reflector stays
-        // orthogonal to the same order as the float32 updates that apply it, and they are on the
-        // critical path of every one of the d - 2 steps
-        float rt, bn;
-        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rt) : "f"(sig));
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(bn) : "f"(fmaf(fabsf(x0), rt, sig)));
-        const float alpha = !reflect ? x0 : (x0 >= 0.f ? -rt : rt);
-        const float v0 = x0 - alpha;
-        bn = reflect ? bn : 0.f;
-#pragma unroll
-        for (int t = T0; t <= T0 + SEG && t < CH; ++t)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) v[t][c] = 4 * (q + TR * t) + c == m0 ? v0 : v[t][c];
-        float p[RW];
-#pragma unroll
-        for (int y = 0; y < RW; ++y) {
-          s0 = s1 = s2 = s3 = 0.f;
-#pragma unroll
-          for (int t = T0; t < CH; ++t) {
-            s0 = fmaf(areg[y][t][0], v[t][0], s0); s1 = fmaf(areg[y][t][1], v[t][1], s1);
-            s2 = fmaf(areg[y][t][2], v[t][2], s2); s3 = fmaf(areg[y][t][3], v[t][3], s3);
-          }
-          p[y] = (s0 + s1) + (s2 + s3);
-        }
-#pragma unroll
-        for (int y = 0; y < RW; ++y) p[y] = bn * sum_row(p[y]);
+        // y = A x and |x|^2 (x is zero before m0); row m0 of A goes to the others as it is
 #pragma unroll
         for (int y = 0; y < RW; ++y)
-          if (q == y) pbuf[r + y] = r + y >= m0 ? p[y] : 0.f;
-        // kept for part 3 in the space of the result
-        if (k - r >= 0 && k - r < RW) {
-          if (q == 0) { de[k] = make_float2(x_k, alpha); beta[k] = bn; }
+          if (r + y == m0) put_row(ak, areg[y], T0);
+        float y_r[RW], sig;
+        {
+          f32x2 s[RW + 1][2];
 #pragma unroll
-          for (int t = 0; t < CH; ++t)
-            *reinterpret_cast<float4*>(&a.W32[mat + (size_t)k * D + 4 * (q + TR * t)]) =
-                t < T0 ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(v[t][0], v[t][1], v[t][2], v[t][3]);
+          for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int y = 0; y < RW; ++y) s[y][h] = mul2(areg[y][T0][h], x[T0][h]);
+            s[RW][h] = mul2(x[T0][h], x[T0][h]);
+#pragma unroll
+            for (int t = T0 + 1; t < CH; ++t) {
+#pragma unroll
+              for (int y = 0; y < RW; ++y) s[y][h] = fma2(areg[y][t][h], x[t][h], s[y][h]);
+              s[RW][h] = fma2(x[t][h], x[t][h], s[RW][h]);
+            }
+          }
+#pragma unroll
+          for (int y = 0; y < RW; ++y) y_r[y] = sum2(add2(s[y][0], s[y][1]));
+          sig = sum2(add2(s[RW][0], s[RW][1]));
         }
+#pragma unroll
+        for (int o = 1; o < TR; o <<= 1) {
+#pragma unroll
+          for (int y = 0; y < RW; ++y) y_r[y] += __shfl_xor_sync(0xffffffffu, y_r[y], o);
+          sig += __shfl_xor_sync(0xffffffffu, sig, o);
+        }
+        float y_q = y_r[0];
+#pragma unroll
+        for (int y = 1; y < RW; ++y) y_q = q == y ? y_r[y] : y_q;
+        if (q < RW) yk[r + q] = y_q;
+        // approximate root and reciprocals (a unit in the last place or two): the reflector stays
+        // orthogonal to the same order as the float32 updates that apply it, and they are on the
+        // critical path of every one of the d - 2 steps
+        float rt, irt;
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rt) : "f"(sig));
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(irt) : "f"(sig));
         named_sync(1, kParties);
-        float p_r[RW];
+        f32x2 p[CH][2];                                // first y
+        float s1;
+        {
+          f32x2 s[2];
 #pragma unroll
-        for (int y = 0; y < RW; ++y) p_r[y] = pbuf[r + y];
-        float pv[CH][4];
+          for (int t = T0; t < CH; ++t) {
+            // (columns before m0 may hold an older y: x is zero there, and the entries it changes are not used again)
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&yk[4 * (q + TR * t)]);
+            p[t][0] = w.x; p[t][1] = w.y;
+          }
 #pragma unroll
-        for (int t = T0; t < CH; ++t) {
-          // (columns below m0 may hold an older p: v is zero there, and the entries they change are not used again)
-          const float4 pp = *reinterpret_cast<const float4*>(&pbuf[4 * (q + TR * t)]);
-          pv[t][0] = pp.x; pv[t][1] = pp.y; pv[t][2] = pp.z; pv[t][3] = pp.w;
+          for (int h = 0; h < 2; ++h) {
+            s[h] = mul2(x[T0][h], p[T0][h]);
+#pragma unroll
+            for (int t = T0 + 1; t < CH; ++t) s[h] = fma2(x[t][h], p[t][h], s[h]);
+          }
+          s1 = sum2(add2(s[0], s[1]));
         }
-        s0 = s1 = s2 = s3 = 0.f;
+        const float* xk = refl + k * LDA;
+        const float x0 = xk[m0], y0 = yk[m0], a0 = ak[m0];
+        float x_own[RW], a_own[RW];
 #pragma unroll
-        for (int t = T0; t < CH; ++t) {
-          s0 = fmaf(v[t][0], pv[t][0], s0); s1 = fmaf(v[t][1], pv[t][1], s1);
-          s2 = fmaf(v[t][2], pv[t][2], s2); s3 = fmaf(v[t][3], pv[t][3], s3);
+        for (int y = 0; y < RW; y += 2) {
+          const float2 xo = *reinterpret_cast<const float2*>(&xk[r + y]), ao = *reinterpret_cast<const float2*>(&ak[r + y]);
+          x_own[y] = xo.x; x_own[y + 1] = xo.y;
+          a_own[y] = ao.x; a_own[y + 1] = ao.y;
         }
-        const float K = 0.5f * bn * sum_row((s0 + s1) + (s2 + s3));
 #pragma unroll
-        for (int y = 0; y < RW; ++y) {
-          // a -= v_r (p - K v) + (p_r - K v_r) v = v_r p + (p_r - 2 K v_r) v
-          const float v_r = r + y > m0 ? x_r[y] : (r + y == m0 ? v0 : 0.f);
-          const float u_r = r + y >= m0 ? fmaf(-2.f * K, v_r, p_r[y]) : 0.f;
-          const bool apply = reflect && r + y >= m0;
+        for (int o = 1; o < TR; o <<= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        // already tridiagonal in this column otherwise, to 1e-12 of the largest diagonal entry (uniform: every
+        // group has added the same numbers); beta = 0 then makes the step do nothing
+        const bool reflect = sig - x0 * x0 > 1e-24f;
+        float bn;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(bn) : "f"(fmaf(fabsf(x0), rt, sig)));
+        bn = reflect ? bn : 0.f;
+        const float alpha = !reflect ? x0 : (x0 >= 0.f ? -rt : rt);
+        const float i_alpha = x0 >= 0.f ? -irt : irt;
+        const float vy = fmaf(-alpha, y0, s1);                               // v . y, v = x - alpha e_m0
+        const float k2 = bn * (bn * fmaf(-alpha, fmaf(-alpha, a0, y0), vy));   // beta^2 v^T A v
+        if (publisher) {
+          // the first entry of a reflector is put in its place a step later, when no thread reads the row any more
+          if (lane == 0) {
+            de[k] = make_float2(d_cur, alpha);
+            beta[k] = bn;
+            if (k > 0) refl[(k - 1) * LDA + k] = v0_prev;
+          }
+          v0_prev = x0 - alpha;
+          if (k % kBlock == 0 && k > 0) { __syncwarp(); named_arrive(kBlockBar + k / kBlock - 1, 32 + kHelpers); }
+        }
+        d_cur = reflect ? s1 * i_alpha * i_alpha : a0;
+        // p = beta A v = beta (y - alpha A e_m0);  A - x_r p - (p_r - k2 x_r) x
+        const float ba = -bn * alpha;
+        if (reflect) {
+          const float g = -bn * vy * i_alpha;
+          // two rows at a time (registers)
+#pragma unroll
+          for (int y0 = 0; y0 < RW; y0 += 2) {
+            const f32x2 bn2 = pack2(bn, bn), ba2 = pack2(ba, ba);
+            f32x2 v2[2], u2[2];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+              const bool live = r + y0 + y > m0;
+              const float v_r = live ? -x_own[y0 + y] : 0.f;
+              const float u_r = live ? fmaf(k2, x_own[y0 + y], -fmaf(ba, a_own[y0 + y], bn * y_r[y0 + y])) : 0.f;
+              v2[y] = pack2(v_r, v_r);
+              u2[y] = pack2(u_r, u_r);
+            }
+#pragma unroll
+            for (int t = T0; t < CH; ++t) {
+              const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&ak[4 * (q + TR * t)]);
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const f32x2 pj = fma2(ba2, h == 0 ? w.x : w.y, mul2(bn2, p[t][h]));
+#pragma unroll
+                for (int y = 0; y < 2; ++y) areg[y0 + y][t][h] = fma2(u2[y], x[t][h], fma2(v2[y], pj, areg[y0 + y][t][h]));
+              }
+            }
+          }
+          const f32x2 g2 = pack2(g, g), ia2 = pack2(i_alpha, i_alpha);
 #pragma unroll
           for (int t = T0; t < CH; ++t)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const float next = fmaf(-v_r, pv[t][c], fmaf(-u_r, v[t][c], areg[y][t][c]));
-              areg[y][t][c] = apply ? next : areg[y][t][c];
-            }
-          if (r + y == m0) {
-            float* xn = xbuf + ((k + 1) & 1) * D;
+            for (int h = 0; h < 2; ++h) x[t][h] = fma2(g2, x[t][h], mul2(ia2, p[t][h]));
+        } else {
 #pragma unroll
-            for (int t = T0; t < CH; ++t)
-              *reinterpret_cast<float4*>(&xn[4 * (q + TR * t)]) = make_float4(areg[y][t][0], areg[y][t][1], areg[y][t][2], areg[y][t][3]);
+          for (int t = T0; t < CH; ++t) {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&ak[4 * (q + TR * t)]);
+            x[t][0] = w.x; x[t][1] = w.y;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                  // the chunk that holds column m0
+          const int j = 4 * (q + TR * T0) + 2 * h;
+          float lo, hi;
+          unpack2(x[T0][h], lo, hi);
+          x[T0][h] = pack2(j > m0 ? lo : 0.f, j + 1 > m0 ? hi : 0.f);
+        }
+        if (publish) put_row(refl + m0 * LDA, x, T0);
+      }
+    };
+    segment(std::integral_constant<int, 0>{});
+    segment(std::integral_constant<int, 1>{});
+    segment(std::integral_constant<int, 2>{});
+    segment(std::integral_constant<int, 3>{});
+    // the last 2 x 2 block
+    if (r + RW == D && q == TR - 1) {
+      float lo, hi, last;
+      unpack2(x[CH - 1][1], lo, hi);
+      unpack2(areg[RW - 1][CH - 1][1], lo, last);
+      de[D - 2] = make_float2(d_cur, hi);
+      de[D - 1] = make_float2(last, 0.f);
+    }
+    named_sync(1, kParties);
+    if (publisher) {
+      if (lane == 0) refl[(D - 3) * LDA + D - 2] = v0_prev;
+      __syncwarp();
+      named_arrive(kBlockBar + 7, 32 + kHelpers);
+    }
+  } else {
+    // The other warps apply the reflectors, a block behind, to the rows of the factor (or the identity), which come
+    // out as F Q, Q = H_0 H_1 ...: two rows per four threads (a row per thread group costs twice the
+    // shared-memory reads, which the reduction feels); one warp to the mean as well, D / 32 entries per lane.
+    constexpr int DC = D / 16;                         // float4 chunks of a row per thread
+    constexpr int kMeanWarp = NT / 32 - 1;
+    const int h = tid - kParties, row = 2 * (h / 4), q = h % 4;
+    const bool has_row = row < D;
+    f32x2 z[2][DC][2];
+    float m[D / 32];
+    if (has_row) {
+#pragma unroll
+      for (int y = 0; y < 2; ++y)
+#pragma unroll
+        for (int t = 0; t < DC; ++t) {
+          const int j = 4 * (q + 4 * t);
+          if (need_e) {
+            z[y][t][0] = pack2(j == row + y ? 1.f : 0.f, j + 1 == row + y ? 1.f : 0.f);
+            z[y][t][1] = pack2(j + 2 == row + y ? 1.f : 0.f, j + 3 == row + y ? 1.f : 0.f);
+          } else {
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&L[(row + y) * LDA + j]);
+            z[y][t][0] = w.x; z[y][t][1] = w.y;
+          }
+        }
+    }
+    if (warp == kMeanWarp) {
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c)
+        m[c] = a.mean_sum ? (float)(a.mean_sum[(size_t)blockIdx.x * D + lane * (D / 32) + c] / a.mean_n) : 0.f;
+    }
+    named_sync(kHelperBar, kHelpers);                  // the factor has been read
+    // zero outside the blocks of the divide and conquer, in both buffers
+    for (int e = 4 * h; e < D * LDA; e += 4 * kHelpers) {
+      *reinterpret_cast<float4*>(&Qt[e]) = make_float4(0.f, 0.f, 0.f, 0.f);
+      *reinterpret_cast<float4*>(&L[e]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    const bool lifted_mean = !need_e && a.mean_lifted;   // (otherwise the mean is multiplied by what comes out)
+    // reflectors k of two blocks, without an entry before chunk T0
+    auto blocks = [&](auto t0c, int b0) {
+      constexpr int T0 = decltype(t0c)::value;
+#pragma unroll 1
+      for (int b = b0; b < b0 + 2; ++b) {
+        named_sync(kBlockBar + b, 32 + kHelpers);
+        const int k_end = min(kBlock * (b + 1), D - 2);
+#pragma unroll 1
+        for (int k = kBlock * b; k < k_end; ++k) {
+          const float* vk = refl + k * LDA;
+          const float bk = -beta[k];
+          if (has_row) {
+            ulonglong2 v[DC];
+            f32x2 s[2][2];
+#pragma unroll
+            for (int t = T0; t < DC; ++t) v[t] = *reinterpret_cast<const ulonglong2*>(&vk[4 * (q + 4 * t)]);
+            float f[2];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+              s[y][0] = mul2(v[T0].x, z[y][T0][0]);
+              s[y][1] = mul2(v[T0].y, z[y][T0][1]);
+#pragma unroll
+              for (int t = T0 + 1; t < DC; ++t) {
+                s[y][0] = fma2(v[t].x, z[y][t][0], s[y][0]);
+                s[y][1] = fma2(v[t].y, z[y][t][1], s[y][1]);
+              }
+              f[y] = sum2(add2(s[y][0], s[y][1]));
+            }
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+              for (int y = 0; y < 2; ++y) f[y] += __shfl_xor_sync(0xffffffffu, f[y], o);
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+              const f32x2 f2 = pack2(f[y] * bk, f[y] * bk);
+#pragma unroll
+              for (int t = T0; t < DC; ++t) {
+                z[y][t][0] = fma2(v[t].x, f2, z[y][t][0]);
+                z[y][t][1] = fma2(v[t].y, f2, z[y][t][1]);
+              }
+            }
+          }
+          if (warp == kMeanWarp && lifted_mean) {
+            float v[D / 32], f = 0.f;
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+              v[c] = vk[lane * (D / 32) + c];
+              f = fmaf(v[c], m[c], f);
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+            f *= bk;
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) m[c] = fmaf(f, v[c], m[c]);
           }
         }
       }
     };
-    segment(std::integral_constant<int, 0>{});
-    segment(std::integral_constant<int, SEG>{});
-    segment(std::integral_constant<int, 2 * SEG>{});
-    segment(std::integral_constant<int, 3 * SEG>{});
-    // the last 2 x 2 block
-    if (q == TR - 1) {
+    blocks(std::integral_constant<int, 0>{}, 0);
+    blocks(std::integral_constant<int, DC / 4>{}, 2);
+    blocks(std::integral_constant<int, DC / 2>{}, 4);
+    blocks(std::integral_constant<int, 3 * DC / 4>{}, 6);
+    if (has_row) {
 #pragma unroll
-      for (int y = 0; y < RW; ++y) {
-        if (r + y == D - 2) de[D - 2] = make_float2(areg[y][CH - 1][2], areg[y][CH - 1][3]);
-        if (r + y == D - 1) de[D - 1] = make_float2(areg[y][CH - 1][3], 0.f);
-      }
+      for (int y = 0; y < 2; ++y)
+#pragma unroll
+        for (int t = 0; t < DC; ++t)                   // (no room in shared memory at d = 128)
+          *reinterpret_cast<ulonglong2*>(&a.W32[mat + (size_t)(row + y) * D + 4 * (q + 4 * t)]) = make_ulonglong2(z[y][t][0], z[y][t][1]);
+    }
+    if (warp == kMeanWarp) {
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c) mean[lane * (D / 32) + c] = m[c];
     }
   }
   __syncthreads();
@@ -829,8 +1027,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     de[k].x -= fabsf(bk);
   }
   __syncthreads();
-#pragma unroll 1
-  for (int w = warp; w < D / kBase; w += NT / 32) ql_block(de, w * kBase, reinterpret_cast<float2*>(rot) + w * kBase, Qt, LDA, lane);
+  if (warp == 0) jacobi_blocks(de, D / kBase, Qt, LDA, lane);
   __syncthreads();
   // merges of a level side by side, T threads per row
 #pragma unroll 1
@@ -841,117 +1038,42 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     float* swap = Qt; Qt = L; L = swap;
   }
 
-  // ---- 3. the reflectors, last one first, on the eigenvectors of T (rows of Qt)
-  for (int e = tid; e < (D - 2) * D / 4; e += NT)
-    *reinterpret_cast<float4*>(&L[(e / (D / 4)) * LDA + 4 * (e % (D / 4))]) = *reinterpret_cast<const float4*>(&a.W32[mat + 4 * (size_t)e]);
+  // ---- 3. the map from the original space, W = F E = (F Q) S, into A, S the eigenvectors of T (rows of Qt); where E is
+  // asked for, E = Q S first, its columns as rows of Qt, and then F E for the sign rule
+  for (int e = tid; e < D * D / 4; e += NT)
+    *reinterpret_cast<float4*>(&L[(4 * e / D) * LDA + 4 * e % D]) = *reinterpret_cast<const float4*>(&a.W32[mat + 4 * (size_t)e]);
   __syncthreads();
-  {
-    // Two reflectors at a time: H_a (H_b z) needs v_a . z and v_b . z only, once v_a . v_b is known.
-    constexpr int T = 8, CB = D / (4 * T);             // threads per two vectors (r, r + d / 2), float4 chunks per thread
-    float* cross = pbuf;                               // [k] = v_k . v_{k+1}
-    {
-      constexpr int TP = NT / (D / 2);
-      const int k = 2 * (tid / TP), q = tid % TP;
-      float dot = 0.f;
-      if (k < D - 2)
-        for (int j = q; j < D; j += TP) dot = fmaf(L[k * LDA + j], L[(k + 1) * LDA + j], dot);
+  // out[i][j] = sum_k L[i][k] Qt[j][k], or its transpose
+  auto product = [&](float* out, bool transposed) {
+    if (tile.live) {
+      float acc[TI][TJ];
+      tile_product_rows<D>(L, Qt, LDA, tile, acc);
 #pragma unroll
-      for (int o = 1; o < TP; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      if (q == 0 && k < D - 2) cross[k] = dot;
-    }
-    __syncthreads();
-    const int r = tid / T, q = tid % T;
-    if (tid < T * D / 2) {
-      float z[2][CB][4];
+      for (int x = 0; x < TI; ++x)
 #pragma unroll
-      for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int t = 0; t < CB; ++t) {
-          const float4 x = *reinterpret_cast<const float4*>(&Qt[(r + y * (D / 2)) * LDA + 4 * (q + T * t)]);
-          z[y][t][0] = x.x; z[y][t][1] = x.y; z[y][t][2] = x.z; z[y][t][3] = x.w;
+        for (int y = 0; y < TJ; ++y) {
+          const int i = TI * tile.i + x, j = tile.j + Tile<D>::COLS * y;
+          out[transposed ? j * LDA + i : i * LDA + j] = acc[x][y];
         }
-      auto segment = [&](auto t0c, int k_first, int k_last) {  // reflectors without an entry before chunk T0
-        constexpr int T0 = decltype(t0c)::value;
-#pragma unroll 1
-        for (int k = k_first; k >= k_last; k -= 2) {
-          const float ba = beta[k], bb = beta[k + 1], cc = cross[k];
-          float4 va[CB], vb[CB];
-#pragma unroll
-          for (int t = T0; t < CB; ++t) {
-            va[t] = *reinterpret_cast<const float4*>(&L[k * LDA + 4 * (q + T * t)]);
-            vb[t] = *reinterpret_cast<const float4*>(&L[(k + 1) * LDA + 4 * (q + T * t)]);
-          }
-          float da[2], db[2];
-#pragma unroll
-          for (int y = 0; y < 2; ++y) {
-            float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
-#pragma unroll
-            for (int t = T0; t < CB; ++t) {
-              a0 = fmaf(va[t].x, z[y][t][0], a0); a1 = fmaf(va[t].y, z[y][t][1], a1);
-              a0 = fmaf(va[t].z, z[y][t][2], a0); a1 = fmaf(va[t].w, z[y][t][3], a1);
-              b0 = fmaf(vb[t].x, z[y][t][0], b0); b1 = fmaf(vb[t].y, z[y][t][1], b1);
-              b0 = fmaf(vb[t].z, z[y][t][2], b0); b1 = fmaf(vb[t].w, z[y][t][3], b1);
-            }
-            da[y] = a0 + a1;
-            db[y] = b0 + b1;
-          }
-#pragma unroll
-          for (int o = 1; o < T; o <<= 1)
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-              da[y] += __shfl_xor_sync(0xffffffffu, da[y], o);
-              db[y] += __shfl_xor_sync(0xffffffffu, db[y], o);
-            }
-#pragma unroll
-          for (int y = 0; y < 2; ++y) {
-            const float fb = -bb * db[y];
-            const float fa = -ba * fmaf(cc, fb, da[y]);
-#pragma unroll
-            for (int t = T0; t < CB; ++t) {
-              z[y][t][0] = fmaf(fa, va[t].x, fmaf(fb, vb[t].x, z[y][t][0])); z[y][t][1] = fmaf(fa, va[t].y, fmaf(fb, vb[t].y, z[y][t][1]));
-              z[y][t][2] = fmaf(fa, va[t].z, fmaf(fb, vb[t].z, z[y][t][2])); z[y][t][3] = fmaf(fa, va[t].w, fmaf(fb, vb[t].w, z[y][t][3]));
-            }
-          }
-        }
-      };
-      // reflector k starts at entry k + 1
-      segment(std::integral_constant<int, CB / 2>{}, D - 4, D / 2);
-      segment(std::integral_constant<int, 0>{}, D / 2 - 2, 0);
-#pragma unroll
-      for (int y = 0; y < 2; ++y)
-#pragma unroll
-        for (int t = 0; t < CB; ++t)
-          *reinterpret_cast<float4*>(&Qt[(r + y * (D / 2)) * LDA + 4 * (q + T * t)]) =
-              make_float4(z[y][t][0], z[y][t][1], z[y][t][2], z[y][t][3]);
     }
-  }
-  __syncthreads();
-  // the factor of the sign rule (its space served the prologue, the merges and the reflectors)
-  if (a.lift) load_factor();
-  __syncthreads();
-
-  // ---- the map from the original space, W = F E (W[i][j] = sum_k F[i][k] Qt[j][k]), into A
-  if (a.lift) {
-#pragma unroll 1
-    for (int tile = tid; tile < TILES; tile += NT) {
-      const int tile_i = tile / (D / 4), tile_j = tile % (D / 4);
-      float acc[4][4];
-      tile_product_rows<D>(L, Qt, LDA, tile_i, tile_j, acc);
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) A[(4 * tile_i + x) * LDA + tile_j + (D / 4) * y] = acc[x][y];
+  };
+  product(A, need_e);
+  if (need_e) {
+    float* swap = Qt; Qt = A; A = swap;
+    if (a.lift) {
+      __syncthreads();
+      load_factor();
+      __syncthreads();
+      product(A, false);
     }
   }
   let_next_start();
   // ---- order, sign, bias
-  double* lam = reinterpret_cast<double*>(xbuf);             // [D] doubles over xbuf's 2D floats
-  int* rank_of = reinterpret_cast<int*>(pbuf);
+  double* lam = reinterpret_cast<double*>(ybuf);             // [D] doubles over ybuf's 2D floats
+  int* rank_of = reinterpret_cast<int*>(abuf);
   float* sign_of = beta;
-  float* mean = rot;                                         // the rotation lists are free now
   if (tid < D) {
     lam[tid] = (double)de[tid].x * a_scale;
-    mean[tid] = a.mean_sum ? (float)(a.mean_sum[(size_t)blockIdx.x * D + tid] / a.mean_n) : 0.f;
   }
   __syncthreads();
   const bool lifted_out = a.lift && a.out_lifted;
@@ -964,7 +1086,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
       rank += (other > mine) || (other == mine && k < tid);
     }
     // sign rule on column tid of F E (of E when no factor is given); bias = -mean . that column, or
-    // . column tid of E where the mean is one of transformed rows
+    // . column tid of E where the mean is one of transformed rows (without E: of S, the mean then is in the basis Q)
     float best = -1.f, sgn = 1.f, dot = 0.f;
 #pragma unroll 8
     for (int i = 0; i < D; ++i) {
@@ -999,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
 }
 
 int launch_pca(const PcaArgs& args, int count, int D, LaunchStream st) {
-  const size_t smem = sizeof(float) * ((size_t)3 * D * (D + 4) + 8 * D + 18 * D);
+  const size_t smem = sizeof(float) * ((size_t)3 * D * (D + 4) + 8 * D + 21 * D);
   auto k = D == 64 ? eigh_tql_kernel<64> : eigh_tql_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, count, kThreads, smem, st, args);

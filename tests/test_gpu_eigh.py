@@ -79,6 +79,28 @@ def test_degenerate_and_structured_matrices(d):
     assert np.abs(ev[3] - want).max() <= 1e-5
 
 
+@pytest.mark.parametrize("multiplicity", [2, 5, 31])
+@pytest.mark.parametrize("d", [64, 128])
+def test_merges_with_many_coinciding_poles(d, multiplicity):
+    """Eigenvalues of some multiplicity under a noise floor of 1e-6: merges that rotate most of their poles away,
+    so that the two halves' lists of rows share many and are filled up at every remainder; and couplings that
+    vanish at some cuts, so that a list is empty."""
+    r = np.random.default_rng(1000 * d + multiplicity)
+    mats = []
+    for i in range(6):
+        Qm, _ = np.linalg.qr(r.standard_normal((d, d)))
+        lam = np.repeat(r.uniform(0.1, 1.0, -(-d // multiplicity)), multiplicity)[:d] + 1e-6 * r.standard_normal(d)
+        mats.append(Qm @ np.diag(lam) @ Qm.T)
+    for cut in (4, d // 2, d - 4):                                 # already tridiagonal, uncoupled at one cut
+        off = r.uniform(0.0, 0.5, d - 1)
+        off[cut - 1] = 0.0
+        mats.append(np.diag(np.repeat(r.uniform(0.5, 1.0, d // 4), 4)) + np.diag(off, 1) + np.diag(off, -1))
+    mats = [(m + m.T) / 2 for m in mats]
+    W, ev = run(mats)
+    for i, (A, w, e) in enumerate(zip(mats, W, ev)):
+        check(A, w, e, f"d={d} multiplicity {multiplicity} matrix {i}", vectors_unique=False)
+
+
 def test_many_matrices_in_one_launch_are_independent():
     r = np.random.default_rng(99)
     d = 64
