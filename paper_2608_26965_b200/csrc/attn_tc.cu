@@ -19,12 +19,15 @@
 // per step (rows to load, masks, additive terms) into a ring, warps 4-15 are the
 // softmax groups.  The roles run ahead of one another across tiles, so that the start
 // of a tile hides behind the end of the one before.
-// The rows of a 64-row query cluster are loaded twice, into both halves of a tile: the
-// upper half takes keys 0-63 of every step and the lower half keys 64-127 (the other
-// probabilities of a row are stored as zeros), so that all four softmax warps of a group
-// work and each on half of the columns; the two halves are independent rows with sums,
-// references and outputs of their own, merged at the end of the tile.  (0 x inf is NaN: where
-// a kept cluster holds an infinite value the merged outputs send the tile to the second pass.)
+// Query clusters of 64 rows go two to a tile, neighbours, one in either half (siblings of the split tree: their lists
+// have 64 to 86 % of their entries in common on the inputs measured).  A key cluster that both lists hold is taken once, by all rows;
+// one that a single list holds by the rows of that half, next to one of the other list (the other probabilities of a row
+// are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
+// loaded into both halves that divided the keys of a step between them, was the form before: 12 heads of 16,385 rows, 33
+// of 257 clusters 348 -> 236 us, 12 heads of 30,592 rows 667 -> 454.  (0 x inf is NaN: where a key cluster of one list holds an infinite
+// value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
+// descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
+// 400 cycles put into each step cost 46 us; now 4).
 // All roles run at the same time on one SM and have to fit its instruction cache
 // together: with the loops of the single-warp roles unrolled (105 KB of code) the same
 // kernel took 1.40 ms where it now takes 0.73 (2 x 16 heads of 20,000 rows, d = 128, 10
@@ -36,7 +39,7 @@
 // exponentials (1,024 of 1,340 cycles per step) and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
 // four at d = 64, half-steps of 64 keys in one chain per CTA): 40 heads of 32,760 rows,
 // d = 128, 32 of 256 clusters kept 2.91 -> 2.44 ms; 8 heads of 16,384 x 131,072, d = 64,
-// 128 of 1,024 kept 0.88 -> 0.82; 12 heads of 16,385 in clusters of 64 0.373 -> 0.356.
+// 128 of 1,024 kept 0.88 -> 0.80.
 //
 // The softmax keeps a reference m per row instead of the exact running maximum: it is
 // measured on a row's first step and raised (by an integer) when a sum of 32
@@ -65,9 +68,8 @@ constexpr int kGroups = 3;                 // softmax groups of 128 threads, sco
 constexpr int kTcThreads = 128 + kGroups * 128;
 constexpr int kTile = 128;                 // query rows per tile, key rows per step
 constexpr int kCen = 64;                   // key centroids per step
-constexpr int kRing = 8;                   // step descriptors in flight
 constexpr int kParts = 6;                  // steps s - 2 .. s + 3 can have row sums on their way while step s ends a tile
-constexpr int kMergeInts = 18;             // row pitch of the hand-over between the halves of a 64-row query cluster
+constexpr int kQueue = 64;                 // list entries of a pair of 64-row query clusters in waiting
 // first rows of a step's boxes (key clusters of 16 rows: eight boxes), of its value centroids, of Q
 constexpr int kRowCenV = 8, kRowQ = 9, kRowInts = 12;
 // A reference is raised when a sum of 32 probabilities exceeds 2^32: P is bf16, O and l are fp32, so
@@ -79,12 +81,18 @@ constexpr float kDangerSum = 7.9228163e28f;  // 2^96
 
 // flags of a step descriptor
 constexpr int kFMasked = 1, kFCentroid = 2, kFFirst = 4, kFLast = 8, kFStop = 16;
+// tiles of 64-row query clusters: the upper half of the rows takes keys 0-63 of the step and the lower half keys
+// 64-127, or only one of the halves takes part
+constexpr int kFSplit = 32, kFUpper = 64, kFLower = 128;
 constexpr int kFIndexShift = 8, kFRestShift = 12;   // min(15, index in the tile), min(15, steps after it)
+constexpr int kFMixed = 1 << 16, kFSingle = 1 << 17;   // the tile has steps of the kinds above; it holds one cluster
 
 // F8: queries, keys and key centroids arrive as E4M3 codes (one byte per element: a 128-byte row
 // of a panel holds 128 of them) and Q K^T runs as kind::f8f6f4 products; values stay bf16.
-template <int D, bool F8 = false>
+template <int D, bool F8, bool HALVES>
 struct TcCfg {
+  // step descriptors in flight (64-row query clusters: four are written at a time)
+  static constexpr int RING = !HALVES ? 8 : D == 64 ? 16 : 12;
   static constexpr int PANELS = D / 64;                      // value panels (bf16: 64 elements per 128-byte row)
   static constexpr int QK_PANELS = F8 ? D / 128 : D / 64;    // query / key panels
   static constexpr int QK_PANEL_COLS = F8 ? 128 : 64;        // elements per panel row
@@ -99,16 +107,16 @@ struct TcCfg {
   static constexpr int OFF_Q = 0;
   static constexpr int OFF_K = OFF_Q + QK_BYTES;
   static constexpr int OFF_V = OFF_K + NK * QK_BYTES;
-  static constexpr int OFF_BIAS = OFF_V + NV * V_BYTES;                  // [kRing][128] floats
-  static constexpr int OFF_LPART = OFF_BIAS + kRing * kTile * 4;         // [kParts steps][128 rows] {row sum, reference}
-  static constexpr int OFF_MERGE = OFF_LPART + kParts * kTile * 8;       // [64 rows][kMergeInts] 16 columns of O, sum, reference
-  static constexpr int OFF_REF = OFF_MERGE + 64 * kMergeInts * 4;        // [128 rows] {reference, step}
-  static constexpr int OFF_ROWS = OFF_REF + kTile * 8;                   // [kRing][kRowInts]
-  static constexpr int OFF_TILE = OFF_ROWS + kRing * kRowInts * 4;       // [kRing] head, first position, redo word, tile
-  static constexpr int OFF_FLAGS = OFF_TILE + kRing * 16;
-  static constexpr int OFF_SCALE = OFF_FLAGS + kRing * 4;                // [kRing][2] scales of the keys (F8)
-  static constexpr int OFF_BAR = OFF_SCALE + kRing * 8;
-  static constexpr int NUM_BARS = 2 + 4 + 2 * kGroups + 2 * kRing + NK + 2 * NV + 4;
+  static constexpr int OFF_BIAS = OFF_V + NV * V_BYTES;                  // [RING][128] floats
+  static constexpr int OFF_LPART = OFF_BIAS + RING * kTile * 4;         // [kParts steps][128 rows] {row sum, reference}
+  static constexpr int OFF_QUEUE = OFF_LPART + kParts * kTile * 8;       // [3][kQueue] {first key row, rows, scale of the keys}
+  static constexpr int OFF_REF = OFF_QUEUE + (HALVES ? 3 * kQueue * 16 : 0);            // [128 rows] {reference, step}
+  static constexpr int OFF_ROWS = OFF_REF + kTile * 8;                   // [RING][kRowInts]
+  static constexpr int OFF_TILE = OFF_ROWS + RING * kRowInts * 4;       // [RING] head, first position, redo word, tile
+  static constexpr int OFF_FLAGS = OFF_TILE + RING * 16;
+  static constexpr int OFF_SCALE = OFF_FLAGS + RING * 4;                // [RING][2] scales of the keys (F8)
+  static constexpr int OFF_BAR = OFF_SCALE + RING * 8;
+  static constexpr int NUM_BARS = 2 + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;                // tmem base, abort flag, redo counts x 4
   static constexpr int OFF_BITMAP = OFF_MISC + 32;
   static_assert(OFF_TILE % 16 == 0 && OFF_BAR % 8 == 0 && OFF_MISC % 8 == 0, "alignment");
@@ -125,6 +133,7 @@ struct TcParams {
   int* next_tile;                 // counter that hands out tiles, zero at the start
   int32_t* redo;                  // [B*H, n_qc, 2] per tile: scores left the range of the fast softmax
   int n_q, n_k, c_q, c_k, keep, list_stride, n_qc, n_kc, cen_tiles, compensate, bitmap_words, n_tiles;
+  int pairs;                      // 64-row query clusters: two to a tile
   float scale_log2;
   // quantised Q K^T: de-quantisation scales of the query rows [B*H*n_qc*c_q], of the key clusters
   // [B*H*n_kc] and of the runs of 64 key centroids [B*H*cen_tiles]; null otherwise
@@ -136,6 +145,7 @@ struct TcParams {
 };
 
 constexpr int kErrBadIndex = 6;   // CA_ERR_BAD_INDEX
+constexpr int kPairBitmapWords = 2048;    // of each list of a pair: 65,536 key clusters (d = 128 leaves 18 KB for both)
 
 // key rows of the selected clusters are consumed in tiles of 128 rows
 __host__ __device__ inline int selected_tiles(int keep, int c_k) {
@@ -146,13 +156,14 @@ __host__ __device__ inline int selected_tiles(int keep, int c_k) {
 // and addresses from it stay in the uniform datapath.
 __device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
-template <int D, bool F8>
+// HALVES: query clusters of 64 rows (an instance of its own: the other sizes run slower with that code in the kernel)
+template <int D, bool F8, bool HALVES>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ck,
                const __grid_constant__ CUtensorMap tm_cv, const TcParams prm) {
   wait_for_previous();
-  using C = TcCfg<D, F8>;
+  using C = TcCfg<D, F8, HALVES>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
@@ -174,34 +185,33 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   auto b_s_full = [&](int b) { return bar1 + 8 * b; };
   auto b_p_ready = [&](int b) { return bar1 + 8 * (kGroups + b); };
   auto b_step_full = [&](int s) { return bar1 + 8 * (2 * kGroups + s); };
-  auto b_step_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + kRing + s); };
-  auto b_k_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + s); };
-  auto b_v_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + s); };
-  auto b_v_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + C::NV + s); };
-  auto b_m_full = [&](int w) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + 2 * C::NV + w); };
-  auto b_m_empty = [&](int w) { return bar1 + 8 * (2 * kGroups + 2 * kRing + C::NK + 2 * C::NV + 2 + w); };
+  auto b_step_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + C::RING + s); };
+  auto b_k_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + s); };
+  auto b_v_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + C::NK + s); };
+  auto b_v_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + C::NK + C::NV + s); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
   int* redo_acc = reinterpret_cast<int*>(smem + C::OFF_MISC + 8);
   unsigned* bitmap = reinterpret_cast<unsigned*>(smem + C::OFF_BITMAP);
 
   const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
-  // a query cluster of 256 rows takes two tiles; one of 64 rows is loaded into both halves of one
+  // a query cluster of 256 rows takes two tiles; two of 64 rows (or one) share one
   const int tiles_per_qc = prm.c_q >= kTile ? prm.c_q / kTile : 1;
-  const bool twice = prm.c_q < kTile;
+  constexpr bool halves = HALVES;
+  const int box_rows = halves ? min(prm.c_k, kTile / 2) : min(prm.c_k, kTile);   // of a load of keys
 
   if (tid == 0) {
     mbar_init(b_q_empty, 1); mbar_init(b_o_empty, 4);
 #pragma unroll 1
     for (int b = 0; b < kGroups; ++b) { mbar_init(b_s_full(b), 1); mbar_init(b_p_ready(b), 4); }
 #pragma unroll 1
-    for (int s = 0; s < kRing; ++s) { mbar_init(b_step_full(s), 1); mbar_init(b_step_empty(s), 6); }
+    for (int s = 0; s < C::RING; ++s) { mbar_init(b_step_full(s), 1); mbar_init(b_step_empty(s), 6); }
 #pragma unroll 1
     for (int s = 0; s < C::NK; ++s) mbar_init(b_k_full(s), 1);
 #pragma unroll 1
     for (int s = 0; s < C::NV; ++s) { mbar_init(b_v_full(s), 1); mbar_init(b_v_empty(s), 1); }
 #pragma unroll 1
-    for (int w = 0; w < 4; ++w) { mbar_init(b_m_full(w), 1); mbar_init(b_o_full(w), 1); }
+    for (int w = 0; w < 4; ++w) mbar_init(b_o_full(w), 1);
     *abort_flag = 0;
     for (int b = 0; b < 4; ++b) redo_acc[b] = 0;
     fence_mbar_init();
@@ -226,7 +236,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (lane == 0) {
         prefetch_tensormap(warp == 0 ? &tm_q : &tm_v);
         prefetch_tensormap(warp == 0 ? &tm_k : &tm_cv);
-        const int boxes = prm.c_k >= kTile ? 1 : kTile / prm.c_k;
+        const int boxes = kTile / box_rows;
         auto produce = [&](auto is_key) {
           constexpr bool key = decltype(is_key)::value;
           constexpr int panels = key ? C::QK_PANELS : C::PANELS, cols = key ? C::QK_PANEL_COLS : 64;
@@ -252,22 +262,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (key && (fl & kFFirst)) {
                 if (tiles > 0 && !relaxed(b_q_empty, tiles - 1)) return;
                 ++tiles;
-                mbar_expect_more(bar, C::QK_BYTES);           // Q arrives with the tile's first keys
+                // Q arrives with the tile's first keys (scores of a half without a cluster are not read)
+                const bool one = halves && (fl & kFSingle) != 0;
+                mbar_expect_more(bar, one ? C::QK_BYTES / 2 : C::QK_BYTES);
 #pragma unroll 1
-                for (int half = 0; half <= (twice ? 1 : 0); ++half)
+                for (int half = 0; half <= (halves && !one ? 1 : 0); ++half)
 #pragma unroll
                   for (int pn = 0; pn < C::QK_PANELS; ++pn)
-                    tma_load_2d(s_q + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ], bar);
+                    tma_load_2d(s_q + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ] + half * 64, bar);
               }
               if (!(fl & kFCentroid)) {
-                // 128 rows: one box, or several boxes of c_k rows
+                // 128 rows: one box, or several boxes
                 if (!key || i != (prm.skip_key_load >> 1)) {     // diagnostic: this slot never fills, its waiters time out
                   mbar_expect_tx(bar, bytes);
 #pragma unroll 1
                   for (int x = 0; x < boxes; ++x)
 #pragma unroll
                     for (int pn = 0; pn < panels; ++pn)
-                      tma_load_2d(dst + pn * C::PANEL_BYTES + x * prm.c_k * 128, key ? &tm_k : &tm_v, pn * cols, rows[x], bar);
+                      tma_load_2d(dst + pn * C::PANEL_BYTES + x * box_rows * 128, key ? &tm_k : &tm_v, pn * cols, rows[x], bar);
                 }
               } else {
                 // keys as bf16: 64 rows of hi parts and 64 rows of lo parts; as codes, and values: 64 rows
@@ -279,7 +291,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               mbar_arrive(b_step_empty(ring));
             }
             if (++slot == slots) { slot = 0; ph_slot ^= 1; }
-            if (++ring == kRing) { ring = 0; ph_ring ^= 1; }
+            if (++ring == C::RING) { ring = 0; ph_ring ^= 1; }
           }
         };
         if (warp == 0) produce(std::true_type{});
@@ -361,7 +373,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         __syncwarp();
         fl0 = fl1; fl1 = fl2; fl2 = fl_s;
         if (++buf == kGroups) { buf = 0; ph_s ^= 1; if (u >= 0) ph_p ^= 1; }
-        if (++ring == kRing) ring = 0;
+        if (++ring == C::RING) ring = 0;
         if (u >= 0) {
           first = (fl & kFLast) != 0;
           if (first) ++o_tiles;
@@ -370,35 +382,195 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
     } else {
       // ---------------------------------------------------------- tiles, lists, step descriptors
-      const int per_head = prm.n_qc * tiles_per_qc;
+      const int per_head = prm.pairs ? (prm.n_qc + 1) >> 1 : prm.n_qc * tiles_per_qc;
       const int ck_shift = __ffs(prm.c_k) - 1;
       const int boxes = prm.c_k >= kTile ? 1 : kTile / prm.c_k;      // list entries per step, at most 8
       int s = 0, ord = 0;
       bool ok = true;
       auto claim = [&]() {
-        if (s >= kRing) ok = __all_sync(0xffffffffu, relaxed(b_step_empty(s % kRing), s / kRing - 1));
+        if (s >= C::RING) ok = __all_sync(0xffffffffu, relaxed(b_step_empty(s % C::RING), s / C::RING - 1));
         return ok;
       };
       auto publish = [&]() {
         __syncwarp();
-        if (lane == 0) mbar_arrive(b_step_full(s % kRing));
+        if (lane == 0) mbar_arrive(b_step_full(s % C::RING));
         ++s;
+      };
+      // centroids [64 i, 64 i + 64) of a step: additive term log2 of the count, the clusters of a list (of
+      // either of two) masked
+      auto centroid_bias = [&](float* bz, const unsigned* in0, const unsigned* in1, const int32_t* cnt, int i) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          const int j = i * kCen + lane + 32 * g;
+          const float w = j < prm.n_kc ? log2f((float)cnt[min(j, prm.n_kc - 1)]) : -INFINITY;
+          bz[lane + 32 * g] = (in0[j >> 5] >> (j & 31)) & 1u ? -INFINITY : w;
+          if (halves) bz[kCen + lane + 32 * g] = (in1[j >> 5] >> (j & 31)) & 1u ? -INFINITY : w;
+        }
+      };
+      auto list_length = [&](size_t at) {
+        int keep = prm.keep_count ? prm.keep_count[at] : prm.keep;
+        if (keep < 0 || keep > prm.list_stride) {            // a list length that does not fit its row
+          if (lane == 0) atomicCAS(prm.status, 0, kErrBadIndex);
+          keep = keep < 0 ? 0 : prm.list_stride;
+        }
+        return keep;
       };
 #pragma unroll 1
       for (int tile = blockIdx.x; tile < prm.n_tiles && ok; ++ord) {
         int next = 0;
         if (lane == 0) next = (int)gridDim.x + atomicAdd(prm.next_tile, 1);
         const int p = tile / per_head, x = tile % per_head;
+        const int32_t* cnt = prm.count_k + (size_t)p * prm.n_kc;
+        const int cen_steps = prm.compensate ? prm.cen_tiles : 0;
+        if constexpr (halves) {
+          // ---- Two 64-row query clusters, one in either half of the tile, or one in the upper half.  Neighbours in
+          // cluster order are siblings of the split tree, and most of their lists are the same: key clusters of both
+          // lists are taken by all rows, those of one list two at a time by a half each.  In runs of 64 keys:
+          //   shared       two runs of both lists per step
+          //   split        a run of the upper list, for the upper half, and one of the lower
+          //   one-sided    two runs of the list that is longer than the other
+          // which are never more steps than two tiles of one cluster each.  (A list that holds a cluster twice
+          // counts it twice: then nothing is shared.)
+          const int qc = prm.pairs ? 2 * x : x;
+          const bool single = !prm.pairs || qc + 1 == prm.n_qc;
+          const size_t at = (size_t)p * prm.n_qc + qc;
+          const int32_t* sel0 = prm.block_idx + at * prm.list_stride;
+          const int32_t* sel1 = sel0 + prm.list_stride;
+          const int keep0 = list_length(at), keep1 = single ? 0 : list_length(at + 1);
+          unsigned* in0 = bitmap;
+          unsigned* in1 = single ? bitmap : bitmap + prm.bitmap_words;
+          __syncwarp();
+#pragma unroll 1
+          for (int w = lane; w < (single ? 1 : 2) * prm.bitmap_words; w += 32) bitmap[w] = 0u;
+          __syncwarp();
+          int n0 = 0, n1 = 0, both = 0;                      // entries of the lists that are key clusters, shared ones
+          bool again = false;
+#pragma unroll 1
+          for (int base = 0; base < max(keep0, keep1); base += 32) {
+            const int e = base + lane;
+            const int j0 = e < keep0 ? sel0[e] : 0, j1 = e < keep1 ? sel1[e] : 0;
+            const bool ok0 = e < keep0 && (unsigned)j0 < (unsigned)prm.n_kc, ok1 = e < keep1 && (unsigned)j1 < (unsigned)prm.n_kc;
+            // not a key cluster: flagged, left out
+            if ((e < keep0 && !ok0) || (e < keep1 && !ok1)) atomicCAS(prm.status, 0, kErrBadIndex);
+            const unsigned bit0 = 1u << (j0 & 31), bit1 = 1u << (j1 & 31);
+            if (ok0) again |= (atomicOr(&in0[j0 >> 5], bit0) & bit0) != 0;
+            if (ok1) again |= (atomicOr(&in1[j1 >> 5], bit1) & bit1) != 0;
+            n0 += __popc(__ballot_sync(0xffffffffu, ok0));
+            n1 += __popc(__ballot_sync(0xffffffffu, ok1));
+          }
+          const bool apart = __any_sync(0xffffffffu, again);
+          __syncwarp();
+          if (!single && !apart) {
+#pragma unroll 1
+            for (int w = lane; w < prm.bitmap_words; w += 32) both += __popc(in0[w] & in1[w]);
+            both = __reduce_add_sync(0xffffffffu, both);
+          }
+          // Entries of the lists in waiting: `taken` have been looked at, those of `kind` (0: not in the other list,
+          // 1: in both, 2: any) are put in, first key row, rows and scale of the keys.
+          auto fill = [&](int4* queue, const int32_t* sel, int keep, const unsigned* other, int kind, int& taken, int& filled, int upto) {
+#pragma unroll 1
+            while (filled < upto && taken < keep) {
+              const int e = taken + lane;
+              const int j = e < keep ? sel[e] : -1;
+              bool in = (unsigned)j < (unsigned)prm.n_kc;
+              if (in && kind != 2) in = ((other[j >> 5] >> (j & 31)) & 1u) == (unsigned)kind;
+              const unsigned found = __ballot_sync(0xffffffffu, in);
+              if (in)
+                queue[(filled + __popc(found & ((1u << lane) - 1u))) % kQueue] =
+                    make_int4((p * prm.n_kc + j) * prm.c_k, min(max(cnt[j], 0), prm.c_k),
+                              F8 ? __float_as_int(prm.k_scale[(size_t)p * prm.n_kc + j]) : 0, 0);
+              filled += __popc(found);
+              taken += 32;
+            }
+          };
+          // runs of 64 keys: a cluster has 2^parts of them, a run holds 2^each clusters
+          const int parts = max(ck_shift - 6, 0), each = max(6 - ck_shift, 0);
+          auto through = [&](int run) { return ((run >> parts) + 1) << each; };                    // entries of runs 0 .. run
+          auto runs = [&](int entries) { return ((entries + (1 << each) - 1) >> each) << parts; };
+          const int all = single ? n0 : both, own0 = single ? 0 : n0 - both, own1 = n1 - both;     // entries
+          const int runs0 = runs(own0), runs1 = runs(own1);
+          const int end_shared = (runs(all) + 1) >> 1, end_split = end_shared + min(runs0, runs1);
+          const int end_runs = end_split + ((abs(runs0 - runs1) + 1) >> 1), n = max(end_runs + cen_steps, 1);
+          const int longer = runs1 > runs0 ? 1 : 0;            // list of the one-sided steps
+          const int kind = apart ? 2 : 0;
+          int4* queue = reinterpret_cast<int4*>(smem + C::OFF_QUEUE);
+          int taken_both = 0, filled_both = 0, taken0 = 0, filled0 = 0, taken1 = 0, filled1 = 0;
+          // Four steps at a time, eight lanes to a step, one to a box: a step by itself takes this warp longer
+          // (1,800 cycles) than the softmax.
+          const int k = lane >> 3, box = lane & 7;
+          const int h = box * box_rows >= kCen ? 1 : 0;        // the box's run of the step
+          const bool a_box = box * box_rows < kTile;
+#pragma unroll 1
+          for (int u0 = 0; u0 < n && ok; u0 += 4) {
+            const int u = u0 + k, last = min(u0 + 3, n - 1);   // this lane's step; the last one of the four
+            if (u0 < end_shared)
+              fill(queue, sel0, keep0, in1, single ? 2 : 1, taken_both, filled_both, min(all, through(2 * min(last, end_shared - 1) + 1)));
+            if (last >= end_shared && u0 < end_runs) {
+              // runs of either list up to step `last`
+              const int v = min(last, end_runs - 1), far = max(v - end_split + 1, 0);
+              const int to = min(v, end_split - 1) - end_shared + 2 * far;
+              fill(queue + kQueue, sel0, keep0, in1, kind, taken0, filled0, min(own0, through(longer == 0 ? to : to - 2 * far)));
+              fill(queue + 2 * kQueue, sel1, keep1, in0, kind, taken1, filled1, min(own1, through(longer == 1 ? to : to - 2 * far)));
+            }
+            __syncwarp();
+            const bool shared = u < end_shared, split = !shared && u < end_split, one = u >= end_split && u < end_runs;
+            const bool cen = u >= end_runs && cen_steps > 0, live = u < n;
+            const int which = shared ? 0 : split ? 1 + h : 1 + longer;
+            const int run = shared ? 2 * u + h : split ? u - end_shared : 2 * (u - end_split) + end_split - end_shared + h;
+            const int entries = shared ? all : !(split || one) ? 0 : which == 2 ? own1 : own0;
+            const int entry = ((run >> parts) << each) + (box & ((1 << each) - 1));
+            const int first = (run & ((1 << parts) - 1)) * kCen;
+            int4 it = make_int4(p * prm.n_kc * prm.c_k, 0, 0, 0);   // (behind the end of a list: rows of the first cluster, masked)
+            if (a_box && entry < entries) it = queue[which * kQueue + entry % kQueue];
+            const int members = entry < entries ? it.y - first : 0;
+            const bool starts = live && box == 0;              // the lane that waits for the step's slot and hands it over
+            const int slot = (s + k) % C::RING;
+            if (starts && s + k >= C::RING) ok = relaxed(b_step_empty(slot), (s + k) / C::RING - 1);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            int* rows = st_rows + slot * kRowInts;
+            const unsigned cut = __ballot_sync(0xffffffffu, live && !cen && a_box && members < box_rows);
+            if (live && !cen && a_box) {
+              rows[box] = it.x + first;
+              if (F8 && box < 2) st_scale[slot * 2 + box] = __int_as_float(it.z);
+            }
+            if (live && cen) {
+              const int i = u - end_runs;
+              if (box == 0) rows[0] = (p * prm.cen_tiles + i) * (F8 ? kCen : kTile);
+              if (box == 1) rows[kRowCenV] = (p * prm.cen_tiles + i) * kCen;
+              if (F8 && box < 2) st_scale[slot * 2 + box] = prm.c_scale[(size_t)p * prm.cen_tiles + i];
+            }
+            if (starts) {
+              st_flags[slot] = (single ? kFSingle | kFUpper : 0) | (runs0 + runs1 > 0 ? kFMixed : 0) | (u == 0 ? kFFirst : 0) |
+                               (u == n - 1 ? kFLast : 0) | (min(u, 15) << kFIndexShift) | (min(n - 1 - u, 15) << kFRestShift) |
+                               (split ? kFSplit : one ? (longer ? kFLower : kFUpper) : 0) | (cen ? kFCentroid : 0) |
+                               (cen || ((cut >> (lane & 24)) & 255u) ? kFMasked : 0);
+              rows[kRowQ] = (int)at * prm.c_q;
+              st_tile[slot] = make_int4(p, qc * prm.c_q, (int)at * 2, ord);
+            }
+            // additive terms of short clusters and of centroids, a step after the other
+#pragma unroll 1
+            for (int kk = 0; kk < 4; ++kk) {
+              float* bz = bias + ((s + kk) % C::RING) * kTile;
+              if ((cut >> (8 * kk)) & 255u) {
+#pragma unroll 1
+                for (int c = lane; c < kTile; c += 32) {
+                  const int m = __shfl_sync(0xffffffffu, members, 8 * kk + c / box_rows);
+                  bz[c] = (c & (box_rows - 1)) < m ? 0.f : -INFINITY;
+                }
+              }
+              if (cen_steps > 0 && u0 + kk >= end_runs && u0 + kk < n) centroid_bias(bz, in0, in1, cnt, u0 + kk - end_runs);
+            }
+            __syncwarp();
+            if (starts) mbar_arrive(b_step_full(slot));
+            s += last - u0 + 1;
+          }
+          tile = __shfl_sync(0xffffffffu, next, 0);
+        } else {
         const int qc = x / tiles_per_qc, half = x % tiles_per_qc;
         const int32_t* sel = prm.block_idx + ((size_t)p * prm.n_qc + qc) * prm.list_stride;
-        const int32_t* cnt = prm.count_k + (size_t)p * prm.n_kc;
-        int keep = prm.keep_count ? prm.keep_count[(size_t)p * prm.n_qc + qc] : prm.keep;
-        if (keep < 0 || keep > prm.list_stride) {            // a list length that does not fit its row
-          if (lane == 0) atomicCAS(prm.status, 0, kErrBadIndex);
-          keep = keep < 0 ? 0 : prm.list_stride;
-        }
+        const int keep = list_length((size_t)p * prm.n_qc + qc);
         const int sel_steps = selected_tiles(keep, prm.c_k);
-        const int cen_steps = prm.compensate ? prm.cen_tiles : 0;
         const int n = max(sel_steps + cen_steps, 1);      // nothing to attend to: one step with every column masked
         if (prm.compensate) {
 #pragma unroll 1
@@ -431,8 +603,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
           }
           if (!claim()) break;
-          int* rows = st_rows + (s % kRing) * kRowInts;
-          float* bz = bias + (s % kRing) * kTile;
+          int* rows = st_rows + (s % C::RING) * kRowInts;
+          float* bz = bias + (s % C::RING) * kTile;
           float sc = 0.f;
           if (u < sel_steps) {
             // filler boxes behind the end of the list repeat its last entry, masked
@@ -460,12 +632,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               const int i = u - sel_steps;
               fl |= kFCentroid;
               __syncwarp();
-#pragma unroll
-              for (int g = 0; g < 2; ++g) {
-                const int j = i * kCen + lane + 32 * g;
-                const bool use = j < prm.n_kc && !((bitmap[j >> 5] >> (j & 31)) & 1u);
-                bz[lane + 32 * g] = use ? log2f((float)cnt[min(j, prm.n_kc - 1)]) : -INFINITY;
-              }
+              centroid_bias(bz, bitmap, bitmap, cnt, i);
               if (lane == 0) rows[0] = (p * prm.cen_tiles + i) * (F8 ? kCen : kTile);
               if (lane == 1) rows[kRowCenV] = (p * prm.cen_tiles + i) * kCen;
               if (F8) sc = prm.c_scale[(size_t)p * prm.cen_tiles + i];
@@ -475,20 +642,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (lane < boxes) rows[lane] = p * prm.n_kc * prm.c_k;
             }
           }
-          if (F8 && lane < 2) st_scale[(s % kRing) * 2 + lane] = sc;
+          if (F8 && lane < 2) st_scale[(s % C::RING) * 2 + lane] = sc;
           if (lane == 0) {
-            st_flags[s % kRing] = fl;
+            st_flags[s % C::RING] = fl;
             rows[kRowQ] = (p * prm.n_qc + qc) * prm.c_q + half * kTile;
-            st_tile[s % kRing] = make_int4(p, qc * prm.c_q + half * kTile, (p * prm.n_qc + qc) * 2 + half, ord);
+            st_tile[s % C::RING] = make_int4(p, qc * prm.c_q + half * kTile, (p * prm.n_qc + qc) * 2 + half, ord);
           }
           publish();
         }
         tile = __shfl_sync(0xffffffffu, next, 0);
+        }
       }
 #pragma unroll 1
       for (int g = 0; g < kGroups && ok; ++g) {
         if (!claim()) break;
-        if (lane == 0) st_flags[s % kRing] = kFStop;
+        if (lane == 0) st_flags[s % C::RING] = kFStop;
         publish();
       }
     }
@@ -497,7 +665,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int group = (warp >> 2) - 1;
     const int quarter = warp & 3;                  // TMEM lanes this warp may touch
     const int row = quarter * 32 + lane;           // row within the tile
-    const int qrow = twice ? row & 63 : row;       // query row
     const int half = quarter >> 1;                 // of the tile
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const uint32_t t_s = tmem_base + group * kTile + lane_addr;
@@ -511,7 +678,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     uint32_t ph_s = 0;
 #pragma unroll 1
     for (int s = group;; s += kGroups) {
-      const int ring = s % kRing;
+      const int ring = s % C::RING;
       if (!wait(b_s_full(group), ph_s)) break;
       ph_s ^= 1;
       tc_fence_after();
@@ -525,7 +692,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         pend = 0.f;
         if (F8) {
           const int4 tl = st_tile[ring];
-          row_sc = prm.scale_log2 * prm.q_scale[(size_t)tl.x * prm.n_qc * prm.c_q + tl.y + qrow];
+          row_sc = prm.scale_log2 * prm.q_scale[(size_t)tl.x * prm.n_qc * prm.c_q + tl.y + (halves && (fl & kFSingle) ? row & 63 : row)];
         }
       }
       // scales of this step's scores, per run of 64 columns.  A zero scale (an all-zero query row or
@@ -541,11 +708,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           sc_h[h] = sc_eff > 0.f ? sc_eff : (masked ? 1.f : 0.f);
         }
       }
-      const float* bz = bias + ring * kTile;
-      // chunks [c_begin, c_end) of 32 columns; of a 64-row query cluster's halves the lower one has no part in
-      // the 64 columns of a centroid step
-      const int c_begin = twice && !cen ? 2 * half : 0;
-      const int c_end = twice ? (cen ? 2 - 2 * half : c_begin + 2) : (cen ? 2 : 4);
+      // (the two lists of a tile of 64-row query clusters leave out different centroids)
+      const float* bz = bias + ring * kTile + (halves && cen ? half * kCen : 0);
+      // chunks [c_begin, c_end) of 32 columns
+      const bool idle = halves && (fl & (half == 0 ? kFLower : kFUpper)) != 0, split = halves && (fl & kFSplit) != 0;
+      // (kept from the compiler that it is 0 in the instances for 128 rows: with the loops below arranged for
+      // that, they are 3 % slower, 807 -> 835 us for 8 heads of 16,384 x 131,072 rows)
+      int c_begin = split ? 2 * half : 0;
+      asm volatile("" : "+r"(c_begin));
+      const int c_end = idle ? 0 : split ? c_begin + 2 : (cen ? 2 : 4);
       // ---- masked or weighted steps: scores of hi and lo parts of centroids are added and the additive
       // term is folded into the scores in tensor memory first, so that the common path below has
       // no bias
@@ -708,10 +879,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         chunk(rb, sc2, t_s + h * 32 + 16);
         tmem_wait_ld32(ra);
       }
-      if (twice && (!cen || half == 1)) {                  // the other half's keys
+      if (split || idle) {                                 // the other half's keys
 #pragma unroll
         for (int j = 0; j < 32; ++j) ra[j] = 0u;
-        tmem_st32(t_s + (cen || half == 1 ? 0 : 32), ra);
+        tmem_st32(t_s + (split && half == 0 ? 32 : 0), ra);
+        if (idle && !cen) tmem_st32(t_s + 32, ra);
       }
       if (big > kSumLimit) pend = ceilf(log2f(big));
       // the group's last step of the tile: its row sums go to the group that ends the tile
@@ -725,8 +897,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (rest > 0) continue;
 
       // ---- epilogue: O / l, rows back to their original positions
-      const int pos = tl.y + qrow;
-      bool live = pos < prm.n_q;                        // rows of the padding are not written
+      const int pos = tl.y + row;
+      // rows of the padding are not written, nor those of a half without a cluster
+      bool live = pos < prm.n_q && !(halves && (fl & kFSingle) && half == 1);
       int orig = live ? prm.perm_q[(size_t)tl.x * prm.n_q + pos] : 0;
       if (orig < 0 || orig >= prm.n_q) {                // not a row of O: flagged, nothing written
         atomicCAS(prm.status, 0, kErrBadIndex);
@@ -743,95 +916,59 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (other.y > -INFINITY) l_run += other.x * ex2_approx(other.y - m_ref);
         }
       }
-      // the halves of a 64-row query cluster: the lower one hands over its sums and 16 columns of O at a
-      // time, scaled to the larger reference by the upper one
-      float* merge = reinterpret_cast<float*>(smem + C::OFF_MERGE) + qrow * kMergeInts;
-      const int pair = quarter & 1, uses = tl.w * (D / 16);
-      bool got = true;
-      if (twice && half == 1) {
-#pragma unroll 1
-        for (int c = 0; c < D / 16 && got; ++c) {
-          const int use = uses + c;
-          uint32_t o[16];
-          tmem_ld16(tmem_o + lane_addr + c * 16, o);
-          tmem_wait_ld();
-          if (use > 0) got = wait(b_m_empty(pair), use - 1);
-          if (!got) break;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) merge[j] = __uint_as_float(o[j]);
-          merge[16] = l_run;
-          merge[17] = m_ref;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(b_m_full(pair));
-        }
-      }
-      float l_all = l_run, m_all = m_ref, w_own = 1.f, w_other = 0.f;
-      if (twice && half == 0) {
-        got = wait(b_m_full(pair), uses);
-        if (!got) break;
-        const float l_other = merge[16], m_other = merge[17];
-        m_all = fmaxf(m_ref, m_other);
-        w_own = m_ref > -INFINITY ? ex2_approx(m_ref - m_all) : 0.f;
-        w_other = m_other > -INFINITY ? ex2_approx(m_other - m_all) : 0.f;
-        l_all = l_run * w_own + l_other * w_other;
-      }
-      if (!got) break;
+      float l_all = l_run;
       // a row without a single live entry (an empty list without compensation): zeros, lse = -inf
       const bool empty = !(l_all > 0.f);
       const float inv = empty ? 0.f : 1.f / l_all;
       __nv_bfloat16* out = prm.O + ((size_t)tl.x * prm.n_q + orig) * D;
-      const bool write = live && !(twice && half == 1);
-      if (!(twice && half == 1)) {
-        const float inv_own = inv * w_own, inv_other = inv * w_other;
+      // 0 x inf, an infinite value among the other half's keys: for the second pass
+      const bool check = halves && (fl & kFMixed) != 0;
 #pragma unroll 1
-        for (int c = 0; c < D / 16; ++c) {
-          uint32_t o[16];
-          tmem_ld16(tmem_o + lane_addr + c * 16, o);
-          tmem_wait_ld();
+      for (int c = 0; c < D / 16; ++c) {
+        uint32_t o[16];
+        tmem_ld16(tmem_o + lane_addr + c * 16, o);
+        tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv_own);
-          if (twice) {
-            if (c > 0) got = wait(b_m_full(pair), uses + c);
-            if (!got) break;
+        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv);
+        if (check) {
+          f32x2 any2 = pack2(0.f, 0.f);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(fmaf(merge[j], inv_other, __uint_as_float(o[j])));
-            // 0 x inf, an infinite value among the other half's keys: for the second pass
-            f32x2 any2 = pack2(0.f, 0.f);
+          for (int j = 0; j < 16; j += 2) any2 = add2(any2, pack2(__uint_as_float(o[j]), __uint_as_float(o[j + 1])));
+          float any, any_odd;
+          unpack2(any2, any, any_odd);
+          any += any_odd;
+          if (any != any) l_all = any;
+        }
+        if (live) {
+          uint4* dst = reinterpret_cast<uint4*>(out + c * 16);
 #pragma unroll
-            for (int j = 0; j < 16; j += 2) any2 = add2(any2, pack2(__uint_as_float(o[j]), __uint_as_float(o[j + 1])));
-            float any, any_odd;
-            unpack2(any2, any, any_odd);
-            any += any_odd;
-            if (any != any) l_all = any;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(b_m_empty(pair));
-          }
-          if (write) {
-            uint4* dst = reinterpret_cast<uint4*>(out + c * 16);
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-              uint4 w;
-              w.x = pack_bf16x2(__uint_as_float(o[8 * v + 0]), __uint_as_float(o[8 * v + 1]));
-              w.y = pack_bf16x2(__uint_as_float(o[8 * v + 2]), __uint_as_float(o[8 * v + 3]));
-              w.z = pack_bf16x2(__uint_as_float(o[8 * v + 4]), __uint_as_float(o[8 * v + 5]));
-              w.w = pack_bf16x2(__uint_as_float(o[8 * v + 6]), __uint_as_float(o[8 * v + 7]));
-              if (empty) w = make_uint4(0u, 0u, 0u, 0u);   // every column masked: the accumulator may hold 0 x inf
-              dst[v] = w;
-            }
+          for (int v = 0; v < 2; ++v) {
+            uint4 w;
+            w.x = pack_bf16x2(__uint_as_float(o[8 * v + 0]), __uint_as_float(o[8 * v + 1]));
+            w.y = pack_bf16x2(__uint_as_float(o[8 * v + 2]), __uint_as_float(o[8 * v + 3]));
+            w.z = pack_bf16x2(__uint_as_float(o[8 * v + 4]), __uint_as_float(o[8 * v + 5]));
+            w.w = pack_bf16x2(__uint_as_float(o[8 * v + 6]), __uint_as_float(o[8 * v + 7]));
+            if (empty) w = make_uint4(0u, 0u, 0u, 0u);   // every column masked: the accumulator may hold 0 x inf
+            dst[v] = w;
           }
         }
       }
-      if (!got) break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(b_o_empty);
-      if (write && prm.lse)
-        prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_all + log2f(l_all)) * 0.6931471805599453f;
-      // one word per tile, written on every launch by the last of its four warps: 1 = recompute (a row left the range)
-      const bool redo = __any_sync(0xffffffffu, !(l_all < INFINITY) && !(twice && half == 1));
+      if (live && prm.lse)
+        prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_ref + log2f(l_all)) * 0.6931471805599453f;
+      // one word per tile or 64-row query cluster, written on every launch by the last of its four warps: 1 = recompute
+      // (a row left the range)
+      const bool redo = __any_sync(0xffffffffu, live && !(l_all < INFINITY));
       if (lane == 0) {
         int* acc = &redo_acc[tl.w & 3];
-        if ((atomicAdd(acc, redo ? 257 : 1) & 255) == 3) prm.redo[tl.z] = atomicExch(acc, 0) >= 256 ? 1 : 0;
+        const int mine = redo ? (halves && half == 1 ? 65537 : 257) : 1;
+        if ((atomicAdd(acc, mine) & 255) == 3) {
+          const int all = atomicExch(acc, 0);
+          prm.redo[tl.z] = (all >> 8) & 255 ? 1 : 0;
+          if (halves && !(fl & kFSingle)) prm.redo[tl.z + 2] = all >> 16 ? 1 : 0;
+        }
       }
     }
   }
@@ -935,11 +1072,11 @@ size_t attn_tc_workspace_bytes(const ca_problem_t& pr) {
   return bytes;
 }
 
-template <int D, bool F8>
+template <int D, bool F8, bool HALVES>
 static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, LaunchStream st) {
-  using C = TcCfg<D, F8>;
-  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4;
-  auto k = attn_tc_kernel<D, F8>;
+  using C = TcCfg<D, F8, HALVES>;
+  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4 * (prm.pairs ? 2 : 1);
+  auto k = attn_tc_kernel<D, F8, HALVES>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, grid, kTcThreads, smem, st, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
   CA_LAUNCH_CHECK();
@@ -988,8 +1125,8 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
     CA_LAUNCH_CHECK();
   }
   CUtensorMap maps[5];
-  const int kbox = pr.cluster_k < kTile ? pr.cluster_k : kTile;
   const int qbox = pr.cluster_q < kTile ? pr.cluster_q : kTile;
+  const int kbox = pr.cluster_k < qbox ? pr.cluster_k : qbox;     // 64-row query clusters: keys in runs of 64
   bool ok = make_map(&maps[2], Vp, (size_t)P * n_kc * pr.cluster_k, D, kbox) &&
             make_map(&maps[4], vb, (size_t)P * cen_tiles * kCen, D, kCen);
   if (f8)
@@ -1013,17 +1150,22 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   prm.skip_key_load = g_skip_key_load;
   prm.q_scale = sq; prm.k_scale = sk; prm.c_scale = sc;
   const int tiles_per_qc = pr.cluster_q >= kTile ? pr.cluster_q / kTile : 1;
-  prm.n_tiles = P * n_qc * tiles_per_qc;
   prm.next_tile = status + kTileWord;
   int sms = 0, dev = 0;
   CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
   CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // 64-row query clusters go two to a tile where there are more of them than SMs (a pair takes up to twice the steps
+  // of one cluster: with fewer, SMs would stand idle), unless the lists' bitmaps do not fit
+  prm.pairs = pr.cluster_q < kTile && (long long)P * n_qc > sms && prm.bitmap_words <= kPairBitmapWords;
+  prm.n_tiles = P * (prm.pairs ? (n_qc + 1) / 2 : n_qc * tiles_per_qc);
   const int grid = prm.n_tiles < sms ? prm.n_tiles : sms;
   int rc;
   {
     ProfScope ps(kProfAttn, st);
-    if (f8) rc = launch_tc_d<128, true>(maps, prm, grid, st);
-    else rc = D == 64 ? launch_tc_d<64, false>(maps, prm, grid, st) : launch_tc_d<128, false>(maps, prm, grid, st);
+    const bool halves = pr.cluster_q < kTile;
+    if (f8) rc = halves ? launch_tc_d<128, true, true>(maps, prm, grid, st) : launch_tc_d<128, true, false>(maps, prm, grid, st);
+    else if (D == 64) rc = halves ? launch_tc_d<64, false, true>(maps, prm, grid, st) : launch_tc_d<64, false, false>(maps, prm, grid, st);
+    else rc = halves ? launch_tc_d<128, false, true>(maps, prm, grid, st) : launch_tc_d<128, false, false>(maps, prm, grid, st);
   }
   if (rc != CA_OK) return rc;
   ProfScope ps(kProfAttnSecond, st);

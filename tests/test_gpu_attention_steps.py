@@ -175,3 +175,44 @@ def test_values_with_infinities(d, c_q, c_k, keep, compensate):
         assert torch.equal(mask(O), mask(want)), mask.__name__
     fine = torch.isfinite(want)
     assert (O - want)[fine].norm() <= 1e-2 * want[fine].norm()
+
+
+@pytest.mark.parametrize("compensate", [False, True])
+@pytest.mark.parametrize("d,c_k,infinite", [(64, 64, False), (64, 16, False), (128, 32, False), (128, 64, False), (64, 128, False), (128, 256, False),
+                                            (64, 64, True), (128, 128, True)])
+def test_pairs_of_64_row_query_clusters(d, c_k, infinite, compensate):
+    """More 64-row query clusters than SMs go two to a tile, with the key clusters of both lists taken once: lists that
+    share everything, something and nothing, of the same and of very different lengths, empty ones, in any order, with a
+    cluster twice, an odd number of clusters per head."""
+    heads, n_qc, n_kc = 9, 35, 45
+    n_q, n_k = 64 * n_qc - 17, c_k * n_kc - 5
+    Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, 64, c_k, d + c_k)
+    if infinite:
+        Vp[0, :, 3 * c_k + 5, 7] = torch.inf
+        Vp[0, :, 8 * c_k, d - 1] = -torch.inf
+    even = lists[:, :, ::2].repeat_interleave(2, dim=2)[:, :, :n_qc]      # both clusters of a pair have one order
+    kind = torch.arange(heads * n_qc, device=DEV).reshape(1, heads, n_qc) // 2 % 5
+    keep = torch.tensor([9, 14, 5, 9, 0], device=DEV)[kind] + torch.arange(n_qc, device=DEV) % 2 * torch.tensor([0, 3, 0, 20, 4], device=DEV)[kind]
+    idx = torch.where((kind % 5 == 2)[..., None], lists, even)      # kind 2: unrelated lists
+    idx = torch.where(((kind == 3) & (torch.arange(n_qc, device=DEV) % 2 == 1))[..., None], even.roll(-4, -1), idx)     # kind 3: shifted
+    idx[:, 1::3, 3, 0] = idx[:, 1::3, 3, 1]                               # a cluster twice
+    keep[:, 1::3, 3] = 37                                                 # (and others behind it in the list's second 32)
+    idx, keep = idx.int().contiguous(), keep.int().contiguous()
+    out = []
+    for flags in (0, binding.CA_ATTN_FP32):
+        plan = binding.Plan(binding.make_problem(1, heads, n_q, n_k, d, "bf16", 64, c_k, 1, compensate, flags=flags), DEV)
+        O, lse = plan.cluster_attention_fwd_ragged(idx, keep, Qp, Kp, Vp, ck, cv, count, perm)
+        torch.cuda.synchronize()
+        assert plan.last_status()["attn"] == 0
+        out.append((O.float(), lse))
+        if flags == 0 and not infinite:
+            assert plan.recomputed_clusters() == 0
+    (O, lse), (want, want_lse) = out
+    for mask in (torch.isnan, torch.isposinf, torch.isneginf):
+        assert torch.equal(mask(O), mask(want)), mask.__name__
+    fine, live = torch.isfinite(want), ~torch.isneginf(want_lse)
+    assert torch.equal(torch.isneginf(lse), ~live)
+    # probabilities and value centroids are bf16 on one side (2^-9 each), results on both
+    assert (O - want)[fine].norm() <= 1e-2 * want[fine].norm()
+    assert (O - want)[fine].abs().max() <= 5e-2
+    assert (lse - want_lse)[live].abs().max() <= 2e-3
