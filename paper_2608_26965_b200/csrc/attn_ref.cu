@@ -5,26 +5,34 @@
 // Serves fp32 storage, unusual cluster sizes, and as an on-device cross-check of
 // the tensor-core kernel.  Flash-style online softmax, fp32 throughout.
 //
-// Bound by the fp32 pipe and by what feeds it from shared memory: 16 threads share RY = 4 query
-// rows, a thread computes 4 x 2 scores and 4 x D / 16 outputs, so that six 16-byte loads feed 32 (scores)
-// and 12 feed 128 (outputs) multiply-adds; the rows of the next tile of keys are fetched from global memory
-// while a tile is computed.  4 heads of 5,003 rows, d = 128, 5 of 40 clusters of 128 kept: 0.80 ->
-// 0.36 ms; 2 heads of 1,024 rows, d = 64: 49 -> 26 us (before: 16 query rows per CTA, scalar loads).
-// A CTA takes 64 query rows where that still gives every SM one, otherwise 32; of a query cluster of 16
-// rows it takes those, with RY = 2: in a tile of 32 half of the threads computed nothing, and calls with such
-// clusters took up to 1.4 times as long as with the scalar kernel (60 shapes: 1.00 of its speed in the mean, 0.71 at worst; with the narrow
-// tile 1.37 and 0.99, with RY = 4 in it 1.35 and 0.94).
+// Bound by the fp32 pipe and by what feeds it from shared memory: 16 threads share RY query
+// rows, a thread computes RY x KT / 16 scores and RY x D / 16 outputs, so that (RY = 4, KT = 64) eight 16-byte loads feed 64
+// (scores) and 12 feed 128 (outputs) multiply-adds.  fp32 storage: the keys of the next tile are copied to shared memory
+// asynchronously while the softmax and the outputs of a tile are computed, its values during the scores of the next, without
+// passing registers, which leaves room for 16 warps per SM; with registers in between (8 to 16 warps, 64 rows per CTA) 4
+// heads of 5,003 rows, d = 128, 5 of 40 clusters of 128 kept took 357 us, now 310, 4 heads of 8,192 rows 805 -> 599, 2 heads of 1,024
+// rows, d = 64 29 -> 23.  (5,003 rows are 628 CTAs, four to an SM: 36 too many for one wave.)  bf16 storage (the cross-check and
+// the second pass behind the tensor-core kernel) converts, so its rows pass through registers.
+// Of a query cluster of 16 rows a CTA takes those, with RY = 2: in a tile of 32 half of the threads would compute nothing.
 #include "kernels.h"
 
 namespace ca {
 
-constexpr int kRefKT = 32;       // keys per staged tile
+// 16 bytes global -> shared memory, zeros where `use` is false
+__device__ __forceinline__ void copy_async16(float* dst, const float* src, bool use) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(use ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void copies_close() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int left>                // all groups of copies but the last `left` have arrived
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(left) : "memory"); }
+
 // Key clusters that the bitmap of the selected ones covers at a time (128 KB, beside the widest tile), so that their number
 // has no bound in shared memory.  With more of them (`many`, an instance of its own: moving the window costs the others
 // registers) the bitmap is set anew per window; a second pass never has as many (the tensor-core kernel takes an eighth).
 constexpr int kRefWindow = 1 << 20;
 
-template <typename T, int D, int QR, int RY, bool many>
+template <typename T, int D, int QR, int RY, int KT, bool direct, bool many>
 __global__ void __launch_bounds__(16 * QR / RY)
 attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __restrict__ Vp,
                 const float* __restrict__ ck, const float* __restrict__ cv,
@@ -37,17 +45,17 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   wait_for_previous();
   constexpr int NT = 16 * QR / RY;       // threads: 16 per RY query rows
   constexpr int LD = D + 4;              // row pitch: rows of eight threads in distinct banks
-  constexpr int LP = kRefKT + 4;
+  constexpr int LP = KT + 4;
   constexpr int CG = D / 64;             // groups of four output columns per thread
-  constexpr int KI = kRefKT / 16;        // keys per thread
-  constexpr int PF = kRefKT * D / 4 / NT;   // float4 of keys (of values) per thread and tile
+  constexpr int KI = KT / 16;            // keys per thread
+  constexpr int PF = KT * D / 4 / NT;    // float4 of keys (of values) per thread and tile
   extern __shared__ __align__(16) float smem[];
   float* qs = smem;                      // [QR][LD]
   float* ks = qs + QR * LD;              // [KT][LD]
-  float* vs = ks + kRefKT * LD;          // [KT][LD]
-  float* ps = vs + kRefKT * LD;          // [QR][LP]
-  float* bias = ps + QR * LP;            // [KT] per-key additive term (ln|c| or -inf)
-  unsigned* selected = reinterpret_cast<unsigned*>(bias + kRefKT);   // bitmap over a window of key clusters
+  float* vs = ks + KT * LD;              // [KT][LD]
+  float* ps = vs + KT * LD;              // [QR][LP]
+  float* bias = ps + QR * LP;            // [2][KT] per-key additive term (ln|c| or -inf), of two tiles in turn
+  unsigned* selected = reinterpret_cast<unsigned*>(bias + 2 * KT);   // bitmap over a window of key clusters
 
   const int n_qc = (n_q + c_q - 1) / c_q, n_kc = (n_k + c_k - 1) / c_k;
   const int tiles_per_cluster = (c_q + QR - 1) / QR;
@@ -133,54 +141,79 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       while (t < keep) {
         const int j = sel[t];
         members = (j < 0 || j >= n_kc) ? 0 : min(max(cnt[j], 0), c_k);       // out of range: flagged above
-        if (t0 < members) { rows = min(kRefKT, members - t0); return; }
+        if (t0 < members) { rows = min(KT, members - t0); return; }
         ++t;
         t0 = 0;
       }
-      rows = compensate ? min(kRefKT, n_kc - t0) : 0;
+      rows = compensate ? min(KT, n_kc - t0) : 0;
     };
-    float4 kf[PF], vf[PF];
-    float next_bias = 0.f;
-    auto fetch = [&]() {
-      const bool cen = t >= keep;
-      const size_t base = cen ? (size_t)t0 * D : ((size_t)sel[t] * c_k + t0) * D;
-#pragma unroll
-      for (int i = 0; i < PF; ++i) {
-        const int e = tid + i * NT, r = e / (D / 4), col = 4 * (e % (D / 4));
-        kf[i] = vf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < rows) {
-          const size_t at = base + (size_t)r * D + col;
-          kf[i] = cen ? load4(ckh + at) : load4(Kh + at);
-          vf[i] = cen ? load4(cvh + at) : load4(Vh + at);
+    float4 kf[direct ? 1 : PF], vf[direct ? 1 : PF];
+    int parity = 0;                        // of the tile that is computed
+    const T *k_src = nullptr, *v_src = nullptr;   // (direct) rows of the next tile
+    int src_rows = 0;
+    auto copy_tile = [&](float* dst, const T* src) {
+      if constexpr (direct) {
+#pragma unroll 4
+        for (int i = 0; i < PF; ++i) {
+          const int e = tid + i * NT, r = e / (D / 4), col = 4 * (e % (D / 4));
+          copy_async16(&dst[r * LD + col], src + (r < src_rows ? (size_t)r * D + col : 0), r < src_rows);
         }
       }
-      if (tid < kRefKT) {
+      copies_close();
+    };
+    auto fetch = [&](int to) {
+      const bool cen = t >= keep;
+      const size_t base = cen ? (size_t)t0 * D : ((size_t)sel[t] * c_k + t0) * D;
+      if constexpr (direct) {
+        k_src = (cen ? ckh : Kh) + base;
+        v_src = (cen ? cvh : Vh) + base;
+        src_rows = rows;
+      } else {
+#pragma unroll
+        for (int i = 0; i < PF; ++i) {
+          const int e = tid + i * NT, r = e / (D / 4), col = 4 * (e % (D / 4));
+          kf[i] = vf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (r < rows) {
+            const size_t at = base + (size_t)r * D + col;
+            kf[i] = cen ? load4(ckh + at) : load4(Kh + at);
+            vf[i] = cen ? load4(cvh + at) : load4(Vh + at);
+          }
+        }
+      }
+      if (tid < KT) {
         bool use = tid < rows;
+        float b = use ? 0.f : -INFINITY;
         if (cen && use) {
           const int j = t0 + tid;
           use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
-          next_bias = use ? logf((float)cnt[j]) : -INFINITY;
-        } else {
-          next_bias = use ? 0.f : -INFINITY;
+          b = use ? logf((float)cnt[j]) : -INFINITY;
         }
+        bias[to * KT + tid] = b;
       }
     };
     settle();
-    if (rows > 0) fetch();
+    if (rows > 0) {
+      fetch(0);
+      if constexpr (direct) { copy_tile(ks, k_src); copy_tile(vs, v_src); }
+    }
     while (rows > 0) {
-      __syncthreads();                     // the tile before has been read
+      if constexpr (direct) {
+        copies_wait<1>();
+        __syncthreads();                   // the keys have arrived
+      } else {
+        __syncthreads();                   // the tile before has been read
 #pragma unroll
-      for (int i = 0; i < PF; ++i) {
-        const int e = tid + i * NT, r = e / (D / 4), col = 4 * (e % (D / 4));
-        *reinterpret_cast<float4*>(&ks[r * LD + col]) = kf[i];
-        *reinterpret_cast<float4*>(&vs[r * LD + col]) = vf[i];
+        for (int i = 0; i < PF; ++i) {
+          const int e = tid + i * NT, r = e / (D / 4), col = 4 * (e % (D / 4));
+          *reinterpret_cast<float4*>(&ks[r * LD + col]) = kf[i];
+          *reinterpret_cast<float4*>(&vs[r * LD + col]) = vf[i];
+        }
+        __syncthreads();
       }
-      if (tid < kRefKT) bias[tid] = next_bias;
-      __syncthreads();
-      t0 += kRefKT;
+      t0 += KT;
       rows = 0;
       if (t < keep) settle();
-      else rows = max(0, min(kRefKT, n_kc - t0));
+      else rows = max(0, min(KT, n_kc - t0));
       if constexpr (many) {
         if (rows > 0 && t >= keep && t0 > 0 && t0 % kRefWindow == 0) {
           __syncthreads();                 // the window before has been read
@@ -188,7 +221,9 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
           __syncthreads();
         }
       }
-      if (rows > 0) fetch();
+      const float* b_tile = bias + parity * KT;
+      parity ^= 1;
+      if (rows > 0) fetch(parity);
 
       // scores of rows RY tr + y, keys tc + 16 i
       float s[RY][KI];
@@ -211,6 +246,11 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
             s[y][i] = fmaf(q4[y].z, k4[i].z, s[y][i]); s[y][i] = fmaf(q4[y].w, k4[i].w, s[y][i]);
           }
       }
+      if constexpr (direct) {
+        copies_wait<0>();
+        __syncthreads();                   // the keys have been read, the values have arrived
+        if (rows > 0) copy_tile(ks, k_src);
+      }
       // online softmax: the 16 threads of a row are half a warp
       float tmax[RY];
 #pragma unroll
@@ -218,7 +258,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         tmax[y] = -INFINITY;
 #pragma unroll
         for (int i = 0; i < KI; ++i) {
-          s[y][i] = s[y][i] * scale + bias[tc + 16 * i];
+          s[y][i] = s[y][i] * scale + b_tile[tc + 16 * i];
           tmax[y] = fmaxf(tmax[y], s[y][i]);
         }
       }
@@ -255,7 +295,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       __syncwarp();
 #pragma unroll 2
-      for (int key = 0; key < kRefKT; key += 4) {
+      for (int key = 0; key < KT; key += 4) {
         float4 p4[RY];
 #pragma unroll
         for (int y = 0; y < RY; ++y) p4[y] = *reinterpret_cast<const float4*>(&ps[(RY * tr + y) * LP + key]);
@@ -271,6 +311,10 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
               acc[y][g][2] = fmaf(pv, v4.z, acc[y][g][2]); acc[y][g][3] = fmaf(pv, v4.w, acc[y][g][3]);
             }
           }
+      }
+      if constexpr (direct) {
+        __syncthreads();                   // the values have been read
+        if (rows > 0) copy_tile(vs, v_src);
       }
     }
 
@@ -296,14 +340,15 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
   }   // clusters of the CTA
 }
 
-template <typename T, int D, int QR, int RY = 4, bool many = false>
+// direct: tiles are copied to shared memory asynchronously, not by way of registers
+template <typename T, int D, int QR, int RY, int KT, bool direct = sizeof(T) == 4, bool many = false>
 static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* Vp, const float* ck,
                        const float* cv, const int32_t* count_k, const int32_t* block_idx,
                        const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
                        float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                        int* redo_count) {
   const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
-  const size_t smem = sizeof(float) * ((size_t)(QR + 2 * kRefKT) * (D + 4) + QR * (kRefKT + 4) + kRefKT) +
+  const size_t smem = sizeof(float) * ((size_t)(QR + 2 * KT) * (D + 4) + QR * (KT + 4) + 2 * KT) +
                       sizeof(unsigned) * (((n_kc < kRefWindow ? n_kc : kRefWindow) + 31) / 32);
   // second pass: some 600 CTAs that look at their share of the marks (10,240 CTAs that each looked at one took 18 us)
   const int n_clusters = pr.batch * pr.heads * n_qc;
@@ -311,7 +356,7 @@ static int launch_rows(const ca_problem_t& pr, const T* Qp, const T* Kp, const T
   const int per_cta = redo ? (ceil_div(n_clusters, 592) < NT ? ceil_div(n_clusters, 592) : NT) : 1;
   const dim3 grid = redo ? dim3(ceil_div(n_clusters, per_cta))
                          : dim3(n_qc * ceil_div(pr.cluster_q, QR), pr.batch * pr.heads);
-  auto k = attn_ref_kernel<T, D, QR, RY, many>;
+  auto k = attn_ref_kernel<T, D, QR, RY, KT, direct, many>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, grid, NT, smem, st, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, pr.n_q, pr.n_k,
                                 pr.cluster_q, pr.cluster_k, pr.keep, pr.compensate, scale, O, lse, status, redo,
@@ -326,18 +371,44 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
                     const int32_t* keep_count, int list_stride, const int32_t* perm_q, float scale, T* O,
                     float* lse, int* status, LaunchStream st, const int32_t* redo, int redo_tiles,
                     int* redo_count) {
-  // 64 query rows per CTA read every key half as often as 32; 32 where 64 would leave SMs without a CTA
-  const int n_kc = ceil_div(pr.n_k, pr.cluster_k);
-  const long long ctas = (long long)pr.batch * pr.heads * ceil_div(pr.n_q, 64);
-  const bool wide = !redo && pr.cluster_q >= 64 && ctas >= 148;
+  const int n_qc = ceil_div(pr.n_q, pr.cluster_q), n_kc = ceil_div(pr.n_k, pr.cluster_k);
   auto go = [&](auto launch) {
     return launch(pr, Qp, Kp, Vp, ck, cv, count_k, block_idx, keep_count, list_stride, perm_q, scale, O, lse, status, st,
                   redo, redo_tiles, redo_count);
   };
+  if (n_kc > kRefWindow) return pr.head_dim == 64 ? go(launch_rows<T, 64, 32, 4, 32, false, true>) : go(launch_rows<T, 128, 32, 4, 32, false, true>);
   const bool narrow = pr.cluster_q < 32;       // (never a second pass: the tensor-core kernel takes 64 rows and more)
-  if (n_kc > kRefWindow) return pr.head_dim == 64 ? go(launch_rows<T, 64, 32, 4, true>) : go(launch_rows<T, 128, 32, 4, true>);
-  if (pr.head_dim == 64) return narrow ? go(launch_rows<T, 64, 16, 2>) : wide ? go(launch_rows<T, 64, 64>) : go(launch_rows<T, 64, 32>);
-  return narrow ? go(launch_rows<T, 128, 16, 2>) : wide ? go(launch_rows<T, 128, 64>) : go(launch_rows<T, 128, 32>);
+  if constexpr (sizeof(T) == 4) {
+    // Query rows per CTA: 8 or 16 where every CTA still has an SM for itself (a CTA is a chain of latencies then, which shared
+    // work shortens), otherwise 32.  Keys per tile: 64 (fewer rounds of the softmax), but 32 where clusters
+    // are smaller (a tile holds one cluster) and at d = 128 with more than two CTAs per SM, of which four
+    // fit with 32 and two with 64.  us, tiles of 32 rows and 32 keys / 64 keys / 16 rows / 8 rows:
+    //   1 head of 1,024 rows, d = 64     20.7 / 19.5 / 16.6 / 14.9      2 heads of 1,024     31 / 27 / 22.8 / 26.8
+    //   4 heads of 1,024                 30 / 26.8 / 28.9 / 37          4 heads of 8,192     619 / 537 / 733
+    //   1 head of 1,500, d = 128         59 / 51 / 41 / 54              2 heads of 2,500     134 / 115 / 146
+    //   2 heads of 5,003, 10 clusters    321 / 395                      4 heads of 8,192     599 / 709
+    //   4 heads of 5,000 in clusters of 32    331 / 671             1 head of 1,000, key clusters of 16     93 / - / 77
+    auto ctas = [&](int rows) { return (long long)pr.batch * pr.heads * n_qc * ceil_div(pr.cluster_q, rows); };
+    // (by way of registers where small clusters leave at most two CTAs to an SM: two barriers per tile instead of three,
+    // 52 against 56 us for 1 head of 2,500 rows, d = 128, key clusters of 32)
+    const bool few = ctas(32) <= 296;
+    if (pr.head_dim == 64) {
+      if (pr.cluster_k < 64)
+        return narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 32>) : few ? go(launch_rows<T, 64, 32, 4, 32, false>) : go(launch_rows<T, 64, 32, 4, 32>);
+      if (ctas(8) <= 148) return go(launch_rows<T, 64, 8, 1, 64>);
+      return narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 64>) : go(launch_rows<T, 64, 32, 4, 64>);
+    }
+    if (pr.cluster_k < 64)
+      return narrow || ctas(16) <= 148 ? go(launch_rows<T, 128, 16, 2, 32>) : few ? go(launch_rows<T, 128, 32, 4, 32, false>) : go(launch_rows<T, 128, 32, 4, 32>);
+    if (ctas(8) <= 148) return go(launch_rows<T, 128, 8, 1, 64>);
+    if (narrow || ctas(16) <= 148) return go(launch_rows<T, 128, 16, 2, 64>);
+    return few ? go(launch_rows<T, 128, 32, 4, 64>) : go(launch_rows<T, 128, 32, 4, 32>);
+  } else {
+    // 64 query rows per CTA read every key half as often as 32; 32 where 64 would leave SMs without a CTA
+    const bool wide = !redo && pr.cluster_q >= 64 && (long long)pr.batch * pr.heads * ceil_div(pr.n_q, 64) >= 148;
+    if (pr.head_dim == 64) return narrow ? go(launch_rows<T, 64, 16, 2, 32>) : wide ? go(launch_rows<T, 64, 64, 4, 32>) : go(launch_rows<T, 64, 32, 4, 32>);
+    return narrow ? go(launch_rows<T, 128, 16, 2, 32>) : wide ? go(launch_rows<T, 128, 64, 4, 32>) : go(launch_rows<T, 128, 32, 4, 32>);
+  }
 }
 
 int launch_attn_ref(const ca_problem_t& pr, const void* Qp, const void* Kp, const void* Vp,

@@ -76,6 +76,10 @@ def test_tiles_of_few_steps_and_many_tiles(d, c_q, c_k, heads, n_q, n_k, compens
     (64, 32, 64, 2, 32 * 4 - 31, 64 * 5, True), (128, 32, 32, 1, 100, 32 * 9 - 1, False),             # of 32
     (64, 256, 64, 1, 300, 64 * 4 - 9, True),
     (128, 64, 128, 5, 64 * 30 - 3, 128 * 3 - 60, True), (64, 128, 32, 3, 128 * 26, 32 * 8, False),    # of 64: from 148 tiles on
+    # fp32 storage: tiles of 8 and 16 rows while there is an SM for each, then 32, with 64 keys and 32
+    (64, 64, 64, 2, 64 * 9 - 5, 64 * 5 - 9, True), (64, 64, 128, 2, 64 * 10 - 9, 128 * 4 - 77, False), (128, 64, 64, 2, 64 * 10 - 9, 64 * 6 - 1, True),
+    (64, 128, 64, 3, 128 * 7 - 5, 64 * 6 - 9, True), (128, 128, 256, 2, 128 * 10, 256 * 3 - 100, True),
+    (128, 128, 64, 5, 128 * 16 - 3, 64 * 5 - 7, True),
 ])
 def test_fp32_kernel_against_float64(d, c_q, c_k, heads, n_q, n_k, compensate, dtype):
     Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, c_q, c_k, d + c_q + c_k + n_q)
