@@ -481,7 +481,7 @@ namespace {
 struct BasicWs {
   int* status;
   float* partial;
-  double *gramQ, *sumQ, *gramK, *sumK, *metric;
+  double *gramQ, *sumQ, *gramK, *sumK;
   float *dirs_q, *dirs_k;
   int32_t *perm_q_tmp, *perm_k_tmp;
   uint32_t *keybuf_q, *keybuf_k;
@@ -499,7 +499,6 @@ BasicWs carve_basic(const ca_problem_t* p, void* base) {
   w.partial = c.take<float>(P * (size_t)(ncq > nck ? ncq : nck) * (DD + D));
   w.gramQ = c.take<double>(P * DD);  w.sumQ = c.take<double>(P * D);
   w.gramK = c.take<double>(P * DD);  w.sumK = c.take<double>(P * D);
-  w.metric = c.take<double>(2 * P * DD);
   const int lq = split_levels_for(p->n_q, p->cluster_q), lk = split_levels_for(p->n_k, p->cluster_k);
   w.nodes_q = (1 << (lq > 0 ? lq : 1)) - 1;
   w.nodes_k = (1 << (lk > 0 ? lk : 1)) - 1;
@@ -537,7 +536,6 @@ int cluster_qk_basic(const ca_problem_t* p, const void* Q, const void* K, const 
   if (ws_bytes < w.bytes) return CA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int P = p->batch * p->heads, D = p->head_dim;
-  const size_t DD = (size_t)D * D;
   CA_RETURN_IF_CUDA(cudaMemsetAsync(w.status, 0, kStatusBytes, st));
   if (!(p->flags & CA_METRIC_IN)) {
     // keys are compared in the query metric Q^T Q / n_q, queries in K_c^T K_c / n_k (Section 3.2.2)
@@ -548,11 +546,7 @@ int cluster_qk_basic(const ca_problem_t* p, const void* Q, const void* K, const 
       CA_TRY(launch_moments(Q, p->dtype, P, p->n_q, D, w.partial, w.gramQ, w.sumQ, st));
       CA_TRY(launch_moments(K, p->dtype, P, p->n_k, D, w.partial, w.gramK, w.sumK, st));
     }
-    double* M = w.metric;
-    double* CK = w.metric + (size_t)P * DD;
-    CA_TRY(launch_metric(w.gramQ, w.gramK, w.sumK, P, D, p->n_q, p->n_k, 1.0 / (double)p->n_k, M, CK, st));
-    CA_TRY(launch_cast_f64_f32(M, A_k, (size_t)P * DD, st));
-    CA_TRY(launch_cast_f64_f32(CK, A_q, (size_t)P * DD, st));
+    CA_TRY(launch_metric(w.gramQ, w.gramK, w.sumK, P, D, p->n_q, p->n_k, 1.0 / (double)p->n_k, A_k, A_q, st));
   }
   CA_TRY(launch_split_basic(Q, K, p->dtype, A_q, A_k, noise_q, noise_k, w.dirs_q, w.dirs_k, iterations, P, D, p->n_q,
                             p->n_k, p->cluster_q, p->cluster_k, perm_q, w.perm_q_tmp, perm_k, w.perm_k_tmp,

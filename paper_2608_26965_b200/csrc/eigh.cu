@@ -187,36 +187,23 @@ int launch_cholesky_factor(const double* gram, const double* sum, double n, doub
 // ---------------------------------------------------------------------------
 // d x d algebra in double (one CTA per problem unless noted).
 // ---------------------------------------------------------------------------
-// M = gramQ / n_q ;  C_K = gramK - sumK sumK^T / n_k   (centred scatter)
+// M = gramQ / n_q ;  C_K = (gramK - sumK sumK^T / n_k) ck_scale   (centred scatter), rounded to float
 __global__ void metric_kernel(const double* __restrict__ gramQ, const double* __restrict__ gramK,
                               const double* __restrict__ sumK, int D, double n_q, double n_k,
-                              double ck_scale, double* __restrict__ M, double* __restrict__ CK) {
+                              double ck_scale, float* __restrict__ M, float* __restrict__ CK) {
   wait_for_previous();
   let_next_start();
-  // either output may be left out (null)
   const int p = blockIdx.y;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= D * D) return;
   const int i = e / D, j = e % D;
   const size_t o = (size_t)p * D * D + e;
-  if (M) M[o] = gramQ[o] / n_q;
-  if (CK) CK[o] = (gramK[o] - sumK[(size_t)p * D + i] * sumK[(size_t)p * D + j] / n_k) * ck_scale;
-}
-
-__global__ void cast_f64_f32_kernel(const double* __restrict__ src, float* __restrict__ dst, size_t count) {
-  wait_for_previous();
-  let_next_start();
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < count) dst[i] = (float)src[i];
-}
-int launch_cast_f64_f32(const double* src, float* dst, size_t count, LaunchStream st) {
-  launch_chained(cast_f64_f32_kernel, (unsigned)((count + 255) / 256), 256, 0, st, src, dst, count);
-  CA_LAUNCH_CHECK();
-  return CA_OK;
+  M[o] = (float)(gramQ[o] / n_q);
+  CK[o] = (float)((gramK[o] - sumK[(size_t)p * D + i] * sumK[(size_t)p * D + j] / n_k) * ck_scale);
 }
 
 int launch_metric(const double* gramQ, const double* gramK, const double* sumK, int P, int D, int n_q,
-                  int n_k, double ck_scale, double* M, double* CK, LaunchStream st) {
+                  int n_k, double ck_scale, float* M, float* CK, LaunchStream st) {
   launch_chained(metric_kernel, dim3(ceil_div(D * D, 256), P), 256, 0, st, gramQ, gramK, sumK, D, (double)n_q,
                  (double)n_k, ck_scale, M, CK);
   CA_LAUNCH_CHECK();

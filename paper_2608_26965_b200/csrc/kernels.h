@@ -54,7 +54,7 @@ int launch_pca(const PcaArgs& args, int count, int D, LaunchStream st);
 
 // eigh.cu
 int launch_metric(const double* gramQ, const double* gramK, const double* sumK, int P, int D, int n_q,
-                  int n_k, double ck_scale, double* M, double* CK, LaunchStream st);
+                  int n_k, double ck_scale, float* M, float* CK, LaunchStream st);
 // factor of gram * scale (sum null) or of (gram - s s^T / n) * scale
 int launch_cholesky_factor(const double* gram, const double* sum, double n, double scale, int count, int D,
                            double* out64, float* out32, void* wt_hi, void* wt_lo, LaunchStream st);
@@ -75,7 +75,6 @@ int launch_split_basic(const void* Q, const void* K, int dtype, const float* A_q
                        int32_t* perm_q_tmp, int32_t* perm_k_out, int32_t* perm_k_tmp, uint32_t* keybuf_q,
                        uint32_t* keybuf_k, LaunchStream st);
 int split_levels_for(int n, int c);
-int launch_cast_f64_f32(const double* src, float* dst, size_t count, LaunchStream st);
 int launch_permute_centroid(const void* X, int dtype, const int32_t* perm, int P, int n, int D, int c,
                             void* Xp, float* cen, int32_t* count, LaunchStream st, const void* X2 = nullptr,
                             void* Xp2 = nullptr, float* cen2 = nullptr);

@@ -1001,18 +1001,36 @@ struct BasicParams {
   int level, problems, iterations;
 };
 
-__device__ __forceinline__ float seq_norm(const float* v, int d) {
-  // d is a multiple of 8; the squares are formed eight at a time and added in order
-  float s = 0.f;
-#pragma unroll 1
-  for (int j0 = 0; j0 < d; j0 += 8) {
-    float sq[8];
+// Sums of the power iteration, terms in order.  The operands come eight at a time in 16-byte loads, so that the
+// additions, one dependent chain, are what takes the time.
+// a . b, n a multiple of 8
+__device__ __forceinline__ float ordered_dot(const float* a, const float* b, int n) {
+  float acc = 0.f;
+#pragma unroll 2
+  for (int k0 = 0; k0 < n; k0 += 8) {
+    float term[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sq[j] = __fmul_rn(v[j0 + j], v[j0 + j]);
+    for (int h = 0; h < 8; h += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(a + k0 + h), y = *reinterpret_cast<const float4*>(b + k0 + h);
+      term[h] = __fmul_rn(x.x, y.x); term[h + 1] = __fmul_rn(x.y, y.y);
+      term[h + 2] = __fmul_rn(x.z, y.z); term[h + 3] = __fmul_rn(x.w, y.w);
+    }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) s = __fadd_rn(s, sq[j]);
+    for (int k = 0; k < 8; ++k) acc = __fadd_rn(acc, term[k]);
   }
-  return __fsqrt_rn(s);
+  return acc;
+}
+__device__ __forceinline__ float seq_norm(const float* v, int d) {
+  float acc = 0.f;
+#pragma unroll 2
+  for (int k0 = 0; k0 < d; k0 += 8) {
+    const float4 x = *reinterpret_cast<const float4*>(v + k0), y = *reinterpret_cast<const float4*>(v + k0 + 4);
+    const float sq[8] = {__fmul_rn(x.x, x.x), __fmul_rn(x.y, x.y), __fmul_rn(x.z, x.z), __fmul_rn(x.w, x.w),
+                         __fmul_rn(y.x, y.x), __fmul_rn(y.y, y.y), __fmul_rn(y.z, y.z), __fmul_rn(y.w, y.w)};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc = __fadd_rn(acc, sq[k]);
+  }
+  return __fsqrt_rn(acc);
 }
 
 // One CTA of D threads per (slot, side, head).
@@ -1020,9 +1038,10 @@ template <typename T, int D>
 __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams prm) {
   wait_for_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* z = reinterpret_cast<float*>(smem_raw);       // [m][D + 1]
-  __shared__ float u[D], v[D], w[D], y[D], g[D];
-  constexpr int LD = D + 1;
+  constexpr int LD = D + 4;
+  float* z = reinterpret_cast<float*>(smem_raw);       // [m][LD]
+  float* As = z + D * LD;                              // [D][LD]   the metric
+  __shared__ __align__(16) float u[D], v[D], w[D], y[D], g[D];
   const int which = blockIdx.y / prm.problems, p = blockIdx.y % prm.problems;
   const BasicSide sd = prm.side[which];
   if (prm.level >= sd.levels) return;
@@ -1046,26 +1065,30 @@ __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams pr
       for (int k8 = 0; k8 < D / 8; ++k8) {
         const uint32_t wds[4] = {q[k8].x, q[k8].y, q[k8].z, q[k8].w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          z[tid * LD + k8 * 8 + 2 * e] = __uint_as_float(wds[e] << 16);
-          z[tid * LD + k8 * 8 + 2 * e + 1] = __uint_as_float(wds[e] & 0xffff0000u);
-        }
+        for (int e = 0; e < 4; e += 2)
+          *reinterpret_cast<float4*>(&z[tid * LD + k8 * 8 + 2 * e]) =
+              make_float4(__uint_as_float(wds[e] << 16), __uint_as_float(wds[e] & 0xffff0000u),
+                          __uint_as_float(wds[e + 1] << 16), __uint_as_float(wds[e + 1] & 0xffff0000u));
       }
     } else {
 #pragma unroll 8
-      for (int k4 = 0; k4 < D / 4; ++k4) {
-        const float4 q = __ldg(reinterpret_cast<const float4*>(xr) + k4);
-        z[tid * LD + k4 * 4] = q.x; z[tid * LD + k4 * 4 + 1] = q.y;
-        z[tid * LD + k4 * 4 + 2] = q.z; z[tid * LD + k4 * 4 + 3] = q.w;
-      }
+      for (int k4 = 0; k4 < D / 4; ++k4)
+        *reinterpret_cast<float4*>(&z[tid * LD + k4 * 4]) = __ldg(reinterpret_cast<const float4*>(xr) + k4);
     }
+  }
+  {
+    const float4* A4 = reinterpret_cast<const float4*>(sd.A + (size_t)p * D * D);
+#pragma unroll 16
+    for (int e = tid; e < D * D / 4; e += D) *reinterpret_cast<float4*>(&As[(e / (D / 4)) * LD + 4 * (e % (D / 4))]) = __ldg(A4 + e);
   }
   g[tid] = sd.noise[((size_t)p * sd.nodes + node) * D + tid];
   __syncthreads();
   {
     float mu = 0.f;                                      // thread k: column k, rows in order
+#pragma unroll 8
     for (int i = 0; i < m; ++i) mu = __fadd_rn(mu, z[i * LD + tid]);
     mu = __fdiv_rn(mu, (float)m);
+#pragma unroll 8
     for (int i = 0; i < m; ++i) z[i * LD + tid] = __fsub_rn(z[i * LD + tid], mu);
     const float gn = __fdiv_rn(g[tid], seq_norm(g, D));
     float start = gn;
@@ -1077,24 +1100,16 @@ __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams pr
   }
   __syncthreads();
   for (int it = 0; it < prm.iterations; ++it) {
-    if (tid < m) {
-      float acc = 0.f;
-      for (int k = 0; k < D; ++k) acc = __fadd_rn(acc, __fmul_rn(z[tid * LD + k], u[k]));
-      v[tid] = acc;
-    }
+    if (tid < m) v[tid] = ordered_dot(&z[tid * LD], u, D);
     __syncthreads();
     {
       float acc = 0.f;
+#pragma unroll 8
       for (int i = 0; i < m; ++i) acc = __fadd_rn(acc, __fmul_rn(z[i * LD + tid], v[i]));
       w[tid] = acc;
     }
     __syncthreads();
-    {
-      const float* Ar = sd.A + ((size_t)p * D + tid) * D;
-      float acc = 0.f;
-      for (int k = 0; k < D; ++k) acc = __fadd_rn(acc, __fmul_rn(Ar[k], w[k]));
-      y[tid] = acc;
-    }
+    y[tid] = ordered_dot(&As[tid * LD], w, D);
     __syncthreads();
     const float nrm = seq_norm(y, D);                    // every thread takes the same sequential sum
     if (nrm > 0.f && isfinite(nrm)) u[tid] = __fdiv_rn(y[tid], nrm);
@@ -1104,51 +1119,104 @@ __global__ void __launch_bounds__(D) basic_direction_kernel(const BasicParams pr
   sd.dirs[((size_t)p * sd.nodes + node) * D + tid] = u[tid];
 }
 
-// Keys of one level: one thread per position; the set of a position follows from the size rule.
+// Keys of 32 R rows by one warp, R per lane (row: none if negative; dir: offset of the row's direction in `dirs`, shared
+// or global memory, a multiple of 4): projection x . u, terms in the order of the columns.  A lane that reads its own row touches 32
+// lines with every load; so the rows are copied to shared memory (2 x 2 KB of the warp), 64 bytes of 32 rows at a time and a piece
+// ahead of the sums, four lanes to a row, 16-byte chunk c of row r at place c ^ (r / 2 & 3).  A level of a subtree
+// of 4,096 rows, d = 64: 60 k -> 18 k cycles; 25 k with the pieces loaded through registers, one after the other.
+template <typename T, int D, int R>
+__device__ __forceinline__ void project_rows(const T* __restrict__ X, const int (&row)[R], const float* dirs, const int (&dir)[R], uint4* buf,
+                                             int lane, uint32_t (&key)[R]) {
+  constexpr int SEGS = D * (int)sizeof(T) / 64, E = 16 / (int)sizeof(T);
+  auto pick = [&](const int (&of)[R], int y) {
+    int v = of[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) v = y == k ? of[k] : v;
+    return v;
+  };
+  auto fetch = [&](int n) {
+    const int mine = pick(row, n / SEGS);
+    const uint4* src = reinterpret_cast<const uint4*>(X) + (n % SEGS) * 4 + (lane & 3);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int at = 8 * k + (lane >> 2), r = __shfl_sync(0xffffffffu, mine, at);
+      if (r >= 0)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(
+                         &buf[(n & 1) * 128 + at * 4 + ((lane & 3) ^ ((at >> 1) & 3))])), "l"(src + (size_t)r * (SEGS * 4)) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float t = 0.f;
+  fetch(0);
+#pragma unroll 1
+  for (int n = 0; n < R * SEGS; ++n) {
+    if (n + 1 < R * SEGS) {
+      fetch(n + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncwarp();
+    const int y = n / SEGS;
+    const float* u = dirs + pick(dir, y) + (n % SEGS) * 4 * E;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint4 x = buf[(n & 1) * 128 + lane * 4 + (c ^ ((lane >> 1) & 3))];
+      const uint32_t wds[4] = {x.x, x.y, x.z, x.w};
+      float uu[E];
+#pragma unroll
+      for (int e = 0; e < E; e += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(u + c * E + e);
+        uu[e] = w.x; uu[e + 1] = w.y; uu[e + 2] = w.z; uu[e + 3] = w.w;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (sizeof(T) == 2) {
+          t = __fadd_rn(t, __fmul_rn(__uint_as_float(wds[e] << 16), uu[2 * e]));
+          t = __fadd_rn(t, __fmul_rn(__uint_as_float(wds[e] & 0xffff0000u), uu[2 * e + 1]));
+        } else {
+          t = __fadd_rn(t, __fmul_rn(__uint_as_float(wds[e]), uu[e]));
+        }
+      }
+    }
+    __syncwarp();                                       // (the piece has been read)
+    if (n % SEGS == SEGS - 1) {
+#pragma unroll
+      for (int k = 0; k < R; ++k) key[k] = y == k ? order_key(t) : key[k];
+      t = 0.f;
+    }
+  }
+}
+
+// Keys of one level, two positions per thread; the set of a position follows from the size rule.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) basic_keys_kernel(const BasicParams prm) {
   wait_for_previous();
   let_next_start();
+  __shared__ uint4 staged[8][256];
   const int which = blockIdx.y / prm.problems, p = blockIdx.y % prm.problems;
   const BasicSide sd = prm.side[which];
-  if (prm.level >= sd.levels) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= sd.n) return;
-  int lo = 0, size = sd.n, slot = 0;
-  for (int l = 0; l < prm.level; ++l) {
-    if (size <= sd.c) return;                           // a final set: nothing to split at this level
-    const int L = sd.c * ((size + sd.c) / (2 * sd.c));
-    if (i < lo + L) { size = L; slot = 2 * slot; } else { lo += L; size -= L; slot = 2 * slot + 1; }
-  }
-  if (size <= sd.c) return;
-  const int node = (1 << prm.level) - 1 + slot;
-  const float* u = sd.dirs + ((size_t)p * sd.nodes + node) * D;
-  const int row = sd.perm_in ? sd.perm_in[(size_t)p * sd.n + i] : i;
-  const T* xr = static_cast<const T*>(sd.X) + ((size_t)p * sd.n + row) * D;
-  float t = 0.f;
-  if (sizeof(T) == 2) {
-    const uint4* x4 = reinterpret_cast<const uint4*>(xr);
-    for (int k8 = 0; k8 < D / 8; ++k8) {
-      const uint4 q = __ldg(x4 + k8);
-      const uint32_t wds[4] = {q.x, q.y, q.z, q.w};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i0 = (blockIdx.x * 8 + warp) * 64 + lane;
+  if (prm.level >= sd.levels || i0 - lane >= sd.n) return;
+  int row[2], node[2];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float a = __uint_as_float(wds[e] << 16), b = __uint_as_float(wds[e] & 0xffff0000u);
-        t = __fadd_rn(t, __fmul_rn(a, __ldg(u + k8 * 8 + 2 * e)));
-        t = __fadd_rn(t, __fmul_rn(b, __ldg(u + k8 * 8 + 2 * e + 1)));
-      }
+  for (int y = 0; y < 2; ++y) {
+    const int i = i0 + 32 * y;
+    int lo = 0, size = sd.n, slot = 0;
+    for (int l = 0; l < prm.level && size > sd.c; ++l) {   // (a final set: nothing to split at this level)
+      const int L = sd.c * ((size + sd.c) / (2 * sd.c));
+      if (i < lo + L) { size = L; slot = 2 * slot; } else { lo += L; size -= L; slot = 2 * slot + 1; }
     }
-  } else {
-    const float4* x4 = reinterpret_cast<const float4*>(xr);
-    for (int k4 = 0; k4 < D / 4; ++k4) {
-      const float4 q = __ldg(x4 + k4);
-      t = __fadd_rn(t, __fmul_rn(q.x, __ldg(u + k4 * 4)));
-      t = __fadd_rn(t, __fmul_rn(q.y, __ldg(u + k4 * 4 + 1)));
-      t = __fadd_rn(t, __fmul_rn(q.z, __ldg(u + k4 * 4 + 2)));
-      t = __fadd_rn(t, __fmul_rn(q.w, __ldg(u + k4 * 4 + 3)));
-    }
+    const bool splits = i < sd.n && size > sd.c;
+    node[y] = splits ? ((1 << prm.level) - 1 + slot) * D : 0;      // (an offset: of fewer than 2^31 / D nodes)
+    row[y] = !splits ? -1 : sd.perm_in ? sd.perm_in[(size_t)p * sd.n + i] : i;
   }
-  sd.keybuf[(size_t)p * sd.n + i] = order_key(t);
+  const float* dirs = sd.dirs + (size_t)p * sd.nodes * D;
+  uint32_t key[2] = {0u, 0u};
+  project_rows<T, D, 2>(static_cast<const T*>(sd.X) + (size_t)p * sd.n * D, row, dirs, node, staged[warp], lane, key);
+#pragma unroll
+  for (int y = 0; y < 2; ++y)
+    if (row[y] >= 0) sd.keybuf[(size_t)p * sd.n + i0 + 32 * y] = key[y];
 }
 
 // ---------------------------------------------------------------------------
@@ -1323,16 +1391,18 @@ __device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_s
 // subset's direction (the sum of basic_keys_kernel), then the selection and partition of the
 // diagonalized subtree kernel.
 // ---------------------------------------------------------------------------
-// staged sample rows (later the scan and the digit counts): 16 subsets of 64 bf16 rows at d = 64, 4 at d = 128
-template <int D> struct BasicStage { static constexpr int BYTES = D == 64 ? 135168 : 133120; };
+// staged sample rows: 16 subsets of 64 bf16 rows at d = 64, 4 of 128 at d = 128 (then the rows that are projected, 4 KB
+// per warp; then the scan and the digit counts).  16-byte chunk c of row r stands at place c ^ (r & 7).
+constexpr int kBasicStage = 131072;
 
 template <int D>
 struct BasicTailSmem {
   static constexpr int TEAMS = kSplitThreads / D;
   int32_t rows[2][kTailRowsMax];
-  __align__(16) unsigned char stage[BasicStage<D>::BYTES];
+  __align__(16) unsigned char stage[kBasicStage];
   float dirs[2][kTailSegs][D];            // directions of this level's subsets and of the level above
-  float mu[TEAMS][D], u[TEAMS][D], v[TEAMS][D], w[TEAMS][D], y[TEAMS][D], g[TEAMS][D];
+  __align__(16) float mu[TEAMS][D], u[TEAMS][D], v[TEAMS][D], w[TEAMS][D], y[TEAMS][D], g[TEAMS][D];
+  float4 metric[D == 64 ? D * D / 4 : 1];   // d = 64: the metric, chunks of a row placed as above (d = 128: no room)
   int seg_lo[2][2 * kTailSegs + 2];
   int seg_slot[2][2 * kTailSegs + 2];     // slot of a subset in the tree, at the level it stands on
   int seg_par[2][2 * kTailSegs + 2];      // subset of the level above it came from
@@ -1347,13 +1417,6 @@ struct BasicTailSmem {
   int more;
 };
 
-template <typename T>
-__device__ __forceinline__ float stored_value(const T* p);
-template <>
-__device__ __forceinline__ float stored_value<float>(const float* p) { return *p; }
-template <>
-__device__ __forceinline__ float stored_value<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
 template <typename T, int D>
 __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicParams prm, const SplitParams sp) {
   wait_for_previous();
@@ -1361,12 +1424,13 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Sm& sm = *reinterpret_cast<Sm*>(smem_raw);
   constexpr int nt = kSplitThreads;
-  constexpr int LD = D + (sizeof(T) == 2 ? 2 : 1);      // row stride of the staged rows (elements): odd in 4-byte words
-  constexpr int NODE_BYTES = D * LD * (int)sizeof(T);
-  constexpr int ROUND = (BasicStage<D>::BYTES / NODE_BYTES) < Sm::TEAMS ? (BasicStage<D>::BYTES / NODE_BYTES) : Sm::TEAMS;
+  constexpr int V = D * (int)sizeof(T) / 16;            // 16-byte chunks of a row
+  constexpr int E = 16 / (int)sizeof(T);                // elements of a chunk
+  constexpr int NODE_BYTES = D * V * 16;
+  constexpr int ROUND = (kBasicStage / NODE_BYTES) < Sm::TEAMS ? (kBasicStage / NODE_BYTES) : Sm::TEAMS;
   static_assert(ROUND >= 1, "a subset's sample must fit the staging area");
   constexpr int PT = kTailRowsMax / kSplitThreads;
-  static_assert(PT == 4 && kTailRowsMax * 4 + kTailSegs * 256 * 4 <= BasicStage<D>::BYTES, "scan and digit counts live in the staging area");
+  static_assert(PT == 4 && kTailRowsMax * 4 + kTailSegs * 256 * 4 <= kBasicStage && nt / 32 * 4096 <= kBasicStage, "scan, digit counts and projected rows live in the staging area");
   uint32_t* scan = reinterpret_cast<uint32_t*>(sm.stage);
   int* hist = reinterpret_cast<int*>(sm.stage + kTailRowsMax * 4);
 
@@ -1379,6 +1443,8 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
   if (!root.active) return;
   const int tid = threadIdx.x;
   const int team = tid / D, member = tid % D;
+  // where half of a team works, it is the second half of every other team, so that all four sub-cores have part in it
+  const int half_member = (D == 64 ? team >> 1 : team) & 1 ? (member + D / 2) % D : member;
   const int c = sd.c;
   const T* X = static_cast<const T*>(bs.X) + (size_t)p * sd.n * D;
   const float* Am = bs.A + (size_t)p * D * D;
@@ -1388,6 +1454,11 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
   const int lo = root.lo, s0 = root.size;
 
   for (int i = tid; i < s0; i += nt) sm.rows[0][i] = pin ? pin[lo + i] : lo + i;
+  if (D == 64 && s0 > c) {
+#pragma unroll
+    for (int e = tid; e < D * D / 4; e += nt)
+      sm.metric[(e & ~7) | ((e & 7) ^ ((e / (D / 4)) & 7))] = __ldg(reinterpret_cast<const float4*>(Am) + e);
+  }
   if (tid == 0) {
     sm.seg_lo[0][0] = 0; sm.seg_lo[0][1] = s0; sm.nseg[0] = 1; sm.more = s0 > c;
     sm.seg_slot[0][0] = (int)blockIdx.x; sm.seg_par[0][0] = -1;
@@ -1411,35 +1482,49 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
       const bool active = team < ROUND && r0 + team < nsplit;
       const int g = active ? sm.split_list[r0 + team] : 0;
       const int a = slo[g], sz = slo[g + 1] - a, m = min(D, sz);
-      T* xs = reinterpret_cast<T*>(sm.stage + (size_t)(team < ROUND ? team : 0) * NODE_BYTES);
+      uint4* xs = reinterpret_cast<uint4*>(sm.stage + (size_t)(team < ROUND ? team : 0) * NODE_BYTES);   // [D][V]
+      const uint32_t* xw = reinterpret_cast<const uint32_t*>(xs);
+      // Columns: a word per thread and row, two columns of bf16 (by half of the team) or one
+      const bool columns = active && half_member < 4 * V;
+      auto word = [&](int i) { return xw[i * (4 * V) + (((half_member >> 2) ^ (i & 7)) << 2) + (half_member & 3)]; };
+      auto first_of = [&](uint32_t x) { return sizeof(T) == 2 ? __uint_as_float(x << 16) : __uint_as_float(x); };
+      auto second_of = [&](uint32_t x) { return __uint_as_float(x & 0xffff0000u); };
+      const int col = sizeof(T) == 2 ? 2 * half_member : half_member;
       if (active) {
-        if (member < m) {
-          const int pos = a + (int)(((long long)member * sz) / m);
-          const T* xr = X + (size_t)rows[pos] * D;
-          uint32_t* dst = reinterpret_cast<uint32_t*>(xs + (size_t)member * LD);     // LD * sizeof(T) is a multiple of 4
-          constexpr int V = D * (int)sizeof(T) / 16;                                 // 16-byte loads of a row
+        // a row index per lane, the rows by 128 bytes and more of neighbouring lanes
+        const int lane = tid & 31;
+        const int sample = member < m ? rows[a + (int)(((long long)member * sz) / m)] : -1;
+        const uint4* X4 = reinterpret_cast<const uint4*>(X);
 #pragma unroll
-          for (int k0 = 0; k0 < V; k0 += 8) {
-            uint4 q[8];
+        for (int k0 = 0; k0 < V; k0 += 8) {
+          uint4 q[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) if (k0 + k < V) q[k] = __ldg(reinterpret_cast<const uint4*>(xr) + k0 + k);
+          for (int k = 0; k < 8; ++k) {
+            const int r = __shfl_sync(0xffffffffu, sample, (k0 + k) * (32 / V) + lane / V);
+            q[k] = r >= 0 ? __ldg(X4 + (size_t)r * V + lane % V) : make_uint4(0u, 0u, 0u, 0u);
+          }
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              if (k0 + k < V) {
-                dst[(k0 + k) * 4 + 0] = q[k].x; dst[(k0 + k) * 4 + 1] = q[k].y;
-                dst[(k0 + k) * 4 + 2] = q[k].z; dst[(k0 + k) * 4 + 3] = q[k].w;
-              }
+          for (int k = 0; k < 8; ++k) {
+            const int r = (member & ~31) + (k0 + k) * (32 / V) + lane / V;
+            xs[r * V + ((lane % V) ^ (r & 7))] = q[k];
           }
         }
         const int node = (1 << level) - 1 + sm.seg_slot[cur][g];
         sm.g[team][member] = noise[(size_t)node * D + member];
       }
       __syncthreads();
+      if (columns) {                                         // means, rows in order
+        float mu = 0.f, mu2 = 0.f;
+#pragma unroll 8
+        for (int i = 0; i < m; ++i) {
+          const uint32_t x = word(i);
+          mu = __fadd_rn(mu, first_of(x));
+          if (sizeof(T) == 2) mu2 = __fadd_rn(mu2, second_of(x));
+        }
+        sm.mu[team][col] = __fdiv_rn(mu, (float)m);
+        if (sizeof(T) == 2) sm.mu[team][col + 1] = __fdiv_rn(mu2, (float)m);
+      }
       if (active) {
-        float mu = 0.f;                                      // column `member`, rows in order
-        for (int i = 0; i < m; ++i) mu = __fadd_rn(mu, stored_value(xs + i * LD + member));
-        mu = __fdiv_rn(mu, (float)m);
-        sm.mu[team][member] = mu;
         const float gn = __fdiv_rn(sm.g[team][member], seq_norm(sm.g[team], D));
         float start = gn;
         if (level > 0) {
@@ -1452,53 +1537,80 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
       }
       __syncthreads();
       for (int it = 0; it < prm.iterations; ++it) {
-        if (active && member < m) {
-          // (terms formed eight at a time, then added in order: the loads do not wait for the sum)
-          float acc = 0.f;
+        if (active && half_member < D / 2) {
+          // (two rows per thread, which share the loads of mean and direction; the terms of a chunk are formed, then
+          // added in order: the loads do not wait for the sum)
+          float acc[2] = {0.f, 0.f};
 #pragma unroll 1
-          for (int k0 = 0; k0 < D; k0 += 8) {
-            float term[8];
+          for (int c8 = 0; c8 < V; ++c8) {
+            float mu[E], u[E];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              term[k] = __fmul_rn(__fsub_rn(stored_value(xs + member * LD + k0 + k), sm.mu[team][k0 + k]), sm.u[team][k0 + k]);
+            for (int e = 0; e < E; e += 4) {
+              *reinterpret_cast<float4*>(&mu[e]) = *reinterpret_cast<const float4*>(&sm.mu[team][c8 * E + e]);
+              *reinterpret_cast<float4*>(&u[e]) = *reinterpret_cast<const float4*>(&sm.u[team][c8 * E + e]);
+            }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc = __fadd_rn(acc, term[k]);
+            for (int y = 0; y < 2; ++y) {
+              const int r = half_member + y * (D / 2);
+              const uint4 x = xs[r * V + (c8 ^ (r & 7))];
+              const uint32_t wds[4] = {x.x, x.y, x.z, x.w};
+              float term[E];
+#pragma unroll
+              for (int e = 0; e < E; ++e) {
+                const float xe = sizeof(T) == 4 ? __uint_as_float(wds[e & 3]) : e % 2 ? second_of(wds[e / 2]) : first_of(wds[e / 2]);
+                term[e] = __fmul_rn(__fsub_rn(xe, mu[e]), u[e]);
+              }
+#pragma unroll
+              for (int e = 0; e < E; ++e) acc[y] = __fadd_rn(acc[y], term[e]);
+            }
           }
-          sm.v[team][member] = acc;
+          sm.v[team][half_member] = acc[0];                       // (rows behind a smaller sample: not used)
+          sm.v[team][half_member + D / 2] = acc[1];
         }
         __syncthreads();
-        if (active) {
-          const float mk = sm.mu[team][member];
-          float acc = 0.f;
+        if (columns) {
+          const float mk = sm.mu[team][col], mk2 = sizeof(T) == 2 ? sm.mu[team][col + 1] : 0.f;
+          float acc = 0.f, acc2 = 0.f;
           int i = 0;
-#pragma unroll 1
-          for (; i + 8 <= m; i += 8) {
-            float term[8];
+#pragma unroll 2
+          for (; i + 4 <= m; i += 4) {
+            const float4 v4 = *reinterpret_cast<const float4*>(&sm.v[team][i]);
+            const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
+            uint32_t x[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-              term[k] = __fmul_rn(__fsub_rn(stored_value(xs + (i + k) * LD + member), mk), sm.v[team][i + k]);
+            for (int k = 0; k < 4; ++k) x[k] = word(i + k);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc = __fadd_rn(acc, term[k]);
+            for (int k = 0; k < 4; ++k) {
+              acc = __fadd_rn(acc, __fmul_rn(__fsub_rn(first_of(x[k]), mk), vv[k]));
+              if (sizeof(T) == 2) acc2 = __fadd_rn(acc2, __fmul_rn(__fsub_rn(second_of(x[k]), mk2), vv[k]));
+            }
           }
-          for (; i < m; ++i)
-            acc = __fadd_rn(acc, __fmul_rn(__fsub_rn(stored_value(xs + i * LD + member), mk), sm.v[team][i]));
-          sm.w[team][member] = acc;
+          for (; i < m; ++i) {
+            const uint32_t x = word(i);
+            acc = __fadd_rn(acc, __fmul_rn(__fsub_rn(first_of(x), mk), sm.v[team][i]));
+            if (sizeof(T) == 2) acc2 = __fadd_rn(acc2, __fmul_rn(__fsub_rn(second_of(x), mk2), sm.v[team][i]));
+          }
+          sm.w[team][col] = acc;
+          if (sizeof(T) == 2) sm.w[team][col + 1] = acc2;
         }
         __syncthreads();
-        if (active) {
-          const float4* Ar = reinterpret_cast<const float4*>(Am + (size_t)member * D);
-          float acc = 0.f;
-#pragma unroll 1
-          for (int k0 = 0; k0 < D; k0 += 8) {
-            const float4 a0 = __ldg(Ar + k0 / 4), a1 = __ldg(Ar + k0 / 4 + 1);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            float term[8];
+        if (active && half_member < D / 2) {
+          float acc[2] = {0.f, 0.f};
+#pragma unroll 2
+          for (int c4 = 0; c4 < D / 4; ++c4) {
+            const float4 w4 = *reinterpret_cast<const float4*>(&sm.w[team][4 * c4]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) term[k] = __fmul_rn(av[k], sm.w[team][k0 + k]);
+            for (int y = 0; y < 2; ++y) {
+              const int j = half_member + y * (D / 2);
+              const float4 av = D == 64 ? sm.metric[j * (D / 4) + ((c4 & ~7) | ((c4 & 7) ^ (j & 7)))]
+                                        : __ldg(reinterpret_cast<const float4*>(Am + (size_t)j * D) + c4);
+              const float term[4] = {__fmul_rn(av.x, w4.x), __fmul_rn(av.y, w4.y), __fmul_rn(av.z, w4.z), __fmul_rn(av.w, w4.w)};
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc = __fadd_rn(acc, term[k]);
+              for (int k = 0; k < 4; ++k) acc[y] = __fadd_rn(acc[y], term[k]);
+            }
           }
-          sm.y[team][member] = acc;
+          sm.y[team][half_member] = acc[0];
+          sm.y[team][half_member + D / 2] = acc[1];
         }
         __syncthreads();
         if (active) {
@@ -1518,6 +1630,7 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
     }
 
     // ---- 2. keys: the projection of a row onto its subset's direction, terms in the order of the columns
+    // (the staged samples have been read)
     int my_seg[PT];
     uint32_t my_key[PT];
     {
@@ -1527,45 +1640,28 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
         int hi = nseg;                                  // slo[g] <= i0 < slo[g+1]
         while (hi - g > 1) { const int mid = (g + hi) >> 1; if (slo[mid] <= i0) g = mid; else hi = mid; }
       }
-#pragma unroll 1
+#pragma unroll
       for (int u = 0; u < PT; ++u) {
         const int i = i0 + u;
         my_key[u] = 0u;
         if (i < s0) {
           while (slo[g + 1] <= i) ++g;
           const bool splits = slo[g + 1] - slo[g] > c;
-          if (splits) {
-            const T* xr = X + (size_t)rows[i] * D;
-            const float* uu = dir_now[g];
-            float t = 0.f;
-            constexpr int E = 16 / (int)sizeof(T);       // elements of a 16-byte load
-#pragma unroll
-            for (int k0 = 0; k0 < D; k0 += 4 * E) {      // four loads in flight, then their terms in order
-              uint4 q[4];
-#pragma unroll
-              for (int k = 0; k < 4; ++k) q[k] = __ldg(reinterpret_cast<const uint4*>(xr + k0) + k);
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const uint32_t wds[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  if (sizeof(T) == 2) {
-                    const float x0 = __uint_as_float(wds[e] << 16), x1 = __uint_as_float(wds[e] & 0xffff0000u);
-                    t = __fadd_rn(t, __fmul_rn(x0, uu[k0 + k * E + 2 * e]));
-                    t = __fadd_rn(t, __fmul_rn(x1, uu[k0 + k * E + 2 * e + 1]));
-                  } else {
-                    t = __fadd_rn(t, __fmul_rn(__uint_as_float(wds[e]), uu[k0 + k * E + e]));
-                  }
-                }
-              }
-            }
-            my_key[u] = order_key(t);
-          }
           my_seg[u] = splits ? g : -1 - g;              // final subset: carried over unchanged
         } else {
           my_seg[u] = INT_MIN;
         }
       }
+      int row[PT], dir[PT];
+      bool any = false;
+#pragma unroll
+      for (int u = 0; u < PT; ++u) {
+        row[u] = my_seg[u] >= 0 ? rows[i0 + u] : -1;
+        dir[u] = max(my_seg[u], 0) * D;
+        any |= row[u] >= 0;
+      }
+      if (__any_sync(0xffffffffu, any))
+        project_rows<T, D, PT>(X, row, dir_now[0], dir, reinterpret_cast<uint4*>(sm.stage + (tid >> 5) * 4096), tid & 31, my_key);
     }
     __syncthreads();                                    // the staging area becomes the scan and the digit counts
 
@@ -1657,7 +1753,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
   for (int level = 0; level < top; ++level) {
     fill(level);
     bp.level = level;
-    const size_t dsmem = (size_t)D * (D + 1) * sizeof(float);
+    const size_t dsmem = (size_t)2 * D * (D + 4) * sizeof(float);
     if (D == 64) {
       auto dk = basic_direction_kernel<T, 64>;
       CA_RETURN_IF_CUDA(cudaFuncSetAttribute(dk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsmem));
@@ -1669,7 +1765,7 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
     }
     CA_LAUNCH_CHECK();
     const int n_max = n_q > n_k ? n_q : n_k;
-    launch_chained(D == 64 ? basic_keys_kernel<T, 64> : basic_keys_kernel<T, 128>, dim3(ceil_div(n_max, 256), 2 * problems), 256,
+    launch_chained(D == 64 ? basic_keys_kernel<T, 64> : basic_keys_kernel<T, 128>, dim3(ceil_div(n_max, 512), 2 * problems), 256,
                    0, st, bp);
     CA_LAUNCH_CHECK();
     int max_seg = 1;

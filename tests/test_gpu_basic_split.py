@@ -35,6 +35,9 @@ CASES = [
     (1, 2048, 40000, 64, 128, 128, "bf16", 1),       # sets larger than the shared-memory window
     (1, 640, 704, 128, 256, 16, "bf16", 0),          # no iteration: the start vectors decide
     (1, 700, 5000, 128, 64, 128, "fp32", 2),         # float32 rows at d = 128: two subsets staged per round
+    (2, 4033, 4097, 64, 64, 64, "bf16", 2),          # 32 subsets per subtree, whose edges fall inside a lane's four rows
+    (1, 65, 12345, 64, 16, 32, "bf16", 3),           # subtrees that end early, samples of fewer rows than coordinates
+    (1, 129, 8193, 64, 32, 128, "fp32", 1),          # float32 rows in four pieces, a single row in the last one
 ]
 
 
