@@ -18,24 +18,28 @@ namespace ca {
 // Besides F in double and float, F^T can be written as bf16 hi + lo parts, the layout in which the
 // tensor-core projection takes its weights (the query representation multiplies by F).
 //
-// The elimination goes by panels of eight columns.  One warp factors a panel with its rows in
-// registers and shuffles instead of barriers (the chain of a column: pivot, reciprocal, update), then all
-// threads take the eight columns off the trailing block at once: two barriers per eight columns.  With a
-// column and a barrier of 1,024 threads per step, and the one division of the step in its chain, a factor
-// took 26 us at d = 64 and 59 us at d = 128 (per launch); now 17.5 and 50.  Warp w keeps the entries (w + NW a, q + 32 b) of the trailing block in
-// registers, rows dealt out cyclically, so that the shrinking block stays spread over all warps and tests on
-// rows are uniform; finished columns stay in shared memory, unscaled, and are scaled by 1 / sqrt(pivot)
+// The elimination goes by panels of eight columns, a row per lane in registers; every lane factors the panel's 8 x 8 head for itself
+// as well, so that the chain of a column (pivot, reciprocal, update: some 80 cycles) waits for no other lane.  Then all
+// threads take the eight columns off the trailing block at once: two barriers per eight columns.  (With the panel's rows in one
+// warp and pivots and heads by shuffles a factor took 15 us at d = 64 and 50 us at d = 128; now 12.5 and 33.)  The trailing block is kept
+// in registers as the accumulators of double-precision matrix instructions, tiles of 8 x 8 of the lower triangle dealt out so
+// that the shrinking block stays spread over all warps; finished columns stay in shared memory, unscaled, and are scaled by 1 / sqrt(pivot)
 // on the way out.  The trailing block takes A[r][k] -= A[r][j] A[k][j] / pivot_j with the unscaled columns;
 // a dropped pivot (reciprocal 0) leaves it alone and gives a zero column.
 // ---------------------------------------------------------------------------
 constexpr int kPanel = 8;
 
-// reciprocal by Newton's iteration on the hardware's estimate (relative error of a few 1e-16)
+// reciprocal: the hardware's estimate (a relative error e of 2^-20) and one step of third order, 1 + e + e^2
 __device__ __forceinline__ double reciprocal(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// C (8 x 8) += A (8 x 4) B (4 x 8) in double: lane l holds A[l / 4][l % 4], B[l % 4][l / 4], C[l / 4][2 (l % 4) + 0, 1]
+__device__ __forceinline__ void mma_f64(double (&c)[2], double a, double b) {
+  asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c[0]), "+d"(c[1]) : "d"(a), "d"(b));
 }
 
 template <int D>
@@ -46,31 +50,53 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
                                                                 __nv_bfloat16* __restrict__ wt_hi,
                                                                 __nv_bfloat16* __restrict__ wt_lo) {
   constexpr int NT = 4 * D, NW = NT / 32;
-  constexpr int RT = D / NW, CT = D / 32;     // rows and columns of a thread's tile
+  constexpr int NB = D / kPanel;              // blocks of eight rows, of eight columns
+  constexpr int TILES = NB * (NB + 1) / 2, SLOTS = (TILES + NW - 1) / NW;
   constexpr int LD = D + 1;                   // pitch of a column
+  constexpr int LP = D + 8;                   // of a panel column: the four columns of a fragment in two runs of banks
   extern __shared__ __align__(16) double chol_smem[];
-  double* F = chol_smem;                      // [D][LD]  finished columns and the panel, column-major, unscaled
-  double* G = F + D * LD;                     // [kPanel][D]  panel columns over their pivots
-  double* pivots = G + kPanel * D;            // [D]
+  double* F = chol_smem;                      // [D][LD]  finished columns, column-major, unscaled; a panel before it is factored
+  double* P = F + D * LD;                     // [kPanel][LP]  panel columns
+  double* G = P + kPanel * LP;                // [kPanel][LP]  ... over their pivots
+  double* pivots = G + kPanel * LP;           // [D]
   __shared__ double s_tol;
   constexpr double kDrop = 1e-12;             // share of the largest diagonal entry below which a pivot drops out
-  wait_for_previous();
-  const int tid = threadIdx.x, w = tid >> 5, q = tid & 31;
+  const int tid = threadIdx.x, w = tid >> 5, q = tid & 31, fr = q >> 2, fk = q & 3;
   const double* A = gram + (size_t)blockIdx.x * D * D;
   const double* sm = sum ? sum + (size_t)blockIdx.x * D : nullptr;
-  double a[RT][CT];
+  // Tiles (I, J), I >= J, of eight rows by eight columns, the last column of blocks first: those that a step still
+  // has to do are the first ones of the list, dealt out to the warps in turn.
+  int row0[SLOTS], col0[SLOTS];
+  double a[SLOTS][2];
   const double per_n = sm ? scale / n : 0.0;
 #pragma unroll
-  for (int ta = 0; ta < RT; ++ta) {
-    const int r = w + NW * ta;
-    // the centring needs double precision: the Gram matrix is n mean^2 + scatter
-    const double row_term = sm ? sm[r] * per_n : 0.0;
+  for (int i = 0; i < SLOTS; ++i) {
+    const int t = w + NW * i;
+    const int m = (int)((sqrtf((float)(8 * t + 1)) - 1.f) * 0.5f) + 1;   // blocks in the tile's column of blocks
+    col0[i] = t < TILES ? kPanel * (NB - m) : -1;
+    row0[i] = t < TILES ? kPanel * (NB - m + t - m * (m - 1) / 2) : 0;
+  }
+  wait_for_previous();                        // (what stands above needs nothing of the kernel before)
+  {
+    double2 g[SLOTS];
+    double sr[SLOTS], s0[SLOTS], s1[SLOTS];
 #pragma unroll
-    for (int tb = 0; tb < CT; ++tb) {
-      const int k = q + 32 * tb;
-      a[ta][tb] = 0.0;
-      if (k <= r) a[ta][tb] = sm ? fma(-row_term, sm[k], A[r * D + k] * scale) : A[r * D + k] * scale;
-      if (k == r) pivots[r] = a[ta][tb];
+    for (int i = 0; i < SLOTS; ++i) {
+      const int r = row0[i] + fr, k = max(col0[i], 0) + 2 * fk;
+      g[i] = *reinterpret_cast<const double2*>(&A[r * D + k]);
+      // the centring needs double precision: the Gram matrix is n mean^2 + scatter
+      sr[i] = sm ? sm[r] : 0.0;
+      s0[i] = sm ? sm[k] : 0.0;
+      s1[i] = sm ? sm[k + 1] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < SLOTS; ++i) {
+      const int r = row0[i] + fr, k = col0[i] + 2 * fk;
+      const double row_term = sr[i] * per_n;
+      a[i][0] = fma(-row_term, s0[i], g[i].x * scale);
+      a[i][1] = fma(-row_term, s1[i], g[i].y * scale);
+      if (k == r) pivots[r] = a[i][0];
+      if (k + 1 == r && col0[i] >= 0) pivots[r] = a[i][1];
     }
   }
   __syncthreads();
@@ -83,68 +109,53 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
 #pragma unroll 1
   for (int p0 = 0; p0 < D; p0 += kPanel) {
     // the panel's columns, from their owners to shared memory
-    const int b0 = p0 >> 5, at = q - (p0 & 31);
-    if (at >= 0 && at < kPanel) {
 #pragma unroll
-      for (int ta = 0; ta < RT; ++ta) {
-        double v = a[ta][0];
-#pragma unroll
-        for (int tb = 1; tb < CT; ++tb) v = tb == b0 ? a[ta][tb] : v;
-        F[(p0 + at) * LD + w + NW * ta] = v;
+    for (int i = 0; i < SLOTS; ++i)
+      if (col0[i] == p0) {
+        F[(p0 + 2 * fk) * LD + row0[i] + fr] = a[i][0];
+        F[(p0 + 2 * fk + 1) * LD + row0[i] + fr] = a[i][1];
       }
-    }
     __syncthreads();
-    if (w == 0) {
+    if (tid < D && (w + 1) * 32 > p0) {
+      // row `tid` of the panel, and its 8 x 8 head, which every lane factors for itself
       const double tol = s_tol;
-      double x[CT][kPanel];                   // rows q + 32 s
-#pragma unroll
-      for (int s = 0; s < CT; ++s)
-#pragma unroll
-        for (int c = 0; c < kPanel; ++c) x[s][c] = F[(p0 + c) * LD + q + 32 * s];
+      double head[kPanel][kPanel], x[kPanel];
 #pragma unroll
       for (int c = 0; c < kPanel; ++c) {
-        // rows p0 .. p0 + 7 of the panel lie in slot b0 of eight neighbouring lanes
-        double own = x[0][c];
+        x[c] = F[(p0 + c) * LD + tid];
 #pragma unroll
-        for (int s = 1; s < CT; ++s) own = s == b0 ? x[s][c] : own;
-        const double pivot = __shfl_sync(0xffffffffu, own, (p0 + c) & 31);
-        double head[kPanel];
+        for (int k = c; k < kPanel; ++k) head[c][k] = F[(p0 + c) * LD + p0 + k];
+      }
+      __syncwarp();
 #pragma unroll
-        for (int k = c + 1; k < kPanel; ++k) head[k] = __shfl_sync(0xffffffffu, own, (p0 + k) & 31);
+      for (int c = 0; c < kPanel; ++c) {
+        const double pivot = head[c][c];
         const double ip = pivot > tol ? reciprocal(pivot) : 0.0;
+        const double f = x[c] * ip;
 #pragma unroll
-        for (int s = 0; s < CT; ++s) {
-          const double f = x[s][c] * ip;
+        for (int j = c + 1; j < kPanel; ++j) {
+          const double fj = head[c][j] * ip;
 #pragma unroll
-          for (int k = c + 1; k < kPanel; ++k) x[s][k] = fma(-f, head[k], x[s][k]);
-          F[(p0 + c) * LD + q + 32 * s] = x[s][c];
-          G[c * D + q + 32 * s] = f;
+          for (int k = c + 1; k <= j; ++k) head[k][j] = fma(-fj, head[c][k], head[k][j]);
+          x[j] = fma(-f, head[c][j], x[j]);
         }
-        if (q == 0) pivots[p0 + c] = pivot > tol ? pivot : 0.0;
+        P[c * LP + tid] = x[c];
+        G[c * LP + tid] = -f;
+        if (tid >= p0 + kPanel) F[(p0 + c) * LD + tid] = x[c];
+        if (tid == p0 + c) pivots[tid] = pivot > tol ? pivot : 0.0;
       }
     }
     __syncthreads();
-    // trailing block: columns from p0 + 8 on
+    if (tid < kPanel * kPanel) F[(p0 + tid / kPanel) * LD + p0 + tid % kPanel] = P[(tid / kPanel) * LP + p0 + tid % kPanel];
+    // trailing block, by groups of a warp's tiles without a branch in between (tiles that are done take anything)
+    constexpr int GROUP = D == 64 ? SLOTS : 3;
 #pragma unroll
-    for (int half = 0; half < kPanel; half += 4) {
-      double cv[CT][4];
+    for (int i0 = 0; i0 < SLOTS; i0 += GROUP) {
+      if (col0[i0] <= p0) break;
 #pragma unroll
-      for (int tb = 0; tb < CT; ++tb)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) cv[tb][c] = q + 32 * tb >= p0 + kPanel ? F[(p0 + half + c) * LD + q + 32 * tb] : 0.0;
-#pragma unroll
-      for (int ta = 0; ta < RT; ++ta) {
-        const int r = w + NW * ta;
-        if (r < p0 + kPanel) continue;        // uniform over the warp
-        double f[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) f[c] = G[(half + c) * D + r];
-#pragma unroll
-        for (int tb = 0; tb < CT; ++tb) {
-          if (32 * tb > r || 32 * tb + 31 < p0 + kPanel) continue;   // uniform: above the diagonal, or finished
-#pragma unroll
-          for (int c = 0; c < 4; ++c) a[ta][tb] = fma(-f[c], cv[tb][c], a[ta][tb]);
-        }
+      for (int i = i0; i < i0 + GROUP && i < SLOTS; ++i) {
+        mma_f64(a[i], G[fk * LP + row0[i] + fr], P[fk * LP + max(col0[i], 0) + fr]);
+        mma_f64(a[i], G[(4 + fk) * LP + row0[i] + fr], P[(4 + fk) * LP + max(col0[i], 0) + fr]);
       }
     }
   }
@@ -153,7 +164,7 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
   if (tid < D) pivots[tid] = pivots[tid] > 0.0 ? rsqrt(pivots[tid]) : 0.0;
   __syncthreads();
   const size_t mat = (size_t)blockIdx.x * D * D;
-#pragma unroll 4
+#pragma unroll 8
   for (int e = tid; e < D * D; e += NT) {
     const int r = e / D, k = e % D;
     const double v = k <= r ? F[k * LD + r] * pivots[k] : 0.0;
@@ -161,7 +172,7 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
     if (out32) out32[mat + e] = (float)v;
   }
   if (wt_hi) {                                // F^T [out k][in r] = F[r][k] as bf16 hi + lo
-#pragma unroll 4
+#pragma unroll 8
     for (int e = tid; e < D * D; e += NT) {
       const int k = e / D, r = e % D;
       const float vf = k <= r ? (float)(F[k * LD + r] * pivots[k]) : 0.f;
@@ -176,7 +187,7 @@ int launch_cholesky_factor(const double* gram, const double* sum, double n, doub
                            double* out64, float* out32, void* wt_hi, void* wt_lo, LaunchStream st) {
   __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(wt_hi);
   __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(wt_lo);
-  const size_t smem = sizeof(double) * ((size_t)D * (D + 1) + kPanel * D + D);
+  const size_t smem = sizeof(double) * ((size_t)D * (D + 1) + 2 * kPanel * (D + 8) + D);
   auto k = D == 64 ? cholesky_factor_kernel<64> : cholesky_factor_kernel<128>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, count, 4 * D, smem, st, gram, sum, n, scale, out64, out32, hi, lo);
