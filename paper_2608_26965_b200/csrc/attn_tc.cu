@@ -14,7 +14,7 @@
 // four softmax warps, each with a score buffer of its own (3 x 128 + D columns of
 // tensor memory), and the tensor core works up to three steps ahead: neither the
 // products nor the hand-offs between the units are on a softmax warp's path.  Roles:
-// warp 0 loads Q and K, warp 3 V (TMA, 128-byte swizzle, 64-column panels), warp 1
+// warp 0 loads Q and K, warp 3 V (TMA, 128-byte swizzle, 64-column panels), one thread of warp 1
 // issues all products, warp 2 walks over tiles and block lists and writes a descriptor
 // per step (rows to load, masks, additive terms) into a ring, warps 4-15 are the
 // softmax groups.  The roles run ahead of one another across tiles, so that the start
@@ -24,22 +24,23 @@
 // one that a single list holds by the rows of that half, next to one of the other list (the other probabilities of a row
 // are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
 // loaded into both halves that divided the keys of a step between them, was the form before: 12 heads of 16,385 rows, 33
-// of 257 clusters 348 -> 236 us, 12 heads of 30,592 rows 667 -> 454.  (0 x inf is NaN: where a key cluster of one list holds an infinite
+// of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454.  (0 x inf is NaN: where a key cluster of one list holds an infinite
 // value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
 // descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
 // 400 cycles put into each step cost 46 us; now 4).
 // All roles run at the same time on one SM and have to fit its instruction cache
 // together: with the loops of the single-warp roles unrolled (105 KB of code) the same
-// kernel took 1.40 ms where it now takes 0.73 (2 x 16 heads of 20,000 rows, d = 128, 10
+// kernel took 1.40 ms where it now takes 0.72 (2 x 16 heads of 20,000 rows, d = 128, 10
 // clusters of 256 kept), so loops stay rolled unless a step is shorter for it.
 // What bounds it: at d = 128 no unit by itself.  A step brings 64 KB through L2, since every tile
-// loads its lists for itself, and takes 0.96 us (1,850 cycles of 1.92 GHz): 10.0 TB/s over the SMs of the
-// 14.6 that plain bulk loads of L2-resident data reach (51 bytes per cycle and SM, 0.66 us),
-// with the tensor pipe 62 % and the exponentials 61 % busy; the rest are hand-offs.  At d = 64 the
-// exponentials (1,024 of 1,340 cycles per step) and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
+// loads its lists for itself, and takes 0.945 us: 10.2 TB/s over the SMs of the
+// 14.6 that plain bulk loads of L2-resident data reach (0.66 us),
+// with the tensor pipe 63 % and the exponentials 62 % busy; the rest are hand-offs, and launches in a row
+// run at the power limit (745 us alone, 857 behind one another).  At d = 64 the
+// exponentials (1,024 of 1,270 cycles per step) and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
 // four at d = 64, half-steps of 64 keys in one chain per CTA): 40 heads of 32,760 rows,
-// d = 128, 32 of 256 clusters kept 2.91 -> 2.44 ms; 8 heads of 16,384 x 131,072, d = 64,
-// 128 of 1,024 kept 0.88 -> 0.80.
+// d = 128, 32 of 256 clusters kept 2.91 -> 2.40 ms; 8 heads of 16,384 x 131,072, d = 64,
+// 128 of 1,024 kept 0.88 -> 0.76.
 //
 // The softmax keeps a reference m per row instead of the exact running maximum: it is
 // measured on a row's first step and raised (by an integer) when a sum of 32
@@ -102,10 +103,13 @@ struct TcCfg {
   static constexpr int V_BYTES = PANELS * PANEL_BYTES;       // a value tile
   static constexpr uint32_t TMEM_COLS = 512;                 // kGroups x 128 score columns (P over 64 of them), D of O
   static constexpr int NK = kGroups;                         // key tiles in shared memory: one per score buffer
-  static constexpr int NV = (D == 64 || F8) ? 3 : 2;         // value tiles
+  static constexpr int NV = D == 64 ? 4 : F8 ? 3 : 2;        // value tiles
+  // Query tiles: two where there is room, so that the scores of a tile do not wait until its queries have come behind the last
+  // scores of the one before (with four value tiles for three, 8 heads of 16,384 x 131,072 rows 788 -> 758 us)
+  static constexpr int NQ = (D == 64 || F8) ? 2 : 1;
   // shared memory layout (offsets from a 1024-byte aligned base)
   static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + QK_BYTES;
+  static constexpr int OFF_K = OFF_Q + NQ * QK_BYTES;
   static constexpr int OFF_V = OFF_K + NK * QK_BYTES;
   static constexpr int OFF_BIAS = OFF_V + NV * V_BYTES;                  // [RING][128] floats
   static constexpr int OFF_LPART = OFF_BIAS + RING * kTile * 4;         // [kParts steps][128 rows] {row sum, reference}
@@ -116,7 +120,7 @@ struct TcCfg {
   static constexpr int OFF_FLAGS = OFF_TILE + RING * 16;
   static constexpr int OFF_SCALE = OFF_FLAGS + RING * 4;                // [RING][2] scales of the keys (F8)
   static constexpr int OFF_BAR = OFF_SCALE + RING * 8;
-  static constexpr int NUM_BARS = 2 + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV;
+  static constexpr int NUM_BARS = 1 + NQ + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;                // tmem base, abort flag, redo counts x 4
   static constexpr int OFF_BITMAP = OFF_MISC + 32;
   static_assert(OFF_TILE % 16 == 0 && OFF_BAR % 8 == 0 && OFF_MISC % 8 == 0, "alignment");
@@ -177,11 +181,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   int* st_flags = reinterpret_cast<int*>(smem + C::OFF_FLAGS);
   float* st_scale = reinterpret_cast<float*>(smem + C::OFF_SCALE);
   const uint32_t bar0 = s_base + C::OFF_BAR;
-  const uint32_t b_q_empty = bar0, b_o_empty = bar0 + 8;
+  const uint32_t b_o_empty = bar0;
+  auto b_q_empty = [&](int t) { return bar0 + 8 + 8 * (t % C::NQ); };   // the scores of tile t are complete
   // O of tile t is complete.  With tiles of one step three groups wait for three tiles at a time: a
   // barrier for each, so that no parity stands for two of them.
-  auto b_o_full = [&](int t) { return bar0 + 16 + 8 * (t & 3); };
-  const uint32_t bar1 = bar0 + 48;
+  auto b_o_full = [&](int t) { return bar0 + 8 + 8 * C::NQ + 8 * (t & 3); };
+  const uint32_t bar1 = bar0 + 40 + 8 * C::NQ;
   auto b_s_full = [&](int b) { return bar1 + 8 * b; };
   auto b_p_ready = [&](int b) { return bar1 + 8 * (kGroups + b); };
   auto b_step_full = [&](int s) { return bar1 + 8 * (2 * kGroups + s); };
@@ -201,7 +206,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const int box_rows = halves ? min(prm.c_k, kTile / 2) : min(prm.c_k, kTile);   // of a load of keys
 
   if (tid == 0) {
-    mbar_init(b_q_empty, 1); mbar_init(b_o_empty, 4);
+    mbar_init(b_o_empty, 4);
+#pragma unroll 1
+    for (int w = 0; w < C::NQ; ++w) mbar_init(b_q_empty(w), 1);
 #pragma unroll 1
     for (int b = 0; b < kGroups; ++b) { mbar_init(b_s_full(b), 1); mbar_init(b_p_ready(b), 4); }
 #pragma unroll 1
@@ -260,7 +267,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (++stops == kGroups) return;
             } else {
               if (key && (fl & kFFirst)) {
-                if (tiles > 0 && !relaxed(b_q_empty, tiles - 1)) return;
+                if (tiles >= C::NQ && !relaxed(b_q_empty(tiles), tiles / C::NQ - 1)) return;
+                const uint32_t q_dst = s_q + tiles % C::NQ * C::QK_BYTES;
                 ++tiles;
                 // Q arrives with the tile's first keys (scores of a half without a cluster are not read)
                 const bool one = halves && (fl & kFSingle) != 0;
@@ -269,7 +277,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 for (int half = 0; half <= (halves && !one ? 1 : 0); ++half)
 #pragma unroll
                   for (int pn = 0; pn < C::QK_PANELS; ++pn)
-                    tma_load_2d(s_q + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ] + half * 64, bar);
+                    tma_load_2d(q_dst + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ] + half * 64, bar);
               }
               if (!(fl & kFCentroid)) {
                 // 128 rows: one box, or several boxes
@@ -299,87 +307,106 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       }
     } else if (warp == 1) {
       // ---------------------------------------------------------- MMA issuer
-      // Every lane runs the loop (descriptor arithmetic stays warp-uniform); one elected lane issues
-      // the tensor-core instructions.  A wait on a barrier that has completed costs some 130
-      // cycles, so everything a step needs is waited for at once, one barrier per lane.
-      constexpr uint32_t idesc_qk = F8 ? idesc_e4m3_f32(kTile, kTile) : idesc_bf16_f32(kTile, kTile, 0, 0);
-      constexpr uint32_t idesc_qc = F8 ? idesc_e4m3_f32(kTile, kCen) : idesc_qk;      // centroid steps
-      constexpr uint32_t idesc_pv = idesc_bf16_f32(kTile, D, 0, 1);
-      auto wait = [&](uint32_t bar, uint32_t phase) {
-        return __all_sync(0xffffffffu, mbar_wait(bar, phase & 1, abort_flag, prm.status, prm.wait_limit));
-      };
-      // descriptors differ from a base one only in the start-address field (units of 16 bytes):
-      // the base descriptors are built once, the per-instruction part is an addition
-      const uint64_t q_desc0 = smem_desc_sw128(s_q, 16, 1024);
-      const uint64_t k_desc0 = smem_desc_sw128(s_k, 16, 1024);
-      const uint64_t v_desc0 = smem_desc_sw128(s_v, C::PANEL_BYTES, 1024);
-      int o_tiles = 0;
-      // scores of step u + kGroups, by one thread, into the buffer that P V (u) was issued from just before
-      auto scores = [&](int fl, int buf) {
-        if (fl & kFStop) {                    // wakes the group of this step, which ends with it
-          mbar_arrive(b_s_full(buf));
-          return;
-        }
-        const uint32_t d_cols = tmem_base + buf * kTile;
-        const uint64_t kd = k_desc0 + ((buf * C::QK_BYTES) >> 4);
-        const uint32_t idesc = (fl & kFCentroid) ? idesc_qc : idesc_qk;
-#pragma unroll
-        for (int ks = 0; ks < D / C::QK_KSTEP; ++ks) {
-          // K-major operands: 32 bytes (16 bf16 or 32 E4M3 elements) per instruction, four per panel
-          const uint32_t off = ((ks / 4) * C::PANEL_BYTES + (ks % 4) * 32) >> 4;
-          if (F8) mma_ss_f8(d_cols, q_desc0 + off, kd + off, idesc, ks > 0 ? 1u : 0u);
-          else mma_ss(d_cols, q_desc0 + off, kd + off, idesc, ks > 0 ? 1u : 0u);
-        }
-        mma_commit(b_s_full(buf));
-        if (fl & kFLast) mma_commit(b_q_empty);
-      };
-      static_assert(C::NK == kGroups, "key slots and score buffers go round together");
-      bool ok = true, first = true;           // `first`: P V of this step is the first one of a tile
-      int buf = 0, slot_v = 0, ring = 0;      // of the scores to issue; of P V
-      int fl0 = 0, fl1 = 0, fl2 = 0;          // flags of steps u, u + 1, u + 2
-      uint32_t ph_s = 0, ph_p = 0, ph_v = 0;  // phases of the keys of step u + kGroups, of P and of V of step u
-#pragma unroll 1
-      for (int u = -kGroups; ok; ++u) {
-        uint32_t bar = b_k_full(buf), phase = ph_s;
-        const int fl = fl0;
-        if (u >= 0) {
-          if (fl & kFStop) break;
-          if (lane == 1) { bar = b_p_ready(buf); phase = ph_p; }
-          if (lane == 2) { bar = b_v_full(slot_v); phase = ph_v; }
-        }
-        ok = wait(bar, phase);
-        if (u >= 0 && first && o_tiles > 0) ok = ok && wait(b_o_empty, o_tiles - 1);   // O of the tile before has been read
-        if (!ok) break;
-        const int fl_s = warp_uniform(st_flags[ring]);      // published: its keys have arrived
-        tc_fence_after();
-        if (elect_one()) {
-          if (u >= 0) {
+      // One thread issues all products: P V in the order of the steps, scores in the order of the steps and up to three
+      // steps ahead, either as soon as what it needs is there.  An instruction is issued when the one before it
+      // has been taken in, so that all that this thread does between products leaves the tensor core idle: with a warp that
+      // waited for one barrier after the other, voted and read the flags by shuffles 500 to 600 of the 1,600
+      // cycles of a step at d = 128.  It looks at all barriers at once and waits for none.  40 heads of 32,760
+      // rows, 32 of 256 clusters, d = 128 2,483 -> 2,395 us, 2 x 16 heads of 20,000 rows, 10 clusters of 256 749 -> 717, 12 heads of
+      // 16,385 rows, d = 64, clusters of 64 226 -> 221.  (One thread and one barrier after the other: 2,414, 727, 228.)
+      if (elect_one()) {
+        constexpr uint32_t idesc_qk = F8 ? idesc_e4m3_f32(kTile, kTile) : idesc_bf16_f32(kTile, kTile, 0, 0);
+        constexpr uint32_t idesc_qc = F8 ? idesc_e4m3_f32(kTile, kCen) : idesc_qk;      // centroid steps
+        constexpr uint32_t idesc_pv = idesc_bf16_f32(kTile, D, 0, 1);
+        // descriptors differ from a base one only in the start-address field (units of 16 bytes):
+        // the base descriptors are built once, the per-instruction part is an addition
+        const uint64_t q_desc0 = smem_desc_sw128(s_q, 16, 1024);
+        const uint64_t k_desc0 = smem_desc_sw128(s_k, 16, 1024);
+        const uint64_t v_desc0 = smem_desc_sw128(s_v, C::PANEL_BYTES, 1024);
+        int o_tiles = 0, q_tiles = 0;
+        // scores of step n, into the buffer that P V (n - kGroups) was issued from
+        auto scores = [&](int fl, int buf) {
+          if (fl & kFStop) {                    // wakes the group of this step, which ends with it
+            mbar_arrive(b_s_full(buf));
+            return;
+          }
+          const uint32_t d_cols = tmem_base + buf * kTile;
+          const uint64_t kd = k_desc0 + ((buf * C::QK_BYTES) >> 4);
+          const uint64_t qd = q_desc0 + (uint64_t)((q_tiles % C::NQ * C::QK_BYTES) >> 4);
+          const uint32_t idesc = (fl & kFCentroid) ? idesc_qc : idesc_qk;
+  #pragma unroll
+          for (int ks = 0; ks < D / C::QK_KSTEP; ++ks) {
+            // K-major operands: 32 bytes (16 bf16 or 32 E4M3 elements) per instruction, four per panel
+            const uint32_t off = ((ks / 4) * C::PANEL_BYTES + (ks % 4) * 32) >> 4;
+            if (F8) mma_ss_f8(d_cols, qd + off, kd + off, idesc, ks > 0 ? 1u : 0u);
+            else mma_ss(d_cols, qd + off, kd + off, idesc, ks > 0 ? 1u : 0u);
+          }
+          mma_commit(b_s_full(buf));
+          if (fl & kFLast) mma_commit(b_q_empty(q_tiles));
+        };
+        static_assert(C::NK == kGroups, "key slots and score buffers go round together");
+        bool first = true;                      // P V of step u is the first one of a tile
+        int u = 0, n = 0;                       // steps of the next P V, of the next scores
+        int buf_u = 0, buf_n = 0, slot_v = 0, ring = 0;
+        uint32_t ph_s = 0, ph_p = 0, ph_v = 0;  // phases of the keys of step n, of P and of V of step u
+        unsigned long long flags = 0;           // of steps u .. n - 1, 21 bits each
+        uint32_t idle = 0;
+        long long t0 = 0;
+  #pragma unroll 1
+        for (;;) {
+          const int fl = (int)flags & 0x1fffff;
+          if (n == u + kGroups && (fl & kFStop)) break;
+          const bool keys = mbar_test_wait(b_k_full(buf_n), ph_s);
+          const bool probabilities = mbar_test_wait(b_p_ready(buf_u), ph_p), value_rows = mbar_test_wait(b_v_full(slot_v), ph_v);
+          const int fl_n = reinterpret_cast<volatile int*>(st_flags)[ring];    // published when the keys have arrived
+          // (behind the first P V of a tile: O of the tile before has been read)
+          bool go = n > u && !(fl & kFStop) && probabilities && value_rows;
+          if (go && first && o_tiles > 0) go = mbar_test_wait(b_o_empty, (o_tiles - 1) & 1);
+          tc_fence_after();
+          if (go) {
             // V is MN-major: 16 key rows (2048 bytes) per instruction; panels along d
             const uint64_t vd = v_desc0 + ((slot_v * C::V_BYTES) >> 4);
-            const uint32_t p_cols = tmem_base + buf * kTile;
-#pragma unroll
+            const uint32_t p_cols = tmem_base + buf_u * kTile;
+  #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               mma_ts(tmem_o, p_cols + ks * 8, vd + (uint64_t)(ks * (2048 >> 4)), idesc_pv, (ks > 0 || !first) ? 1u : 0u);
             if (!(fl & kFCentroid)) {
-#pragma unroll
+  #pragma unroll
               for (int ks = 4; ks < 8; ++ks)
                 mma_ts(tmem_o, p_cols + ks * 8, vd + (uint64_t)(ks * (2048 >> 4)), idesc_pv, 1u);
             }
             mma_commit(b_v_empty(slot_v));
             if (fl & kFLast) mma_commit(b_o_full(o_tiles));
+            first = (fl & kFLast) != 0;
+            if (first) ++o_tiles;
+            flags >>= 21;
+            ++u;
+            if (++buf_u == kGroups) { buf_u = 0; ph_p ^= 1; }
+            if (++slot_v == C::NV) { slot_v = 0; ph_v ^= 1; }
           }
-          scores(fl_s, buf);
-        }
-        __syncwarp();
-        fl0 = fl1; fl1 = fl2; fl2 = fl_s;
-        if (++buf == kGroups) { buf = 0; ph_s ^= 1; if (u >= 0) ph_p ^= 1; }
-        if (++ring == C::RING) ring = 0;
-        if (u >= 0) {
-          first = (fl & kFLast) != 0;
-          if (first) ++o_tiles;
-          if (++slot_v == C::NV) { slot_v = 0; ph_v ^= 1; }
+          const bool more = keys && n < u + kGroups;
+          if (more) {
+            scores(fl_n, buf_n);
+            flags |= (unsigned long long)fl_n << (21 * (n - u));
+            if (C::NQ > 1 && (fl_n & kFLast)) ++q_tiles;
+            ++n;
+            if (++buf_n == kGroups) { buf_n = 0; ph_s ^= 1; }
+            if (++ring == C::RING) ring = 0;
+          }
+          if (go || more) { idle = 0; continue; }
+          if ((idle++ & 255u) == 0) {           // bounded, as every wait
+            const long long t = clock64();
+            if (idle == 1) t0 = t;
+            if (*abort_flag) break;
+            if (t - t0 > prm.wait_limit) {
+              *abort_flag = 1;
+              atomicExch(prm.status, 5 /* CA_ERR_TIMEOUT */);
+              break;
+            }
+          }
         }
       }
+      __syncwarp();
     } else {
       // ---------------------------------------------------------- tiles, lists, step descriptors
       const int per_head = prm.pairs ? (prm.n_qc + 1) >> 1 : prm.n_qc * tiles_per_qc;
