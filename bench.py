@@ -279,14 +279,15 @@ class ClockSampler:
 # ------------------------------------------------------------------------------
 # per-kernel rooflines of the clustering and selection stages
 # ------------------------------------------------------------------------------
-def split_level_counts(n, c):
+def split_level_counts(n, c, heads):
     """(levels run as per-level launches over whole sets, levels finished inside the subtree kernel):
-    sets of more than min(32 c, 4096) rows take a launch per level."""
+    sets of more than min(16 c, 1024) rows take a launch per level, or of more than 512 rows where the
+    subtrees of both sides then fit the 148 SMs one each."""
     def nxt(big):
         L = c * ((big + c) // (2 * c))
         return max(L, big - L)
     levels, top, big = 0, 0, n
-    tail_rows = min(32 * c, 4096)
+    tail_rows = min(16 * c, 512 if 2 * heads * -(-n // 512) <= 148 else 1024)
     while big > c:
         if big > tail_rows:
             top += 1
@@ -301,8 +302,8 @@ def stage_rooflines(w, heads, group_ms, hbm_gbs, peak_kind):
     alone), and the fraction of the roof that bounds it."""
     b = 2 if w.dtype == "bf16" else 4
     d, nq, nk, c = w.head_dim, w.n_q, w.n_k, w.cluster
-    top_q, tail_q = split_level_counts(nq, c)
-    top_k, tail_k = split_level_counts(nk, c)
+    top_q, tail_q = split_level_counts(nq, c, heads)
+    top_k, tail_k = split_level_counts(nk, c, heads)
     sub = lambda nodes: nodes * d * d * 4                      # subsample rows read by `nodes` sets
     algo = {
         # Gram matrices of Q, K and of the query representation r(q): bf16 reads Q once more, fp32 reads

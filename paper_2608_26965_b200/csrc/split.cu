@@ -37,8 +37,10 @@ constexpr int kSmemRowsMax = 24576;      // rows a CTA stages (8 bytes each)
 constexpr int kMaxCluster = 8;
 constexpr int kLevelBins = 1024;
 constexpr int kLevelList = 512;          // candidates that the level kernel ranks from a list
-constexpr int kTailRowsMax = 4096;
-constexpr int kTailSegs = 32;            // subsets a tail CTA splits side by side
+constexpr int kTailRowsMax = 1024;       // rows of a subtree
+constexpr int kTailSegs = 16;            // subsets a tail CTA splits side by side
+constexpr int kBasicRowsMax = 4096;      // the same of the basic variant
+constexpr int kBasicSegs = 32;
 
 struct SegmentRef { int lo, size, active; };
 
@@ -572,7 +574,7 @@ __device__ __forceinline__ bool pick_bin(uint32_t* hist, int rank, int lane, int
   uint4* h4 = reinterpret_cast<uint4*>(hist) + lane;
   const uint4 h = *h4;
   *h4 = make_uint4(0u, 0u, 0u, 0u);
-  const uint32_t pairs = (h.x + h.y) + (h.z + h.w);      // at most 4,096 rows: the halves do not overflow
+  const uint32_t pairs = (h.x + h.y) + (h.z + h.w);      // at most 1,024 rows: the halves do not overflow
   const int sum = (int)((pairs & 0xffffu) + (pairs >> 16));
   int incl = sum;
 #pragma unroll
@@ -644,7 +646,7 @@ __device__ __noinline__ void tail_thresholds_by_digits(TailSmem& sm, unsigned cr
 }
 
 // Subtree of a set of at most kTailRowsMax rows, finished by one CTA.  A level is a chain of short
-// stages between barriers (at most 32 subsets side by side), so its time is latency: loads from L2,
+// stages between barriers (at most 16 subsets side by side), so its time is latency: loads from L2,
 // shuffles, barriers, and the instruction fetch of a long loop body, which has to stay well below the
 // 32 KB that the SM keeps: the position loops are rolled and their state lives in shared memory.  Per level:
 // sample variances by independent warps (unit_variance); values gathered by asynchronous copies; the
@@ -652,13 +654,16 @@ __device__ __noinline__ void tail_thresholds_by_digits(TailSmem& sm, unsigned cr
 // the L-th value; the rows in that bin, ranked by one warp; the partition from ballots, where the
 // rows that go down before a subset are known beforehand (the L of the subsets to its left).  A bin with
 // more than 64 rows (values repeat, or far outliers stretch s) is resolved digit by digit.
-// Two CTAs of 512 threads share an SM; where all CTAs of both sides fit the SMs one each, 1,024 threads
-// (12 heads of 1,370 rows, d = 64: 43 -> 35 us a side).  With the earlier form (samples read twice between
-// barriers, two digits of counting, one CTA of 1,024 threads an SM) 12 x 1,370 rows took 52 us, 12 x
-// 16,385 rows 90 and now 47.  At d = 128 the sample rows are read from HBM (40 heads of 32,760 rows, 0.65 GB in
-// pieces of one row: 356 -> 315 us).
+// Four CTAs of 256 threads share an SM, or two of 512 where all CTAs of both sides fit that way (256 instead: 2 heads of
+// 1,024 rows 27 -> 33 us a side).  Subtrees of at most 4,096 rows, two CTAs of 512 threads to an SM, were the form before: CTAs
+// that run long leave the last wave nearly empty (40 heads of 32,760 rows, d = 128, 320 CTAs on 296 places: 285 us
+// a side, and 197 for 37 heads), and twice their 90 KB of shared memory leave too little L1 for the pieces of sample
+// rows in flight (1,024 rows to a CTA with 48 KB 285 us a side, with 33 KB 193).  Levels and subtrees of a side, before ->
+// after: 12 heads of 1,370 rows, d = 64: 36 -> 35 us, 12 x 16,385: 98 -> 94; 8 x 131,072 keys and 16,384 queries: 178 -> 161, 4 x
+// 5,003, d = 128: 83 -> 58; 40 x 32,760, d = 128: 373 -> 341.  At d = 128 the sample rows are read from HBM (0.65 GB a side in
+// pieces of one row).
 template <int D, int nt>
-__global__ void __launch_bounds__(nt, nt == 1024 ? 1 : 2) split_tail_kernel(const SplitParams prm) {
+__global__ void __launch_bounds__(nt, 1024 / nt) split_tail_kernel(const SplitParams prm) {
   wait_for_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TailSmem& sm = *reinterpret_cast<TailSmem*>(smem_raw);
@@ -871,15 +876,20 @@ static int max_segment_at_level(int n, int c, int level) {
   return big;
 }
 
-static int tail_rows_for(int c) {
-  const int r = kTailSegs * c;
-  return r < kTailRowsMax ? r : kTailRowsMax;
+// Rows of the sets that the subtree kernel starts from: at most 1,024, and half of that where all CTAs of both
+// sides then have an SM to themselves (a level costs a CTA with few rows less than it costs a launch; 4 heads of 5,003
+// rows, d = 128, clustering 465 us from 4,096 rows, 437 from 1,024, 436 from 512; 2 heads of 1,024 rows, d = 64 130, 129, 126;
+// 8 heads of 131,072 rows 573, 558, 567; 40 heads of 32,760 rows, d = 128 1,681, 1,662, 1,690).
+static int tail_rows_for(int n, int c, int problems) {
+  const int most = 2LL * problems * ceil_div(n, kTailRowsMax / 2) <= 148 ? kTailRowsMax / 2 : kTailRowsMax;
+  return min(kTailSegs * c, most);
 }
+static int basic_rows_for(int c) { return min(kBasicSegs * c, kBasicRowsMax); }
 
-// Levels [0, tail_level) run as per-level launches; the tail kernel finishes the rest.
-static int tail_level_for(int n, int c) {
+// Levels [0, tail_level) run as per-level launches; a subtree kernel finishes sets of at most `rows` rows.
+static int tail_level_for(int n, int c, int rows) {
   int level = 0;
-  for (int big = n; big > tail_rows_for(c); big = next_size(big, c)) ++level;
+  for (int big = n; big > rows; big = next_size(big, c)) ++level;
   return level;
 }
 
@@ -918,7 +928,8 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
                  const float* Ytq, const float* Ytk) {
   // sides: bit 0 = queries, bit 1 = keys
   const bool do_q = (sides & 1) != 0, do_k = (sides & 2) != 0;
-  const int tail_q = tail_level_for(n_q, c_q), tail_k = tail_level_for(n_k, c_k);
+  const int tail_q = tail_level_for(n_q, c_q, tail_rows_for(n_q, c_q, problems));
+  const int tail_k = tail_level_for(n_k, c_k, tail_rows_for(n_k, c_k, problems));
   const int top_q = do_q ? tail_q : 0, top_k = do_k ? tail_k : 0;
   const int top_levels = top_q > top_k ? top_q : top_k;
   SplitParams prm;
@@ -965,12 +976,11 @@ int launch_split(const float* Yq, const float* Yk, int problems, int D, int n_q,
   prm.level = top_levels;
   prm.smem_rows = 0;
   const int slots = 1 << ((do_q ? tail_q : 0) > (do_k ? tail_k : 0) ? (do_q ? tail_q : 0) : (do_k ? tail_k : 0));
-  const bool one_wave = 2 * slots * problems <= 148;      // both sides run at the same time
-  const int threads = one_wave ? 1024 : 512;
-  auto tail_kernel = D == 64 ? (one_wave ? split_tail_kernel<64, 1024> : split_tail_kernel<64, 512>)
-                             : (one_wave ? split_tail_kernel<128, 1024> : split_tail_kernel<128, 512>);
+  const bool few = 2LL * slots * problems <= 296;          // both sides run at the same time
+  auto tail_kernel = D == 64 ? (few ? split_tail_kernel<64, 512> : split_tail_kernel<64, 256>)
+                             : (few ? split_tail_kernel<128, 512> : split_tail_kernel<128, 256>);
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TailSmem)));
-  launch_chained(tail_kernel, dim3(slots, prm.sides * problems), threads, sizeof(TailSmem), st, prm);
+  launch_chained(tail_kernel, dim3(slots, prm.sides * problems), few ? 512 : 256, sizeof(TailSmem), st, prm);
   CA_LAUNCH_CHECK();
   return CA_OK;
 }
@@ -1225,12 +1235,12 @@ __global__ void __launch_bounds__(256) basic_keys_kernel(const BasicParams prm) 
 // the stable partition into rows_next.  A thread owns the four consecutive positions 4 tid .. 4 tid + 3
 // (my_seg: subset of a position, -1 - g in a final subset, INT_MIN past the end; my_key: its key).
 template <typename Smem>
-__device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_seg)[kTailRowsMax / kSplitThreads],
-                                                      const uint32_t (&my_key)[kTailRowsMax / kSplitThreads],
+__device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_seg)[kBasicRowsMax / kSplitThreads],
+                                                      const uint32_t (&my_key)[kBasicRowsMax / kSplitThreads],
                                                       int nseg, const int* slo, const int32_t* rows,
                                                       int32_t* rows_next, int tid, int* hist, uint32_t* scan) {
   constexpr int nt = kSplitThreads;
-  constexpr int PT = kTailRowsMax / kSplitThreads;
+  constexpr int PT = kBasicRowsMax / kSplitThreads;
   const int lane = tid & 31, warp = tid >> 5;
   // ---- radix selection, all subsets side by side: two digits of eight bits by counting; then the
   // keys that share those sixteen bits with the threshold are few (a handful per subset unless keys
@@ -1383,7 +1393,7 @@ __device__ __forceinline__ void tail_select_partition(Smem& sm, const int (&my_s
   }
 }
 
-// Subtree of the basic variant: a set of at most kTailRowsMax rows finished by one CTA, so that
+// Subtree of the basic variant: a set of at most kBasicRowsMax rows finished by one CTA, so that
 // the deepest levels are one launch instead of three per level.  Per level: the directions of all
 // subsets that still split (a team of D threads per subset; the operations of
 // basic_direction_kernel in the same order -- the sample rows are staged as stored and centred
@@ -1398,19 +1408,19 @@ constexpr int kBasicStage = 131072;
 template <int D>
 struct BasicTailSmem {
   static constexpr int TEAMS = kSplitThreads / D;
-  int32_t rows[2][kTailRowsMax];
+  int32_t rows[2][kBasicRowsMax];
   __align__(16) unsigned char stage[kBasicStage];
-  float dirs[2][kTailSegs][D];            // directions of this level's subsets and of the level above
+  float dirs[2][kBasicSegs][D];            // directions of this level's subsets and of the level above
   __align__(16) float mu[TEAMS][D], u[TEAMS][D], v[TEAMS][D], w[TEAMS][D], y[TEAMS][D], g[TEAMS][D];
   float4 metric[D == 64 ? D * D / 4 : 1];   // d = 64: the metric, chunks of a row placed as above (d = 128: no room)
-  int seg_lo[2][2 * kTailSegs + 2];
-  int seg_slot[2][2 * kTailSegs + 2];     // slot of a subset in the tree, at the level it stands on
-  int seg_par[2][2 * kTailSegs + 2];      // subset of the level above it came from
-  int seg_digit[kTailSegs], seg_rem[kTailSegs], seg_L[kTailSegs];
-  int seg_cand[kTailSegs];                // candidates left after the first two digits; -1: threshold found
+  int seg_lo[2][2 * kBasicSegs + 2];
+  int seg_slot[2][2 * kBasicSegs + 2];     // slot of a subset in the tree, at the level it stands on
+  int seg_par[2][2 * kBasicSegs + 2];      // subset of the level above it came from
+  int seg_digit[kBasicSegs], seg_rem[kBasicSegs], seg_L[kBasicSegs];
+  int seg_cand[kBasicSegs];                // candidates left after the first two digits; -1: threshold found
   int overflow;                           // some subset has more candidates than a warp takes
-  uint32_t seg_prefix[kTailSegs];
-  int split_list[kTailSegs];              // the subsets that still split
+  uint32_t seg_prefix[kBasicSegs];
+  int split_list[kBasicSegs];              // the subsets that still split
   int warp_tot[32];
   int nseg[2];
   int nsplit;
@@ -1429,10 +1439,10 @@ __global__ void __launch_bounds__(kSplitThreads) basic_tail_kernel(const BasicPa
   constexpr int NODE_BYTES = D * V * 16;
   constexpr int ROUND = (kBasicStage / NODE_BYTES) < Sm::TEAMS ? (kBasicStage / NODE_BYTES) : Sm::TEAMS;
   static_assert(ROUND >= 1, "a subset's sample must fit the staging area");
-  constexpr int PT = kTailRowsMax / kSplitThreads;
-  static_assert(PT == 4 && kTailRowsMax * 4 + kTailSegs * 256 * 4 <= kBasicStage && nt / 32 * 4096 <= kBasicStage, "scan, digit counts and projected rows live in the staging area");
+  constexpr int PT = kBasicRowsMax / kSplitThreads;
+  static_assert(PT == 4 && kBasicRowsMax * 4 + kBasicSegs * 256 * 4 <= kBasicStage && nt / 32 * 4096 <= kBasicStage, "scan, digit counts and projected rows live in the staging area");
   uint32_t* scan = reinterpret_cast<uint32_t*>(sm.stage);
-  int* hist = reinterpret_cast<int*>(sm.stage + kTailRowsMax * 4);
+  int* hist = reinterpret_cast<int*>(sm.stage + kBasicRowsMax * 4);
 
   const int which = blockIdx.y / prm.problems, p = blockIdx.y % prm.problems;
   const BasicSide bs = prm.side[which];
@@ -1709,10 +1719,10 @@ static int launch_split_basic_t(const T* Q, const T* K, const float* A_q, const 
                                 int32_t* perm_k_out, int32_t* perm_k_tmp, uint32_t* keybuf_q, uint32_t* keybuf_k,
                                 LaunchStream st) {
   const int lev_q = split_levels_for(n_q, c_q), lev_k = split_levels_for(n_k, c_k);
-  // Sets of more than kTailRowsMax rows take three launches per level (directions, projections,
+  // Sets of more than kBasicRowsMax rows take three launches per level (directions, projections,
   // select + partition); the subtree kernel finishes the rest.  Per-level launches write alternately
   // to tmp/out so that the subtree kernel, which runs last, reads the buffer that is not the output.
-  const int tail_q = tail_level_for(n_q, c_q), tail_k = tail_level_for(n_k, c_k);
+  const int tail_q = tail_level_for(n_q, c_q, basic_rows_for(c_q)), tail_k = tail_level_for(n_k, c_k, basic_rows_for(c_k));
   const int top = tail_q > tail_k ? tail_q : tail_k;
   BasicParams bp;
   bp.problems = problems; bp.iterations = iterations;

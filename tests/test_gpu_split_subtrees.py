@@ -34,6 +34,9 @@ def _coordinates(kind, heads, n, d, seed):
     ("outliers", 1, 4096, 128, 256), ("outliers", 80, 1030, 64, 64), ("outliers", 40, 2000, 128, 64),
     ("repeated", 2, 4095, 64, 128), ("repeated", 80, 700, 128, 32),
     ("two values", 1, 4096, 64, 128), ("huge", 1, 2049, 64, 64), ("huge", 80, 600, 128, 64),
+    # subtrees of at most 512 rows, of 1,024, and one row more; 512 threads and 256
+    ("normal", 1, 513, 128, 64), ("normal", 24, 1536, 64, 64), ("outliers", 25, 1537, 128, 64), ("normal", 148, 1024, 64, 128),
+    ("repeated", 149, 1024, 128, 64), ("two values", 75, 2049, 64, 256),
 ])
 def test_subtrees_match_the_oracle(kind, heads, n, d, c):
     Y = _coordinates(kind, heads, n, d, n + d)
