@@ -28,6 +28,61 @@ __device__ __forceinline__ void clear_status(int* status) {
   if (status && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(int)) status[threadIdx.x] = 0;
 }
 
+// The `keep` largest of a row's n keys (ties: lower index), in ascending order of index, by one warp.  row[j] the keys in
+// shared memory, 16-byte aligned, 0 from n up to a multiple of 128.  The keep-th largest is found bit by bit from
+// counts of the keys at or above a candidate, until as many as are wanted stand there: no barriers.  (A count is 250
+// cycles and 40 per 128 keys, and 8 to 20 are needed.  Candidates interpolated between the scores, ten counts for eighteen, and
+// three candidates to a count took longer.)
+__device__ __forceinline__ void select_row(const uint32_t* row, int n, int keep, int32_t* __restrict__ out, int lane) {
+  const int quads = (n + 127) >> 7;
+  const uint4* mine = reinterpret_cast<const uint4*>(row) + lane;
+  auto count = [&](uint32_t least) {
+    int c0 = 0, c1 = 0, c2 = 0, c3 = 0;
+#pragma unroll 4
+    for (int i = 0; i < quads; ++i) {
+      const uint4 k = mine[32 * i];
+      c0 += k.x >= least ? 1 : 0;
+      c1 += k.y >= least ? 1 : 0;
+      c2 += k.z >= least ? 1 : 0;
+      c3 += k.w >= least ? 1 : 0;
+    }
+    return (int)__reduce_add_sync(0xffffffffu, (c0 + c1) + (c2 + c3));
+  };
+  uint32_t threshold = 0;
+  int from = 0;                                          // keys at or above it
+#pragma unroll 1
+  for (uint32_t bit = 1u << 31; bit != 0 && from != keep; bit >>= 1) {
+    const int c = count(threshold | bit);
+    if (c >= keep) {
+      threshold |= bit;
+      from = c;
+    }
+  }
+  const unsigned before = (1u << lane) - 1u;
+  if (from == keep) {
+#pragma unroll 4
+    for (int j0 = 0; j0 < n; j0 += 32) {
+      const bool in = (j0 + lane < n ? row[j0 + lane] : 0u) >= threshold;       // (the threshold is not 0)
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (in) out[__popc(b & before)] = j0 + lane;
+      out += __popc(b);
+    }
+    return;
+  }
+  // several keys are equal to the keep-th largest: the first ones of them
+  int wanted = keep - (threshold == 0xffffffffu ? 0 : count(threshold + 1));
+#pragma unroll 1
+  for (int j0 = 0; j0 < n; j0 += 32) {
+    const uint32_t k = j0 + lane < n ? row[j0 + lane] : 0u;            // 0: not above, and the last of its equals
+    const unsigned g = __ballot_sync(0xffffffffu, k > threshold), e = __ballot_sync(0xffffffffu, k == threshold);
+    const int at = __popc(g & before), rank = __popc(e & before);
+    if (k > threshold || (k == threshold && rank < wanted)) out[at + min(rank, wanted)] = j0 + lane;
+    const int taken = min(__popc(e), wanted);
+    out += __popc(g) + taken;
+    wanted -= taken;
+  }
+}
+
 // QT query clusters per CTA: 4 when the CTA computes the scores itself (the key centroids are read
 // once for the four), 1 when the scores come from memory (less shared memory, more CTAs per SM).
 template <int D, int QT>
@@ -39,8 +94,10 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
   let_next_start();
   clear_status(status);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);                       // [QT][n_kc]
-  float* qs = reinterpret_cast<float*>(keys + (size_t)QT * n_kc);        // [QT][D]
+  const bool by_warps = QT > 1 && n_kc <= 128;           // the selection by a warp per row, without barriers
+  const int ld = by_warps ? 128 : n_kc;
+  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);                       // [QT][ld]
+  float* qs = reinterpret_cast<float*>(keys + (size_t)QT * ld);          // [QT][D]
   __shared__ int s_hist[QT][256];
   __shared__ int s_warp[QT][64];
   __shared__ int s_scalar[QT][4];
@@ -65,6 +122,7 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
 #pragma unroll
     for (int t = 0; t < QT; ++t) acc[t] = 0.f;
     const float4* row = reinterpret_cast<const float4*>(ckp + (size_t)j * D);
+#pragma unroll 8
     for (int k4 = 0; k4 < D / 4; ++k4) {
       const float4 kv = __ldg(row + k4);
 #pragma unroll
@@ -77,10 +135,20 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
       }
     }
 #pragma unroll
-    for (int t = 0; t < QT; ++t) keys[(size_t)t * n_kc + j] = score_key(acc[t]);
+    for (int t = 0; t < QT; ++t) keys[(size_t)t * ld + j] = score_key(acc[t]);
   }
   }
   __syncthreads();
+
+  if (by_warps) {
+    if (warp < nq) {
+#pragma unroll 1
+      for (int j = n_kc + lane; j < ld; j += 32) keys[(size_t)warp * ld + j] = 0u;
+      __syncwarp();
+      select_row(keys + (size_t)warp * ld, n_kc, keep, block_idx + ((size_t)p * n_qc + q0 + warp) * keep, lane);
+    }
+    return;
+  }
 
   // ---- radix selection of the keep-th largest key, the QT rows side by side (one set of barriers
   // for all of them: a row on its own is bound by the barriers of its passes, not by work)
@@ -194,8 +262,37 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
   }
 }
 
+// Selection from scores in memory by a warp per row, its keys in shared memory.  A CTA per row counts digits between
+// barriers, 16 to 20 of them: bound by their latency, eight rows to an SM at a time.  A warp takes longer for a long row,
+// with a dozen times as many of them on an SM: taken where the rows are more than the SMs, of more than 512 key clusters
+// where they are more than eight per SM (scores and selection, CTA -> warp per row: 12 heads of 257 x 257 clusters 31 -> 24
+// us, 40 of 256 x 256 85 -> 56, 40 of 591 x 591 345 -> 247, 16 of 1,024 x 1,024 323 -> 255; left as they are: 8 heads of
+// 128 x 1,024 20.2 -> 21.6, 8 of 12 x 181 within a forward pass 267 -> 269).
+constexpr int kWarpRows = 4;
+static bool select_by_warps(int n_kc, long long rows) { return n_kc <= 1024 && rows > (n_kc <= 512 ? 148 : 8 * 148); }
+__global__ void __launch_bounds__(32 * kWarpRows)
+select_rows_kernel(const float* __restrict__ scores, int n_qc, int n_kc, int keep, int32_t* __restrict__ block_idx,
+                   int row0, int chunk_rows, int* __restrict__ status) {
+  wait_for_previous();
+  let_next_start();
+  clear_status(status);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int padded = (n_kc + 127) & ~127;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.y, r = blockIdx.x * kWarpRows + warp, q = row0 + r;
+  if (r >= chunk_rows || q >= n_qc) return;
+  const float* row = scores + ((size_t)p * chunk_rows + r) * n_kc;
+  uint32_t* mine = reinterpret_cast<uint32_t*>(smem_raw) + warp * padded;
+#pragma unroll 8
+  for (int j = lane; j < padded; j += 32) {
+    const float score = __ldg(row + min(j, n_kc - 1));
+    mine[j] = j < n_kc ? score_key(score) : 0u;
+  }
+  __syncwarp();
+  select_row(mine, n_kc, keep, block_idx + ((size_t)p * n_qc + q) * keep, lane);
+}
+
 size_t select_smem_bytes(int n_kc, int D, int qt) {
-  return (size_t)qt * n_kc * sizeof(uint32_t) + (size_t)qt * D * sizeof(float);
+  return (size_t)qt * (qt > 1 && n_kc < 128 ? 128 : n_kc) * sizeof(uint32_t) + (size_t)qt * D * sizeof(float);
 }
 
 // ---------------------------------------------------------------------------
@@ -329,19 +426,27 @@ int launch_score_select(const float* cq, const float* ck, int P, int n_qc, int n
     CA_LAUNCH_CHECK();
     return CA_OK;
   }
-  size_t smem = select_smem_bytes(n_kc, D, 1);
+  const bool by_warps = select_by_warps(n_kc, (long long)min(chunk, n_qc) * P);
+  const size_t warp_smem = (size_t)kWarpRows * ((n_kc + 127) & ~127) * sizeof(uint32_t);
+  size_t smem = by_warps ? warp_smem : select_smem_bytes(n_kc, D, 1);
   if (smem > 200 * 1024) return CA_ERR_UNSUPPORTED;
-  smem = spread_smem(smem, 2048, (long long)min(chunk, n_qc) * P);
+  smem = by_warps ? spread_smem(smem, 0, (long long)ceil_div(min(chunk, n_qc), kWarpRows) * P)
+                  : spread_smem(smem, 2048, (long long)min(chunk, n_qc) * P);
   auto k64 = score_select_kernel<64, 1>;
   auto k128 = score_select_kernel<128, 1>;
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (by_warps) {
+    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(select_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  } else {
+    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  }
   for (int row0 = 0; row0 < n_qc; row0 += chunk) {
     const int rows = min(chunk, n_qc - row0);
     if (D == 64) { int rc = launch_score_tiles<64>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
     else { int rc = launch_score_tiles<128>(cq, ck, P, n_qc, n_kc, row0, chunk, score_ws, st); if (rc != CA_OK) return rc; }
-    dim3 grid(rows, P);
-    if (D == 64) launch_chained(k64, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
+    dim3 grid(by_warps ? ceil_div(rows, kWarpRows) : rows, P);
+    if (by_warps) launch_chained(select_rows_kernel, grid, 32 * kWarpRows, smem, st, score_ws, n_qc, n_kc, keep, block_idx, row0, chunk, status);
+    else if (D == 64) launch_chained(k64, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
     else launch_chained(k128, grid, kSelectThreads, smem, st, cq, ck, n_qc, n_kc, keep, block_idx, score_ws, row0, chunk, status);
     CA_LAUNCH_CHECK();
   }

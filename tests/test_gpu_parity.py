@@ -191,7 +191,10 @@ def test_cluster_qk_transforms_and_split(name, H, n_q, n_k):
 # Block selection on the oracle's centroids (rounded to fp32): exact lists.
 # ----------------------------------------------------------------------------
 @pytest.mark.parametrize("H,n_qc,n_kc,d,keep", [(2, 16, 16, 64, 4), (1, 37, 300, 128, 1), (1, 5, 300, 64, 300),
-                                                  (2, 130, 1024, 64, 128), (1, 9, 2049, 128, 77)])
+                                                  (2, 130, 1024, 64, 128), (1, 9, 2049, 128, 77),
+                                                  # a warp per row: fused, to 512 clusters, to 1,024 for many rows
+                                                  (1, 9, 127, 64, 127), (2, 7, 128, 128, 9), (30, 6, 129, 64, 128), (5, 33, 512, 64, 500),
+                                                  (5, 33, 513, 64, 50), (4, 300, 520, 64, 65), (2, 600, 1024, 128, 1)])
 def test_select_blocks_exact(H, n_qc, n_kc, d, keep):
     r = np.random.default_rng(n_qc * n_kc)
     cq = r.standard_normal((H, n_qc, d)).astype(np.float32)
