@@ -23,8 +23,9 @@
 // have 64 to 86 % of their entries in common on the inputs measured).  A key cluster that both lists hold is taken once, by all rows;
 // one that a single list holds by the rows of that half, next to one of the other list (the other probabilities of a row
 // are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
-// loaded into both halves that divided the keys of a step between them, was the form before: 12 heads of 16,385 rows, 33
-// of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454.  (0 x inf is NaN: where a key cluster of one list holds an infinite
+// in both halves that divide the keys of a step between them and merge their outputs, was the only form before (12 heads of
+// 16,385 rows, 33 of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454) and stays where the clusters are no more than
+// the SMs (4 heads of 512 x 131,072 rows 192 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
 // value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
 // descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
 // 400 cycles put into each step cost 46 us; now 4).
@@ -120,7 +121,7 @@ struct TcCfg {
   static constexpr int OFF_FLAGS = OFF_TILE + RING * 16;
   static constexpr int OFF_SCALE = OFF_FLAGS + RING * 4;                // [RING][2] scales of the keys (F8)
   static constexpr int OFF_BAR = OFF_SCALE + RING * 8;
-  static constexpr int NUM_BARS = 1 + NQ + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV;
+  static constexpr int NUM_BARS = 1 + NQ + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV + (HALVES ? 4 : 0);
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;                // tmem base, abort flag, redo counts x 4
   static constexpr int OFF_BITMAP = OFF_MISC + 32;
   static_assert(OFF_TILE % 16 == 0 && OFF_BAR % 8 == 0 && OFF_MISC % 8 == 0, "alignment");
@@ -194,6 +195,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   auto b_k_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + s); };
   auto b_v_full = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + C::NK + s); };
   auto b_v_empty = [&](int s) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + C::NK + C::NV + s); };
+  // hand-over between the halves of a cluster whose rows stand in both, by warp of a half
+  auto b_m_full = [&](int w) { return bar1 + 8 * (2 * kGroups + 2 * C::RING + C::NK + 2 * C::NV + w); };
+  auto b_m_empty = [&](int w) { return b_m_full(2 + w); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
   int* redo_acc = reinterpret_cast<int*>(smem + C::OFF_MISC + 8);
@@ -203,6 +207,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   // a query cluster of 256 rows takes two tiles; two of 64 rows (or one) share one
   const int tiles_per_qc = prm.c_q >= kTile ? prm.c_q / kTile : 1;
   constexpr bool halves = HALVES;
+  const bool twice = halves && !prm.pairs;     // too few clusters for pairs: the rows of one stand in both halves
   const int box_rows = halves ? min(prm.c_k, kTile / 2) : min(prm.c_k, kTile);   // of a load of keys
 
   if (tid == 0) {
@@ -219,6 +224,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     for (int s = 0; s < C::NV; ++s) { mbar_init(b_v_full(s), 1); mbar_init(b_v_empty(s), 1); }
 #pragma unroll 1
     for (int w = 0; w < 4; ++w) mbar_init(b_o_full(w), 1);
+    if (halves)
+#pragma unroll 1
+      for (int w = 0; w < 4; ++w) mbar_init(b_m_full(w), 1);
     *abort_flag = 0;
     for (int b = 0; b < 4; ++b) redo_acc[b] = 0;
     fence_mbar_init();
@@ -271,13 +279,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 const uint32_t q_dst = s_q + tiles % C::NQ * C::QK_BYTES;
                 ++tiles;
                 // Q arrives with the tile's first keys (scores of a half without a cluster are not read)
-                const bool one = halves && (fl & kFSingle) != 0;
+                const bool one = halves && (fl & kFSingle) != 0 && !twice;
                 mbar_expect_more(bar, one ? C::QK_BYTES / 2 : C::QK_BYTES);
 #pragma unroll 1
                 for (int half = 0; half <= (halves && !one ? 1 : 0); ++half)
 #pragma unroll
                   for (int pn = 0; pn < C::QK_PANELS; ++pn)
-                    tma_load_2d(q_dst + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ] + half * 64, bar);
+                    tma_load_2d(q_dst + pn * C::PANEL_BYTES + half * 64 * 128, &tm_q, pn * C::QK_PANEL_COLS, rows[kRowQ] + (twice ? 0 : half * 64), bar);
               }
               if (!(fl & kFCentroid)) {
                 // 128 rows: one box, or several boxes
@@ -456,7 +464,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           //   shared       two runs of both lists per step
           //   split        a run of the upper list, for the upper half, and one of the lower
           //   one-sided    two runs of the list that is longer than the other
-          // which are never more steps than two tiles of one cluster each.  (A list that holds a cluster twice
+          // which are never more steps than two tiles of one cluster each.  Where clusters are not paired for lack of tiles, the
+          // rows of a cluster stand in both halves (twice): a half takes a run of each step, the upper one the centroids.  (A list that holds a cluster twice
           // counts it twice: then nothing is shared.)
           const int qc = prm.pairs ? 2 * x : x;
           const bool single = !prm.pairs || qc + 1 == prm.n_qc;
@@ -568,7 +577,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (F8 && box < 2) st_scale[slot * 2 + box] = prm.c_scale[(size_t)p * prm.cen_tiles + i];
             }
             if (starts) {
-              st_flags[slot] = (single ? kFSingle | kFUpper : 0) | (runs0 + runs1 > 0 ? kFMixed : 0) | (u == 0 ? kFFirst : 0) |
+              st_flags[slot] = (!single ? 0 : kFSingle | (twice && shared ? kFSplit : kFUpper)) | (twice || runs0 + runs1 > 0 ? kFMixed : 0) | (u == 0 ? kFFirst : 0) |
                                (u == n - 1 ? kFLast : 0) | (min(u, 15) << kFIndexShift) | (min(n - 1 - u, 15) << kFRestShift) |
                                (split ? kFSplit : one ? (longer ? kFLower : kFUpper) : 0) | (cen ? kFCentroid : 0) |
                                (cen || ((cut >> (lane & 24)) & 255u) ? kFMasked : 0);
@@ -943,20 +952,82 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (other.y > -INFINITY) l_run += other.x * ex2_approx(other.y - m_ref);
         }
       }
-      float l_all = l_run;
+      // Rows that stand in both halves: the lower one hands over its sum and reference, then eight columns of O at a time,
+      // which the upper one scales to the larger reference.
+      float l_all = l_run, m_all = m_ref, w_own = 1.f, w_other = 0.f;
+      float* merge = reinterpret_cast<float*>(smem + C::OFF_QUEUE + kQueue * 16) + (row & 63);     // [8][64], no lists wait there
+      const int pair = quarter & 1;
+      int use = tl.w * (1 + D / 8);
+      bool got = true;
+      auto take = [&]() { return wait(b_m_full(pair), use); };
+      auto taken = [&]() {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b_m_empty(pair));
+        ++use;
+      };
+      if (twice && half == 1) {
+        auto room = [&]() { return use == 0 || wait(b_m_empty(pair), use - 1); };
+        auto handed = [&]() {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_m_full(pair));
+          ++use;
+        };
+        got = room();
+        if (!got) break;
+        merge[0] = l_run;
+        merge[64] = m_ref;
+        handed();
+#pragma unroll 1
+        for (int c = 0; c < D / 16 && got; ++c) {
+          uint32_t o[16];
+          tmem_ld16(tmem_o + lane_addr + c * 16, o);
+          tmem_wait_ld();
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            got = got && room();
+            if (!got) break;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) merge[64 * j] = __uint_as_float(o[8 * h + j]);
+            handed();
+          }
+        }
+        if (!got) break;
+      }
+      if (twice && half == 0) {
+        got = take();
+        if (!got) break;
+        const float l_other = merge[0], m_other = merge[64];
+        taken();
+        m_all = fmaxf(m_ref, m_other);
+        w_own = m_ref > -INFINITY ? ex2_approx(m_ref - m_all) : 0.f;
+        w_other = m_other > -INFINITY ? ex2_approx(m_other - m_all) : 0.f;
+        l_all = l_run * w_own + l_other * w_other;
+      }
       // a row without a single live entry (an empty list without compensation): zeros, lse = -inf
       const bool empty = !(l_all > 0.f);
       const float inv = empty ? 0.f : 1.f / l_all;
       __nv_bfloat16* out = prm.O + ((size_t)tl.x * prm.n_q + orig) * D;
       // 0 x inf, an infinite value among the other half's keys: for the second pass
       const bool check = halves && (fl & kFMixed) != 0;
+      const float inv_own = inv * w_own, inv_other = inv * w_other;
 #pragma unroll 1
-      for (int c = 0; c < D / 16; ++c) {
+      for (int c = 0; c < (twice && half == 1 ? 0 : D / 16); ++c) {
         uint32_t o[16];
         tmem_ld16(tmem_o + lane_addr + c * 16, o);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv);
+        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv_own);
+        if (twice) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            got = got && take();
+            if (!got) break;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) o[8 * h + j] = __float_as_uint(fmaf(merge[64 * j], inv_other, __uint_as_float(o[8 * h + j])));
+            taken();
+          }
+          if (!got) break;
+        }
         if (check) {
           f32x2 any2 = pack2(0.f, 0.f);
 #pragma unroll
@@ -980,11 +1051,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           }
         }
       }
+      if (!got) break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(b_o_empty);
       if (live && prm.lse)
-        prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_ref + log2f(l_all)) * 0.6931471805599453f;
+        prm.lse[(size_t)tl.x * prm.n_q + orig] = empty ? -INFINITY : (m_all + log2f(l_all)) * 0.6931471805599453f;
       // one word per tile or 64-row query cluster, written on every launch by the last of its four warps: 1 = recompute
       // (a row left the range)
       const bool redo = __any_sync(0xffffffffu, live && !(l_all < INFINITY));

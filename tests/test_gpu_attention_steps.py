@@ -182,13 +182,14 @@ def test_values_with_infinities(d, c_q, c_k, keep, compensate):
 
 
 @pytest.mark.parametrize("compensate", [False, True])
+@pytest.mark.parametrize("heads", [9, 2])
 @pytest.mark.parametrize("d,c_k,infinite", [(64, 64, False), (64, 16, False), (128, 32, False), (128, 64, False), (64, 128, False), (128, 256, False),
                                             (64, 64, True), (128, 128, True)])
-def test_pairs_of_64_row_query_clusters(d, c_k, infinite, compensate):
+def test_pairs_of_64_row_query_clusters(d, c_k, infinite, compensate, heads):
     """More 64-row query clusters than SMs go two to a tile, with the key clusters of both lists taken once: lists that
     share everything, something and nothing, of the same and of very different lengths, empty ones, in any order, with a
-    cluster twice, an odd number of clusters per head."""
-    heads, n_qc, n_kc = 9, 35, 45
+    cluster twice, an odd number of clusters per head.  Fewer stand in both halves of a tile, each with half of the keys."""
+    n_qc, n_kc = 35, 45
     n_q, n_k = 64 * n_qc - 17, c_k * n_kc - 5
     Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, 64, c_k, d + c_k)
     if infinite:
