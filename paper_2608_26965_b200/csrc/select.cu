@@ -264,12 +264,11 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
 
 // Selection from scores in memory by a warp per row, its keys in shared memory.  A CTA per row counts digits between
 // barriers, 16 to 20 of them: bound by their latency, eight rows to an SM at a time.  A warp takes longer for a long row,
-// with a dozen times as many of them on an SM: taken where the rows are more than the SMs, of more than 512 key clusters
-// where they are more than eight per SM (scores and selection, CTA -> warp per row: 12 heads of 257 x 257 clusters 31 -> 24
-// us, 40 of 256 x 256 85 -> 56, 40 of 591 x 591 345 -> 247, 16 of 1,024 x 1,024 323 -> 255; left as they are: 8 heads of
-// 128 x 1,024 20.2 -> 21.6, 8 of 12 x 181 within a forward pass 267 -> 269).
+// with a dozen times as many of them on an SM: taken where a CTA per row would take more than one round (scores and selection,
+// CTA -> warp per row: 12 heads of 257 x 257 clusters 31 -> 24 us, 40 of 256 x 256 85 -> 56, 40 of 591 x 591 345 -> 247, 16 of
+// 1,024 x 1,024 323 -> 255; left as they are: 8 heads of 128 x 1,024 20.2 -> 21.6, 2 of 140 x 305 12 -> 14).
 constexpr int kWarpRows = 4;
-static bool select_by_warps(int n_kc, long long rows) { return n_kc <= 1024 && rows > (n_kc <= 512 ? 148 : 8 * 148); }
+static bool select_by_warps(int n_kc, long long rows) { return n_kc <= 1024 && rows > 8 * 148; }
 __global__ void __launch_bounds__(32 * kWarpRows)
 select_rows_kernel(const float* __restrict__ scores, int n_qc, int n_kc, int keep, int32_t* __restrict__ block_idx,
                    int row0, int chunk_rows, int* __restrict__ status) {

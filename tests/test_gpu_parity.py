@@ -192,9 +192,9 @@ def test_cluster_qk_transforms_and_split(name, H, n_q, n_k):
 # ----------------------------------------------------------------------------
 @pytest.mark.parametrize("H,n_qc,n_kc,d,keep", [(2, 16, 16, 64, 4), (1, 37, 300, 128, 1), (1, 5, 300, 64, 300),
                                                   (2, 130, 1024, 64, 128), (1, 9, 2049, 128, 77),
-                                                  # a warp per row: fused, to 512 clusters, to 1,024 for many rows
-                                                  (1, 9, 127, 64, 127), (2, 7, 128, 128, 9), (30, 6, 129, 64, 128), (5, 33, 512, 64, 500),
-                                                  (5, 33, 513, 64, 50), (4, 300, 520, 64, 65), (2, 600, 1024, 128, 1)])
+                                                  # a warp per row: fused, and for many rows
+                                                  (1, 9, 127, 64, 127), (2, 7, 128, 128, 9), (60, 20, 129, 64, 128), (8, 148, 512, 64, 500),
+                                                  (8, 149, 513, 64, 500), (4, 300, 520, 64, 65), (2, 600, 1024, 128, 1)])
 def test_select_blocks_exact(H, n_qc, n_kc, d, keep):
     r = np.random.default_rng(n_qc * n_kc)
     cq = r.standard_normal((H, n_qc, d)).astype(np.float32)
