@@ -25,7 +25,7 @@
 // are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
 // in both halves that divide the keys of a step between them and merge their outputs, was the only form before (12 heads of
 // 16,385 rows, 33 of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454) and stays where the clusters are no more than
-// the SMs (4 heads of 512 x 131,072 rows 192 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
+// the SMs (4 heads of 512 x 131,072 rows 188 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
 // value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
 // descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
 // 400 cycles put into each step cost 46 us; now 4).
