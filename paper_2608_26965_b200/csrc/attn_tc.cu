@@ -24,8 +24,8 @@
 // one that a single list holds by the rows of that half, next to one of the other list (the other probabilities of a row
 // are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
 // in both halves that divide the keys of a step between them and merge their outputs, was the only form before (12 heads of
-// 16,385 rows, 33 of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454) and stays where the clusters are no more than
-// the SMs (4 heads of 512 x 131,072 rows 188 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
+// 16,385 rows, 33 of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454) and stays where pairs would take
+// no fewer rounds of tiles (4 heads of 512 x 131,072 rows 188 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
 // value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
 // descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
 // 400 cycles put into each step cost 46 us; now 4).
@@ -1253,9 +1253,12 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   int sms = 0, dev = 0;
   CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
   CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // 64-row query clusters go two to a tile where there are more of them than SMs (a pair takes up to twice the steps
-  // of one cluster: with fewer, SMs would stand idle), unless the lists' bitmaps do not fit
-  prm.pairs = pr.cluster_q < kTile && (long long)P * n_qc > sms && prm.bitmap_words <= kPairBitmapWords;
+  // A pair takes about 1.4 times the steps of one cluster (less the more their lists share), and tiles go in rounds of one per SM:
+  // pairs where their rounds are shorter by that, which they are not up to a cluster per SM, nor up to two where
+  // odd counts per head leave more than one tile per SM (54 heads of 5 clusters 183 us by ones, 239 by pairs); and by
+  // ones where the bitmaps of two lists do not fit.
+  const int rounds_of_pairs = ceil_div(P * ((n_qc + 1) / 2), sms), rounds_of_ones = ceil_div(P * n_qc, sms);
+  prm.pairs = pr.cluster_q < kTile && 7LL * rounds_of_pairs < 5LL * rounds_of_ones && prm.bitmap_words <= kPairBitmapWords;
   prm.n_tiles = P * (prm.pairs ? (n_qc + 1) / 2 : n_qc * tiles_per_qc);
   const int grid = prm.n_tiles < sms ? prm.n_tiles : sms;
   int rc;
