@@ -161,7 +161,8 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       copies_close();
     };
-    auto fetch = [&](int to) {
+    int next_count = 0;                    // of the next tile: of a centroid; -1: in use, -2: not (waited for at the tile's turn)
+    auto fetch = [&]() {
       const bool cen = t >= keep;
       const size_t base = cen ? (size_t)t0 * D : ((size_t)sel[t] * c_k + t0) * D;
       if constexpr (direct) {
@@ -182,21 +183,21 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       if (tid < KT) {
         bool use = tid < rows;
-        float b = use ? 0.f : -INFINITY;
+        next_count = use ? -1 : -2;
         if (cen && use) {
           const int j = t0 + tid;
           use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
-          b = use ? logf((float)cnt[j]) : -INFINITY;
+          next_count = use ? cnt[j] : -2;
         }
-        bias[to * KT + tid] = b;
       }
     };
     settle();
     if (rows > 0) {
-      fetch(0);
+      fetch();
       if constexpr (direct) { copy_tile(ks, k_src); copy_tile(vs, v_src); }
     }
     while (rows > 0) {
+      if (tid < KT) bias[parity * KT + tid] = next_count >= 0 ? logf((float)next_count) : next_count == -1 ? 0.f : -INFINITY;
       if constexpr (direct) {
         copies_wait<1>();
         __syncthreads();                   // the keys have arrived
@@ -223,7 +224,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       const float* b_tile = bias + parity * KT;
       parity ^= 1;
-      if (rows > 0) fetch(parity);
+      if (rows > 0) fetch();
 
       // scores of rows RY tr + y, keys tc + 16 i
       float s[RY][KI];
@@ -390,11 +391,12 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
     //   4 heads of 5,000 in clusters of 32    331 / 671             1 head of 1,000, key clusters of 16     93 / - / 77
     auto ctas = [&](int rows) { return (long long)pr.batch * pr.heads * n_qc * ceil_div(pr.cluster_q, rows); };
     // (by way of registers where small clusters leave at most two CTAs to an SM: two barriers per tile instead of three,
-    // 52 against 56 us for 1 head of 2,500 rows, d = 128, key clusters of 32)
+    // 52 against 56 us for 1 head of 2,500 rows, d = 128, key clusters of 32; 5 heads of 318 x 38,642 rows, clusters of 16 x 32
+    // 735 against 806)
     const bool few = ctas(32) <= 296;
     if (pr.head_dim == 64) {
       if (pr.cluster_k < 64)
-        return narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 32>) : few ? go(launch_rows<T, 64, 32, 4, 32, false>) : go(launch_rows<T, 64, 32, 4, 32>);
+        return narrow && few ? go(launch_rows<T, 64, 16, 2, 32, false>) : narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 32>) : few ? go(launch_rows<T, 64, 32, 4, 32, false>) : go(launch_rows<T, 64, 32, 4, 32>);
       if (ctas(8) <= 148) return go(launch_rows<T, 64, 8, 1, 64>);
       return narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 64>) : go(launch_rows<T, 64, 32, 4, 64>);
     }
