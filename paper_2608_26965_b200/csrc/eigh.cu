@@ -95,8 +95,10 @@ __global__ void __launch_bounds__(4 * D) cholesky_factor_kernel(const double* __
       const double row_term = sr[i] * per_n;
       a[i][0] = fma(-row_term, s0[i], g[i].x * scale);
       a[i][1] = fma(-row_term, s1[i], g[i].y * scale);
-      if (k == r) pivots[r] = a[i][0];
-      if (k + 1 == r && col0[i] >= 0) pivots[r] = a[i][1];
+      if (col0[i] >= 0) {                       // (a slot without a tile holds entries of another one's)
+        if (k == r) pivots[r] = a[i][0];
+        if (k + 1 == r) pivots[r] = a[i][1];
+      }
     }
   }
   __syncthreads();
