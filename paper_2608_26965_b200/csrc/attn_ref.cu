@@ -134,7 +134,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         for (int c = 0; c < 4; ++c) acc[y][g][c] = 0.f;
     }
 
-    // Tiles of keys: the members of the selected clusters in list order (t, row t0), then, 32 at a time, the
+    // Tiles of keys: the members of the selected clusters in list order (t, row t0), then, KT at a time, the
     // centroids (t = keep, first centroid t0).  `rows` = 0: no tile left.
     int t = 0, t0 = 0, rows = 0, members = 0;
     auto settle = [&]() {                  // the first tile at or behind (t, t0)
@@ -161,7 +161,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       copies_close();
     };
-    int next_count = 0;                    // of the next tile: of a centroid; -1: in use, -2: not (waited for at the tile's turn)
+    int next_count = 0;                    // rows that this thread's key of the next tile stands for: 1, or a centroid's; 0: not in use
     auto fetch = [&]() {
       const bool cen = t >= keep;
       const size_t base = cen ? (size_t)t0 * D : ((size_t)sel[t] * c_k + t0) * D;
@@ -182,12 +182,11 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         }
       }
       if (tid < KT) {
-        bool use = tid < rows;
-        next_count = use ? -1 : -2;
-        if (cen && use) {
+        next_count = tid < rows ? 1 : 0;
+        if (cen && tid < rows) {
           const int j = t0 + tid;
-          use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
-          next_count = use ? cnt[j] : -2;
+          const bool use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
+          next_count = use ? cnt[j] : 0;   // (waited for at the tile's turn)
         }
       }
     };
@@ -197,7 +196,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       if constexpr (direct) { copy_tile(ks, k_src); copy_tile(vs, v_src); }
     }
     while (rows > 0) {
-      if (tid < KT) bias[parity * KT + tid] = next_count >= 0 ? logf((float)next_count) : next_count == -1 ? 0.f : -INFINITY;
+      if (tid < KT) bias[parity * KT + tid] = next_count == 1 ? 0.f : logf((float)next_count);   // (of 0: -inf)
       if constexpr (direct) {
         copies_wait<1>();
         __syncthreads();                   // the keys have arrived

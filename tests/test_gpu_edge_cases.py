@@ -224,6 +224,27 @@ def test_forged_indices_are_reported_and_skipped(dtype, d, c):
     assert plan.last_status()["attn"] == 0
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("count", [-1, -2, -3])
+def test_a_negative_count_is_no_number_of_rows(count, dtype):
+    """The logarithm of a negative member count makes the rows that do not keep the cluster NaN, whatever the count is;
+    the others take the cluster as one without members."""
+    d, c, n_kc = 64, 64, 6
+    host, t = _attention_inputs(dtype, d, 4 * c, n_kc * c, c, 3, seed=94)
+    idx = np.array([[0, 1, 2], [1, 3, 5], [0, 2, 4], [2, 3, 4]], np.int32)
+    t["count_k"][0, 0, 3] = count
+    p = binding.make_problem(1, 1, 4 * c, n_kc * c, d, dtype, c, c, 3, True, flags=binding.CA_ATTN_FP32 if dtype == "bf16" else 0)
+    plan = binding.Plan(p, DEV)
+    O, lse = plan.cluster_attention_fwd(t["Qp"], t["Kp"], t["Vp"], t["ck"], t["cv"], t["count_k"], dev(idx[None, None], torch.int32),
+                                        dev(host["perm_q"].astype(np.int32)[None, None], torch.int32))
+    torch.cuda.synchronize()
+    assert plan.last_status()["attn"] == 0
+    bad = torch.zeros(4 * c, dtype=torch.bool, device=DEV)
+    bad[dev(host["perm_q"], torch.int64).reshape(4, c)[[0, 2]].reshape(-1)] = True
+    assert torch.equal(torch.isnan(O[0, 0]).all(-1), bad)
+    assert bool(torch.isfinite(O[0, 0][~bad]).all()) and bool(torch.isfinite(lse[0, 0][~bad]).all())
+
+
 @pytest.mark.parametrize("dtype,compensate", [("bf16", True), ("bf16", False), ("fp32", False)])
 def test_ragged_list_lengths_of_zero_and_beyond_the_row(dtype, compensate):
     """cluster_attention_fwd_ragged with a list of length 0 (with compensation: centroids only;
