@@ -87,7 +87,7 @@ constexpr int kFMasked = 1, kFCentroid = 2, kFFirst = 4, kFLast = 8, kFStop = 16
 // 64-127, or only one of the halves takes part
 constexpr int kFSplit = 32, kFUpper = 64, kFLower = 128;
 constexpr int kFIndexShift = 8, kFRestShift = 12;   // min(15, index in the tile), min(15, steps after it)
-constexpr int kFMixed = 1 << 16, kFSingle = 1 << 17;   // the tile has steps of the kinds above; it holds one cluster
+constexpr int kFSingle = 1 << 16;          // the tile holds one cluster
 
 // F8: queries, keys and key centroids arrive as E4M3 codes (one byte per element: a 128-byte row
 // of a panel holds 128 of them) and Q K^T runs as kind::f8f6f4 products; values stay bf16.
@@ -577,7 +577,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (F8 && box < 2) st_scale[slot * 2 + box] = prm.c_scale[(size_t)p * prm.cen_tiles + i];
             }
             if (starts) {
-              st_flags[slot] = (!single ? 0 : kFSingle | (twice && shared ? kFSplit : kFUpper)) | (twice || runs0 + runs1 > 0 ? kFMixed : 0) | (u == 0 ? kFFirst : 0) |
+              st_flags[slot] = (!single ? 0 : kFSingle | (twice && shared ? kFSplit : kFUpper)) | (u == 0 ? kFFirst : 0) |
                                (u == n - 1 ? kFLast : 0) | (min(u, 15) << kFIndexShift) | (min(n - 1 - u, 15) << kFRestShift) |
                                (split ? kFSplit : one ? (longer ? kFLower : kFUpper) : 0) | (cen ? kFCentroid : 0) |
                                (cen || ((cut >> (lane & 24)) & 255u) ? kFMasked : 0);
@@ -1007,8 +1007,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const bool empty = !(l_all > 0.f);
       const float inv = empty ? 0.f : 1.f / l_all;
       __nv_bfloat16* out = prm.O + ((size_t)tl.x * prm.n_q + orig) * D;
-      // 0 x inf, an infinite value among the other half's keys: for the second pass
-      const bool check = halves && (fl & kFMixed) != 0;
       const float inv_own = inv * w_own, inv_other = inv * w_other;
 #pragma unroll 1
       for (int c = 0; c < (twice && half == 1 ? 0 : D / 16); ++c) {
@@ -1028,7 +1026,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           }
           if (!got) break;
         }
-        if (check) {
+        if (halves) {                                      // 0 x inf, mostly an infinite value among the other half's keys: for the second pass
           f32x2 any2 = pack2(0.f, 0.f);
 #pragma unroll
           for (int j = 0; j < 16; j += 2) any2 = add2(any2, pack2(__uint_as_float(o[j]), __uint_as_float(o[j + 1])));

@@ -221,3 +221,22 @@ def test_pairs_of_64_row_query_clusters(d, c_k, infinite, compensate, heads):
     assert (O - want)[fine].norm() <= 1e-2 * want[fine].norm()
     assert (O - want)[fine].abs().max() <= 5e-2
     assert (lse - want_lse)[live].abs().max() <= 2e-3
+
+
+@pytest.mark.parametrize("heads,n_qc", [(9, 35), (2, 3)])                 # two clusters to a tile, and one
+def test_an_infinite_value_of_negligible_probability(heads, n_qc):
+    """A key 100 below the row's largest logit: exp(-100) is not zero in float32 but is where subnormal numbers are flushed,
+    and 0 x inf is NaN.  64-row query clusters whose outputs are not numbers are recomputed, also where both lists of a
+    tile are the same."""
+    d, n_kc, n_q = 64, 5, 64 * n_qc - 7
+    Qp, Kp, Vp, ck, cv, count, perm, _ = _clustering(heads, n_q, 64 * n_kc, d, 64, 64, n_qc)
+    Qp, Kp = 0.1 * Qp, 0.1 * Kp
+    Qp[:, :, :n_q, 0] = 10.0
+    Kp[:, :, 5, 0] = -80.0
+    Vp[:, :, 5, 7] = torch.inf
+    idx = torch.tensor([0, 3], dtype=torch.int32, device=DEV).expand(1, heads, n_qc, 2).contiguous()
+    plan = binding.Plan(binding.make_problem(1, heads, n_q, 64 * n_kc, d, "bf16", 64, 64, 2, False), DEV)
+    O = plan.cluster_attention_fwd(Qp, Kp, Vp, ck, cv, count, idx, perm)[0]
+    torch.cuda.synchronize()
+    assert plan.last_status()["attn"] == 0 and plan.recomputed_clusters() == heads * n_qc
+    assert bool(torch.isposinf(O[..., 7]).all()) and int(torch.isinf(O).sum()) == heads * n_q
