@@ -22,13 +22,16 @@
 // Query clusters of 64 rows go two to a tile, neighbours, one in either half (siblings of the split tree: their lists
 // have 64 to 86 % of their entries in common on the inputs measured).  A key cluster that both lists hold is taken once, by all rows;
 // one that a single list holds by the rows of that half, next to one of the other list (the other probabilities of a row
-// are stored as zeros), so that all four softmax warps of a group have work.  A tile of one cluster, its rows
-// in both halves that divide the keys of a step between them and merge their outputs, was the only form before (12 heads of
-// 16,385 rows, 33 of 257 clusters 345 -> 221 us, 12 heads of 30,592 rows 667 -> 454) and stays where pairs would take
-// no fewer rounds of tiles (4 heads of 512 x 131,072 rows 188 us; 236 with half of the warps idle).  (0 x inf is NaN: where a key cluster of one list holds an infinite
-// value, outputs that are not numbers send the tile to the second pass.)  The warp that writes the step
+// are stored as zeros), so that all four softmax warps of a group have work.  The warp that writes the step
 // descriptors has more to do then, and writes four at a time: one by one it was what the others waited for (247 us, and a wait of
-// 400 cycles put into each step cost 46 us; now 4).
+// 400 cycles put into each step cost 46 us; now 4).  Where pairs would take no fewer rounds of tiles, the rows of one cluster
+// stand in both halves of a tile, which divide the keys of a step between them and merge their outputs (12 heads of
+// 16,385 rows, 33 of 257 clusters 345 us in this form, 221 in pairs, 12 heads of 30,592 rows 667 and 454; 4 heads of 512 x 131,072
+// rows 188, and 236 in pairs).  Each form has instances of its own: in one kernel with the pairs' code, which a small
+// call fetches and walks through once, 2 heads of 1,000 rows with lists of one cluster took 14.2 us at d = 64 and 16.3 at
+// d = 128, 8 heads with 12 of 16 clusters 16.8; now 12.2, 13.6 and 15.4.
+// (0 x inf is NaN: where a key cluster of one list holds an infinite value, outputs that are not numbers send the
+// query cluster to the second pass.)
 // All roles run at the same time on one SM and have to fit its instruction cache
 // together: with the loops of the single-warp roles unrolled (105 KB of code) the same
 // kernel took 1.40 ms where it now takes 0.72 (2 x 16 heads of 20,000 rows, d = 128, 10
@@ -72,6 +75,7 @@ constexpr int kTile = 128;                 // query rows per tile, key rows per 
 constexpr int kCen = 64;                   // key centroids per step
 constexpr int kParts = 6;                  // steps s - 2 .. s + 3 can have row sums on their way while step s ends a tile
 constexpr int kQueue = 64;                 // list entries of a pair of 64-row query clusters in waiting
+constexpr int kMergeInts = 18;             // row pitch of the hand-over between the halves of a 64-row query cluster
 // first rows of a step's boxes (key clusters of 16 rows: eight boxes), of its value centroids, of Q
 constexpr int kRowCenV = 8, kRowQ = 9, kRowInts = 12;
 // A reference is raised when a sum of 32 probabilities exceeds 2^32: P is bf16, O and l are fp32, so
@@ -83,7 +87,7 @@ constexpr float kDangerSum = 7.9228163e28f;  // 2^96
 
 // flags of a step descriptor
 constexpr int kFMasked = 1, kFCentroid = 2, kFFirst = 4, kFLast = 8, kFStop = 16;
-// tiles of 64-row query clusters: the upper half of the rows takes keys 0-63 of the step and the lower half keys
+// pairs of 64-row query clusters: the upper half of the rows takes keys 0-63 of the step and the lower half keys
 // 64-127, or only one of the halves takes part
 constexpr int kFSplit = 32, kFUpper = 64, kFLower = 128;
 constexpr int kFIndexShift = 8, kFRestShift = 12;   // min(15, index in the tile), min(15, steps after it)
@@ -91,10 +95,12 @@ constexpr int kFSingle = 1 << 16;          // the tile holds one cluster
 
 // F8: queries, keys and key centroids arrive as E4M3 codes (one byte per element: a 128-byte row
 // of a panel holds 128 of them) and Q K^T runs as kind::f8f6f4 products; values stay bf16.
-template <int D, bool F8, bool HALVES>
+// MODE: how query clusters stand in tiles of 128 rows: a cluster of 128 (half of one of 256) in one; two clusters of 64 in one, or
+// in both halves of one
+constexpr int kWhole = 0, kPairs = 1, kTwice = 2;
+template <int D, bool F8, int MODE>
 struct TcCfg {
-  // step descriptors in flight (64-row query clusters: four are written at a time)
-  static constexpr int RING = !HALVES ? 8 : D == 64 ? 16 : 12;
+  static constexpr int RING = MODE != kPairs ? 8 : D == 64 ? 16 : 12;   // step descriptors in flight (pairs: four are written at a time)
   static constexpr int PANELS = D / 64;                      // value panels (bf16: 64 elements per 128-byte row)
   static constexpr int QK_PANELS = F8 ? D / 128 : D / 64;    // query / key panels
   static constexpr int QK_PANEL_COLS = F8 ? 128 : 64;        // elements per panel row
@@ -114,14 +120,15 @@ struct TcCfg {
   static constexpr int OFF_V = OFF_K + NK * QK_BYTES;
   static constexpr int OFF_BIAS = OFF_V + NV * V_BYTES;                  // [RING][128] floats
   static constexpr int OFF_LPART = OFF_BIAS + RING * kTile * 4;         // [kParts steps][128 rows] {row sum, reference}
-  static constexpr int OFF_QUEUE = OFF_LPART + kParts * kTile * 8;       // [3][kQueue] {first key row, rows, scale of the keys}
-  static constexpr int OFF_REF = OFF_QUEUE + (HALVES ? 3 * kQueue * 16 : 0);            // [128 rows] {reference, step}
+  static constexpr int OFF_QUEUE = OFF_LPART + kParts * kTile * 8;       // pairs: [3][kQueue] {first key row, rows, scale of the keys}
+  static constexpr int OFF_MERGE = OFF_QUEUE;                            // twice: [64 rows][kMergeInts] 16 columns of O, sum, reference
+  static constexpr int OFF_REF = OFF_QUEUE + (MODE == kPairs ? 3 * kQueue * 16 : MODE == kTwice ? 64 * kMergeInts * 4 : 0);   // [128 rows] {reference, step}
   static constexpr int OFF_ROWS = OFF_REF + kTile * 8;                   // [RING][kRowInts]
   static constexpr int OFF_TILE = OFF_ROWS + RING * kRowInts * 4;       // [RING] head, first position, redo word, tile
   static constexpr int OFF_FLAGS = OFF_TILE + RING * 16;
   static constexpr int OFF_SCALE = OFF_FLAGS + RING * 4;                // [RING][2] scales of the keys (F8)
   static constexpr int OFF_BAR = OFF_SCALE + RING * 8;
-  static constexpr int NUM_BARS = 1 + NQ + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV + (HALVES ? 4 : 0);
+  static constexpr int NUM_BARS = 1 + NQ + 4 + 2 * kGroups + 2 * RING + NK + 2 * NV + (MODE == kTwice ? 4 : 0);
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;                // tmem base, abort flag, redo counts x 4
   static constexpr int OFF_BITMAP = OFF_MISC + 32;
   static_assert(OFF_TILE % 16 == 0 && OFF_BAR % 8 == 0 && OFF_MISC % 8 == 0, "alignment");
@@ -138,7 +145,6 @@ struct TcParams {
   int* next_tile;                 // counter that hands out tiles, zero at the start
   int32_t* redo;                  // [B*H, n_qc, 2] per tile: scores left the range of the fast softmax
   int n_q, n_k, c_q, c_k, keep, list_stride, n_qc, n_kc, cen_tiles, compensate, bitmap_words, n_tiles;
-  int pairs;                      // 64-row query clusters: two to a tile
   float scale_log2;
   // quantised Q K^T: de-quantisation scales of the query rows [B*H*n_qc*c_q], of the key clusters
   // [B*H*n_kc] and of the runs of 64 key centroids [B*H*cen_tiles]; null otherwise
@@ -161,14 +167,13 @@ __host__ __device__ inline int selected_tiles(int keep, int c_k) {
 // and addresses from it stay in the uniform datapath.
 __device__ __forceinline__ int warp_uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
-// HALVES: query clusters of 64 rows (an instance of its own: the other sizes run slower with that code in the kernel)
-template <int D, bool F8, bool HALVES>
+template <int D, bool F8, int MODE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ck,
                const __grid_constant__ CUtensorMap tm_cv, const TcParams prm) {
   wait_for_previous();
-  using C = TcCfg<D, F8, HALVES>;
+  using C = TcCfg<D, F8, MODE>;
   extern __shared__ unsigned char smem_unaligned[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_unaligned) + 1023) & ~uintptr_t(1023));
@@ -206,9 +211,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
   const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
   // a query cluster of 256 rows takes two tiles; two of 64 rows (or one) share one
   const int tiles_per_qc = prm.c_q >= kTile ? prm.c_q / kTile : 1;
-  constexpr bool halves = HALVES;
-  const bool twice = halves && !prm.pairs;     // too few clusters for pairs: the rows of one stand in both halves
-  const int box_rows = halves ? min(prm.c_k, kTile / 2) : min(prm.c_k, kTile);   // of a load of keys
+  constexpr bool pairs = MODE == kPairs, twice = MODE == kTwice, halves = pairs || twice;
+  const int box_rows = min(prm.c_k, pairs ? kTile / 2 : kTile);   // of a load of keys
 
   if (tid == 0) {
     mbar_init(b_o_empty, 4);
@@ -224,7 +228,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     for (int s = 0; s < C::NV; ++s) { mbar_init(b_v_full(s), 1); mbar_init(b_v_empty(s), 1); }
 #pragma unroll 1
     for (int w = 0; w < 4; ++w) mbar_init(b_o_full(w), 1);
-    if (halves)
+    if (twice)
 #pragma unroll 1
       for (int w = 0; w < 4; ++w) mbar_init(b_m_full(w), 1);
     *abort_flag = 0;
@@ -279,7 +283,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 const uint32_t q_dst = s_q + tiles % C::NQ * C::QK_BYTES;
                 ++tiles;
                 // Q arrives with the tile's first keys (scores of a half without a cluster are not read)
-                const bool one = halves && (fl & kFSingle) != 0 && !twice;
+                const bool one = pairs && (fl & kFSingle) != 0;
                 mbar_expect_more(bar, one ? C::QK_BYTES / 2 : C::QK_BYTES);
 #pragma unroll 1
                 for (int half = 0; half <= (halves && !one ? 1 : 0); ++half)
@@ -417,7 +421,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       __syncwarp();
     } else {
       // ---------------------------------------------------------- tiles, lists, step descriptors
-      const int per_head = prm.pairs ? (prm.n_qc + 1) >> 1 : prm.n_qc * tiles_per_qc;
+      const int per_head = pairs ? (prm.n_qc + 1) >> 1 : prm.n_qc * tiles_per_qc;
       const int ck_shift = __ffs(prm.c_k) - 1;
       const int boxes = prm.c_k >= kTile ? 1 : kTile / prm.c_k;      // list entries per step, at most 8
       int s = 0, ord = 0;
@@ -439,7 +443,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           const int j = i * kCen + lane + 32 * g;
           const float w = j < prm.n_kc ? log2f((float)cnt[min(j, prm.n_kc - 1)]) : -INFINITY;
           bz[lane + 32 * g] = (in0[j >> 5] >> (j & 31)) & 1u ? -INFINITY : w;
-          if (halves) bz[kCen + lane + 32 * g] = (in1[j >> 5] >> (j & 31)) & 1u ? -INFINITY : w;
+          if (pairs) bz[kCen + lane + 32 * g] = (in1[j >> 5] >> (j & 31)) & 1u ? -INFINITY : w;
         }
       };
       auto list_length = [&](size_t at) {
@@ -457,18 +461,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const int p = tile / per_head, x = tile % per_head;
         const int32_t* cnt = prm.count_k + (size_t)p * prm.n_kc;
         const int cen_steps = prm.compensate ? prm.cen_tiles : 0;
-        if constexpr (halves) {
+        if constexpr (pairs) {
           // ---- Two 64-row query clusters, one in either half of the tile, or one in the upper half.  Neighbours in
           // cluster order are siblings of the split tree, and most of their lists are the same: key clusters of both
           // lists are taken by all rows, those of one list two at a time by a half each.  In runs of 64 keys:
           //   shared       two runs of both lists per step
           //   split        a run of the upper list, for the upper half, and one of the lower
           //   one-sided    two runs of the list that is longer than the other
-          // which are never more steps than two tiles of one cluster each.  Where clusters are not paired for lack of tiles, the
-          // rows of a cluster stand in both halves (twice): a half takes a run of each step, the upper one the centroids.  (A list that holds a cluster twice
-          // counts it twice: then nothing is shared.)
-          const int qc = prm.pairs ? 2 * x : x;
-          const bool single = !prm.pairs || qc + 1 == prm.n_qc;
+          // which are never more steps than two tiles of one cluster each.  (A list that holds a cluster twice counts it twice: then
+          // nothing is shared.)
+          const int qc = 2 * x;
+          const bool single = qc + 1 == prm.n_qc;
           const size_t at = (size_t)p * prm.n_qc + qc;
           const int32_t* sel0 = prm.block_idx + at * prm.list_stride;
           const int32_t* sel1 = sel0 + prm.list_stride;
@@ -577,7 +580,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
               if (F8 && box < 2) st_scale[slot * 2 + box] = prm.c_scale[(size_t)p * prm.cen_tiles + i];
             }
             if (starts) {
-              st_flags[slot] = (!single ? 0 : kFSingle | (twice && shared ? kFSplit : kFUpper)) | (u == 0 ? kFFirst : 0) |
+              st_flags[slot] = (!single ? 0 : kFSingle | kFUpper) | (u == 0 ? kFFirst : 0) |
                                (u == n - 1 ? kFLast : 0) | (min(u, 15) << kFIndexShift) | (min(n - 1 - u, 15) << kFRestShift) |
                                (split ? kFSplit : one ? (longer ? kFLower : kFUpper) : 0) | (cen ? kFCentroid : 0) |
                                (cen || ((cut >> (lane & 24)) & 255u) ? kFMasked : 0);
@@ -728,7 +731,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         pend = 0.f;
         if (F8) {
           const int4 tl = st_tile[ring];
-          row_sc = prm.scale_log2 * prm.q_scale[(size_t)tl.x * prm.n_qc * prm.c_q + tl.y + (halves && (fl & kFSingle) ? row & 63 : row)];
+          row_sc = prm.scale_log2 * prm.q_scale[(size_t)tl.x * prm.n_qc * prm.c_q + tl.y + (twice || (pairs && (fl & kFSingle)) ? row & 63 : row)];
         }
       }
       // scales of this step's scores, per run of 64 columns.  A zero scale (an all-zero query row or
@@ -745,9 +748,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
       }
       // (the two lists of a tile of 64-row query clusters leave out different centroids)
-      const float* bz = bias + ring * kTile + (halves && cen ? half * kCen : 0);
+      const float* bz = bias + ring * kTile + (pairs && cen ? half * kCen : 0);
       // chunks [c_begin, c_end) of 32 columns
-      const bool idle = halves && (fl & (half == 0 ? kFLower : kFUpper)) != 0, split = halves && (fl & kFSplit) != 0;
+      const bool idle = pairs ? (fl & (half == 0 ? kFLower : kFUpper)) != 0 : twice && cen && half == 1;
+      const bool split = pairs ? (fl & kFSplit) != 0 : twice && !cen;
       // (kept from the compiler that it is 0 in the instances for 128 rows: with the loops below arranged for
       // that, they are 3 % slower, 807 -> 835 us for 8 heads of 16,384 x 131,072 rows)
       int c_begin = split ? 2 * half : 0;
@@ -933,9 +937,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       if (rest > 0) continue;
 
       // ---- epilogue: O / l, rows back to their original positions
-      const int pos = tl.y + row;
-      // rows of the padding are not written, nor those of a half without a cluster
-      bool live = pos < prm.n_q && !(halves && (fl & kFSingle) && half == 1);
+      const int pos = tl.y + (twice ? row & 63 : row);
+      // rows of the padding are not written, nor those of a half without a cluster of its own
+      bool live = pos < prm.n_q && !((twice || (pairs && (fl & kFSingle))) && half == 1);
       int orig = live ? prm.perm_q[(size_t)tl.x * prm.n_q + pos] : 0;
       if (orig < 0 || orig >= prm.n_q) {                // not a row of O: flagged, nothing written
         atomicCAS(prm.status, 0, kErrBadIndex);
@@ -952,52 +956,34 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
           if (other.y > -INFINITY) l_run += other.x * ex2_approx(other.y - m_ref);
         }
       }
-      // Rows that stand in both halves: the lower one hands over its sum and reference, then eight columns of O at a time,
-      // which the upper one scales to the larger reference.
-      float l_all = l_run, m_all = m_ref, w_own = 1.f, w_other = 0.f;
-      float* merge = reinterpret_cast<float*>(smem + C::OFF_QUEUE + kQueue * 16) + (row & 63);     // [8][64], no lists wait there
-      const int pair = quarter & 1;
-      int use = tl.w * (1 + D / 8);
+      // Rows that stand in both halves: the lower one hands over its sum and reference and 16 columns of O at a time, which
+      // the upper one scales to the larger reference.
+      float* merge = reinterpret_cast<float*>(smem + C::OFF_MERGE) + (row & 63) * kMergeInts;
+      const int pair = quarter & 1, uses = tl.w * (D / 16);
       bool got = true;
-      auto take = [&]() { return wait(b_m_full(pair), use); };
-      auto taken = [&]() {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b_m_empty(pair));
-        ++use;
-      };
       if (twice && half == 1) {
-        auto room = [&]() { return use == 0 || wait(b_m_empty(pair), use - 1); };
-        auto handed = [&]() {
-          __syncwarp();
-          if (lane == 0) mbar_arrive(b_m_full(pair));
-          ++use;
-        };
-        got = room();
-        if (!got) break;
-        merge[0] = l_run;
-        merge[64] = m_ref;
-        handed();
 #pragma unroll 1
         for (int c = 0; c < D / 16 && got; ++c) {
+          const int use = uses + c;
           uint32_t o[16];
           tmem_ld16(tmem_o + lane_addr + c * 16, o);
           tmem_wait_ld();
+          if (use > 0) got = wait(b_m_empty(pair), use - 1);
+          if (!got) break;
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            got = got && room();
-            if (!got) break;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) merge[64 * j] = __uint_as_float(o[8 * h + j]);
-            handed();
-          }
+          for (int j = 0; j < 16; ++j) merge[j] = __uint_as_float(o[j]);
+          merge[16] = l_run;
+          merge[17] = m_ref;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_m_full(pair));
         }
         if (!got) break;
       }
+      float l_all = l_run, m_all = m_ref, w_own = 1.f, w_other = 0.f;
       if (twice && half == 0) {
-        got = take();
+        got = wait(b_m_full(pair), uses);
         if (!got) break;
-        const float l_other = merge[0], m_other = merge[64];
-        taken();
+        const float l_other = merge[16], m_other = merge[17];
         m_all = fmaxf(m_ref, m_other);
         w_own = m_ref > -INFINITY ? ex2_approx(m_ref - m_all) : 0.f;
         w_other = m_other > -INFINITY ? ex2_approx(m_other - m_all) : 0.f;
@@ -1016,15 +1002,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
         for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * inv_own);
         if (twice) {
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            got = got && take();
-            if (!got) break;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) o[8 * h + j] = __float_as_uint(fmaf(merge[64 * j], inv_other, __uint_as_float(o[8 * h + j])));
-            taken();
-          }
+          if (c > 0) got = wait(b_m_full(pair), uses + c);
           if (!got) break;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(fmaf(merge[j], inv_other, __uint_as_float(o[j])));
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_m_empty(pair));
         }
         if (halves) {                                      // 0 x inf, mostly an infinite value among the other half's keys: for the second pass
           f32x2 any2 = pack2(0.f, 0.f);
@@ -1060,11 +1043,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
       const bool redo = __any_sync(0xffffffffu, live && !(l_all < INFINITY));
       if (lane == 0) {
         int* acc = &redo_acc[tl.w & 3];
-        const int mine = redo ? (halves && half == 1 ? 65537 : 257) : 1;
+        const int mine = redo ? (pairs && half == 1 ? 65537 : 257) : 1;
         if ((atomicAdd(acc, mine) & 255) == 3) {
           const int all = atomicExch(acc, 0);
           prm.redo[tl.z] = (all >> 8) & 255 ? 1 : 0;
-          if (halves && !(fl & kFSingle)) prm.redo[tl.z + 2] = all >> 16 ? 1 : 0;
+          if (pairs && !(fl & kFSingle)) prm.redo[tl.z + 2] = all >> 16 ? 1 : 0;
         }
       }
     }
@@ -1169,11 +1152,11 @@ size_t attn_tc_workspace_bytes(const ca_problem_t& pr) {
   return bytes;
 }
 
-template <int D, bool F8, bool HALVES>
+template <int D, bool F8, int MODE>
 static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, LaunchStream st) {
-  using C = TcCfg<D, F8, HALVES>;
-  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4 * (prm.pairs ? 2 : 1);
-  auto k = attn_tc_kernel<D, F8, HALVES>;
+  using C = TcCfg<D, F8, MODE>;
+  const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4 * (MODE == kPairs ? 2 : 1);
+  auto k = attn_tc_kernel<D, F8, MODE>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   launch_chained(k, grid, kTcThreads, smem, st, maps[0], maps[1], maps[2], maps[3], maps[4], prm);
   CA_LAUNCH_CHECK();
@@ -1221,9 +1204,19 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
                    D, kmix, vb, status);
     CA_LAUNCH_CHECK();
   }
+  const int bitmap_words = (cen_tiles * kCen + 31) / 32;
+  int sms = 0, dev = 0;
+  CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
+  CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // A pair takes about 1.4 times the steps of one cluster (less the more their lists share), and tiles go in rounds of one per SM:
+  // pairs where their rounds are shorter by that, which they are not up to a cluster per SM, nor up to two where
+  // odd counts per head leave more than one tile per SM (54 heads of 5 clusters 183 us by ones, 239 by pairs); and by
+  // ones where the bitmaps of two lists do not fit.
+  const int rounds_of_pairs = ceil_div(P * ((n_qc + 1) / 2), sms), rounds_of_ones = ceil_div(P * n_qc, sms);
+  const bool pairs = pr.cluster_q < kTile && 7LL * rounds_of_pairs < 5LL * rounds_of_ones && bitmap_words <= kPairBitmapWords;
   CUtensorMap maps[5];
   const int qbox = pr.cluster_q < kTile ? pr.cluster_q : kTile;
-  const int kbox = pr.cluster_k < qbox ? pr.cluster_k : qbox;     // 64-row query clusters: keys in runs of 64
+  const int kbox = min(pr.cluster_k, pairs ? kTile / 2 : kTile);  // pairs: keys in runs of 64
   bool ok = make_map(&maps[2], Vp, (size_t)P * n_kc * pr.cluster_k, D, kbox) &&
             make_map(&maps[4], vb, (size_t)P * cen_tiles * kCen, D, kCen);
   if (f8)
@@ -1241,31 +1234,25 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   prm.O = static_cast<__nv_bfloat16*>(O); prm.lse = lse; prm.status = status; prm.redo = redo;
   prm.n_q = pr.n_q; prm.n_k = pr.n_k; prm.c_q = pr.cluster_q; prm.c_k = pr.cluster_k; prm.keep = pr.keep;
   prm.n_qc = n_qc; prm.n_kc = n_kc; prm.cen_tiles = cen_tiles; prm.compensate = pr.compensate;
-  prm.bitmap_words = (cen_tiles * kCen + 31) / 32;
+  prm.bitmap_words = bitmap_words;
   prm.scale_log2 = scale * 1.4426950408889634f;
   prm.wait_limit = g_wait_limit;
   prm.skip_key_load = g_skip_key_load;
   prm.q_scale = sq; prm.k_scale = sk; prm.c_scale = sc;
   const int tiles_per_qc = pr.cluster_q >= kTile ? pr.cluster_q / kTile : 1;
   prm.next_tile = status + kTileWord;
-  int sms = 0, dev = 0;
-  CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
-  CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  // A pair takes about 1.4 times the steps of one cluster (less the more their lists share), and tiles go in rounds of one per SM:
-  // pairs where their rounds are shorter by that, which they are not up to a cluster per SM, nor up to two where
-  // odd counts per head leave more than one tile per SM (54 heads of 5 clusters 183 us by ones, 239 by pairs); and by
-  // ones where the bitmaps of two lists do not fit.
-  const int rounds_of_pairs = ceil_div(P * ((n_qc + 1) / 2), sms), rounds_of_ones = ceil_div(P * n_qc, sms);
-  prm.pairs = pr.cluster_q < kTile && 7LL * rounds_of_pairs < 5LL * rounds_of_ones && prm.bitmap_words <= kPairBitmapWords;
-  prm.n_tiles = P * (prm.pairs ? (n_qc + 1) / 2 : n_qc * tiles_per_qc);
+  prm.n_tiles = P * (pairs ? (n_qc + 1) / 2 : n_qc * tiles_per_qc);
   const int grid = prm.n_tiles < sms ? prm.n_tiles : sms;
   int rc;
   {
     ProfScope ps(kProfAttn, st);
-    const bool halves = pr.cluster_q < kTile;
-    if (f8) rc = halves ? launch_tc_d<128, true, true>(maps, prm, grid, st) : launch_tc_d<128, true, false>(maps, prm, grid, st);
-    else if (D == 64) rc = halves ? launch_tc_d<64, false, true>(maps, prm, grid, st) : launch_tc_d<64, false, false>(maps, prm, grid, st);
-    else rc = halves ? launch_tc_d<128, false, true>(maps, prm, grid, st) : launch_tc_d<128, false, false>(maps, prm, grid, st);
+    auto go = [&](auto mode) {
+      constexpr int M = decltype(mode)::value;
+      if (f8) return launch_tc_d<128, true, M>(maps, prm, grid, st);
+      return D == 64 ? launch_tc_d<64, false, M>(maps, prm, grid, st) : launch_tc_d<128, false, M>(maps, prm, grid, st);
+    };
+    if (pairs) rc = go(std::integral_constant<int, kPairs>{});
+    else rc = pr.cluster_q < kTile ? go(std::integral_constant<int, kTwice>{}) : go(std::integral_constant<int, kWhole>{});
   }
   if (rc != CA_OK) return rc;
   ProfScope ps(kProfAttnSecond, st);
