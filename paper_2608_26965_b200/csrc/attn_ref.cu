@@ -161,7 +161,13 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       }
       copies_close();
     };
-    int next_count = 0;                    // rows that this thread's key of the next tile stands for: 1, or a centroid's; 0: not in use
+    // Of this thread's key of the next tile: how many rows it stands for (1, or a centroid's; 0: not in use), waited for at the tile's
+    // turn; or its additive term, formed where the rows are fetched.  bf16, us, at the tile's turn / at the fetch: 5 heads of 318 x
+    // 38,642 rows, clusters of 16, d = 128 (16 rows) 390 / 314, d = 64 193 / 199; 4 heads of 8,000 rows, d = 128, clusters of
+    // 64 (64 rows) 687 / 828; fp32, 2 heads of 2,500 rows, d = 64, clusters of 64 x 32 (32 rows) 51.2 / 49.7.
+    constexpr bool late = direct || QR == 64 || (QR == 16 && D == 64);
+    int next_count = 0;
+    float next_bias = 0.f;
     auto fetch = [&]() {
       const bool cen = t >= keep;
       const size_t base = cen ? (size_t)t0 * D : ((size_t)sel[t] * c_k + t0) * D;
@@ -182,11 +188,15 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         }
       }
       if (tid < KT) {
-        next_count = tid < rows ? 1 : 0;
-        if (cen && tid < rows) {
-          const int j = t0 + tid;
-          const bool use = !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u);
-          next_count = use ? cnt[j] : 0;   // (waited for at the tile's turn)
+        const int j = t0 + tid;
+        const bool centroid = cen && tid < rows;
+        const bool use = centroid ? !((selected[(many ? j % kRefWindow : j) >> 5] >> (j & 31)) & 1u) : tid < rows;
+        if constexpr (late) {
+          next_count = use ? 1 : 0;
+          if (centroid && use) next_count = cnt[j];
+        } else {
+          next_bias = use ? 0.f : -INFINITY;
+          if (centroid && use) next_bias = logf((float)cnt[j]);
         }
       }
     };
@@ -196,7 +206,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
       if constexpr (direct) { copy_tile(ks, k_src); copy_tile(vs, v_src); }
     }
     while (rows > 0) {
-      if (tid < KT) bias[parity * KT + tid] = next_count == 1 ? 0.f : logf((float)next_count);   // (of 0: -inf)
+      if (late && tid < KT) bias[parity * KT + tid] = next_count == 1 ? 0.f : logf((float)next_count);   // (of 0: -inf)
       if constexpr (direct) {
         copies_wait<1>();
         __syncthreads();                   // the keys have arrived
@@ -208,6 +218,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
           *reinterpret_cast<float4*>(&ks[r * LD + col]) = kf[i];
           *reinterpret_cast<float4*>(&vs[r * LD + col]) = vf[i];
         }
+        if (!late && tid < KT) bias[tid] = next_bias;
         __syncthreads();
       }
       t0 += KT;
@@ -222,7 +233,7 @@ attn_ref_kernel(const T* __restrict__ Qp, const T* __restrict__ Kp, const T* __r
         }
       }
       const float* b_tile = bias + parity * KT;
-      parity ^= 1;
+      if constexpr (late) parity ^= 1;
       if (rows > 0) fetch();
 
       // scores of rows RY tr + y, keys tc + 16 i
@@ -380,30 +391,37 @@ static int launch_t(const ca_problem_t& pr, const T* Qp, const T* Kp, const T* V
   const bool narrow = pr.cluster_q < 32;       // (never a second pass: the tensor-core kernel takes 64 rows and more)
   if constexpr (sizeof(T) == 4) {
     // Query rows per CTA: 8 or 16 where every CTA still has an SM for itself (a CTA is a chain of latencies then, which shared
-    // work shortens), otherwise 32.  Keys per tile: 64 (fewer rounds of the softmax), but 32 where clusters
-    // are smaller (a tile holds one cluster) and at d = 128 with more than two CTAs per SM, of which four
-    // fit with 32 and two with 64.  us, tiles of 32 rows and 32 keys / 64 keys / 16 rows / 8 rows:
+    // work shortens) and of clusters of 16, otherwise 32.  Keys per tile: 64 (fewer rounds of the softmax), but 32 where
+    // clusters are smaller (a tile holds one cluster), at d = 128 with more than two CTAs per SM, of which four fit with 32 and two
+    // with 64, and where lists and centroids fill tiles of 64 so badly that an eighth of the columns is added (12 heads of
+    // 1,370 rows, 2 of 22 clusters of 64, d = 64 35.2 us with 32, 37.2 with 64), unless every CTA has an SM for itself.
+    // us, tiles of 32 rows and 32 keys / 64 keys / 16 rows and 64 keys / 8 rows:
     //   1 head of 1,024 rows, d = 64     20.7 / 19.5 / 16.6 / 14.9      2 heads of 1,024     31 / 27 / 22.8 / 26.8
     //   4 heads of 1,024                 30 / 26.8 / 28.9 / 37          4 heads of 8,192     619 / 537 / 733
     //   1 head of 1,500, d = 128         59 / 51 / 41 / 54              2 heads of 2,500     134 / 115 / 146
     //   2 heads of 5,003, 10 clusters    321 / 395                      4 heads of 8,192     599 / 709
     //   4 heads of 5,000 in clusters of 32    331 / 671             1 head of 1,000, key clusters of 16     93 / - / 77
+    // Query clusters of 16, d = 128, 16 rows and 32 keys / 64 keys: 2 heads of 1,400 rows, key clusters of 128 (176 CTAs) 80 / 74,
+    // 2 of 2,500 (314 CTAs, 18 more than two to an SM) 60 / 76, 4 of 8,000 688 / 720.
+    // By way of registers where small clusters leave at most two CTAs to an SM: two barriers per tile instead of three (2 heads of
+    // 2,500 rows, clusters of 64 x 32, d = 64 49.6 us, and 51 with asynchronous copies, d = 128 76.2 and 78; at
+    // d = 128 16 rows take the same time either way).
+    auto columns = [&](int keys) {       // of a list in tiles of `keys`
+      return (long long)pr.keep * ceil_div(pr.cluster_k, keys) * keys + (pr.compensate ? (long long)ceil_div(n_kc, keys) * keys : 0);
+    };
+    const bool full = keep_count || 7 * columns(64) <= 8 * columns(32);     // (lists of lengths not known here: taken as long)
     auto ctas = [&](int rows) { return (long long)pr.batch * pr.heads * n_qc * ceil_div(pr.cluster_q, rows); };
-    // (by way of registers where small clusters leave at most two CTAs to an SM: two barriers per tile instead of three,
-    // 52 against 56 us for 1 head of 2,500 rows, d = 128, key clusters of 32; 5 heads of 318 x 38,642 rows, clusters of 16 x 32
-    // 735 against 806)
-    const bool few = ctas(32) <= 296;
+    const bool few = ctas(32) <= 296, short_rows = narrow || ctas(16) <= 148, wide_keys = pr.cluster_k >= 64;
+    if (wide_keys && ctas(8) <= 148) return pr.head_dim == 64 ? go(launch_rows<T, 64, 8, 1, 64>) : go(launch_rows<T, 128, 8, 1, 64>);
     if (pr.head_dim == 64) {
-      if (pr.cluster_k < 64)
-        return narrow && few ? go(launch_rows<T, 64, 16, 2, 32, false>) : narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 32>) : few ? go(launch_rows<T, 64, 32, 4, 32, false>) : go(launch_rows<T, 64, 32, 4, 32>);
-      if (ctas(8) <= 148) return go(launch_rows<T, 64, 8, 1, 64>);
-      return narrow || ctas(16) <= 148 ? go(launch_rows<T, 64, 16, 2, 64>) : go(launch_rows<T, 64, 32, 4, 64>);
+      if (short_rows && wide_keys && (full || ctas(16) <= 148)) return go(launch_rows<T, 64, 16, 2, 64>);
+      if (short_rows) return few ? go(launch_rows<T, 64, 16, 2, 32, false>) : go(launch_rows<T, 64, 16, 2, 32>);
+      if (wide_keys && full) return go(launch_rows<T, 64, 32, 4, 64>);
+      return few ? go(launch_rows<T, 64, 32, 4, 32, false>) : go(launch_rows<T, 64, 32, 4, 32>);
     }
-    if (pr.cluster_k < 64)
-      return narrow || ctas(16) <= 148 ? go(launch_rows<T, 128, 16, 2, 32>) : few ? go(launch_rows<T, 128, 32, 4, 32, false>) : go(launch_rows<T, 128, 32, 4, 32>);
-    if (ctas(8) <= 148) return go(launch_rows<T, 128, 8, 1, 64>);
-    if (narrow || ctas(16) <= 148) return go(launch_rows<T, 128, 16, 2, 64>);
-    return few ? go(launch_rows<T, 128, 32, 4, 64>) : go(launch_rows<T, 128, 32, 4, 32>);
+    if (short_rows) return wide_keys && (ctas(16) <= 148 || (full && ctas(16) <= 296)) ? go(launch_rows<T, 128, 16, 2, 64>) : go(launch_rows<T, 128, 16, 2, 32>);
+    if (!few) return go(launch_rows<T, 128, 32, 4, 32>);
+    return wide_keys && full ? go(launch_rows<T, 128, 32, 4, 64>) : go(launch_rows<T, 128, 32, 4, 32, false>);
   } else {
     // 64 query rows per CTA read every key half as often as 32; 32 where 64 would leave SMs without a CTA
     const bool wide = !redo && pr.cluster_q >= 64 && (long long)pr.batch * pr.heads * ceil_div(pr.n_q, 64) >= 148;

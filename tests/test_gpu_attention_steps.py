@@ -80,6 +80,8 @@ def test_tiles_of_few_steps_and_many_tiles(d, c_q, c_k, heads, n_q, n_k, compens
     (64, 64, 64, 2, 64 * 9 - 5, 64 * 5 - 9, True), (64, 64, 128, 2, 64 * 10 - 9, 128 * 4 - 77, False), (128, 64, 64, 2, 64 * 10 - 9, 64 * 6 - 1, True),
     (64, 128, 64, 3, 128 * 7 - 5, 64 * 6 - 9, True), (128, 128, 256, 2, 128 * 10, 256 * 3 - 100, True),
     (128, 128, 64, 5, 128 * 16 - 3, 64 * 5 - 7, True),
+    # ... 16 rows and 32 keys where there are many CTAs; 32 rows by way of registers
+    (64, 16, 32, 5, 16 * 60 - 3, 32 * 5 - 9, True), (64, 64, 32, 3, 64 * 30 - 1, 32 * 5 - 3, True), (128, 64, 32, 3, 64 * 30 - 1, 32 * 4, False),
 ])
 def test_fp32_kernel_against_float64(d, c_q, c_k, heads, n_q, n_k, compensate, dtype):
     Qp, Kp, Vp, ck, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, c_q, c_k, d + c_q + c_k + n_q)
