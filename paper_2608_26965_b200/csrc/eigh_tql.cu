@@ -69,6 +69,9 @@ __device__ __forceinline__ void named_arrive(int id, int count) {
 constexpr int kThreads = 512;
 constexpr int kBaseLog = 2, kBase = 1 << kBaseLog;   // rows of a base block of the divide and conquer
 constexpr int kMaxSweeps = 12;
+// The reduction multiplies up to three entries (x . A x), of which those of directions with little variance are small: it runs on
+// the matrix with 2^20 as its largest diagonal entry, so that products of entries down to 1e-15 of that are normal numbers.
+constexpr float kReduceScale = 1048576.f;
 
 // Eigenvalues that are not numbers (the covariance of rows with infinities, or whose sums overflow) stand as +inf: the
 // rank of a pole among the others is then a permutation for every input, and indexes stay in range.
@@ -93,7 +96,7 @@ __device__ __forceinline__ void jacobi_blocks(float2* de, int blocks, float* Qt,
     m[i][i] = d.x;
   }
   // zero to rounding: of the two diagonal entries, or of the whole matrix, whose largest diagonal entry is 1
-  auto negligible = [&](int p, int q) { return !(fabsf(m[p][q]) > fmaxf(1e-8f * (fabsf(m[p][p]) + fabsf(m[q][q])), 1e-15f)); };
+  auto negligible = [&](int p, int q) { return !(fabsf(m[p][q]) > fmaxf(1e-8f * (fabsf(m[p][p]) + fabsf(m[q][q])), 1e-18f)); };
   auto rotate = [&](int p, int q) {
     const float x = m[p][q], d = m[q][q] - m[p][p];
     float root, inv;
@@ -612,6 +615,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
   // what is multiplied by the reduction's Q on the way: the factor F, or the identity where E itself is asked for
   const bool need_e = !(a.lift && a.out_lifted);
   __shared__ double s_scale;
+  __shared__ unsigned s_largest;
   __shared__ float s_rho[D / kBase], s_theta[D / kBase];   // cut before row i kBase
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -676,14 +680,24 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     }
   } else {
     const double* Ain = a.A_in + mat;
-    for (int e = tid; e < D * D; e += NT) A[(e / D) * LDA + e % D] = (float)Ain[e];
+    if (tid == 0) s_largest = 0u;
+    __syncthreads();
+    float largest = 0.f;
+    for (int e = tid; e < D * D; e += NT) {
+      const float v = (float)Ain[e];
+      A[(e / D) * LDA + e % D] = v;
+      largest = fmaxf(largest, fabsf(v));
+    }
+    atomicMax(&s_largest, __float_as_uint(largest));
   }
   __syncthreads();
-  // scale so that the largest diagonal entry is 1 (eigenvectors unchanged, eigenvalues scaled back at the end)
+  // scale so that the largest diagonal entry is 1 (eigenvectors unchanged, eigenvalues scaled back at the end); of a matrix
+  // of the caller's, which need not be a covariance, the largest entry
   if (tid < 32) {
     float mx = 0.f;
     for (int i = tid; i < D; i += 32) mx = fmaxf(mx, fabsf(A[i * LDA + i]));
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (a.mode == kPcaMatrix) mx = fmaxf(mx, __uint_as_float(s_largest));
     if (tid == 0) s_scale = mx > 0.f ? (double)mx : 1.0;
   }
   __syncthreads();
@@ -706,7 +720,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
     f32x2 areg[RW][CH][2], x[CH][2];
     float d_cur;
     {
-      const float inv = (float)(1.0 / a_scale);
+      const float inv = (float)((double)kReduceScale / a_scale);
       auto entry = [&](int i, int j) { return 0.5f * (A[i * LDA + j] + A[j * LDA + i]) * inv; };
 #pragma unroll
       for (int t = 0; t < CH; ++t)
@@ -813,9 +827,9 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
         }
 #pragma unroll
         for (int o = 1; o < TR; o <<= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        // already tridiagonal in this column otherwise, to 1e-12 of the largest diagonal entry (uniform: every
+        // already tridiagonal in this column otherwise, to 1e-15 of the largest diagonal entry (uniform: every
         // group has added the same numbers); beta = 0 then makes the step do nothing
-        const bool reflect = sig - x0 * x0 > 1e-24f;
+        const bool reflect = sig - x0 * x0 > 1e-30f * kReduceScale * kReduceScale;
         float bn;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(bn) : "f"(fmaf(fabsf(x0), rt, sig)));
         bn = reflect ? bn : 0.f;
@@ -826,7 +840,7 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
         if (publisher) {
           // the first entry of a reflector is put in its place a step later, when no thread reads the row any more
           if (lane == 0) {
-            de[k] = make_float2(d_cur, alpha);
+            de[k] = make_float2(d_cur / kReduceScale, alpha / kReduceScale);
             beta[k] = bn;
             if (k > 0) refl[(k - 1) * LDA + k] = v0_prev;
           }
@@ -893,8 +907,8 @@ __global__ void __launch_bounds__(kThreads) eigh_tql_kernel(const PcaArgs a) {
       float lo, hi, last;
       unpack2(x[CH - 1][1], lo, hi);
       unpack2(areg[RW - 1][CH - 1][1], lo, last);
-      de[D - 2] = make_float2(d_cur, hi);
-      de[D - 1] = make_float2(last, 0.f);
+      de[D - 2] = make_float2(d_cur / kReduceScale, hi / kReduceScale);
+      de[D - 1] = make_float2(last / kReduceScale, 0.f);
     }
     named_sync(1, kParties);
     if (publisher) {

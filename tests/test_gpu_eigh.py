@@ -119,3 +119,25 @@ def test_argument_errors():
     A = torch.zeros((1, 32, 32), dtype=torch.float64, device=DEV)
     with pytest.raises(binding.ClusterAttnError):
         binding.debug_eigh(A)                                      # d = 32 is not built
+
+
+@pytest.mark.parametrize("variance", [1e-8, 1e-12, 1e-13])
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_direction_of_little_variance_beside_a_dominant_channel(d, variance):
+    """One channel of variance 1 and one direction of all others, uncoupled (and not mixed by the first reflector): its eigenvector and eigenvalue are as accurate as
+    float32 gives them although it is 1e-13 of the matrix (entries down to 1e-15 of the largest one are not taken for zero, and
+    products of three of them stay normal numbers)."""
+    r = np.random.default_rng(d)
+    mats, want = [], []
+    for channel in (0, d // 2, d - 1):
+        v = r.uniform(0.5, 1.0, d) * r.choice([-1.0, 1.0], d)
+        v[channel] = 0.0
+        v /= np.linalg.norm(v)
+        A = variance * np.outer(v, v)
+        A[channel, channel] = 1.0
+        mats.append(A)
+        want.append(v)
+    W, ev = run(mats)
+    for w, e, v in zip(W, ev, want):
+        assert abs(e[0] - 1.0) <= 1e-6 and abs(e[1] / variance - 1.0) <= 1e-5
+        assert abs(abs(w[:, 1] @ v) - 1.0) <= 1e-5
