@@ -113,7 +113,7 @@ score_select_kernel(const float* __restrict__ cq, const float* __restrict__ ck, 
       const float* srow = scores + ((size_t)p * chunk_rows + (q0 - row0 + t)) * n_kc;
       for (int j = tid; j < n_kc; j += kSelectThreads) keys[(size_t)t * n_kc + j] = score_key(__ldg(srow + j));
     }
-  } else {
+  } else if constexpr (QT > 1) {
   for (int e = tid; e < QT * D; e += kSelectThreads) qs[e] = (e < nq * D) ? cqp[e] : 0.f;
   __syncthreads();
 
