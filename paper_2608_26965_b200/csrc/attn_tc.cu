@@ -156,7 +156,8 @@ struct TcParams {
 };
 
 constexpr int kErrBadIndex = 6;   // CA_ERR_BAD_INDEX
-constexpr int kPairBitmapWords = 2048;    // of each list of a pair: 65,536 key clusters (d = 128 leaves 18 KB for both)
+constexpr int kBitmapWords = 4096;        // of a list: 131,072 key clusters (d = 128 leaves 17 KB)
+constexpr int kPairBitmapWords = 2048;    // of each list of a pair
 
 // key rows of the selected clusters are consumed in tiles of 128 rows
 __host__ __device__ inline int selected_tiles(int keep, int c_k) {
@@ -1126,7 +1127,7 @@ bool attn_tc_supported(const ca_problem_t& pr) {
   if (pr.cluster_q != 64 && pr.cluster_q != 128 && pr.cluster_q != 256) return false;
   if (pr.cluster_k < 16 || pr.cluster_k > 256) return false;
   const int n_kc = ceil_div(pr.n_k, pr.cluster_k);
-  if ((n_kc + 31) / 32 * 4 > 16384) return false;          // selected-cluster bitmap in shared memory
+  if ((n_kc + 31) / 32 > kBitmapWords) return false;       // selected-cluster bitmap in shared memory
   return true;
 }
 
@@ -1155,6 +1156,7 @@ size_t attn_tc_workspace_bytes(const ca_problem_t& pr) {
 template <int D, bool F8, int MODE>
 static int launch_tc_d(const CUtensorMap* maps, const TcParams& prm, int grid, LaunchStream st) {
   using C = TcCfg<D, F8, MODE>;
+  static_assert(1024 + C::OFF_BITMAP + 4 * (MODE == kPairs ? 2 * kPairBitmapWords : kBitmapWords) <= 227 * 1024, "bitmaps of the largest number of key clusters");
   const size_t smem = 1024 + C::OFF_BITMAP + (size_t)prm.bitmap_words * 4 * (MODE == kPairs ? 2 : 1);
   auto k = attn_tc_kernel<D, F8, MODE>;
   CA_RETURN_IF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
