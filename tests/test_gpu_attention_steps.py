@@ -7,6 +7,7 @@ import ctypes
 import pytest
 import torch
 
+from oracle import clusterattn_oracle as orc
 from paper_2608_26965_b200 import binding
 
 pytestmark = pytest.mark.gpu
@@ -242,3 +243,45 @@ def test_an_infinite_value_of_negligible_probability(heads, n_qc):
     torch.cuda.synchronize()
     assert plan.last_status()["attn"] == 0 and plan.recomputed_clusters() == heads * n_qc
     assert bool(torch.isposinf(O[..., 7]).all()) and int(torch.isinf(O).sum()) == heads * n_q
+
+
+@pytest.mark.parametrize("c_k,compensate", [(64, True), (64, False), (128, True), (256, True)])
+def test_quantised_pairs_of_64_row_query_clusters(c_k, compensate):
+    """Quantised Q K^T with two 64-row query clusters to a tile: the scales go with the rows of either cluster and with the
+    runs of 64 keys of shared, split and one-sided steps.  Rows, key clusters and centroids of very different size, and
+    ones that are zero."""
+    d, heads, n_qc, n_kc = 128, 9, 35, 45
+    n_q, n_k = 64 * n_qc - 17, c_k * n_kc - 5
+    Qp, Kp, Vp, _, cv, count, perm, lists = _clustering(heads, n_q, n_k, d, 64, c_k, c_k)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(c_k)
+    gain = lambda n: (2.0 * torch.rand((1, heads, n, 1), generator=g, device=DEV) - 1.0).exp()
+    Qp = (Qp * gain(64 * n_qc)).bfloat16()
+    Kp = (Kp * gain(n_kc).repeat_interleave(c_k, dim=2)).bfloat16()
+    Qp[:, :, 70] = 0
+    Kp[:, :, 4 * c_k:5 * c_k] = 0
+    ck = (Kp.float().reshape(1, heads, n_kc, c_k, d).sum(3) / count[..., None]).contiguous()
+    kind = torch.arange(heads * n_qc, device=DEV).reshape(1, heads, n_qc) // 2 % 4
+    odd = torch.arange(n_qc, device=DEV) % 2
+    keep = torch.tensor([9, 14, 5, 3], device=DEV)[kind] + odd * torch.tensor([0, 3, 0, 20], device=DEV)[kind]
+    even = lists[:, :, ::2].repeat_interleave(2, dim=2)[:, :, :n_qc]
+    idx = torch.where((kind == 2)[..., None], lists, even)                # the same lists, longer ones, unrelated ones
+    idx, keep = idx.int().contiguous(), keep.int().contiguous()
+    plan = binding.Plan(binding.make_problem(1, heads, n_q, n_k, d, "bf16", 64, c_k, 1, compensate, flags=binding.CA_ATTN_FP8_QK), DEV)
+    O, lse = plan.cluster_attention_fwd_ragged(idx, keep, Qp, Kp, Vp, ck, cv, count, perm)
+    torch.cuda.synchronize()
+    assert plan.last_status()["attn"] == 0 and plan.recomputed_clusters() == 0
+    pos, row = torch.arange(n_k, device=DEV), torch.arange(n_q, device=DEV)
+    for h in (0, 4, 8):
+        host = lambda t, n: t[0, h, :n].float().cpu().numpy()
+        Qd, Kd, cd = (torch.from_numpy(a).to(DEV) for a in orc.quantize_qk(host(Qp, n_q), host(Kp, n_k), range(n_k), c_k, host(ck, n_kc)))
+        kept = torch.zeros((n_qc, n_kc), dtype=torch.bool, device=DEV)
+        kept.scatter_(1, idx[0, h].long(), torch.arange(n_kc, device=DEV) < keep[0, h, :, None])
+        x = torch.cat([Qd @ Kd.T, Qd @ cd.T + count[0, h].double().log() * d ** 0.5], dim=1) / d ** 0.5
+        x = x.masked_fill(~torch.cat([kept[:, pos // c_k], ~kept & compensate], dim=1)[row // 64], -torch.inf)
+        want_lse = x.logsumexp(1)
+        want = (x - want_lse[:, None]).exp() @ torch.cat([Vp[0, h, :n_k], cv[0, h]]).double()
+        got, got_lse = O[0, h].double()[perm[0, h].long()], lse[0, h].double()[perm[0, h].long()]
+        # the codes and their products are the same on both sides; probabilities, value centroids and results are bf16
+        assert (got - want).norm() <= 1e-2 * want.norm() and (got - want).abs().max() <= 5e-2
+        assert (got_lse - want_lse).abs().max() <= 2e-3
