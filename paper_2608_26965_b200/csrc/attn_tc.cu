@@ -1211,11 +1211,14 @@ int launch_attn_tc(const ca_problem_t& pr, const void* Qp, const void* Kp, const
   CA_RETURN_IF_CUDA(cudaGetDevice(&dev));
   CA_RETURN_IF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   // A pair takes about 1.4 times the steps of one cluster (less the more their lists share), and tiles go in rounds of one per SM:
-  // pairs where their rounds are shorter by that, which they are not up to a cluster per SM, nor up to two where
-  // odd counts per head leave more than one tile per SM (54 heads of 5 clusters 183 us by ones, 239 by pairs); and by
-  // ones where the bitmaps of two lists do not fit.
+  // pairs where their rounds are shorter by that, which they are not up to a cluster per SM, nor up to two where odd counts per
+  // head leave more than one tile per SM (54 heads of 5 clusters, 32 of 256 clusters of 64, d = 64 42 us by ones, 55 in pairs); and by
+  // ones where the bitmaps of two lists do not fit.  At d = 64 three rounds against two are worth it from four steps on, since a
+  // pair's tile takes 2 us longer to start (9 heads of 35 clusters, us by ones / in pairs, lists of 2 clusters of 64 17.1 / 20.4,
+  // 6 of 64 21.6 / 22.9, 6 of 128 27.0 / 25.3; at d = 128 1 of 64 22.6 / 21.2, 6 of 128 41 / 34).
   const int rounds_of_pairs = ceil_div(P * ((n_qc + 1) / 2), sms), rounds_of_ones = ceil_div(P * n_qc, sms);
-  const bool pairs = pr.cluster_q < kTile && 7LL * rounds_of_pairs < 5LL * rounds_of_ones && bitmap_words <= kPairBitmapWords;
+  const bool long_lists = D == 128 || keep_count || (long long)pr.keep * pr.cluster_k >= 4 * kTile;    // (of lengths not known here: taken as long)
+  const bool pairs = pr.cluster_q < kTile && (long_lists ? 7LL : 8LL) * rounds_of_pairs < 5LL * rounds_of_ones && bitmap_words <= kPairBitmapWords;
   CUtensorMap maps[5];
   const int qbox = pr.cluster_q < kTile ? pr.cluster_q : kTile;
   const int kbox = min(pr.cluster_k, pairs ? kTile / 2 : kTile);  // pairs: keys in runs of 64

@@ -226,7 +226,7 @@ def test_pairs_of_64_row_query_clusters(d, c_k, infinite, compensate, heads):
     assert (lse - want_lse)[live].abs().max() <= 2e-3
 
 
-@pytest.mark.parametrize("heads,n_qc", [(9, 35), (2, 3)])                 # two clusters to a tile, and one
+@pytest.mark.parametrize("heads,n_qc", [(4, 73), (2, 3)])                 # two clusters to a tile, and one
 def test_an_infinite_value_of_negligible_probability(heads, n_qc):
     """A key 100 below the row's largest logit: exp(-100) is not zero in float32 but is where subnormal numbers are flushed,
     and 0 x inf is NaN.  64-row query clusters whose outputs are not numbers are recomputed, also where both lists of a
