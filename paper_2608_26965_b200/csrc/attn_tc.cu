@@ -40,7 +40,7 @@
 // loads its lists for itself, and takes 0.945 us: 10.2 TB/s over the SMs of the
 // 14.6 that plain bulk loads of L2-resident data reach (0.66 us),
 // with the tensor pipe 63 % and the exponentials 62 % busy; the rest are hand-offs, and launches in a row
-// run at the power limit (745 us alone, 857 behind one another).  At d = 64 the
+// run at the power limit (717 us alone, 809 behind one another).  At d = 64 the
 // exponentials (1,024 of 1,270 cycles per step) and the hand-offs.  Measured against the kernel before (two CTAs per SM at d = 128,
 // four at d = 64, half-steps of 64 keys in one chain per CTA): 40 heads of 32,760 rows,
 // d = 128, 32 of 256 clusters kept 2.91 -> 2.40 ms; 8 heads of 16,384 x 131,072, d = 64,
