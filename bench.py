@@ -44,8 +44,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # was captured from: sha256 of csrc/attn_tc.cu + csrc/tc_ptx.cuh, first 16 hex digits.  When the
 # source has changed since, the bench prints null instead of a stale figure.
 NCU_TRAFFIC = {
-    "tabular": {"bytes": 309.1e6, "source": "663f1b922b6cc8c8", "commit": "63d7a69"},
-    "video480": {"bytes": 1273.4e6, "source": "663f1b922b6cc8c8", "commit": "63d7a69"},
+    "tabular": {"bytes": 306.7e6, "source": "6b865b23704c7b2f", "commit": "52e955c"},
+    "video480": {"bytes": 1269.1e6, "source": "6b865b23704c7b2f", "commit": "52e955c"},
 }
 # FP32 FMA rate of the CUDA cores, the roof of kernels bound by plain arithmetic (centroid scoring,
 # the fp32 attention kernel): 148 SMs x 128 FMA lanes x 2 flops x 1.965 GHz (the maximum SM clock).
