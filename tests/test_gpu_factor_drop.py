@@ -30,7 +30,7 @@ def test_one_dominant_direction_leaves_one_column(d, dtype):
     """Keys along (1, 1, 1) and queries along (1, -1, 0) of three coordinates: both metrics are of rank one, and each maps
     the other side's rows to zero, exactly.  The second pivot is zero or what rounding leaves of the first (its sign
     depends on the head's numbers); a factor that keeps it makes unit vectors of the queries' representations, which are
-    normalised, and splits by them.  The three coordinates stand at all positions, those of the largest diagonal entry."""
+    normalised, and splits by them.  The three coordinates, those of the largest diagonal entries, stand all along the diagonal."""
     r = np.random.default_rng(7 + d)
     at = [(i, (i + 2) % d, (i + 4) % d) for i in range(0, d, 1 if d == 64 else 2)] + [(1, 3, 5)] * 24
     H, n_q, n_k = len(at), 130, 262
